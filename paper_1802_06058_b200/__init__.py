@@ -1,20 +1,22 @@
 """Variance-based gradient compression hot path on NVIDIA B200 -- Python binding.
 
-Thin ctypes marshalling over the C ABI declared in ``include/vgc.h`` (same entry-point names).
-Every step of the path runs in the CUDA library ``libvgc.so`` built from ``csrc/``; this module
-only checks tensors, passes pointers and sizes, and raises on a non-zero status.  PyTorch is
+Thin marshalling over the C ABI declared in ``include/vgc.h`` (same entry-point names).
+Every step of the path runs in the CUDA library ``libvgc.so`` built from ``csrc/``; the extension module
+``_vgc_native`` checks tensors and passes pointers and sizes, this module raises on a non-zero status
+(workspace sizes and other plain queries go through ctypes).  PyTorch is
 used for device memory and streams.  There is no CPU fallback: if the library is missing or
 was not built, every call raises.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional, Sequence
 
 import torch
 
-from ._build import LIB_PATH, build  # noqa: F401  (build is re-exported)
+from ._build import LIB_PATH, NATIVE_PATH, build  # noqa: F401  (build is re-exported)
 
 VGC_OK = 0
 VGC_DEV_CAPACITY = 1
@@ -135,6 +137,24 @@ def load_library():
     return lib
 
 
+_native = None
+
+
+def load_native():
+    """Load the extension module that marshals the calls (raises if it has not been built)."""
+    global _native
+    if _native is None:
+        load_library()
+        if not os.path.exists(NATIVE_PATH):
+            raise RuntimeError(f"{NATIVE_PATH} is missing: run paper_1802_06058_b200.build(); there is no fallback path")
+        spec = importlib.util.spec_from_file_location("_vgc_native", NATIVE_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        mod.use_classes(MessageBuffers, HybridMessageBuffers)
+        _native = mod
+    return _native
+
+
 def _status_string(status: int) -> str:
     try:
         return load_library().vgc_status_string(int(status)).decode()
@@ -145,30 +165,6 @@ def _status_string(status: int) -> str:
 def _check(status: int, where: str):
     if status != VGC_OK:
         raise VgcError(status, where)
-
-
-def _dev(t: torch.Tensor, dtype, name: str) -> int:
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
-        raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
-        raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
-    if not t.is_contiguous():
-        raise ValueError(f"{name} must be contiguous")
-    return t.data_ptr()
-
-
-def _stream(stream) -> int:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
-    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
-
-
-def _ws(ws: Optional[torch.Tensor]):
-    if ws is None:
-        return None, 0
-    if not ws.is_cuda or not ws.is_contiguous():
-        raise ValueError("workspace must be a contiguous CUDA tensor")
-    return ws.data_ptr(), ws.numel() * ws.element_size()
 
 
 def vgc_version() -> int:
@@ -186,15 +182,9 @@ def vgc_sqgrad_linear_workspace_bytes(B: int, n_in: int, n_out: int) -> int:
 
 def vgc_sqgrad_linear(x, delta, scale: float, S, accumulate: bool = False, ws=None, stream=None):
     """S[out,in] (+)= scale * sum_z delta[z,:]^2 (outer) x[z,:]^2 ; x [B,in], delta [B,out]."""
-    B, n_in = x.shape
-    B2, n_out = delta.shape
-    if B != B2 or S.numel() != n_in * n_out:
-        raise ValueError("shape mismatch")
-    wp, wb = _ws(ws)
-    st = load_library().vgc_sqgrad_linear(_dev(x, torch.float32, "x"), _dev(delta, torch.float32, "delta"),
-                                          B, n_in, n_out, float(scale), int(bool(accumulate)),
-                                          _dev(S, torch.float32, "S"), wp, wb, _stream(stream))
-    _check(st, "vgc_sqgrad_linear")
+    st = (_native or load_native()).sqgrad_linear(x, delta, scale, S, accumulate, ws, stream)
+    if st:
+        _check(st, "vgc_sqgrad_linear")
     return S
 
 
@@ -205,21 +195,9 @@ def vgc_sqgrad_conv_workspace_bytes(B, C, H, W, Cout, Kh, Kw, sh, sw, ph, pw) ->
 def vgc_sqgrad_conv(x, delta, kernel, stride, padding, scale: float, S, accumulate: bool = False,
                     ws=None, stream=None):
     """S[Cout,C,Kh,Kw] (+)= scale * sum over (example, output position) of squared contributions."""
-    B, C, H, W = x.shape
-    B2, Cout, Ho, Wo = delta.shape
-    Kh, Kw = kernel
-    sh, sw = stride
-    ph, pw = padding
-    if B != B2 or S.numel() != Cout * C * Kh * Kw:
-        raise ValueError("shape mismatch")
-    if Ho != (H + 2 * ph - Kh) // sh + 1 or Wo != (W + 2 * pw - Kw) // sw + 1:
-        raise ValueError("delta spatial shape does not match the convolution geometry")
-    wp, wb = _ws(ws)
-    st = load_library().vgc_sqgrad_conv(_dev(x, torch.float32, "x"), _dev(delta, torch.float32, "delta"),
-                                        B, C, H, W, Cout, Kh, Kw, sh, sw, ph, pw, float(scale),
-                                        int(bool(accumulate)), _dev(S, torch.float32, "S"), wp, wb,
-                                        _stream(stream))
-    _check(st, "vgc_sqgrad_conv")
+    st = (_native or load_native()).sqgrad_conv(x, delta, kernel, stride, padding, scale, S, accumulate, ws, stream, False)
+    if st:
+        _check(st, "vgc_sqgrad_conv")
     return S
 
 
@@ -230,21 +208,9 @@ def vgc_sqgrad_conv_exact_workspace_bytes(B, C, H, W, Cout, Kh, Kw, sh, sw, ph, 
 def vgc_sqgrad_conv_exact(x, delta, kernel, stride, padding, scale: float, S, accumulate: bool = False,
                           ws=None, stream=None):
     """S[Cout,C,Kh,Kw] (+)= scale * sum over examples of the squared per-example weight gradient."""
-    B, C, H, W = x.shape
-    B2, Cout, Ho, Wo = delta.shape
-    Kh, Kw = kernel
-    sh, sw = stride
-    ph, pw = padding
-    if B != B2 or S.numel() != Cout * C * Kh * Kw:
-        raise ValueError("shape mismatch")
-    if Ho != (H + 2 * ph - Kh) // sh + 1 or Wo != (W + 2 * pw - Kw) // sw + 1:
-        raise ValueError("delta spatial shape does not match the convolution geometry")
-    wp, wb = _ws(ws)
-    st = load_library().vgc_sqgrad_conv_exact(_dev(x, torch.float32, "x"), _dev(delta, torch.float32, "delta"),
-                                              B, C, H, W, Cout, Kh, Kw, sh, sw, ph, pw, float(scale),
-                                              int(bool(accumulate)), _dev(S, torch.float32, "S"), wp, wb,
-                                              _stream(stream))
-    _check(st, "vgc_sqgrad_conv_exact")
+    st = (_native or load_native()).sqgrad_conv(x, delta, kernel, stride, padding, scale, S, accumulate, ws, stream, True)
+    if st:
+        _check(st, "vgc_sqgrad_conv_exact")
     return S
 
 
@@ -270,31 +236,14 @@ def vgc_sqgrad_conv_batch(xs, deltas, kernel, stride, padding, scale: float, Ss,
                           ws=None, stream=None, exact: bool = False):
     """vgc_sqgrad_conv for several layers of one geometry (lists of tensors of equal shapes) in one call
     (``exact``: the per-example statistic, vgc_sqgrad_conv_exact_batch)."""
-    n = len(xs)
-    if len(deltas) != n or len(Ss) != n:
+    if len(deltas) != len(xs) or len(Ss) != len(xs):
         raise ValueError("xs, deltas, Ss must have the same length")
-    if n == 0:
+    if not len(xs):
         return Ss
-    B, C, H, W = xs[0].shape
-    B2, Cout, Ho, Wo = deltas[0].shape
-    Kh, Kw = kernel
-    sh, sw = stride
-    ph, pw = padding
-    if B != B2 or Ho != (H + 2 * ph - Kh) // sh + 1 or Wo != (W + 2 * pw - Kw) // sw + 1:
-        raise ValueError("delta shape does not match the convolution geometry")
-    for x, d, S in zip(xs, deltas, Ss):
-        if tuple(x.shape) != (B, C, H, W) or tuple(d.shape) != (B, Cout, Ho, Wo) or S.numel() != Cout * C * Kh * Kw:
-            raise ValueError("all layers of a batch must have the same shapes")
-    ptrs = ctypes.c_void_p * n
-    xp = ptrs(*[_dev(x, torch.float32, "x") for x in xs])
-    dp = ptrs(*[_dev(d, torch.float32, "delta") for d in deltas])
-    sp = ptrs(*[_dev(S, torch.float32, "S") for S in Ss])
-    wp, wb = _ws(ws)
-    lib = load_library()
-    fn = lib.vgc_sqgrad_conv_exact_batch if exact else lib.vgc_sqgrad_conv_batch
-    st = fn(n, xp, dp, sp, B, C, H, W, Cout, Kh, Kw, sh, sw, ph, pw, float(scale), int(bool(accumulate)), wp, wb,
-            _stream(stream))
-    _check(st, "vgc_sqgrad_conv_exact_batch" if exact else "vgc_sqgrad_conv_batch")
+    st = (_native or load_native()).sqgrad_conv_batch(xs, deltas, kernel, stride, padding, scale, Ss, accumulate, ws, stream,
+                                                      exact)
+    if st:
+        _check(st, "vgc_sqgrad_conv_exact_batch" if exact else "vgc_sqgrad_conv_batch")
     return Ss
 
 
@@ -338,21 +287,9 @@ def vgc_compress_workspace_bytes(n: int, K: int) -> int:
 def vgc_compress(g, s, r, v, group_offsets, alpha: float, zeta: float, out: MessageBuffers, ws, stream=None):
     """One step of Algorithm 1 over the flat buffer + Encode(); r, v updated in place.
     ``s=None``: v already contains this step's squared-gradient sums (sqgrad with accumulate into v)."""
-    n = g.numel()
-    if (s is not None and s.numel() != n) or r.numel() != n or v.numel() != n:
-        raise ValueError("g, s, r, v must have the same length")
-    K = group_offsets.numel() - 1
-    if out.K != K:
-        raise ValueError("message buffers were made for a different number of groups")
-    if out.mask is not None and out.mask.numel() != n:
-        raise ValueError("mask length")
-    wp, wb = _ws(ws)
-    msg = out.struct()
-    st = load_library().vgc_compress(_dev(g, torch.float32, "g"), None if s is None else _dev(s, torch.float32, "s"),
-                                     _dev(r, torch.float32, "r"), _dev(v, torch.float32, "v"), n,
-                                     _dev(group_offsets, torch.int32, "group_offsets"), K, float(alpha),
-                                     float(zeta), ctypes.byref(msg), wp, wb, _stream(stream))
-    _check(st, "vgc_compress")
+    st = (_native or load_native()).compress(g, s, r, v, group_offsets, alpha, zeta, out, ws, stream)
+    if st:
+        _check(st, "vgc_compress")
     return out
 
 
@@ -366,18 +303,9 @@ def vgc_compress_static(g, s, r, v, group_offsets, alpha: float, zeta: float, ou
     array inside the library, so n is limited to VGC_COMPRESS_STATIC_MAX_PARAMS.  Nothing is allocated by
     this call -- the binding passes pointers only.  Calls on one device share the scratch: do not let
     two of them overlap on the GPU.  Make the first call on a device outside any stream capture."""
-    n = g.numel()
-    if s.numel() != n or r.numel() != n or v.numel() != n:
-        raise ValueError("g, s, r, v must have the same length")
-    K = group_offsets.numel() - 1
-    if out.K != K:
-        raise ValueError("message buffers were made for a different number of groups")
-    msg = out.struct()
-    st = load_library().vgc_compress_static(_dev(g, torch.float32, "g"), _dev(s, torch.float32, "s"),
-                                            _dev(r, torch.float32, "r"), _dev(v, torch.float32, "v"), n,
-                                            _dev(group_offsets, torch.int32, "group_offsets"), K, float(alpha),
-                                            float(zeta), ctypes.byref(msg), _stream(stream))
-    _check(st, "vgc_compress_static")
+    st = (_native or load_native()).compress_static(g, s, r, v, group_offsets, alpha, zeta, out, stream)
+    if st:
+        _check(st, "vgc_compress_static")
     return out
 
 
@@ -390,21 +318,9 @@ def vgc_decode_accumulate(messages: Sequence, group_offsets, scale: float, u, de
     decoder reads at most as many words as the words tensor holds.
     ``dev_status``: int32[1] device tensor (zeroed by the caller) receiving VGC_DEV_* bits.
     ``overwrite``: write u = scale * sum instead (vgc_decode_sum): u is neither read nor needs clearing."""
-    W = len(messages)
-    views = (_ViewStruct * max(W, 1))()
-    for w, m in enumerate(messages):
-        if isinstance(m, MessageBuffers):
-            views[w] = m.view()
-        else:
-            words, nnz, gexp = m
-            views[w] = _ViewStruct(_dev(words, torch.int32, "words"), _dev(nnz, torch.int32, "nnz"),
-                                   _dev(gexp, torch.int32, "group_exp"), words.numel())
-    K = group_offsets.numel() - 1
-    lib = load_library()
-    fn = lib.vgc_decode_sum if overwrite else lib.vgc_decode_accumulate
-    st = fn(views, W, _dev(group_offsets, torch.int32, "group_offsets"), K, float(scale), _dev(u, torch.float32, "u"),
-            u.numel(), _dev(dev_status, torch.int32, "dev_status"), _stream(stream))
-    _check(st, "vgc_decode_sum" if overwrite else "vgc_decode_accumulate")
+    st = (_native or load_native()).decode(messages, group_offsets, scale, u, dev_status, stream, overwrite)
+    if st:
+        _check(st, "vgc_decode_sum" if overwrite else "vgc_decode_accumulate")
     return u
 
 
@@ -444,18 +360,9 @@ def vgc_compress_hybrid_workspace_bytes(n: int) -> int:
 def vgc_compress_hybrid(g, s, r, v, alpha: float, zeta: float, tau: float, out: HybridMessageBuffers, ws,
                         correction_from_updated_r: bool = False, stream=None):
     """One step of Algorithm 2 over the flat buffer; r, v updated in place.  ``s=None`` as for vgc_compress."""
-    n = g.numel()
-    if (s is not None and s.numel() != n) or r.numel() != n or v.numel() != n:
-        raise ValueError("g, s, r, v must have the same length")
-    if out.mask is not None and out.mask.numel() != n:
-        raise ValueError("mask length")
-    wp, wb = _ws(ws)
-    msg = out.struct()
-    st = load_library().vgc_compress_hybrid(
-        _dev(g, torch.float32, "g"), None if s is None else _dev(s, torch.float32, "s"), _dev(r, torch.float32, "r"),
-        _dev(v, torch.float32, "v"), n, float(alpha), float(zeta), float(tau), int(bool(correction_from_updated_r)),
-        ctypes.byref(msg), wp, wb, _stream(stream))
-    _check(st, "vgc_compress_hybrid")
+    st = (_native or load_native()).compress_hybrid(g, s, r, v, alpha, zeta, tau, correction_from_updated_r, out, ws, stream)
+    if st:
+        _check(st, "vgc_compress_hybrid")
     return out
 
 
@@ -467,19 +374,9 @@ def vgc_decode_sum_hybrid(messages: Sequence, tau: float, scale: float, u, dev_s
 def vgc_decode_accumulate_hybrid(messages: Sequence, tau: float, scale: float, u, dev_status, stream=None,
                                  overwrite: bool = False):
     """u[idx] += scale * (+-tau) over all words of all messages (HybridMessageBuffers or (words, nnz) pairs)."""
-    W = len(messages)
-    views = (_ViewStruct * max(W, 1))()
-    for w, m in enumerate(messages):
-        if isinstance(m, HybridMessageBuffers):
-            views[w] = m.view()
-        else:
-            words, nnz = m
-            views[w] = _ViewStruct(_dev(words, torch.int32, "words"), _dev(nnz, torch.int32, "nnz"), None, words.numel())
-    lib = load_library()
-    fn = lib.vgc_decode_sum_hybrid if overwrite else lib.vgc_decode_accumulate_hybrid
-    st = fn(views, W, float(tau), float(scale), _dev(u, torch.float32, "u"), u.numel(),
-            _dev(dev_status, torch.int32, "dev_status"), _stream(stream))
-    _check(st, "vgc_decode_accumulate_hybrid")
+    st = (_native or load_native()).decode_hybrid(messages, tau, scale, u, dev_status, stream, overwrite)
+    if st:
+        _check(st, "vgc_decode_accumulate_hybrid")
     return u
 
 
@@ -495,28 +392,18 @@ def vgc_pack_workspace_bytes(max_words: int) -> int:
 def vgc_pack_indices(words, nnz, packed, packed_bytes, dev_status, ws, stream=None):
     """words int32 [max_words] + nnz int32 [1] (device) -> packed uint8 (device): the index field as differences in
     the base-128 code; packed_bytes int32 [1] (device) receives the stream's length."""
-    wp, wb = _ws(ws)
-    st = load_library().vgc_pack_indices(_dev(words, torch.int32, "words"), _dev(nnz, torch.int32, "nnz"), words.numel(),
-                                         _dev(packed, torch.uint8, "packed"), packed.numel(),
-                                         _dev(packed_bytes, torch.int32, "packed_bytes"),
-                                         _dev(dev_status, torch.int32, "dev_status"), wp, wb, _stream(stream))
-    _check(st, "vgc_pack_indices")
+    st = (_native or load_native()).pack_indices(words, nnz, packed, packed_bytes, dev_status, ws, stream)
+    if st:
+        _check(st, "vgc_pack_indices")
     return packed
 
 
 def vgc_unpack_indices(packed, nnz, words, dev_status, stream=None):
     """The inverse of vgc_pack_indices: rebuilds min(nnz, words.numel()) words (device int32)."""
-    st = load_library().vgc_unpack_indices(_dev(packed, torch.uint8, "packed"), _dev(nnz, torch.int32, "nnz"), words.numel(),
-                                           _dev(words, torch.int32, "words"), _dev(dev_status, torch.int32, "dev_status"),
-                                           _stream(stream))
-    _check(st, "vgc_unpack_indices")
+    st = (_native or load_native()).unpack_indices(packed, nnz, words, dev_status, stream)
+    if st:
+        _check(st, "vgc_unpack_indices")
     return words
-
-
-def _host(t: torch.Tensor, dtype, name: str) -> int:
-    if not isinstance(t, torch.Tensor) or t.is_cuda or t.dtype != dtype or not t.is_contiguous():
-        raise TypeError(f"{name} must be a contiguous CPU tensor of {dtype}")
-    return t.data_ptr()
 
 
 def vgc_step_host(layers, g_host, g_dev, s_dev, r, v, group_offsets, alpha, zeta, scale, out: MessageBuffers,
@@ -524,26 +411,10 @@ def vgc_step_host(layers, g_host, g_dev, s_dev, r, v, group_offsets, alpha, zeta
     """One worker step from host buffers.  ``layers``: list of dicts with keys is_conv, B, C, H, W, Cout,
     Kh, Kw, stride, pad, x_host, delta_host (CPU, ideally pinned) and x_dev, delta_dev (CUDA staging).
     Returns (nnz, n_criterion, n_dropped, dev_status) as read back into ``counters_host``."""
-    arr = (_LayerHostStruct * max(len(layers), 1))()
-    for k, L in enumerate(layers):
-        arr[k] = _LayerHostStruct(int(L["is_conv"]), L["B"], L["C"], L.get("H", 1), L.get("W", 1), L["Cout"],
-                                  L.get("Kh", 1), L.get("Kw", 1), L.get("stride", 1), L.get("stride", 1),
-                                  L.get("pad", 0), L.get("pad", 0),
-                                  _host(L["x_host"], torch.float32, "x_host"), _host(L["delta_host"], torch.float32, "delta_host"),
-                                  _dev(L["x_dev"], torch.float32, "x_dev"), _dev(L["delta_dev"], torch.float32, "delta_dev"))
-    n = g_dev.numel()
-    K = group_offsets.numel() - 1
-    wsp, wsb = _ws(ws_sqgrad)
-    wcp, wcb = _ws(ws_compress)
-    msg = out.struct()
-    st = load_library().vgc_step_host(arr, len(layers), _host(g_host, torch.float32, "g_host"),
-                                      _dev(g_dev, torch.float32, "g_dev"), _dev(s_dev, torch.float32, "s_dev"),
-                                      _dev(r, torch.float32, "r"), _dev(v, torch.float32, "v"), n,
-                                      _dev(group_offsets, torch.int32, "group_offsets"), K, float(alpha), float(zeta),
-                                      float(scale), ctypes.byref(msg), _host(words_host, torch.int32, "words_host"),
-                                      _host(counters_host, torch.int32, "counters_host"), wsp, wsb, wcp, wcb,
-                                      _stream(stream))
-    _check(st, "vgc_step_host")
+    st = (_native or load_native()).step_host(layers, g_host, g_dev, s_dev, r, v, group_offsets, alpha, zeta, scale, out,
+                                              words_host, counters_host, ws_sqgrad, ws_compress, stream)
+    if st:
+        _check(st, "vgc_step_host")
     return tuple(int(c) & 0xFFFFFFFF for c in counters_host.tolist())
 
 

@@ -1,4 +1,4 @@
-"""Builds the CUDA library in-tree with nvcc for sm_100a (no JIT cache, no torch extension).
+"""Builds the CUDA library in-tree with nvcc for sm_100a and the Python binding with g++ (no JIT cache).
 
 Every csrc/*.cu is compiled to an object file of its own (in parallel; an object is rebuilt only when its
 source, a shared header or the flags changed) and the objects are linked into libvgc.so next to this file."""
@@ -7,13 +7,17 @@ from __future__ import annotations
 import concurrent.futures
 import glob
 import hashlib
+import importlib.util
 import os
 import subprocess
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 INCLUDE = os.path.join(os.path.dirname(PKG_DIR), "include")
 LIB_PATH = os.path.join(PKG_DIR, "libvgc.so")
+NATIVE_SRC = os.path.join(CSRC, "vgc_binding.cpp")
+NATIVE_PATH = os.path.join(PKG_DIR, "_vgc_native.so")
 OBJ_DIR = os.path.join(PKG_DIR, "build")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -57,9 +61,26 @@ def _compile(nvcc: str, src: str, verbose: bool) -> str:
     return obj
 
 
+def _build_native(force: bool) -> None:
+    """The extension module that marshals the Python calls: compiled against torch's headers, linked to libvgc.so."""
+    if not force and os.path.exists(NATIVE_PATH) and os.path.getmtime(NATIVE_PATH) >= _newest([NATIVE_SRC] + _headers()):
+        return
+    torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
+    torch_inc, torch_lib = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = NATIVE_PATH + ".tmp.%d" % os.getpid()
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+                    "-I", INCLUDE, "-isystem", torch_inc, "-isystem", os.path.join(torch_inc, "torch", "csrc", "api", "include"),
+                    "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), NATIVE_SRC, "-o", tmp,
+                    "-L", torch_lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-L", PKG_DIR, "-lvgc",
+                    "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + torch_lib], check=True)
+    os.replace(tmp, NATIVE_PATH)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile csrc/*.cu into libvgc.so next to this file; returns its path."""
+    """Compile csrc/*.cu into libvgc.so next to this file and the binding beside it; returns the library's path."""
     if not force and not _stale():
+        _build_native(False)
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "nvcc")
     os.makedirs(OBJ_DIR, exist_ok=True)
@@ -72,6 +93,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB_PATH + ".tmp.%d" % os.getpid()
     subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp, *objs], check=True)
     os.replace(tmp, LIB_PATH)
+    _build_native(force)
     return LIB_PATH
 
 
