@@ -44,6 +44,45 @@ inline void report_cuda_error(cudaError_t e, const char *what, const char *file,
 extern unsigned long long g_launches;
 inline void count_launch(unsigned k = 1) { g_launches += k; }
 
+// How many blocks of a kernel the current device holds at a time -- what a cooperative launch may use.  Looked up once
+// per device (a race between two threads looks it up twice); 0 on an error.
+struct ResidentBlocks {
+    static constexpr int kMaxDevices = 64;
+    uint32_t blocks[kMaxDevices];
+    uint32_t get(const void *fn, int threads, size_t smem)
+    {
+        int dev = -1, per_sm = 0, sms = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+        if (dev < kMaxDevices && blocks[dev]) return blocks[dev];
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return 0;
+        const uint32_t all = (uint32_t)(per_sm * sms);
+        if (dev < kMaxDevices) blocks[dev] = all;
+        return all;
+    }
+};
+
+// A buffer of n parameters cut into one contiguous range per block: whole tiles while there are fewer of them than
+// blocks to hold them; beyond that every block takes the same share (a multiple of 128 parameters: 512 B of every
+// stream), cut into tiles of equal size.
+struct Ranges {
+    uint32_t grid, per_block, tile;
+};
+inline Ranges even_ranges(size_t n, uint32_t most_blocks, uint32_t tile_max)
+{
+    Ranges R;
+    const size_t tiles = (n + tile_max - 1) / tile_max;
+    const size_t blocks = tiles < most_blocks ? tiles : most_blocks;
+    const size_t per = round_up((n + blocks - 1) / blocks, 128);
+    const size_t tiles_per = (per + tile_max - 1) / tile_max;
+    R.per_block = (uint32_t)per;
+    R.grid = (uint32_t)((n + per - 1) / per);
+    R.tile = (uint32_t)round_up((per + tiles_per - 1) / tiles_per, 128);
+    return R;
+}
+
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
 
 __device__ __forceinline__ uint64_t ld_volatile_u64(const uint64_t *p)
