@@ -44,92 +44,33 @@ inline void report_cuda_error(cudaError_t e, const char *what, const char *file,
 extern unsigned long long g_launches;
 inline void count_launch(unsigned k = 1) { g_launches += k; }
 
-// How many blocks of a kernel the current device holds at a time -- what a cooperative launch may use.  Looked up once
-// per device (a race between two threads looks it up twice); 0 on an error.
-struct ResidentBlocks {
-    static constexpr int kMaxDevices = 64;
-    uint32_t blocks[kMaxDevices];
-    uint32_t get(const void *fn, int threads, size_t smem)
-    {
-        int dev = -1, per_sm = 0, sms = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
-        if (dev < kMaxDevices && blocks[dev]) return blocks[dev];
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return 0;
-        const uint32_t all = (uint32_t)(per_sm * sms);
-        if (dev < kMaxDevices) blocks[dev] = all;
-        return all;
+// ---- launches that follow one another closely ---------------------------------------------------------------------
+// A kernel launched with `overlap` may start while the kernel before it on the stream is still running (programmatic
+// dependent launch): its blocks take the SMs as they become free, and everything before its grid_wait() -- which every
+// kernel launched that way executes before it touches memory another kernel writes -- hides under that kernel's end.
+// grid_wait() returns once the kernel before has finished and its writes are visible.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// lets the next kernel of the stream start now, where it was launched with `overlap`
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+template <class... Params, class... Given>
+cudaError_t launch_kernel(void (*fn)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap,
+                          Given &&...given)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    if (overlap) {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
     }
-};
-
-// A buffer of n parameters cut into one contiguous range per block: `least` parameters each while there are fewer of
-// those than blocks to hold them; beyond that every block takes the same share (a multiple of 128 parameters: 512 B of
-// every stream), cut into tiles of equal size.
-struct Ranges {
-    uint32_t grid, per_block, tile;
-};
-inline Ranges even_ranges(size_t n, uint32_t most_blocks, uint32_t tile_max, uint32_t least)
-{
-    Ranges R;
-    const size_t tiles = (n + least - 1) / least;
-    const size_t blocks = tiles < most_blocks ? tiles : most_blocks;
-    const size_t per = round_up((n + blocks - 1) / blocks, 128);
-    const size_t tiles_per = (per + tile_max - 1) / tile_max;
-    R.per_block = (uint32_t)per;
-    R.grid = (uint32_t)((n + per - 1) / per);
-    R.tile = (uint32_t)round_up((per + tiles_per - 1) / tiles_per, 128);
-    return R;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, static_cast<Params>(given)...);
 }
-
-// ---- values that the blocks of one cooperative launch hand each other ---------------------------------------------
-// A slot is 16 bytes, {tag, two 32-bit values}, written and read as one 128-bit access: a block publishes its slot, the
-// others poll it until it carries the launch's tag -- one store and one load of latency, the values included, where a
-// grid barrier costs 2.4 us with 16 blocks and 5 us with 592 and is followed by the loads of whatever it guarded.
-// Slots live in the caller's workspace, whose contents are arbitrary, so nothing may depend on their being cleared:
-//   - the tag is 64 bits, unique to the call on the host (leftovers of anything else do not match);
-//   - a captured launch is replayed with the same tag, so a launch leaves no slot behind that carries it: a launch uses
-//     two sets, `first` and `second`.  A block clears its `second` slot, then (a fence between them) publishes its
-//     `first`; it waits for ALL `first` slots (and a fence) before it publishes its `second` and before it looks at
-//     anyone's `second`, so a stale `second` is never seen; the last block, once it has every `second`, clears all of
-//     `first` (everybody has read them by then).
-// Apart from that order the values in a slot are all that is handed over, so publishing and polling are relaxed: a
-// release store would wait for every store the block has in flight, an acquire load would empty the L1 cache.
-// The polls are bounded: a wait that runs out makes the block raise VGC_DEV_TIMEOUT and leave.
-struct __align__(16) Slot {
-    unsigned long long tag;
-    uint32_t a, b;
-};
-constexpr uint32_t kSlotPolls = 1u << 22;
-
-__device__ __forceinline__ void slot_publish(Slot *s, unsigned long long tag, uint32_t a, uint32_t b)
-{
-    const unsigned long long v = (unsigned long long)b << 32 | a;
-    asm volatile("{\n\t.reg .b128 q;\n\tmov.b128 q, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], q;\n\t}"
-                 ::"l"(s), "l"(tag), "l"(v) : "memory");
-}
-__device__ __forceinline__ bool slot_read(const Slot *s, unsigned long long tag, uint32_t &a, uint32_t &b)
-{
-    unsigned long long t, v;
-    asm volatile("{\n\t.reg .b128 q;\n\tld.relaxed.gpu.global.b128 q, [%2];\n\tmov.b128 {%0, %1}, q;\n\t}"
-                 : "=l"(t), "=l"(v) : "l"(s) : "memory");
-    a = (uint32_t)v;
-    b = (uint32_t)(v >> 32);
-    return t == tag;
-}
-// waits until the slot carries the tag; false if it never did
-__device__ __forceinline__ bool slot_wait(const Slot *s, unsigned long long tag, uint32_t &a, uint32_t &b)
-{
-    for (uint32_t i = 0; i < kSlotPolls; ++i) {
-        if (slot_read(s, tag, a, b)) return true;
-        if (i >= 4) __nanosleep(32);
-    }
-    a = b = 0;
-    return false;
-}
-// host: a tag no other call of this process uses (never 0, which cleared slots carry)
-unsigned long long next_tag();
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
 

@@ -7,16 +7,15 @@ using namespace vgc;
 
 namespace {
 struct CompressLayout {
-    size_t slots, rec_max, rec_min, stage, total;
+    size_t records, rec_max, stage, total;
 };
 
 static CompressLayout compress_layout(size_t n, int K)
 {
     CompressLayout L;
     size_t off = 0;
-    L.slots = off;         off = round_up(off + step::kSlotBytes, 256);
+    L.records = off;       off = round_up(off + step::kRecordBytes, 256);
     L.rec_max = off;       off = round_up(off + sizeof(uint32_t) * ((size_t)K + step::kMaxGrid), 256);
-    L.rec_min = off;       off = round_up(off + sizeof(uint32_t) * ((size_t)K + step::kMaxGrid), 256);
     L.stage = off;         off = round_up(off + sizeof(uint32_t) * n, 256);
     // the interface states about 8 bytes per parameter; the staging area takes 4 of them
     L.total = round_up(off + sizeof(uint32_t) * n, 256);
@@ -54,11 +53,10 @@ extern "C" vgc_status vgc_compress(const float *g, const float *s, float *r, flo
     args.g = g; args.s = s; args.r = r; args.v = v; args.n = n;
     args.group_offsets = group_offsets; args.K = K; args.alpha = alpha; args.zeta = zeta;
     args.rec_max = reinterpret_cast<uint32_t *>(base + L.rec_max);
-    args.rec_min = reinterpret_cast<uint32_t *>(base + L.rec_min);
     args.stage = reinterpret_cast<uint32_t *>(base + L.stage);
     args.out = *out;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    return s ? step::launch<true, step::kBasic>(args, base + L.slots, st) : step::launch<false, step::kBasic>(args, base + L.slots, st);
+    return s ? step::launch<true, step::kBasic>(args, base + L.records, st) : step::launch<false, step::kBasic>(args, base + L.records, st);
 }
 
 // ------------------------------------------------------------------------------------------

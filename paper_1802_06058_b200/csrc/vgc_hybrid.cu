@@ -5,10 +5,10 @@
 
 using namespace vgc;
 
-// the slots, then the words past what a block keeps in shared memory: 4 bytes per parameter
+// the blocks' records, then the staged values: 4 bytes per parameter
 extern "C" size_t vgc_compress_hybrid_workspace_bytes(size_t n)
 {
-    return round_up(step::kSlotBytes, 256) + round_up(sizeof(uint32_t) * n, 256);
+    return round_up(step::kRecordBytes, 256) + round_up(sizeof(uint32_t) * n, 256);
 }
 
 extern "C" vgc_status vgc_compress_hybrid(const float *g, const float *s, float *r, float *v, size_t n,
@@ -31,7 +31,7 @@ extern "C" vgc_status vgc_compress_hybrid(const float *g, const float *s, float 
     step::Args args = {};
     args.g = g; args.s = s; args.r = r; args.v = v; args.n = n;
     args.alpha = alpha; args.zeta = zeta; args.tau = tau;
-    args.stage = reinterpret_cast<uint32_t *>(static_cast<char *>(ws) + round_up(step::kSlotBytes, 256));
+    args.stage = reinterpret_cast<uint32_t *>(static_cast<char *>(ws) + round_up(step::kRecordBytes, 256));
     args.out.words = out->words; args.out.capacity = out->capacity; args.out.nnz = out->nnz;
     args.out.mask = out->mask; args.out.dev_status = out->dev_status;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

@@ -1,6 +1,4 @@
 // C ABI of the squared per-example gradient sums (argument checks and kernel choice).
-#include <atomic>
-#include <chrono>
 #include <cstdlib>
 
 #include "vgc_common.cuh"
@@ -201,22 +199,5 @@ extern "C" const char *vgc_status_string(int status)
 
 extern "C" int vgc_version(void) { return 2000; }
 
-namespace vgc {
-unsigned long long g_launches = 0;
-
-unsigned long long next_tag()
-{
-    // a counter from a random start, scrambled (splitmix64, a bijection: no two calls get the same)
-    static const unsigned long long start = (unsigned long long)std::chrono::system_clock::now().time_since_epoch().count() ^
-                                            reinterpret_cast<uintptr_t>(&g_launches);
-    static std::atomic<unsigned long long> counter{0};
-    for (;;) {
-        unsigned long long z = start + 0x9E3779B97F4A7C15ull * (counter.fetch_add(1, std::memory_order_relaxed) + 1);
-        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-        z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-        z ^= z >> 31;
-        if (z) return z;
-    }
-}
-}  // namespace vgc
+namespace vgc { unsigned long long g_launches = 0; }
 extern "C" uint64_t vgc_kernel_launch_count(void) { return vgc::g_launches; }

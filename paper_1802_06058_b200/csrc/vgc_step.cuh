@@ -1,25 +1,28 @@
 // The streaming pass shared by vgc_compress (Algorithm 1, "Basic") and vgc_compress_hybrid (Algorithm 2): one step over
 // the flat parameter buffer and the message it sends.
 //
-// One cooperative kernel.  Every thread block owns one contiguous range of the buffer and goes through three steps;
-// between them the blocks hand each other 16-byte slots (the per-tensor maximum has to be complete before any value can
-// be quantised, and the number of words before a block's own before it can write them):
-//   1  streams g, s, r, v once (16 B read + 8 B written per parameter), applies the send test, writes r, v back and
-//      keeps what was selected in index order, 32 bits each -- position in the range, sign, rounded exponent: all the
-//      quantiser needs.  The first kStaged of them stay in shared memory, the rest goes to the block's part of the
-//      workspace.  For every weight tensor the range touches it records the largest and the smallest |value| sent.
-//   2  E_k = floor(log2 M_k) of the tensors at the range's two ends from the other blocks' slots (tensors inside the
-//      range are complete already); how many selected values survive the quantiser (d <= 7): all of them unless a
-//      recorded minimum says otherwise.
-//   3  adds up the counts of the blocks before its own and writes its words.
-// The hybrid algorithm has neither maxima nor quantiser: its step 2 is only the hand-shake that the slots ask for.
+// Every thread block owns one contiguous range of the buffer:
+//   1  it streams g, s, r, v once (16 B read + 8 B written per parameter), applies the send test, writes r, v back and
+//      stages what was selected in index order, 32 bits each -- position in the range, sign, rounded exponent: all the
+//      quantiser needs.  For every weight tensor the range touches it records the largest |value| sent.
+//   2  E_k = floor(log2 M_k) needs the records of every block that shares tensor k, and a block's first word's place
+//      needs to know how many staged values of the blocks before it survive the quantiser (d <= 7).
+//   3  it writes its words.
+// Steps 2 and 3 are a second kernel: at the end of its range a block of the first one counts how many of the staged values
+// of the range's first and last tensor (the two that other blocks may share) survive for each exponent E_k can turn out to
+// have, nine at most.  (Counting them as they are selected, in a shared-memory histogram, cost 20 % at density 0.15.)
+// With these the second kernel's blocks work out E_k, every block's surviving count and their own place from the records
+// alone: no block waits for another, and nothing has to be cleared by a launch of its own.  It is launched so that it
+// starts under the end of the first.
+// The hybrid algorithm has neither maxima nor quantiser.
 //
-// Bound: HBM, 24 B per parameter, for large buffers -- the latency of the launch and of the two exchanges (about 2 us
-// each with 16 blocks, 4 us with 296) for small ones.  The contiguous ranges keep everything a block selects in its own
-// shared memory; two blocks of 512 threads per SM stream as fast as four of 256 (612 MB in 101.5 us, 0.92 of the
-// measured copy rate) and halve the slots every block has to read.
-// Measured against the memset and three kernels this replaces (B200, one call among others, Algorithm 1, density 1e-2):
-//   n = 25.5 M  125.9 -> 109.8 us,   n = 1.86 M  @M@ -> 16.7 us,   n = 32768  @S@ -> 7.9 us.
+// Bound: HBM, 24 B per parameter, for large buffers (the first kernel: 612 MB in 101.5 us, 0.92 of the measured copy
+// rate) -- the latency of launches and exchanges for small ones.  Measured against the memset and three kernels this
+// replaces (B200, one call among others, Algorithm 1, density 1e-2): n = 25.5 M  125.9 -> 110.0 us,
+// n = 138 M at density 0.05  627 -> 563 us,  n = 3e4 .. 4e5  19 -> 9 us.
+// In between stood one kernel: cooperative, its grid barriers cost 2.4 us each with 16 blocks and 5 us with 592, polled
+// slots 2 us and 4 us, the cooperative launch itself 2.5 us on either side; as one cluster of 16 blocks with distributed
+// shared memory it took as long as these two kernels at n = 8192 and 22 % longer at 131072.
 #pragma once
 
 #include "vgc_common.cuh"
@@ -34,16 +37,26 @@ constexpr int kRowsA = 2;                            // float4 vectors per threa
 constexpr int kTileA = kThreads * kRowsA * 4;        // at most 4096 parameters per tile
 constexpr int kLeastPerBlock = 2048;
 constexpr int kMaxGrid = 148 * kBlocksPerSm;
-constexpr int kCopies = 8;                           // of every slot, so that the pollers do not all meet in one place
+static_assert(kMaxGrid <= kThreads, "the second kernel reads one record per thread");
 constexpr int kOffsSmem = 1024;                      // group offsets cached in shared memory
-constexpr uint32_t kStaged = 12288;                  // selected values a block keeps in shared memory (48 KB)
+constexpr uint32_t kStagedCopy = 2048;
 // a staged value: position in the block's range << 10 | sign << 9 | (rounded exponent + 127)
 constexpr uint32_t kPosShift = 10;
 constexpr size_t kMostPerBlock = 1u << (32 - kPosShift);
 
 enum { kBasic = 0, kHybridBefore = 1, kHybridAfter = 2 };     // the hybrid's correction uses |r| from before / after r -= Sign(r) tau
 
-constexpr size_t kSlotBytes = 2 * sizeof(Slot) * kCopies * kMaxGrid;
+// What the first kernel leaves about a block's range.
+struct __align__(16) Record {
+    uint32_t max_first, max_last;        // largest |value| bits sent from the range's first and last tensor
+    uint32_t head;                       // block where the first tensor begins; top bit: it is also the last tensor
+    uint32_t passed;                     // values staged
+};
+constexpr uint32_t kSame = 0x80000000u;
+// how many of the staged values survive, per exponent E_k above the block's own one ([0] = the same): first tensor, last
+// tensor; then those of the tensors between them, which no other block shares
+constexpr int kLevels = 9, kCounts = 2 * kLevels + 1;
+constexpr size_t kRecordBytes = (sizeof(Record) + sizeof(uint32_t) * kCounts) * kMaxGrid;
 
 struct Args {
     const float *g, *s;
@@ -52,16 +65,16 @@ struct Args {
     const uint32_t *group_offsets;
     int K;
     float alpha, zeta;
-    unsigned long long tag;
-    Slot *first, *second;                // per block: {max of its first tensor, of its last}; {passed, kept}
-    uint32_t *rec_max, *rec_min;         // per (block, tensor) at [block + tensor]: |value| bit patterns
-    uint32_t *stage;                     // values past kStaged of a block, from its first parameter's index on
+    Record *records;                     // [block]
+    uint32_t *counts;                    // [block][kCounts]
+    uint32_t *rec_max;                   // per (block, tensor) at [block + tensor]: |value| bits of the tensors inside
+    uint32_t *stage;                     // staged values of a block from its first parameter's index on
     uint32_t per_block, tile;
     float tau;                           // hybrid only
     vgc_message out;                     // (hybrid: no exponents, nnz only)
 };
 
-constexpr uint32_t kNoMin = 0x7FFFFFFFu;
+// Blocks and the tensors they touch advance together, so that index block + tensor of rec_max is nobody else's.
 
 __device__ __forceinline__ int32_t exponent_of(uint32_t max_bits)       // floor(log2 M_k)
 {
@@ -72,6 +85,60 @@ __device__ __forceinline__ int32_t rounded_exponent(uint32_t bits)      // neare
     return (int32_t)((bits + 0x00400000u) >> 23) - 127;
 }
 
+// exponents of the tensors that begin in [lo, hi) (empty tensors at the buffer's end belong to the last block)
+template <class MaxOf>
+__device__ __forceinline__ void write_exponents(const Args &a, const uint32_t *offs, uint32_t lo, uint32_t hi, bool last,
+                                                const MaxOf &max_of)
+{
+    int k0 = 0, k1 = a.K;                               // first k with offs[k] >= lo
+    while (k0 < k1) {
+        const int mid = (k0 + k1) >> 1;
+        if (offs[mid] < lo) k0 = mid + 1; else k1 = mid;
+    }
+    for (int k = k0 + (int)threadIdx.x; k < a.K && (last || offs[k] < hi); k += kThreads)
+        a.out.group_exp[k] = offs[k] < offs[k + 1] ? exponent_of(max_of(k)) : VGC_EXP_NONE;
+}
+
+// staged value -> word; true if the word is emitted (d <= 7).  Holds the tensor of the last value it saw.
+template <bool kQuantise>
+struct Encoder {
+    const uint32_t *offs;
+    int K, k_first, k_last, k;
+    uint32_t lo;
+    int32_t Ek;
+    __device__ __forceinline__ Encoder(const uint32_t *offs_, int K_, uint32_t lo_, int k_first_, int k_last_)
+        : offs(offs_), K(K_), k_first(k_first_), k_last(k_last_), k(-1), lo(lo_), Ek(0) {}
+    template <class MaxOf>
+    __device__ __forceinline__ bool operator()(uint32_t staged, const MaxOf &max_of, uint32_t &word)
+    {
+        const uint32_t idx = lo + (staged >> kPosShift);
+        word = (idx << 4) | ((staged >> 6) & 8u);
+        if (!kQuantise) return true;
+        if (k < 0 || (k_first != k_last && (idx < offs[k] || idx >= offs[k + 1]))) {
+            k = k_first == k_last ? k_first : group_of(offs, K, idx);
+            Ek = exponent_of(max_of(k));
+        }
+        const int32_t e1 = (int32_t)(staged & 0x1FFu) - 127;
+        const int32_t d = Ek - (e1 < Ek ? e1 : Ek);                        // cut at 2^E_k
+        word |= (uint32_t)(d & 7);
+        return d <= 7;
+    }
+};
+
+// counters of the message: passed and kept values up to and with this block's
+__device__ __forceinline__ void finish(const Args &a, bool last, bool quantise, uint32_t passed, uint32_t kept)
+{
+    if (threadIdx.x != 0) return;
+    if (kept > a.out.capacity) atomicOr(a.out.dev_status, VGC_DEV_CAPACITY);
+    if (last) {
+        *a.out.nnz = kept;
+        if (quantise) {
+            *a.out.n_criterion = passed;
+            *a.out.n_dropped = passed - kept;
+        }
+    }
+}
+
 // kHasS = false: the caller accumulated this step's squared-gradient sums straight into v (the sqgrad entry
 // points with accumulate = 1), so the pass reads 12 instead of 16 bytes per parameter.
 template <bool kHasS, int kAlgorithm>
@@ -79,18 +146,16 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
 compress_step(const __grid_constant__ Args a)
 {
     constexpr bool kQuantise = kAlgorithm == kBasic;
-    extern __shared__ uint32_t sm_staged[];             // kStaged values
     __shared__ uint32_t sm_offs[kOffsSmem];
     __shared__ uint32_t sm_part[2][kRowsA * kWarps];    // per-(row, warp) counts, double buffered
     __shared__ uint32_t sm_wmax[2][kWarps];
-    __shared__ uint32_t sm_wmin[2][kWarps];             // smallest |value| bit pattern sent by each warp
-    __shared__ uint32_t sm_rec_max[2], sm_rec_min[2];   // extremes of the range's first and last tensor, this block's ...
-    __shared__ uint32_t sm_end_max[2];                  // ... and M_k bits, from all blocks
-    __shared__ uint32_t sm_kept[kWarps];
-    __shared__ uint32_t sm_passed_before[kWarps], sm_kept_before[kWarps];
+    __shared__ uint32_t sm_rec_max[2];                  // maxima of the range's first and last tensor
+    __shared__ uint32_t sm_fields[kWarps][7];
+    __shared__ uint32_t sm_staged[kStagedCopy];         // the first staged values once more, for the count at the end
 
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x;
     const int K = a.K;
+    grid_release();
     const bool offs_in_smem = kQuantise && (K + 1) <= kOffsSmem;
     if (offs_in_smem) {                                 // asynchronously: the first tile's loads go out before they arrive
         for (int i = tid; i <= K; i += kThreads)
@@ -100,26 +165,20 @@ compress_step(const __grid_constant__ Args a)
     const uint32_t *offs = offs_in_smem ? sm_offs : a.group_offsets;
     const uint32_t lo = b * a.per_block;
     const uint32_t hi = (uint32_t)((size_t)lo + a.per_block < a.n ? (size_t)lo + a.per_block : a.n);
-    if (tid < 2) { sm_end_max[tid] = 0; sm_rec_max[tid] = 0; sm_rec_min[tid] = kNoMin; }
-    Slot *const my_first = a.first + tid * kMaxGrid + b, *const my_second = a.second + tid * kMaxGrid + b;     // tid < kCopies
-    const Slot *const firsts = a.first + (b % kCopies) * kMaxGrid, *const seconds = a.second + (b % kCopies) * kMaxGrid;
-    if (tid < kCopies) slot_publish(my_second, 0, 0, 0);
-    uint32_t *const rec_max = a.rec_max + b, *const rec_min = a.rec_min + b;     // this block's records, by tensor
+    if (tid < 2) sm_rec_max[tid] = 0;
+    uint32_t *const rec_max = a.rec_max + b;            // this block's records, by tensor
     int k_first = 0, k_last = 0;
 
     const float tau_sq = __fmul_rn(a.tau, a.tau);
 
-    // ---- step 1
-    uint32_t run = 0;                                   // values staged by the block so far
+        uint32_t run = 0;                                   // values staged by the block so far
     int k_tile = 0;                                     // tensor of the tile's first parameter
-    int k_held = 0;                                     // thread 0: the tensor whose extremes it holds
-    uint32_t held_max = 0, held_min = kNoMin;
-    // largest and smallest |value| bits of tensor k: the range's first and last tensor in shared memory (all there is,
-    // mostly), the ones between them in the workspace
-    auto record = [&](int k, uint32_t most, uint32_t least) {
-        const bool end = k == k_first || k == k_last;
-        atomicMax(end ? sm_rec_max + (k != k_first) : rec_max + k, most);
-        atomicMin(end ? sm_rec_min + (k != k_first) : rec_min + k, least);
+    int k_held = 0;                                     // thread 0: the tensor whose maximum it holds
+    uint32_t held_max = 0;
+    // largest |value| bits of tensor k: the range's first and last tensor in shared memory (all there is, mostly), the
+    // ones between them in the workspace
+    auto record = [&](int k, uint32_t most) {
+        atomicMax(k == k_first ? sm_rec_max : k == k_last ? sm_rec_max + 1 : rec_max + k, most);
     };
     uint32_t buf = 0;
     for (uint32_t base = lo; base < hi; base += a.tile, buf ^= 1) {
@@ -148,7 +207,6 @@ compress_step(const __grid_constant__ Args a)
             }
         }
         if (base == lo) {
-            if (tid < kCopies) __threadfence();         // the cleared `second` slot before the `first` one
             if (offs_in_smem) asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
             __syncthreads();
         }
@@ -156,7 +214,7 @@ compress_step(const __grid_constant__ Args a)
             k_first = group_of(offs, K, lo);
             k_last = hi <= offs[k_first + 1] ? k_first : group_of(offs, K, hi - 1);
             k_tile = k_held = k_first;
-            for (int k = k_first + 1 + (int)tid; k < k_last; k += kThreads) { rec_max[k] = 0; rec_min[k] = kNoMin; }
+            for (int k = k_first + 1 + (int)tid; k < k_last; k += kThreads) rec_max[k] = 0;
         }
         if (kQuantise)
             while (offs[k_tile + 1] <= base) ++k_tile;  // block-uniform
@@ -165,7 +223,7 @@ compress_step(const __grid_constant__ Args a)
         // loop body of Algorithm 1 / Algorithm 2; every operation rounded on its own (no FMA)
         uint32_t send_bits = 0;          // bit j*4+q
         uint32_t packed = 0;             // per-row counts, 8 bits each
-        uint32_t my_max = 0, my_min = kNoMin;
+        uint32_t my_max = 0;
 #pragma unroll
         for (int j = 0; j < kRowsA; ++j) {
             const uint32_t e = base + (j * kThreads + tid) * 4;
@@ -185,10 +243,7 @@ compress_step(const __grid_constant__ Args a)
                 if (kQuantise) {
                     Rj[q] = send ? 0.f : r1;
                     Vj[q] = send ? 0.f : __fmul_rn(v1, a.zeta);
-                    if (send) {
-                        my_max = max(my_max, __float_as_uint(r1) & 0x7FFFFFFFu);
-                        my_min = min(my_min, __float_as_uint(r1) & 0x7FFFFFFFu);
-                    }
+                    if (send) my_max = max(my_max, __float_as_uint(r1) & 0x7FFFFFFFu);
                 } else {
                     const float r2 = r1 < 0.f ? __fadd_rn(r1, a.tau) : __fsub_rn(r1, a.tau);     // r -= Sign(r) tau
                     const float cross = __fmul_rn(__fmul_rn(2.0f, kAlgorithm == kHybridBefore ? fabsf(r1) : fabsf(r2)), a.tau);
@@ -228,12 +283,10 @@ compress_step(const __grid_constant__ Args a)
             if (lane >= d) incl += up;
         }
         const uint32_t warp_max = kQuantise ? __reduce_max_sync(0xffffffffu, my_max) : 0u;
-        const uint32_t warp_min = kQuantise ? __reduce_min_sync(0xffffffffu, my_min) : 0u;
         if (lane == 31) {
 #pragma unroll
             for (int j = 0; j < kRowsA; ++j) sm_part[buf][j * kWarps + warp] = (incl >> (8 * j)) & 0xFFu;
             sm_wmax[buf][warp] = warp_max;
-            sm_wmin[buf][warp] = warp_min;
         }
         __syncthreads();
         static_assert(kRowsA * kWarps == 32, "one count per lane");
@@ -260,206 +313,253 @@ compress_step(const __grid_constant__ Args a)
                         const uint32_t bits = __float_as_uint(Gj[q]);
                         const uint32_t staged = (e + q - lo) << kPosShift | (bits >> 31) << 9 |
                                                 (uint32_t)(rounded_exponent(bits & 0x7FFFFFFFu) + 127);
-                        if (at < kStaged) sm_staged[at] = staged;
-                        else a.stage[lo + at] = staged;
+                        a.stage[lo + at] = staged;
+                        if (kQuantise && at < kStagedCopy) sm_staged[at] = staged;
                         ++at;
-                        if (kQuantise && grp < 0) {
-                            const int k = group_of(offs, K, e + q);
-                            record(k, bits & 0x7FFFFFFFu, bits & 0x7FFFFFFFu);
-                        }
+                        if (kQuantise && grp < 0) record(group_of(offs, K, e + q), bits & 0x7FFFFFFFu);
                     }
             }
         }
         if (kQuantise && tid == 0 && grp >= 0 && total) {
             if (grp != k_held) {
-                if (held_max) record(k_held, held_max, held_min);
-                k_held = grp; held_max = 0; held_min = kNoMin;
+                if (held_max) record(k_held, held_max);
+                k_held = grp; held_max = 0;
             }
 #pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                held_max = max(held_max, sm_wmax[buf][w]);
-                held_min = min(held_min, sm_wmin[buf][w]);
-            }
+            for (int w = 0; w < kWarps; ++w) held_max = max(held_max, sm_wmax[buf][w]);
         }
         run += total;
     }
-    if (tid == 0 && held_max) record(k_held, held_max, held_min);
+    if (tid == 0 && held_max) record(k_held, held_max);
     __syncthreads();
-    const int i_last = k_first == k_last ? 0 : 1;
-    if (tid < kCopies) slot_publish(my_first, a.tag, sm_rec_max[0], sm_rec_max[i_last]);
+    const bool same = k_first == k_last;
 
-    // ---- step 2: M_k of the range's first and last tensor, which other blocks may share.  A tensor that spans several
-    // blocks is the last tensor of the block it begins in and the first one of the others
-    {
-        uint32_t f0 = 1, f1 = 0, l0 = 1, l1 = 0;
-        if (kQuantise) {
-            f0 = offs[k_first] / a.per_block; f1 = (offs[k_first + 1] - 1) / a.per_block;
-            l0 = offs[k_last] / a.per_block;  l1 = (offs[k_last + 1] - 1) / a.per_block;
-        }
-        uint32_t m_first = 0, m_last = 0;
-        bool late = false;
-        for (uint32_t c = tid; c < gridDim.x; c += kThreads) {
-            uint32_t of_first, of_last;
-            if (!slot_wait(firsts + c, a.tag, of_first, of_last)) { late = true; break; }
-            if (c >= f0 && c <= f1) m_first = max(m_first, c == f0 && f0 < f1 ? of_last : of_first);
-            if (c >= l0 && c <= l1) m_last = max(m_last, c == l0 ? of_last : of_first);
-        }
-        __threadfence();                                // ... before anyone's `second` slot is looked at
-        __syncwarp();
-        if (kQuantise) {
-            m_first = __reduce_max_sync(0xffffffffu, m_first);
-            m_last = __reduce_max_sync(0xffffffffu, m_last);
-        }
-        if (kQuantise && lane == 0) {
-            if (m_first) atomicMax(&sm_end_max[0], m_first);
-            if (m_last) atomicMax(&sm_end_max[1], m_last);
-        }
-        if (__syncthreads_or(late)) {
-            if (tid == 0) atomicOr(a.out.dev_status, VGC_DEV_TIMEOUT);
-            return;
-        }
-    }
-    auto max_of = [&](int k) -> uint32_t {
-        return k == k_first ? sm_end_max[0] : k == k_last ? sm_end_max[1] : __ldcg(rec_max + k);
-    };
-    bool drops = false;
+    // ---- what the second kernel needs to know
     if (kQuantise) {
-        // exponents of the tensors that begin in this range (empty tensors at the buffer's end belong to the last block)
-        int k0 = 0, k1 = K;                             // first k with offs[k] >= lo
-        while (k0 < k1) {
-            const int mid = (k0 + k1) >> 1;
-            if (offs[mid] < lo) k0 = mid + 1; else k1 = mid;
-        }
-        const bool last = b == gridDim.x - 1;
-        for (int k = k0 + (int)tid; k < K && (last || offs[k] < hi); k += kThreads)
-            a.out.group_exp[k] = offs[k] < offs[k + 1] ? exponent_of(max_of(k)) : VGC_EXP_NONE;
-        // nothing is dropped when even the smallest value sent from each tensor is within 7 binades of its exponent
-        for (int k = k_first + (int)tid; k <= k_last; k += kThreads) {
-            const uint32_t m = k == k_first ? sm_rec_min[0] : k == k_last ? sm_rec_min[1] : __ldcg(rec_min + k);
-            if (m != kNoMin && rounded_exponent(m) < exponent_of(max_of(k)) - 7) drops = true;
-        }
-        drops = __syncthreads_or(drops);
-    }
-
-    // staged value i of the block -> its word; true if a word is emitted.  k: the tensor of the last value looked at
-    auto staged_at = [&](uint32_t i) -> uint32_t { return i < kStaged ? sm_staged[i] : a.stage[lo + i]; };
-    auto encode = [&](uint32_t staged, int &k, int32_t &Ek, uint32_t &word) -> bool {
-        const uint32_t idx = lo + (staged >> kPosShift);
-        if (!kQuantise) { word = (idx << 4) | ((staged >> 6) & 8u); return true; }
-        if (Ek == INT32_MIN || idx < offs[k] || idx >= offs[k + 1]) {
-            k = k_first == k_last ? k_first : group_of(offs, K, idx);
-            Ek = exponent_of(max_of(k));
-        }
-        const int32_t e1 = (int32_t)(staged & 0x1FFu) - 127;
-        const int32_t d = Ek - (e1 < Ek ? e1 : Ek);                        // cut at 2^E_k
-        word = (idx << 4) | ((staged >> 6) & 8u) | (uint32_t)(d & 7);
-        return d <= 7;
-    };
-    // with drops every warp walks a section of the values, four 32-wide slices per round
-    const uint32_t section = ((run + kWarps - 1) / kWarps + 31u) & ~31u;
-    const uint32_t s0 = min(run, warp * section), s1 = min(run, s0 + section);
-    auto walk = [&](auto emit) {
-        int k = k_first;
-        int32_t Ek = INT32_MIN;
-        uint32_t kept = 0;
-        for (uint32_t i0 = s0; i0 < s1; i0 += 128) {
-            uint32_t p[4];
+        // a value survives E_k = own + j (own: this block's exponent for the tensor) if e >= own + j - 7, and e <= own + 1.
+        // A thread counts its values by e - own + 7 in nine 7-bit fields per tensor; a warp adds them in fields of ten
+        // bits (at most 24 values per thread in between), three to a word
+        const uint32_t first_end = offs[k_first + 1], last_begin = offs[k_last];
+        const int own_first = (int)(sm_rec_max[0] >> 23), own_last = (int)(sm_rec_max[1] >> 23);         // biased
+        constexpr uint32_t kBatch = 8, kRound = 3 * kBatch * kThreads;
+        uint32_t sums = 0;                               // thread j of the first kCounts: entry j
+        for (uint32_t i0 = 0; i0 < run; i0 += kRound) {  // block-uniform
+            unsigned long long of_first = 0, of_last = 0;
+            uint32_t inside = 0;
+            const uint32_t i1 = min(run, i0 + kRound);
+            for (uint32_t i = i0 + tid; i < i1; i += kBatch * kThreads) {
+                uint32_t staged[kBatch];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t i = i0 + u * 32 + lane;
-                p[u] = i < s1 ? staged_at(i) : 0u;
+                for (uint32_t u = 0; u < kBatch; ++u) {
+                    const uint32_t at = i + u * kThreads;
+                    staged[u] = at >= i1 ? 0u : at < kStagedCopy ? sm_staged[at] : __ldcg(a.stage + lo + at);
+                }
+#pragma unroll
+                for (uint32_t u = 0; u < kBatch; ++u) {
+                    if (i + u * kThreads >= i1) break;
+                    const uint32_t idx = lo + (staged[u] >> kPosShift);
+                    const int e = (int)(staged[u] & 0x1FFu);
+                    if (idx < first_end) {
+                        const int level = e - own_first + 7;
+                        if (level >= 0) of_first += 1ull << (7 * level);
+                    } else if (idx >= last_begin) {
+                        const int level = e - own_last + 7;
+                        if (level >= 0) of_last += 1ull << (7 * level);
+                    } else {                             // a tensor wholly inside: E_k is this block's
+                        const int own = (int)(__ldcg(rec_max + group_of(offs, K, idx)) >> 23);
+                        inside += e >= own - 7 ? 1u : 0u;
+                    }
+                }
             }
+            auto add_up = [&](unsigned long long f, uint32_t *to) {
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                bool keep = false;
-                uint32_t word = 0;
-                if (i0 + u * 32 + lane < s1) keep = encode(p[u], k, Ek, word);
-                const uint32_t ballot = __ballot_sync(0xffffffffu, keep);
-                if (keep) emit(kept + __popc(ballot & ((1u << lane) - 1u)), word);
-                kept += __popc(ballot);
+                for (int w = 0; w < 3; ++w) {
+                    const uint32_t g = (uint32_t)(f >> (21 * w));
+                    const uint32_t sum = __reduce_add_sync(0xffffffffu, (g & 0x7Fu) | (g & 0x3F80u) << 3 | (g & 0x1FC000u) << 6);
+                    if (lane == 0) to[w] = sum;
+                }
+            };
+            add_up(of_first, sm_fields[warp]);
+            if (!same) {
+                add_up(of_last, sm_fields[warp] + 3);
+                inside = __reduce_add_sync(0xffffffffu, inside);
+                if (lane == 0) sm_fields[warp][6] = inside;
             }
-        }
-        return kept;
-    };
-    uint32_t kept = run;
-    if (drops) {
-        const uint32_t mine = walk([](uint32_t, uint32_t) {});
-        if (lane == 0) sm_kept[warp] = mine;
-        __syncthreads();
-        kept = 0;
+            __syncthreads();
+            if (tid < (uint32_t)kCounts && !(same && tid >= (uint32_t)kLevels)) {
+                const int j = (int)tid % kLevels;
+                const uint32_t at = tid < 2u * kLevels ? 3 * (tid / kLevels) + j / 3 : 6, shift = tid < 2u * kLevels ? 10 * (j % 3) : 0;
+                const uint32_t field = tid < 2u * kLevels ? 0x3FFu : 0xFFFFFFFFu;
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) kept += sm_kept[w];
-    }
-    if (tid < kCopies) slot_publish(my_second, a.tag, run, kept);
-
-    // ---- step 3: counts of the blocks before this one, then the words
-    uint32_t passed_before = 0, kept_before = 0;
-    bool late = false;
-    for (uint32_t c = tid; c < b; c += kThreads) {
-        uint32_t passed_c, kept_c;
-        if (!slot_wait(seconds + c, a.tag, passed_c, kept_c)) { late = true; break; }
-        passed_before += passed_c;
-        kept_before += kept_c;
-    }
-    __syncwarp();
-    passed_before = __reduce_add_sync(0xffffffffu, passed_before);
-    kept_before = __reduce_add_sync(0xffffffffu, kept_before);
-    if (lane == 0) { sm_passed_before[warp] = passed_before; sm_kept_before[warp] = kept_before; }
-    if (__syncthreads_or(late)) {
-        if (tid == 0) atomicOr(a.out.dev_status, VGC_DEV_TIMEOUT);
-        return;
-    }
-    uint32_t pos = 0;
-    passed_before = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) { pos += sm_kept_before[w]; passed_before += sm_passed_before[w]; }
-    if (tid == 0 && pos + kept > a.out.capacity) atomicOr(a.out.dev_status, VGC_DEV_CAPACITY);
-    if (b == gridDim.x - 1) {
-        if (tid == 0) {
-            *a.out.nnz = pos + kept;
-            if (kQuantise) {
-                *a.out.n_criterion = passed_before + run;
-                *a.out.n_dropped = passed_before + run - (pos + kept);
+                for (int w = 0; w < kWarps; ++w) sums += (sm_fields[w][at] >> shift) & field;
             }
+            if (i0 + kRound < run) __syncthreads();
         }
-        for (uint32_t c = tid; c < kCopies * kMaxGrid; c += kThreads) slot_publish(a.first + c, 0, 0, 0);   // everyone has read them
-    }
-    if (drops) {
+        // entry j of a tensor: the values of levels >= j
+        if (warp == 0) {
+            const int level = (int)lane % kLevels;
 #pragma unroll
-        for (uint32_t w = 0; w < kWarps; ++w) pos += w < warp ? sm_kept[w] : 0u;
-        walk([&](uint32_t at, uint32_t word) {
-            if (pos + at < a.out.capacity) a.out.words[pos + at] = word;
-        });
-    } else {
-        int k = k_first;
-        int32_t Ek = INT32_MIN;
-        for (uint32_t i = tid; i < run; i += kThreads) {
-            uint32_t word;
-            encode(staged_at(i), k, Ek, word);
-            if (pos + i < a.out.capacity) a.out.words[pos + i] = word;
+            for (int d = 1; d < kLevels; d <<= 1) {
+                const uint32_t up = __shfl_down_sync(0xffffffffu, sums, d);
+                if (lane < 2u * kLevels && level + d < kLevels) sums += up;
+            }
+            if (lane < (uint32_t)kCounts) a.counts[b * kCounts + lane] = sums;
         }
+    }
+    if (tid == 0) {
+        Record rec;
+        rec.max_first = sm_rec_max[0];
+        rec.max_last = sm_rec_max[same ? 0 : 1];
+        rec.head = (kQuantise ? offs[k_first] / a.per_block : 0u) | (same ? kSame : 0u);
+        rec.passed = run;
+        a.records[b] = rec;
     }
 }
 
-// Enqueues one step.  a: everything but the tag, the slots and the ranges, which are set here; `slots`: kSlotBytes.
-template <bool kHasS, int kAlgorithm>
-vgc_status launch(Args a, void *slots, cudaStream_t st)
+// The second kernel: same blocks, same ranges.
+template <bool kQuantise>
+__global__ void __launch_bounds__(kThreads, kBlocksPerSm)
+encode_step(const __grid_constant__ Args a)
 {
-    const void *fn = reinterpret_cast<const void *>(compress_step<kHasS, kAlgorithm>);
-    constexpr size_t smem = kStaged * sizeof(uint32_t);
-    static ResidentBlocks resident;
-    const uint32_t most = resident.get(fn, kThreads, smem);
-    if (most == 0) return VGC_ERR_CUDA;
-    const Ranges R = even_ranges(a.n, most < (uint32_t)kMaxGrid ? most : (uint32_t)kMaxGrid, kTileA, kLeastPerBlock);
-    if (R.per_block > kMostPerBlock) return VGC_ERR_UNSUPPORTED;         // a device with room for fewer than 64 blocks
-    a.tag = next_tag();
-    a.first = static_cast<Slot *>(slots);
-    a.second = a.first + kCopies * kMaxGrid;
-    a.per_block = R.per_block;
-    a.tile = R.tile;
-    void *params[] = {&a};
-    VGC_CUDA_OK(cudaLaunchCooperativeKernel(fn, dim3(R.grid), dim3(kThreads), params, smem, st));
-    count_launch();
+    __shared__ uint32_t sm_offs[kOffsSmem];
+    __shared__ uint32_t sm_begun[kMaxGrid];             // M_k bits of the last tensor of every block
+    __shared__ uint32_t sm_end_max[2];                  // ... of this block's first and last tensor
+    __shared__ uint32_t sm_passed[kWarps], sm_kept[kWarps], sm_own[2];
+    constexpr int kPerRound = 4;
+    __shared__ __align__(8) uint32_t sm_part[2][kPerRound * kWarps];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x, blocks = gridDim.x;
+    const int K = a.K;
+    const bool offs_in_smem = kQuantise && (K + 1) <= kOffsSmem;
+    if (offs_in_smem)
+        for (int i = tid; i <= K; i += kThreads) sm_offs[i] = a.group_offsets[i];
+    const uint32_t *offs = offs_in_smem ? sm_offs : a.group_offsets;
+    const uint32_t lo = b * a.per_block;
+    const uint32_t hi = (uint32_t)((size_t)lo + a.per_block < a.n ? (size_t)lo + a.per_block : a.n);
+    if (kQuantise && tid < blocks) sm_begun[tid] = 0;
+    __syncthreads();
+    int k_first = 0, k_last = 0;
+    if (kQuantise) { k_first = group_of(offs, K, lo); k_last = hi <= offs[k_first + 1] ? k_first : group_of(offs, K, hi - 1); }
+    grid_wait();
+
+    // the values of the first round are asked for together with the records
+    const uint32_t *staged = a.stage + lo;
+    uint32_t next[kPerRound];
+#pragma unroll
+    for (int u = 0; u < kPerRound; ++u) next[u] = u * kThreads + tid < hi - lo ? __ldcg(staged + u * kThreads + tid) : 0u;
+    Record rec = {0, 0, 0, 0};
+    if (tid < blocks) {
+        const uint4 q = __ldcg(reinterpret_cast<const uint4 *>(a.records) + tid);
+        rec.max_first = q.x; rec.max_last = q.y; rec.head = q.z; rec.passed = q.w;
+    }
+    const uint32_t head = rec.head & ~kSame;
+    const bool same = rec.head & kSame, shared_first = head < tid;
+    uint32_t kept = rec.passed;
+    if (kQuantise) {
+        if (tid < blocks) {
+            // a tensor that spans several blocks is the last one of the block it begins in and the first one of the others
+            if (shared_first) atomicMax(&sm_begun[head], rec.max_first);
+            if (!(same && shared_first)) atomicMax(&sm_begun[tid], rec.max_last);
+        }
+        __syncthreads();
+        kept = 0;
+        if (tid <= b) {
+            const uint32_t m_first = shared_first ? sm_begun[head] : same ? sm_begun[tid] : rec.max_first;
+            const uint32_t m_last = same ? m_first : sm_begun[tid];
+            const uint32_t *counts = a.counts + tid * kCounts;
+            const uint32_t up_first = (m_first >> 23) - (rec.max_first >> 23), up_last = (m_last >> 23) - (rec.max_last >> 23);
+            const uint32_t of_first = up_first < kLevels ? __ldcg(counts + up_first) : 0u;
+            const uint32_t of_last = !same && up_last < kLevels ? __ldcg(counts + kLevels + up_last) : 0u;
+            kept = of_first + of_last + __ldcg(counts + 2 * kLevels);
+            if (tid == b) { sm_end_max[0] = m_first; sm_end_max[1] = m_last; }
+        }
+    }
+    if (tid == b) { sm_own[0] = rec.passed; sm_own[1] = kept; }
+    const uint32_t passed_w = __reduce_add_sync(0xffffffffu, tid < b ? rec.passed : 0u);
+    const uint32_t kept_w = __reduce_add_sync(0xffffffffu, tid < b ? kept : 0u);
+    if (lane == 0) { sm_passed[warp] = passed_w; sm_kept[warp] = kept_w; }
+    __syncthreads();
+    uint32_t passed_before = 0, pos = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) { passed_before += sm_passed[w]; pos += sm_kept[w]; }
+    const uint32_t run = sm_own[0];
+    finish(a, b == blocks - 1, kQuantise, passed_before + run, pos + sm_own[1]);
+    const uint32_t *rec_max = a.rec_max + b;
+    auto max_of = [&](int k) -> uint32_t {
+        return k == k_first ? sm_end_max[0] : k == k_last ? sm_end_max[1] : __ldcg(rec_max + k);
+    };
+    if (kQuantise) write_exponents(a, offs, lo, hi, b == blocks - 1, max_of);
+
+    // words, 4 x 512 values a round (a thread's are 512 apart: neighbouring lanes write neighbouring words); where some are
+    // dropped, a scan over the (512 values, warp) counts of the survivors gives the places
+    Encoder<kQuantise> enc(offs, K, lo, k_first, k_last);
+    const bool drops = kQuantise && sm_own[1] != run;
+    uint32_t buf = 0;
+    for (uint32_t i0 = 0; i0 < run; i0 += kPerRound * kThreads, buf ^= 1) {
+        uint32_t now[kPerRound], word[kPerRound], ballot[kPerRound];
+#pragma unroll
+        for (int u = 0; u < kPerRound; ++u) {
+            now[u] = next[u];
+            const uint32_t i = i0 + (kPerRound + u) * kThreads + tid;
+            next[u] = i < run ? __ldcg(staged + i) : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < kPerRound; ++u) {
+            const bool keep = i0 + u * kThreads + tid < run && enc(now[u], max_of, word[u]);
+            ballot[u] = __ballot_sync(0xffffffffu, keep);
+        }
+        if (!drops) {
+#pragma unroll
+            for (int u = 0; u < kPerRound; ++u) {
+                const uint32_t i = i0 + u * kThreads + tid;
+                if (i < run && pos + i < a.out.capacity) a.out.words[pos + i] = word[u];
+            }
+            continue;
+        }
+        if (lane < (uint32_t)kPerRound) {
+            uint32_t c = 0;
+#pragma unroll
+            for (int u = 0; u < kPerRound; ++u) c = lane == (uint32_t)u ? (uint32_t)__popc(ballot[u]) : c;
+            sm_part[buf][lane * kWarps + warp] = c;
+        }
+        __syncthreads();
+        static_assert(kPerRound * kWarps == 64, "two counts per lane");
+        const uint2 two = *reinterpret_cast<const uint2 *>(&sm_part[buf][2 * lane]);
+        uint32_t incl = two.x + two.y;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t up = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += up;
+        }
+        const uint32_t before_two = incl - two.x - two.y;
+#pragma unroll
+        for (int u = 0; u < kPerRound; ++u) {
+            const uint32_t entry = u * kWarps + warp;
+            uint32_t at = __shfl_sync(0xffffffffu, before_two, entry >> 1);
+            const uint32_t even = __shfl_sync(0xffffffffu, two.x, entry >> 1);
+            at += pos + (entry & 1u ? even : 0u) + __popc(ballot[u] & ((1u << lane) - 1u));
+            if ((ballot[u] >> lane & 1u) && at < a.out.capacity) a.out.words[at] = word[u];
+        }
+        pos += __shfl_sync(0xffffffffu, incl, 31);
+    }
+}
+
+// Enqueues one step.  a: everything but the ranges; records: kRecordBytes, 16-byte aligned.
+template <bool kHasS, int kAlgorithm>
+vgc_status launch(Args a, void *records, cudaStream_t st)
+{
+    a.records = static_cast<Record *>(records);
+    a.counts = reinterpret_cast<uint32_t *>(a.records + kMaxGrid);
+    // every block the same share (to 128 parameters: 512 B of every stream), cut into tiles of equal size
+    const size_t shares = (a.n + kLeastPerBlock - 1) / kLeastPerBlock;
+    const size_t blocks = shares < (size_t)kMaxGrid ? shares : (size_t)kMaxGrid;
+    const size_t per = round_up((a.n + blocks - 1) / blocks, 128);
+    const size_t tiles = (per + kTileA - 1) / kTileA;
+    a.per_block = (uint32_t)per;
+    a.tile = (uint32_t)round_up((per + tiles - 1) / tiles, 128);
+    const dim3 grid((unsigned)((a.n + per - 1) / per));
+    VGC_CUDA_OK(launch_kernel(compress_step<kHasS, kAlgorithm>, grid, dim3(kThreads), 0, st, false, a));
+    VGC_CUDA_OK(launch_kernel(encode_step<kAlgorithm == kBasic>, grid, dim3(kThreads), 0, st, true, a));
+    count_launch(2);
     return VGC_OK;
 }
 

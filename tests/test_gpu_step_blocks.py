@@ -1,7 +1,7 @@
 """The streaming kernel of both compressors at the sizes where its partition changes: one parameter, around one block's
-least share (2048), around one tile per block (4096 x 296 blocks), more values than a block keeps in shared memory
-(12288), tensors that begin and end in the middle of tiles and blocks; and a captured launch replayed, whose slots still
-lie in the workspace when the next replay starts.  Bit-exact against the oracle (whole numbers; fp32 operations rounded
+least share (2048), around one tile per block (4096 x 296 blocks), several rounds of the second kernel,
+tensors that begin and end in the middle of tiles and blocks; and a
+captured launch replayed, which finds what it left in the workspace.  Bit-exact against the oracle (whole numbers; fp32 operations rounded
 one by one on both sides)."""
 import numpy as np
 import pytest
@@ -28,7 +28,7 @@ def test_compress_over_block_borders(n, K, alpha):
         assert_same_state(gpu, cpu)
 
 
-@pytest.mark.parametrize("n,tau", [(1, 1e-3), (2049, 1e-3), (FULL + 5, 1e-3), (4_500_001, 0.0)])
+@pytest.mark.parametrize("n,tau", [(1, 1e-3), (2049, 1e-3), (1 << 18, 0.0), (FULL + 5, 1e-3), (4_500_001, 0.0)])
 def test_hybrid_over_block_borders(n, tau):
     r, v = torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda")
     rc, vc = np.zeros(n, np.float32), np.zeros(n, np.float32)
@@ -45,7 +45,7 @@ def test_hybrid_over_block_borders(n, tau):
         assert np.array_equal(v.cpu().numpy().view(np.uint32), vc.view(np.uint32))
 
 
-def test_replayed_launch_finds_its_own_slots():
+def test_replayed_launch():
     n, K = 700_001, 9
     offs = random_offsets(np.random.default_rng(3), n, K)
     gpu, cpu = GpuCompressor(n, offs), OracleCompressor(n, offs)
