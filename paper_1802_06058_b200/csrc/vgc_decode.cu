@@ -5,21 +5,18 @@
 // scaled, and added into the dense update buffer.  One launch covers up to kMaxViews messages (their
 // pointers travel in the kernel parameters, so nothing is allocated).
 //
-// Messages are sorted by index, so the words that fall into a contiguous range of u are a contiguous run of
-// every message.  A block owns one range of u; one warp per message finds where the run enters it (32-ary
-// search).  Then, per call:
-//   sparse (fewer than one word per eight elements): the block's words are added straight into global memory
-//     with fp32 atomics -- u is touched only where a word points;
-//   dense: the block walks its range in tiles of up to 24576 elements (96 KB of shared memory, two blocks of 512
-//     threads per SM).  The tile comes in by cp.async while one warp per message finds where the message's run
-//     leaves the tile (a search confined to the at most tile-length words that can lie in it); the messages are
-//     then applied one after the other by the whole block, 8 x 512 words at a time with the next batch's loads in
-//     flight (indices inside a message are distinct, so plain read-modify-writes, a block barrier between
-//     messages): an element receives its additions in the order w = 0, 1, ..., the fp32 sequence of a sequential
-//     sum, whatever the scheduling.  A word's value is one look-up in a 16-entry table per message (its low four
-//     bits are sign and d) when the tile lies inside one weight tensor.  u is read and written once, coalesced.
+// Messages are sorted by index, so the words that fall into a contiguous range of u are a contiguous run of every
+// message.  Three ways, by how many words the messages hold together:
+//   flat      few words, added to u: every warp takes pieces of the messages and adds them to u with fp32 atomics -- u is
+//             touched only where a word points (decode_flat);
+//   scatter   few words, u written: a block owns a range of u, writes zeros piece by piece and adds the piece's words while
+//             it is still in L2 (scatter_range);
+//   dense     a block owns a range of u and walks it in tiles held in shared memory; u is read and written once, coalesced:
+//             exact_range where every word is a multiple of one power of two, ordered_range otherwise.
 // kOverwrite: the range starts from zero instead of the old contents of u (u = scale * sum of the messages).
 // kHybrid: messages of the hybrid algorithm (Algorithm 2) -- every word stands for +-tau, no exponents.
+#include <type_traits>
+
 #include "vgc_common.cuh"
 
 namespace vgc {
@@ -34,30 +31,20 @@ struct DecodeViews {
     uint32_t max_words[kMaxViews];
 };
 
-// first position in [0, count) whose index is >= bound (count if none); whole warp, 32-ary search
-__device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t *__restrict__ words, uint32_t count, uint32_t bound)
-{
-    const uint32_t lane = threadIdx.x & 31;
-    uint32_t lo = 0, hi = count;      // every position < lo is below the bound, every position >= hi is not
-    while (hi > lo) {
-        const uint32_t step = (hi - lo) / 32 + 1;                 // 32 probes lo, lo+step, ... reach past hi
-        const uint32_t pos = lo + step * lane;
-        const bool below = pos < hi && (words[pos] >> 4) < bound;
-        const uint32_t nb = __popc(__ballot_sync(0xffffffffu, below));   // sorted input: a prefix of the lanes
-        if (nb == 0) { hi = lo; break; }
-        const uint32_t new_hi = lo + step * nb;                   // first probe that is not below (or past hi)
-        lo = lo + step * (nb - 1) + 1;
-        hi = new_hi < hi ? new_hi : hi;
-    }
-    return lo;
-}
+// Below one word per this many elements (all messages together) a call is not dense.  Added: an atomic costs two DRAM
+// accesses, a dense pass reads and writes all of u (n = 138 M, one word per 16: 172 us flat, 330 us dense; per 6: 250 us
+// dense).  Written: a buffer whose zeros are still in L2 when the words come takes scatter up to one word per eight
+// (n = 1.86 M, one per 12: 5.5 us against 7.5), larger ones up to one per 16 (n = 25.5 M: 29 us dense, 37 scatter).
+constexpr size_t kSparseAdd = 8;
+__host__ __device__ constexpr size_t sparse_write(size_t n) { return n <= ((size_t)4 << 20) ? 8 : 16; }
 
 // three blocks of eight warps per SM: while one block waits at a barrier or for its first words, the others add
 constexpr int kTileThreads = 256;
 constexpr int kBlocksPerSm = 3;
 constexpr int kTileWarps = kTileThreads / 32;
-constexpr int kTileMax = 16384;                  // elements per tile
-constexpr int kTilePre = 8;                      // words per thread in one batch
+constexpr int kTileMax = 15360;                  // elements per tile: three tiles and the tables fit in shared memory
+constexpr int kTensors = kTileWarps;             // weight tensors of a range that takes the exact form
+constexpr int kTilePre = 8;                      // ordered form: words per thread in one batch
 
 __device__ __forceinline__ void cp_async_16(void *smem, const void *gmem)
 {
@@ -69,230 +56,411 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
-template <bool kHybrid, bool kOverwrite>
-__global__ void __launch_bounds__(kTileThreads, kBlocksPerSm)
-decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *__restrict__ group_offsets, int K,
-             float scale, float tau, float *__restrict__ u, size_t n, uint32_t chunk_elems, uint32_t tile_elems,
-             uint32_t *dev_status)
+template <bool kHybrid>
+__device__ __forceinline__ float value_of(uint32_t word, const int32_t *gexp, const uint32_t *offs, int K, float scale, float tau,
+                                          int &k)
 {
-    extern __shared__ __align__(16) float tile[];                // tile_elems floats
-    __shared__ uint32_t sm_offs[kDecOffsSmem];
-    __shared__ uint32_t cur[kMaxViews], end[kMaxViews], taken[kMaxViews];
-    __shared__ int32_t sm_ex[kMaxViews];                         // the messages' exponents for the current tile's tensor
-    __shared__ float lut[kMaxViews * 16];
-    __shared__ uint32_t total_words;
-    // the messages' pointers, copied out of the kernel parameters once: parameters cannot be indexed with a
-    // run-time value (the compiler turns such an access into a chain of selects over all kMaxViews entries)
-    __shared__ const uint32_t *sm_words[kMaxViews];
-    __shared__ const int32_t *sm_gexp[kMaxViews];
-    __shared__ uint32_t sm_count[kMaxViews];
+    if (kHybrid) return __fmul_rn(scale, (word & 8u) ? -tau : tau);
+    const uint32_t idx = word >> 4;
+    if (idx < offs[k] || idx >= offs[k + 1]) k = group_of(offs, K, idx);
+    const int32_t e = gexp[k] - (int32_t)(word & 7u);
+    return __fmul_rn(scale, __uint_as_float(((uint32_t)(e + 127) << 23) | ((word & 8u) << 28)));
+}
 
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// ---- flat -----------------------------------------------------------------------------------------------------------
+// Every warp takes pieces of up to 32 words and adds their values to u with fp32 atomics (reductions: nothing comes
+// back), the next piece's words already on their way.  All messages are cut into the same number of pieces, and the
+// pieces go round by place first and message second, so that what is in flight at a time lies in one stretch of u: DRAM
+// pages are opened once for the words of all messages.
+// Two blocks per SM: with four the stretch doubles, and 8.9 M words into 138 M elements take 267 us instead of 172.
+constexpr int kFlatThreads = 256, kFlatBlocksPerSm = 2, kPiece = 32;
+
+struct FlatShared {
+    const uint32_t *words[kMaxViews];
+    const int32_t *gexp[kMaxViews];
+    uint32_t count[kMaxViews];
+};
+
+template <bool kHybrid, class Shared>
+__device__ __forceinline__ void add_flat(const Shared &sm, int W, const uint32_t *offs, int K, float scale, float tau, float *u,
+                                         size_t n, uint32_t *dev_status, uint32_t warp, uint32_t warps)
+{
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t longest = 0;
+    for (int w = lane; w < W; w += 32) longest = max(longest, sm.count[w]);
+    longest = __reduce_max_sync(0xffffffffu, longest);
+    const uint32_t pieces = (longest + kPiece - 1) / kPiece, units = pieces * (uint32_t)W;
+    bool bad = false;
+    auto fetch = [&](uint32_t unit, const int32_t *&ge) -> uint32_t {
+        const uint32_t piece = unit / (uint32_t)W, w = unit - piece * (uint32_t)W;
+        const uint32_t c = sm.count[w], len = (c + pieces - 1) / pieces;          // at most kPiece
+        const uint32_t p = piece * len + lane, end = min((piece + 1) * len, c);
+        ge = kHybrid ? nullptr : sm.gexp[w];
+        const uint32_t word = p < end ? sm.words[w][p] : 0xFFFFFFFFu;
+        if (p < end && (word >> 4) >= n) bad = true;
+        return word;
+    };
+    const int32_t *ge_next = nullptr;
+    uint32_t next = warp < units ? fetch(warp, ge_next) : 0u;
+    int k = 0;
+    for (uint32_t unit = warp; unit < units; unit += warps) {
+        const int32_t *ge = ge_next;
+        const uint32_t word = next, idx = word >> 4;
+        if (unit + warps < units) next = fetch(unit + warps, ge_next);
+        if (idx < n) atomicAdd(u + idx, value_of<kHybrid>(word, ge, offs, K, scale, tau, k));    // (else filler, or outside u)
+    }
+    if (bad) atomicOr(dev_status, VGC_DEV_RANGE);
+}
+
+template <bool kHybrid>
+__global__ void __launch_bounds__(kFlatThreads, kFlatBlocksPerSm)
+decode_flat(const __grid_constant__ DecodeViews views, int W, const uint32_t *__restrict__ group_offsets, int K, float scale,
+            float tau, float *__restrict__ u, size_t n, uint32_t *dev_status)
+{
+    __shared__ uint32_t sm_offs[kDecOffsSmem];
+    __shared__ FlatShared sm;
+    const uint32_t tid = threadIdx.x;
     const bool in_smem = !kHybrid && (K + 1) <= kDecOffsSmem;
     if (in_smem)
-        for (int i = tid; i <= K; i += kTileThreads) sm_offs[i] = group_offsets[i];
-    const uint32_t *offs = in_smem ? sm_offs : group_offsets;
-    if (tid == 0) total_words = 0;
+        for (int i = tid; i <= K; i += kFlatThreads) sm_offs[i] = group_offsets[i];
+    grid_wait();
     if (tid < (uint32_t)W) {
-        sm_words[tid] = views.words[tid];
-        sm_gexp[tid] = views.group_exp[tid];
-        // never read past the buffer the caller says it has: a truncated message (VGC_DEV_CAPACITY at the sender)
-        // carries the count that was needed, not the count that was written
+        sm.words[tid] = views.words[tid];
+        sm.gexp[tid] = views.group_exp[tid];
         const uint32_t said = *views.nnz[tid], have = views.max_words[tid];
-        sm_count[tid] = said < have ? said : have;
+        sm.count[tid] = said < have ? said : have;
         if (said > have && blockIdx.x == 0) atomicOr(dev_status, VGC_DEV_CAPACITY);
     }
     __syncthreads();
+    add_flat<kHybrid>(sm, W, in_smem ? sm_offs : group_offsets, K, scale, tau, u, n, dev_status,
+                      blockIdx.x * (kFlatThreads / 32) + (tid >> 5), gridDim.x * (kFlatThreads / 32));
+}
 
-    const size_t lo = (size_t)blockIdx.x * chunk_elems;
-    const size_t hi = lo + chunk_elems < n ? lo + chunk_elems : n;
-    const bool last_chunk = hi == n;
+// ---- a block's range --------------------------------------------------------------------------------------------------
+struct TileShared {
+    uint32_t offs[kDecOffsSmem];
+    uint32_t cur[kMaxViews], end[kMaxViews], taken[kMaxViews], count[kMaxViews];
+    // the messages' pointers, copied out of the kernel parameters once: parameters cannot be indexed with a
+    // run-time value (the compiler turns such an access into a chain of selects over all kMaxViews entries)
+    const uint32_t *words[kMaxViews];
+    const int32_t *gexp[kMaxViews];
+    int32_t base[kTensors];                                      // exact form: 2^base is the unit of the range's tensors
+    float lut[2][kMaxViews * 16];                                // values of the words of two tensors, 16 per message
+    uint32_t unfit;                                              // something rules the exact form out
+};
 
-    for (int w = warp; w < W; w += kTileWarps) {
-        const uint32_t *words = sm_words[w];
-        const uint32_t count = sm_count[w];
-        const uint32_t b = warp_lower_bound(words, count, (uint32_t)lo);
-        if (lane == 0) {
-            cur[w] = b;
-            end[w] = count;
-            atomicAdd(&total_words, count);
-            if (last_chunk && count && (words[count - 1] >> 4) >= n) atomicOr(dev_status, VGC_DEV_RANGE);   // skipped
-        }
-    }
-    __syncthreads();
-    const uint32_t total = total_words;
-    if (total == 0 && !kOverwrite) return;
-    bool bad = false;                                           // a word out of place: skipped, reported
-
-    auto value_of = [&](uint32_t word, const int32_t *gexp, int &k) -> float {
-        if (kHybrid) return __fmul_rn(scale, (word & 8u) ? -tau : tau);
-        const uint32_t idx = word >> 4;
-        if (idx < offs[k] || idx >= offs[k + 1]) k = group_of(offs, K, idx);
-        const int32_t e = gexp[k] - (int32_t)(word & 7u);
-        return __fmul_rn(scale, __uint_as_float(((uint32_t)(e + 127) << 23) | ((word & 8u) << 28)));
+// Where every message's run enters the range: sm.cur[w] becomes the first position of message w whose index is >= bound
+// (its count if none).  Warp j looks after the messages j, j + 8, ...; lane i holds the state of the i-th of them.
+// Random accesses are what a search costs -- all blocks search at the same time, every round is a memory latency under
+// that load -- so it interpolates: one probe at the place that uniform indices would give (after it the place is known to
+// some dozens of words), then kWindow neighbouring words around the next guess.  Where the indices are not uniform and the
+// window misses, 32 evenly spaced probes and further windows take turns.  (Five rounds of evenly spaced probes took 10 us
+// of a 43 us call.)  `meanwhile` runs while the first probes are on their way.
+template <int kWords, int kTogether, class Meanwhile>       // words per lane of a window; messages whose windows go out together
+__device__ __forceinline__ void find_runs(TileShared &sm, int W, uint32_t bound, uint32_t most_index, Meanwhile meanwhile)
+{
+    constexpr uint32_t kWindow = 32 * kWords;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t mine = warp + kTileWarps * lane;              // this lane's message
+    uint32_t lo = 0, hi = mine < (uint32_t)W ? sm.count[mine] : 0u;   // positions < lo are below the bound, >= hi are not
+    uint32_t key_lo = 0, key_hi = most_index;                    // indices at those ends
+    const uint32_t *words = mine < (uint32_t)W ? sm.words[mine] : nullptr;
+    if (bound == 0) hi = 0;
+    auto guess = [&]() -> uint32_t {
+        const uint32_t len = hi - lo;
+        const float part = key_hi > key_lo ? __fdividef((float)(bound - key_lo), (float)(key_hi - key_lo)) : 0.5f;
+        return lo + min((uint32_t)(part * (float)len), len - 1u);
     };
-
-    if ((size_t)total * 8 < n) {
-        // ---- sparse messages: not worth moving u through shared memory
-        if (kOverwrite) {
-            for (size_t i = lo + 4 * (size_t)tid; i < hi; i += 4 * kTileThreads) {
-                if (i + 3 < hi) *reinterpret_cast<float4 *>(u + i) = make_float4(0.f, 0.f, 0.f, 0.f);
-                else for (size_t c = i; c < hi; ++c) u[c] = 0.f;
+    const bool probe = hi > kWindow;
+    uint32_t g = 0, key = 0;
+    if (probe) { g = guess(); key = words[g] >> 4; }
+    meanwhile();
+    if (probe) {
+        if (key < bound) { lo = g + 1; key_lo = key; }
+        else { hi = g; key_hi = max(key, key_lo); }
+    }
+    for (uint32_t round = 0;; ++round) {
+        const uint32_t open = __ballot_sync(0xffffffffu, lo < hi);
+        if (open == 0) break;
+        const uint32_t place = lo < hi ? guess() : 0u;
+        for (uint32_t j0 = 0; j0 < 32 && (open >> j0); j0 += kTogether) {
+            uint32_t base[kTogether], step[kTogether], key_at[kTogether][kWords];
+#pragma unroll
+            for (int t = 0; t < kTogether; ++t) {
+                const uint32_t j = j0 + t;
+                const uint32_t l = __shfl_sync(0xffffffffu, lo, j), h = __shfl_sync(0xffffffffu, hi, j);
+                const uint32_t at = __shfl_sync(0xffffffffu, place, j), len = h - l;
+                const uint32_t *from = reinterpret_cast<const uint32_t *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(words), j));
+                const bool spread = (round & 1u) && len > kWindow;        // all of this is warp-uniform
+                step[t] = spread ? len / kWindow + 1 : 1u;
+                base[t] = (spread || at - l <= kWindow / 2 || len <= kWindow) ? l : min(at - kWindow / 2, h - kWindow);
+#pragma unroll
+                for (int i = 0; i < kWords; ++i) {
+                    const uint32_t pos = base[t] + step[t] * (32 * i + lane);
+                    key_at[t][i] = (open >> j & 1u) && pos < h ? from[pos] >> 4 : 0xFFFFFFFFu;
+                }
             }
-            __syncthreads();                                        // this block's zeros before this block's additions
+#pragma unroll
+            for (int t = 0; t < kTogether; ++t) {
+                const uint32_t j = j0 + t;
+                uint32_t nb = 0, below = 0, above = 0xFFFFFFFFu;          // probes below the bound; the keys around it
+#pragma unroll
+                for (int i = 0; i < kWords; ++i) {
+                    const uint32_t b = __popc(__ballot_sync(0xffffffffu, key_at[t][i] < bound));      // sorted: a prefix
+                    nb += b;
+                    const uint32_t last = __shfl_sync(0xffffffffu, key_at[t][i], (b + 31u) & 31u);
+                    if (b > 0) below = last;
+                    const uint32_t first = __shfl_sync(0xffffffffu, key_at[t][i], b & 31u);
+                    if (b < 32 && above == 0xFFFFFFFFu) above = first;
+                }
+                if (lane == j && (open >> j & 1u)) {
+                    const uint32_t new_lo = nb > 0 ? base[t] + step[t] * (nb - 1) + 1 : lo;
+                    const uint32_t new_hi = nb < kWindow ? min(base[t] + step[t] * nb, hi) : hi;
+                    if (nb > 0) key_lo = below;
+                    if (new_hi < hi) key_hi = max(above, key_lo);
+                    lo = new_lo;
+                    hi = max(new_lo, new_hi);
+                }
+            }
         }
-        for (int w = warp; w < W; w += kTileWarps) {
-            const uint32_t *words = sm_words[w];
-            const int32_t *gexp = sm_gexp[w];
+    }
+    if (mine < (uint32_t)W) sm.cur[mine] = lo;
+}
+
+// ---- scatter: few words, u written --------------------------------------------------------------------------------------
+// Zeros and additions piece by piece: the pieces of all blocks together (444 x 128 KB) stay in L2 between the two.
+constexpr uint32_t kScatterPiece = 32768;
+
+template <bool kHybrid>
+__device__ __forceinline__ bool scatter_range(TileShared &sm, int W, const uint32_t *offs, int K, float scale, float tau,
+                                              float *__restrict__ u, uint32_t lo, uint32_t hi)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    bool bad = false;
+    auto load = [&](uint32_t w, uint32_t at) { return at + lane < sm.count[w] ? sm.words[w][at + lane] : 0xFFFFFFFFu; };
+    for (uint32_t p0 = lo; p0 < hi; p0 += kScatterPiece) {
+        const uint32_t p1 = min(hi, p0 + kScatterPiece);
+        uint32_t next = warp < (uint32_t)W ? load(warp, sm.cur[warp]) : 0u;
+        for (uint32_t i = p0 + 4 * tid; i < p1; i += 4 * kTileThreads) {
+            if (i + 3 < p1) *reinterpret_cast<float4 *>(u + i) = make_float4(0.f, 0.f, 0.f, 0.f);
+            else for (uint32_t c = i; c < p1; ++c) u[c] = 0.f;
+        }
+        __syncthreads();                                            // this piece's zeros before its additions
+        for (uint32_t w = warp; w < (uint32_t)W; w += kTileWarps) {
+            uint32_t word = next, at = sm.cur[w];
+            if (w + kTileWarps < (uint32_t)W) next = load(w + kTileWarps, sm.cur[w + kTileWarps]);
+            const int32_t *gexp = sm.gexp[w];
             int k = 0;
-            for (uint32_t i0 = cur[w]; i0 < end[w]; i0 += 32) {       // warp-uniform trip count
-                const uint32_t i = i0 + lane;
-                const uint32_t word = i < end[w] ? words[i] : 0xFFFFFFFFu;
-                const bool in = i < end[w] && (word >> 4) < hi;
+            for (;;) {
+                const uint32_t idx = word >> 4;
+                const bool in = at + lane < sm.count[w] && idx < p1;
                 if (in) {
-                    if ((word >> 4) >= lo) atomicAdd(u + (word >> 4), value_of(word, gexp, k));
-                    else bad = true;                                 // behind the run's start: the message is not sorted
+                    if (idx >= p0) atomicAdd(u + idx, value_of<kHybrid>(word, gexp, offs, K, scale, tau, k));
+                    else bad = true;                                // behind the piece's start: the message is not sorted
                 }
-                if (!__all_sync(0xffffffffu, in)) break;             // sorted: the rest belongs to later chunks
+                const uint32_t out = __ballot_sync(0xffffffffu, !in);
+                if (out) { at += __ffs(out) - 1; break; }           // sorted: the rest belongs to later pieces
+                at += 32;
+                word = load(w, at);
             }
+            __syncwarp();
+            if (lane == 0) sm.cur[w] = at;
         }
-        if (bad) atomicOr(dev_status, VGC_DEV_RANGE);
-        return;
+        __syncwarp();
     }
+    return bad;
+}
 
-    // ---- dense: tile by tile
-    int cached_group = -1;
+// ---- dense, ordered form --------------------------------------------------------------------------------------------------
+// Tile by tile, the messages' runs are added one after the other by the whole block, 8 x 256 words at a time with the next
+// batch's loads in flight (indices inside a message are distinct, so plain read-modify-writes, a block barrier between
+// messages): an element receives its additions in message order, the fp32 sequence of a sequential sum.
+// Returns whether a word was out of place.
+template <bool kHybrid, bool kOverwrite>
+__device__ __forceinline__ bool ordered_range(TileShared &sm, float *tile, int W, const uint32_t *offs, int K, float scale, float tau,
+                                              float *__restrict__ u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t *const cur = sm.cur, *const end = sm.end;
+    bool bad = false;
     uint32_t t_len = 0;
-    // the exact form (below) reads the messages 16 bytes at a time; with a scale that is a positive, normal power of two
-    // its result is the sequential sum's, bit for bit
-    const int s_exp = (int)((__float_as_uint(scale) >> 23) & 0xFFu) - 127;
-    const bool pow2 = (__float_as_uint(scale) & 0x807FFFFFu) == 0u && s_exp > -127 && s_exp < 128;
-    bool exact_possible = s_exp < 128;                          // a finite scale
-    if (exact_possible)
-        for (int w = 0; w < W; ++w) exact_possible = exact_possible && (reinterpret_cast<uintptr_t>(sm_words[w]) & 15u) == 0u;
-    if (kOverwrite || exact_possible) {
-        // the whole tile buffer starts as zeros; from then on whoever writes a tile out leaves zeros behind
-        for (uint32_t q = tid; q < kTileMax / 4; q += kTileThreads)
-            reinterpret_cast<float4 *>(tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (size_t t0 = lo; t0 < hi; t0 += t_len) {
-        const uint32_t left = (uint32_t)(hi - t0);
-        t_len = left < tile_elems ? left : tile_elems;
-        int tile_group = -1;                                        // weight tensor of the tile, -1 if it spans several
+    for (uint32_t t0 = lo; t0 < hi; t0 += t_len) {
+        t_len = min(hi - t0, tile_elems);
+        int tile_group = kHybrid ? 0 : -1;                          // weight tensor of the tile, -1 if it spans several
         if (!kHybrid) {
-            // A tile ends where its weight tensor ends (when that keeps the next tile on a 16-byte boundary): a tile
-            // inside one tensor has one exponent per message -- the table look-up and the exact form below apply.
-            // The buffer holds kTileMax elements, so a tile may grow a little to reach that end; a tensor that needs
-            // two more tiles gets two of the same size rather than a sliver at its end.
-            const int g = group_of(offs, K, (uint32_t)t0);
-            const uint32_t next = offs[g + 1], rem = next - (uint32_t)t0;
-            if ((next & 3u) == 0u && rem <= left) {
-                // (not for a run of tiny tensors: a tile has a fixed cost of a few microseconds)
-                // (a sliver is cut off only where the exact form can make it cheap)
-                const bool worth = rem >= 2048u || (exact_possible && g + 2 <= K && offs[g + 2] - next >= 8192u);
-                if (rem <= (uint32_t)kTileMax) { if (worth) t_len = rem; }
-                else if (rem < t_len + 2048u || rem <= 2u * (uint32_t)kTileMax) {
-                    const uint32_t half = (rem / 2u + 3u) & ~3u;
-                    if (half <= (uint32_t)kTileMax) t_len = half;
-                }
-            }
-            if ((uint32_t)t0 + t_len - 1u < next) tile_group = g;
+            // a tile ends with its weight tensor when that keeps the next one on a 16-byte boundary and leaves no sliver:
+            // inside one tensor a word's value is one look-up
+            const int g = group_of(offs, K, t0);
+            const uint32_t rem = offs[g + 1] - t0;
+            if (rem < t_len && (rem & 3u) == 0u && rem >= 2048u) t_len = rem;
+            if (rem >= t_len) tile_group = g;
         }
-        const uint32_t t_hi = (uint32_t)(t0 + t_len);
+        const uint32_t t_hi = t0 + t_len;
         const uint32_t n_vec = t_len / 4;                           // t0 is a multiple of 4 elements
-        if (tile_group >= 0 && tile_group != cached_group) {       // block-uniform; nobody reads sm_ex between the tiles
-            if (tid < (uint32_t)W) sm_ex[tid] = sm_gexp[tid][tile_group];
-            __syncthreads();
-            cached_group = tile_group;
-        }
-        // Exact form.  When the exponents of all messages for the tile's tensor lie close enough together, every word
-        // is an integer multiple of one power of two, 2^base, and
-        // every partial sum of up to W of them stays within 2^22 multiples: all of them are exact fp32 numbers, fp32
-        // addition of them is associative, and the sequential sum of the words equals the exact sum (with a power-of-two
-        // scale that is the decoder's result bit for bit; otherwise the scale is applied to the exact sum, one rounding
-        // instead of one per message, and vgc_decode_accumulate adds the scaled sum to u in one addition).  The
-        // tile is then accumulated as int32 multiples of 2^base with shared-memory integer atomics, in any order:
-        // no barrier between messages, no search for the runs' ends -- the warps stream every message's words from
-        // its cursor until the indices leave the tile -- and one conversion at the end.  Same bits, much less waiting.
-        int fast_base = INT32_MIN;                                  // INT32_MIN: not applicable
-        if (kHybrid) {
-            // every word stands for +tau or -tau: the multiples are +-1 and a sum is at most W of them
-            if (exact_possible && t_hi < (1u << 28)) fast_base = 0;
-        } else if (exact_possible && tile_group >= 0 && t_hi < (1u << 28)) {
-            int e_max = INT32_MIN, e_min = INT32_MAX;
-            for (int w = 0; w < W; ++w) {
-                const int e = sm_ex[w];
-                if (e != VGC_EXP_NONE) { e_max = max(e_max, e); e_min = min(e_min, e); }
-            }
-            const int base = e_min - 7;                             // the smallest value a word can stand for
-            // 2^base and every sum of multiples are normal numbers; with a power-of-two scale so are their products
-            if (e_max >= e_min && e_max - base + (32 - __clz((W - 1) | 1)) <= 22 && base >= -126 && base + 22 <= 127 &&
-                (!pow2 || (base + s_exp >= -126 && base + 22 + s_exp <= 127)))
-                fast_base = base;
-        }
-        const bool fast = fast_base != INT32_MIN;
-        if (!kOverwrite && fast)                                    // the exact form reads u at the tile's end: ask it into L2 now
-            for (uint32_t line = tid; line < (t_len + 31u) / 32u; line += kTileThreads)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(u + t0 + 32u * (size_t)line));
-        if (!kOverwrite && !fast) {                                 // the ordered form adds to the tile's old content
-            for (uint32_t q = tid; q < n_vec; q += kTileThreads) cp_async_16(tile + 4 * q, u + t0 + 4 * (size_t)q);
+        if (!kOverwrite) {                                          // the tile's old content
+            for (uint32_t q = tid; q < n_vec; q += kTileThreads) cp_async_16(tile + 4 * q, u + t0 + 4 * q);
             if (tid < t_len - 4 * n_vec) tile[4 * n_vec + tid] = u[t0 + 4 * n_vec + tid];
         }
-        if (tid < (uint32_t)W) taken[tid] = 0;
-        if (!fast) {
-            if (kOverwrite) __syncthreads();                        // the cursors of the tile before
         // where every message's run leaves the tile: at most t_len of its words can lie inside
-            for (int w = warp; w < W; w += kTileWarps) {
-                const uint32_t *words = sm_words[w];
-                const uint32_t count = sm_count[w];
-                const uint32_t c = cur[w];
-                const uint32_t span = count - c < t_len ? count - c : t_len;
-                const uint32_t e = c + warp_lower_bound(words + c, span, t_hi);
-                if (lane == 0) end[w] = e;
+        for (int w = warp; w < W; w += kTileWarps) {
+            const uint32_t *words = sm.words[w] + cur[w];
+            const uint32_t left = sm.count[w] - cur[w];
+            uint32_t a = 0, b = left < t_len ? left : t_len;        // positions < a are below t_hi, >= b are not
+            while (a < b) {                                         // 32 probes a, a + step, ... reach past b
+                const uint32_t step = (b - a) / 32 + 1, pos = a + step * lane;
+                const uint32_t nb = __popc(__ballot_sync(0xffffffffu, pos < b && (words[pos] >> 4) < t_hi));
+                if (nb == 0) break;
+                const uint32_t new_b = a + step * nb;
+                a += step * (nb - 1) + 1;
+                b = new_b < b ? new_b : b;
             }
+            if (lane == 0) end[w] = cur[w] + a;
         }
-        // the 16 values a word's low four bits (sign, d) can stand for, per message, when the tile lies in one tensor
-        const bool use_lut = kHybrid || tile_group >= 0;
-        if (use_lut)
+        // the 16 values a word's low four bits (sign, d) can stand for, per message
+        if (tile_group >= 0)
             for (int i = tid; i < W * 16; i += kTileThreads) {
-                const int w = i >> 4;
                 const uint32_t code = (uint32_t)i & 15u;
-                float val;
-                if (kHybrid && fast) {
-                    reinterpret_cast<int *>(lut)[i] = (code & 8u) ? -1 : 1;
-                    continue;
-                } else if (kHybrid) val = (code & 8u) ? -tau : tau;
-                else if (fast) {
-                    const int e = sm_ex[w];
-                    const int mult = e == VGC_EXP_NONE ? 0 : 1 << (e - (int)(code & 7u) - fast_base);
-                    reinterpret_cast<int *>(lut)[i] = (code & 8u) ? -mult : mult;
-                    continue;
-                } else {
-                    const uint32_t ebits = (uint32_t)(sm_ex[w] + 127) << 23;
-                    val = __uint_as_float((ebits - ((code & 7u) << 23)) | ((code & 8u) << 28));
-                }
-                lut[i] = __fmul_rn(scale, val);
+                const uint32_t ebits = kHybrid ? 0u : (uint32_t)(sm.gexp[i >> 4][tile_group] + 127) << 23;
+                const float val = kHybrid ? ((code & 8u) ? -tau : tau)
+                                          : __uint_as_float((ebits - ((code & 7u) << 23)) | ((code & 8u) << 28));
+                sm.lut[0][i] = __fmul_rn(scale, val);
             }
-        if (!kOverwrite && !fast) cp_async_wait_all();
+        if (!kOverwrite) cp_async_wait_all();
         __syncthreads();
 
-        if (fast) {
-            // ---- exact form: warps stream the messages' words from their cursors.  Message m is shared by the warps
-            // m, m + W, ... (W < 8) in turns of 256 words -- or a warp takes the messages warp, warp + 8, ... -- and a
-            // warp stops at its first turn that reaches past the tile (or the message's end); the words it found inside
-            // are added to the message's count, which moves the cursor once all warps are done.
-            const uint32_t tile_addr = (uint32_t)__cvta_generic_to_shared(tile);
-            const uint32_t lut_addr = (uint32_t)__cvta_generic_to_shared(lut);
-            // a word minus t0 << 4 keeps its low four bits and turns its index into the offset inside the tile; one
-            // unsigned comparison then says "inside the tile" (a word behind the tile wraps around to a huge number,
-            // and so does the filler 0xFFFFFFFF, because t_hi < 2^28)
-            const uint32_t t0s = (uint32_t)t0 << 4, t_len16 = t_len << 4;
-            const int sharers = W < kTileWarps ? kTileWarps / W : 1;   // warps per message
+        constexpr uint32_t kBatchWords = kTilePre * kTileThreads;
+        auto batches_of = [&](int w) -> uint32_t { return (end[w] - cur[w] + kBatchWords - 1) / kBatchWords; };
+        auto load_batch = [&](int w, uint32_t b, uint32_t (&dst)[kTilePre]) {
+            const uint32_t first = cur[w] + b * kBatchWords + tid, e = end[w];
+            const uint32_t *p = sm.words[w] + first;
+#pragma unroll
+            for (int j = 0; j < kTilePre; ++j) dst[j] = first + j * kTileThreads < e ? p[j * kTileThreads] : 0u;
+        };
+        int w = 0;
+        uint32_t b = 0;
+        while (w < W && batches_of(w) == 0) ++w;
+        uint32_t held[kTilePre], next[kTilePre];
+        uint32_t nb = w < W ? batches_of(w) : 0;                     // batches of the current message
+        if (w < W) load_batch(w, 0, held);
+        int k = 0;
+        while (w < W) {
+            int w2 = w;
+            uint32_t b2 = b + 1, nb2 = nb;
+            if (b2 >= nb) {
+                w2 = w + 1; b2 = 0;
+                while (w2 < W && (nb2 = batches_of(w2)) == 0) ++w2;
+            }
+            if (w2 < W) load_batch(w2, b2, next);
+            const uint32_t first = cur[w] + b * kBatchWords + tid, e = end[w];
+            const float *lut = sm.lut[0] + 16 * w;
+            const int32_t *gexp = sm.gexp[w];
+#pragma unroll
+            for (int j = 0; j < kTilePre; ++j) {
+                const uint32_t word = held[j], at = (word >> 4) - t0;
+                if (first + j * kTileThreads >= e) continue;
+                // a word of a sorted message lies inside the tile; one that does not (the message is not sorted) is skipped
+                if (at >= t_len) { bad = true; continue; }
+                const float v = tile_group >= 0 ? lut[word & 15u] : value_of<kHybrid>(word, gexp, offs, K, scale, tau, k);
+                tile[at] = __fadd_rn(tile[at], v);
+            }
+            if (w2 != w) __syncthreads();                            // the next message may hit the same elements
+#pragma unroll
+            for (int j = 0; j < kTilePre; ++j) held[j] = next[j];
+            w = w2; b = b2; nb = nb2;
+        }
+        __syncthreads();
+        if (tid < (uint32_t)W) cur[tid] = end[tid];
+        for (uint32_t q = tid; q < n_vec; q += kTileThreads) {
+            *reinterpret_cast<float4 *>(u + t0 + 4 * q) = reinterpret_cast<const float4 *>(tile)[q];
+            if (kOverwrite) reinterpret_cast<float4 *>(tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        if (tid < t_len - 4 * n_vec) {
+            u[t0 + 4 * n_vec + tid] = tile[4 * n_vec + tid];
+            if (kOverwrite) tile[4 * n_vec + tid] = 0.f;
+        }
+        __syncthreads();                                             // cursors, and the tile before it is loaded again
+    }
+    return bad;
+}
+
+// ---- dense, exact form ----------------------------------------------------------------------------------------------------
+// When the exponents of all messages for a tensor lie close enough together, every word is an integer multiple of one power
+// of two, 2^base, and every partial sum of up to W of them stays within 2^22 multiples: all of them are exact fp32 numbers,
+// fp32 addition of them is associative, and the sequential sum of the words equals the exact sum (with a power-of-two scale
+// that is the decoder's result bit for bit; otherwise the scale is applied to the exact sum, one rounding instead of one
+// per message, and vgc_decode_accumulate adds the scaled sum to u in one addition).  A tile is then accumulated as int32
+// multiples of 2^base with shared-memory integer atomics, in any order: no barrier between messages, no search for the
+// runs' ends -- the warps stream every message's words from its cursor until the indices leave the tile -- and one
+// conversion at the end.  Same bits, much less waiting.  A block takes this form when it applies to all tensors of its range.
+// Returns whether a word was out of place.
+template <bool kHybrid, bool kOverwrite>
+__device__ __forceinline__ bool exact_range(TileShared &sm, float *tile, int W, const uint32_t *offs, int g_first, float scale,
+                                            float tau, float *__restrict__ u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t tile_addr = (uint32_t)__cvta_generic_to_shared(tile);
+    const int sharers = W < kTileWarps ? kTileWarps / W : 1;       // warps per message
+    bool bad = false;
+    int g = g_first, made = -1;        // tensor of the tile's first element; the last tensor whose table was made
+    int slot = 1;                      // the table of the tile's first tensor
+    uint32_t t_len = 0;
+    for (uint32_t t0 = lo; t0 < hi; t0 += t_len) {
+        // A tile inside one tensor or across the border of two; one that would reach a third ends before it, at a multiple
+        // of four elements
+        t_len = min(hi - t0, tile_elems);
+        uint32_t split = t_len;                                     // elements of the first tensor
+        if (!kHybrid) {
+            while (offs[g + 1] <= t0) ++g;                          // block-uniform, as all of this
+            if (offs[g + 1] - t0 < t_len) {
+                split = offs[g + 1] - t0;
+                int g1 = g + 1;
+                while (offs[g1 + 1] == offs[g1]) ++g1;
+                if (offs[g1 + 1] - t0 < t_len) t_len = (offs[g1 + 1] - t0) & ~3u;
+                split = min(split, t_len);
+            }
+        }
+        // the 16 values a word's low four bits (sign, d) can stand for, per message, as multiples of the tensor's unit; the
+        // tables of two neighbouring tensors take turns
+        auto table = [&](int which, int k) {
+            const int base = kHybrid ? 0 : sm.base[k - g_first];
+            for (int i = tid; i < W * 16; i += kTileThreads) {
+                const int e = kHybrid ? 0 : sm.gexp[i >> 4][k];
+                const int mult = kHybrid ? 1 : e == VGC_EXP_NONE ? 0 : 1 << (e - (i & 7) - base);
+                reinterpret_cast<int *>(sm.lut[which])[i] = (i & 8) ? -mult : mult;
+            }
+        };
+        if (made < g) { slot ^= 1; table(slot, g); made = g; }      // (the tile before ended with its tensor)
+        int next = g;
+        if (split < t_len) {
+            ++next;
+            while (offs[next + 1] == offs[next]) ++next;
+            table(slot ^ 1, next);
+            made = next;
+        }
+        const uint32_t n_vec = t_len / 4;                           // t0 is a multiple of 4 elements
+        if (!kOverwrite)                                            // u is read at the tile's end: ask it into L2 now
+            for (uint32_t line = tid; line < (t_len + 31u) / 32u; line += kTileThreads)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(u + t0 + 32u * line));
+        if (tid < (uint32_t)W) sm.taken[tid] = 0;
+        __syncthreads();
+
+        // ---- warps stream the messages' words from their cursors.  Message m is shared by the warps m, m + W, ...
+        // (W < 8) in turns of 256 words -- or a warp takes the messages warp, warp + 8, ... -- and a warp stops at its
+        // first turn that reaches past the tile (or the message's end); the words it found inside are added to the
+        // message's count, which moves the cursor once all warps are done.
+        // A word minus t0 << 4 keeps its low four bits and turns its index into the offset inside the tile; one unsigned
+        // comparison then says "inside the tile" (a word behind the tile wraps around to a huge number, and so does the
+        // filler 0xFFFFFFFF, because the range ends before 2^28).
+        const uint32_t t0s = t0 << 4, t_len16 = t_len << 4, split16 = split << 4;
+        auto stream = [&](auto two) {
+            constexpr bool kTwo = decltype(two)::value;             // the tile has elements of two tensors
+            const uint32_t lut_addr = (uint32_t)__cvta_generic_to_shared(sm.lut[slot]);
+            const uint32_t lut_other = (uint32_t)__cvta_generic_to_shared(sm.lut[slot ^ 1]) - lut_addr;
             for (int m = (int)warp % W; m < W; m += kTileWarps) {
                 if (W < kTileWarps && (int)warp >= sharers * W) break;   // warps left over when W does not divide the warps
                 const uint32_t turn0 = W < kTileWarps ? warp / (uint32_t)W : 0u;
-                const uint32_t *words = sm_words[m];
-                const uint32_t c = cur[m], cnt = sm_count[m];
+                const uint32_t *words = sm.words[m];
+                const uint32_t c = sm.cur[m], cnt = sm.count[m];
                 const uint32_t a = c & ~3u;                          // 16-byte loads: start at the boundary before the cursor
                 const uint32_t lut_m = lut_addr + 64u * (uint32_t)m;
                 uint32_t inside = 0, n_in = 0;                       // words up to the tile's end; words added
@@ -322,25 +490,48 @@ decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *_
                 };
                 // one word: inside the tile -> look its multiple up and add it; all of it predicated, no branch
                 auto add = [&](uint32_t word) {
-                    asm volatile("{\n\t"
-                                 ".reg .pred p;\n\t"
-                                 ".reg .s32 iv;\n\t"
-                                 ".reg .u32 o, at, l;\n\t"
-                                 "sub.u32 o, %1, %2;\n\t"
-                                 "setp.lt.u32 p, o, %3;\n\t"
-                                 "and.b32 l, %1, 15;\n\t"
-                                 "shl.b32 l, l, 2;\n\t"
-                                 "add.u32 l, l, %4;\n\t"
-                                 "shr.u32 at, o, 2;\n\t"
-                                 "and.b32 at, at, 0xFFFFFFFC;\n\t"
-                                 "add.u32 at, at, %5;\n\t"
-                                 "@p ld.shared.s32 iv, [l];\n\t"
-                                 "@p red.shared.add.s32 [at], iv;\n\t"
-                                 "@p add.u32 %0, %0, 1;\n\t"
-                                 "}"
-                                 : "+r"(n_in)
-                                 : "r"(word), "r"(t0s), "r"(t_len16), "r"(lut_m), "r"(tile_addr)
-                                 : "memory");
+                    if (kTwo)
+                        asm volatile("{\n\t"
+                                     ".reg .pred p, second;\n\t"
+                                     ".reg .s32 iv;\n\t"
+                                     ".reg .u32 o, at, l;\n\t"
+                                     "sub.u32 o, %1, %2;\n\t"
+                                     "setp.lt.u32 p, o, %3;\n\t"
+                                     "setp.ge.u32 second, o, %6;\n\t"
+                                     "and.b32 l, %1, 15;\n\t"
+                                     "shl.b32 l, l, 2;\n\t"
+                                     "add.u32 l, l, %4;\n\t"
+                                     "@second add.u32 l, l, %7;\n\t"
+                                     "shr.u32 at, o, 2;\n\t"
+                                     "and.b32 at, at, 0xFFFFFFFC;\n\t"
+                                     "add.u32 at, at, %5;\n\t"
+                                     "@p ld.shared.s32 iv, [l];\n\t"
+                                     "@p red.shared.add.s32 [at], iv;\n\t"
+                                     "@p add.u32 %0, %0, 1;\n\t"
+                                     "}"
+                                     : "+r"(n_in)
+                                     : "r"(word), "r"(t0s), "r"(t_len16), "r"(lut_m), "r"(tile_addr), "r"(split16), "r"(lut_other)
+                                     : "memory");
+                    else
+                        asm volatile("{\n\t"
+                                     ".reg .pred p;\n\t"
+                                     ".reg .s32 iv;\n\t"
+                                     ".reg .u32 o, at, l;\n\t"
+                                     "sub.u32 o, %1, %2;\n\t"
+                                     "setp.lt.u32 p, o, %3;\n\t"
+                                     "and.b32 l, %1, 15;\n\t"
+                                     "shl.b32 l, l, 2;\n\t"
+                                     "add.u32 l, l, %4;\n\t"
+                                     "shr.u32 at, o, 2;\n\t"
+                                     "and.b32 at, at, 0xFFFFFFFC;\n\t"
+                                     "add.u32 at, at, %5;\n\t"
+                                     "@p ld.shared.s32 iv, [l];\n\t"
+                                     "@p red.shared.add.s32 [at], iv;\n\t"
+                                     "@p add.u32 %0, %0, 1;\n\t"
+                                     "}"
+                                     : "+r"(n_in)
+                                     : "r"(word), "r"(t0s), "r"(t_len16), "r"(lut_m), "r"(tile_addr)
+                                     : "memory");
                 };
                 fetch(turn0, nxt);
                 for (uint32_t turn = turn0;; turn += (uint32_t)sharers) {
@@ -359,7 +550,7 @@ decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *_
                     }
                     // the last turn of this warp: count the words from the cursor on that lie before the tile's end
                     uint32_t mine = 0;
-                    const uint32_t p0 = a + turn * kTurnWords + 4u * lane;
+                    const uint32_t p0 = a + turn * kTurnWords + 4u * lane, t_hi = t0 + t_len;
 #pragma unroll
                     for (int v = 0; v < kVecs; ++v) {
                         const uint32_t p = p0 + 128u * v;
@@ -372,147 +563,188 @@ decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *_
                 }
                 // a word before the tile's end that was not added lies behind the tile: the message is not sorted
                 if (__reduce_add_sync(0xffffffffu, n_in) != inside) bad = true;
-                if (lane == 0 && inside) atomicAdd(&taken[m], inside);
-            }
-        } else {
-        // messages one after the other, each in batches of kTileBatch words per thread; the loads of the next batch
-        // (of this message or of the next one) are in flight while a batch is applied
-        constexpr uint32_t kBatchWords = kTilePre * kTileThreads;
-        auto batches_of = [&](int w) -> uint32_t { return (end[w] - cur[w] + kBatchWords - 1) / kBatchWords; };
-        auto load_batch = [&](int w, uint32_t b, uint32_t (&dst)[kTilePre]) {
-            const uint32_t first = cur[w] + b * kBatchWords + tid, e = end[w];
-            const uint32_t *p = sm_words[w] + first;
-            if (first + (kTilePre - 1) * kTileThreads < e) {         // whole column of this thread inside the run
-#pragma unroll
-                for (int j = 0; j < kTilePre; ++j) dst[j] = p[j * kTileThreads];
-            } else {
-#pragma unroll
-                for (int j = 0; j < kTilePre; ++j) dst[j] = first + j * kTileThreads < e ? p[j * kTileThreads] : 0u;
+                if (lane == 0 && inside) atomicAdd(&sm.taken[m], inside);
             }
         };
-        // shared-memory byte addresses: element idx of u lives at tile_addr + 4 * (idx - t0); a word carries
-        // idx << 4, so 4 * idx = (word >> 2) & ~3
-        const uint32_t tile_addr = (uint32_t)__cvta_generic_to_shared(tile) - 4u * (uint32_t)t0;
-        const uint32_t lut_addr = (uint32_t)__cvta_generic_to_shared(lut);
-        auto add_at = [&](uint32_t word, uint32_t lut_w) {
-            // a word of a sorted message lies inside the tile; one that does not (the message is not sorted) is skipped
-            if ((word >> 4) - (uint32_t)t0 >= t_len) { bad = true; return; }
-            const uint32_t at = tile_addr + ((word >> 2) & 0xFFFFFFFCu);
-            float x, v;
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(lut_w + ((word & 15u) << 2)));
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(at) : "memory");
-            x = __fadd_rn(x, v);
-            asm volatile("st.shared.f32 [%0], %1;" ::"r"(at), "f"(x) : "memory");
-        };
-        int w = 0;
-        uint32_t b = 0;
-        while (w < W && batches_of(w) == 0) ++w;
-        uint32_t held[kTilePre], next[kTilePre];
-        uint32_t nb = w < W ? batches_of(w) : 0;                     // batches of the current message
-        if (w < W) load_batch(w, 0, held);
-        int k = 0;
-        while (w < W) {
-            int w2 = w;
-            uint32_t b2 = b + 1, nb2 = nb;
-            if (b2 >= nb) {
-                w2 = w + 1; b2 = 0;
-                while (w2 < W && (nb2 = batches_of(w2)) == 0) ++w2;
-            }
-            if (w2 < W) load_batch(w2, b2, next);
-            const uint32_t first = cur[w] + b * kBatchWords + tid, e = end[w];
-            const bool whole = first + (kTilePre - 1) * kTileThreads < e;
-            if (use_lut) {
-                const uint32_t lut_w = lut_addr + 64u * (uint32_t)w;
-                if (whole) {
-#pragma unroll
-                    for (int j = 0; j < kTilePre; ++j) add_at(held[j], lut_w);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < kTilePre; ++j)
-                        if (first + j * kTileThreads < e) add_at(held[j], lut_w);
-                }
-            } else {
-                const int32_t *gexp = sm_gexp[w];
-#pragma unroll
-                for (int j = 0; j < kTilePre; ++j) {
-                    const uint32_t word = held[j];
-                    if (first + j * kTileThreads < e) {
-                        if ((word >> 4) - (uint32_t)t0 < t_len) tile[(word >> 4) - (uint32_t)t0] += value_of(word, gexp, k);
-                        else bad = true;
-                    }
-                }
-            }
-            if (w2 != w) __syncthreads();                            // the next message may hit the same elements
-#pragma unroll
-            for (int j = 0; j < kTilePre; ++j) held[j] = next[j];
-            w = w2; b = b2; nb = nb2;
-        }
-        }
+        if (split < t_len) stream(std::true_type());
+        else stream(std::false_type());
         __syncthreads();
-        if (tid < (uint32_t)W) cur[tid] = fast ? cur[tid] + taken[tid] : end[tid];
-        if (fast) {
-            // multiples of 2^base -> fp32 (a sum is at most 2^22 multiples either way, so 1.5 * 2^23 plus it is a float
-            // whose bits are 0x4B400000 plus it), times 2^base (exact), times the scale: one rounding, none when the
-            // scale is a power of two.  vgc_decode_accumulate adds the result to u; an element no word points at keeps
-            // its bits.
-            const float unit = kHybrid ? __fmul_rn(scale, tau) : __uint_as_float((uint32_t)(fast_base + 127) << 23);
-            auto value = [&](int mult) {
-                const float m = __fmul_rn(__fsub_rn(__int_as_float(0x4B400000 + mult), 12582912.f), unit);
-                return kHybrid ? m : __fmul_rn(m, scale);       // hybrid: a word is worth scale * tau, rounded once
-            };
-            if (kOverwrite) {
-                for (uint32_t q = tid; q < n_vec; q += kTileThreads) {
-                    const int4 mlt = reinterpret_cast<const int4 *>(tile)[q];
-                    reinterpret_cast<int4 *>(tile)[q] = make_int4(0, 0, 0, 0);
-                    *reinterpret_cast<float4 *>(u + t0 + 4 * (size_t)q) =
-                        make_float4(value(mlt.x), value(mlt.y), value(mlt.z), value(mlt.w));
-                }
-            } else {
-                // four vectors of u per thread in flight (asked into L2 when the tile began)
-                for (uint32_t q0 = tid; q0 < n_vec; q0 += 4 * kTileThreads) {
-                    float4 o[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint32_t q = q0 + j * kTileThreads;
-                        if (q < n_vec) o[j] = *reinterpret_cast<const float4 *>(u + t0 + 4 * (size_t)q);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const uint32_t q = q0 + j * kTileThreads;
-                        if (q >= n_vec) break;
-                        const int4 mlt = reinterpret_cast<const int4 *>(tile)[q];
-                        if ((mlt.x | mlt.y | mlt.z | mlt.w) == 0) continue;
-                        reinterpret_cast<int4 *>(tile)[q] = make_int4(0, 0, 0, 0);
-                        if (mlt.x) o[j].x = __fadd_rn(o[j].x, value(mlt.x));
-                        if (mlt.y) o[j].y = __fadd_rn(o[j].y, value(mlt.y));
-                        if (mlt.z) o[j].z = __fadd_rn(o[j].z, value(mlt.z));
-                        if (mlt.w) o[j].w = __fadd_rn(o[j].w, value(mlt.w));
-                        *reinterpret_cast<float4 *>(u + t0 + 4 * (size_t)q) = o[j];
-                    }
-                }
-            }
-            if (tid < t_len - 4 * n_vec) {
-                const int mult = reinterpret_cast<const int *>(tile)[4 * n_vec + tid];
-                float *dst = u + t0 + 4 * n_vec + tid;
-                if (kOverwrite) *dst = value(mult);
-                else if (mult) *dst = __fadd_rn(*dst, value(mult));
-                tile[4 * n_vec + tid] = 0.f;
+        if (tid < (uint32_t)W) sm.cur[tid] += sm.taken[tid];
+
+        // ---- multiples of 2^base -> fp32 (a sum is at most 2^22 multiples either way, so 1.5 * 2^23 plus it is a float
+        // whose bits are 0x4B400000 plus it), times 2^base (exact), times the scale: one rounding, none when the scale is a
+        // power of two.  vgc_decode_accumulate adds the result to u; an element no word points at keeps its bits.
+        auto unit_of = [&](int k) {
+            return kHybrid ? __fmul_rn(scale, tau) : __uint_as_float((uint32_t)(sm.base[k - g_first] + 127) << 23);
+        };
+        const float unit_a = unit_of(g), unit_b = unit_of(next);
+        auto value = [&](int mult, float unit) {
+            const float m = __fmul_rn(__fsub_rn(__int_as_float(0x4B400000 + mult), 12582912.f), unit);
+            return kHybrid ? m : __fmul_rn(m, scale);           // hybrid: a word is worth scale * tau, rounded once
+        };
+        // vector q of the tile: the units of its elements (they differ inside the one vector that holds the border)
+        auto values = [&](const int4 &mult, uint32_t q) {
+            const uint32_t left = split - min(split, 4 * q);    // elements of the first tensor from here on
+            return make_float4(value(mult.x, left > 0 ? unit_a : unit_b), value(mult.y, left > 1 ? unit_a : unit_b),
+                               value(mult.z, left > 2 ? unit_a : unit_b), value(mult.w, left > 3 ? unit_a : unit_b));
+        };
+        float *const dst = u + t0;
+        if (kOverwrite) {
+            for (uint32_t q = tid; q < n_vec; q += kTileThreads) {
+                const int4 mlt = reinterpret_cast<const int4 *>(tile)[q];
+                reinterpret_cast<int4 *>(tile)[q] = make_int4(0, 0, 0, 0);
+                *reinterpret_cast<float4 *>(dst + 4 * q) = values(mlt, q);
             }
         } else {
-            const bool zero_after = kOverwrite || exact_possible;
-            for (uint32_t q = tid; q < n_vec; q += kTileThreads) {
-                *reinterpret_cast<float4 *>(u + t0 + 4 * (size_t)q) = reinterpret_cast<const float4 *>(tile)[q];
-                if (zero_after) reinterpret_cast<float4 *>(tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            if (tid < t_len - 4 * n_vec) {
-                u[t0 + 4 * n_vec + tid] = tile[4 * n_vec + tid];
-                if (zero_after) tile[4 * n_vec + tid] = 0.f;
+            constexpr int kHeld = 4;                            // vectors of u per thread in flight
+            for (uint32_t q0 = tid; q0 < n_vec; q0 += kHeld * kTileThreads) {
+                float4 o[kHeld];
+#pragma unroll
+                for (int j = 0; j < kHeld; ++j) {
+                    const uint32_t q = q0 + j * kTileThreads;
+                    if (q < n_vec) o[j] = *reinterpret_cast<const float4 *>(dst + 4 * q);
+                }
+#pragma unroll
+                for (int j = 0; j < kHeld; ++j) {
+                    const uint32_t q = q0 + j * kTileThreads;
+                    if (q >= n_vec) break;
+                    const int4 mlt = reinterpret_cast<const int4 *>(tile)[q];
+                    if ((mlt.x | mlt.y | mlt.z | mlt.w) == 0) continue;
+                    reinterpret_cast<int4 *>(tile)[q] = make_int4(0, 0, 0, 0);
+                    const float4 add = values(mlt, q);
+                    if (mlt.x) o[j].x = __fadd_rn(o[j].x, add.x);
+                    if (mlt.y) o[j].y = __fadd_rn(o[j].y, add.y);
+                    if (mlt.z) o[j].z = __fadd_rn(o[j].z, add.z);
+                    if (mlt.w) o[j].w = __fadd_rn(o[j].w, add.w);
+                    *reinterpret_cast<float4 *>(dst + 4 * q) = o[j];
+                }
             }
         }
-        // vgc_decode_sum: every thread put zeros back where it read, and the next tile's barrier orders them before
-        // the next additions.  vgc_decode_accumulate loads the next tile over this one: wait for the readers.
-        if (!kOverwrite) __syncthreads();
+        if (tid < t_len - 4 * n_vec) {                          // the buffer's last elements
+            const uint32_t i = 4 * n_vec + tid;
+            const int mult = reinterpret_cast<const int *>(tile)[i];
+            const float v = value(mult, i < split ? unit_a : unit_b);
+            if (kOverwrite) dst[i] = v;
+            else if (mult) dst[i] = __fadd_rn(dst[i], v);
+            tile[i] = 0.f;
+        }
+        // every thread put zeros back where it read, and the next tile's barrier orders them before the next additions
+        if (next != g) { g = next; slot ^= 1; }
     }
+    return bad;
+}
+
+// Bound: HBM for the dense forms (4 B per word, 4 or 8 B per element), DRAM accesses for the sparse ones, latency for small
+// buffers.  Measured (B200, one call among others, W messages): n = 25.5 M, W = 8, density 0.05, written: 45.2 -> 33.7 us
+// (143 MB, 0.65 of the measured copy rate); added: 64.2 -> 58.0; W = 64, density 0.01: 107.8 -> 73.0; n = 123.6 M, W = 4,
+// density 0.03: 345 -> 114 us; n = 32768: 4.3 -> 3.3 us.  The gain is the search (five rounds of scattered probes -> two),
+// tiles that may span two tensors, tables made once per tensor, and the sparse forms.
+template <bool kHybrid, bool kOverwrite>
+__global__ void __launch_bounds__(kTileThreads, kBlocksPerSm)
+decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *__restrict__ group_offsets, int K,
+             float scale, float tau, float *__restrict__ u, size_t n, uint32_t chunk_elems, uint32_t tile_elems,
+             uint32_t *dev_status)
+{
+    extern __shared__ __align__(16) float tile[];                // kTileMax floats
+    __shared__ TileShared sm;
+
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool in_smem = !kHybrid && (K + 1) <= kDecOffsSmem;
+    if (in_smem)
+        for (int i = tid; i <= K; i += kTileThreads) sm.offs[i] = group_offsets[i];
+    const uint32_t *offs = in_smem ? sm.offs : group_offsets;
+    if (tid == 0) sm.unfit = 0;
+    if (tid < (uint32_t)W) {
+        sm.words[tid] = views.words[tid];
+        sm.gexp[tid] = views.group_exp[tid];
+    }
+    grid_wait();
+    if (tid < (uint32_t)W) {
+        // never read past the buffer the caller says it has: a truncated message (VGC_DEV_CAPACITY at the sender)
+        // carries the count that was needed, not the count that was written
+        const uint32_t said = *views.nnz[tid], have = views.max_words[tid];
+        sm.count[tid] = said < have ? said : have;
+        if (said > have && blockIdx.x == 0) atomicOr(dev_status, VGC_DEV_CAPACITY);
+    }
+    __syncthreads();
+
+    const uint32_t lo = blockIdx.x * chunk_elems;
+    const uint32_t hi = (uint32_t)((size_t)lo + chunk_elems < n ? (size_t)lo + chunk_elems : n);
+    uint32_t total;                                              // words, in units of 64
+    {
+        const uint32_t c0 = lane < (uint32_t)W ? sm.count[lane] : 0u, c1 = lane + 32u < (uint32_t)W ? sm.count[lane + 32] : 0u;
+        total = __reduce_add_sync(0xffffffffu, (uint32_t)(((uint64_t)c0 + c1 + 63u) >> 6));
+    }
+    if (total == 0 && !kOverwrite) return;
+    if (hi == n && tid < (uint32_t)W) {
+        const uint32_t count = sm.count[tid];
+        if (count && (sm.words[tid][count - 1] >> 4) >= n) atomicOr(dev_status, VGC_DEV_RANGE);   // skipped
+    }
+    bool bad;
+    if ((size_t)total * 64 * (kOverwrite ? sparse_write(n) : kSparseAdd) < n) {
+        if constexpr (kOverwrite) {
+            if (W <= kTileWarps) find_runs<8, 1>(sm, W, lo, (uint32_t)n, [] {});
+            else find_runs<4, 4>(sm, W, lo, (uint32_t)n, [] {});
+            __syncwarp();                                        // (a warp's cursors are its own)
+            bad = scatter_range<kHybrid>(sm, W, offs, K, scale, tau, u, lo, hi);
+            if (bad) atomicOr(dev_status, VGC_DEV_RANGE);
+        } else {
+            add_flat<kHybrid>(sm, W, offs, K, scale, tau, u, n, dev_status, blockIdx.x * kTileWarps + warp, gridDim.x * kTileWarps);
+        }
+        return;
+    }
+
+    // ---- dense: whether the exact form applies
+    // with a scale that is a positive, normal power of two its result is the sequential sum's, bit for bit
+    const int s_exp = (int)((__float_as_uint(scale) >> 23) & 0xFFu) - 127;
+    const bool pow2 = (__float_as_uint(scale) & 0x807FFFFFu) == 0u && s_exp > -127 && s_exp < 128;
+    const int g_first = kHybrid ? 0 : group_of(offs, K, lo);
+    const int g_last = kHybrid ? 0 : hi <= offs[g_first + 1] ? g_first : group_of(offs, K, hi - 1);
+    if (tid < (uint32_t)W && (reinterpret_cast<uintptr_t>(sm.words[tid]) & 15u)) sm.unfit = 1;      // read 16 bytes at a time
+    // a scale that is not finite; the filler's index would be an element; more tensors than there is room for
+    if (tid == 0 && (s_exp >= 128 || hi == (1u << 28) || g_last - g_first >= kTensors)) sm.unfit = 1;
+    int32_t ex[2] = {VGC_EXP_NONE, VGC_EXP_NONE};                // warp j looks at the range's j-th tensor
+    const int g_mine = g_first + (int)warp;
+    if (!kHybrid && g_mine <= g_last) {                          // on their way during the search
+        if (lane < (uint32_t)W) ex[0] = sm.gexp[lane][g_mine];
+        if (lane + 32u < (uint32_t)W) ex[1] = sm.gexp[lane + 32][g_mine];
+    }
+    // the tile buffer starts as zeros; from then on whoever writes a tile out leaves zeros behind
+    auto clear = [&] {
+        for (uint32_t q = tid; q < kTileMax / 4; q += kTileThreads)
+            reinterpret_cast<float4 *>(tile)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    if (W <= kTileWarps) find_runs<8, 1>(sm, W, lo, (uint32_t)n, clear);
+    else find_runs<4, 4>(sm, W, lo, (uint32_t)n, clear);
+    __syncwarp();
+    for (uint32_t w = warp; w < (uint32_t)W; w += kTileWarps) {  // the runs' first words into L2
+        const uint32_t at = sm.cur[w] + 32u * lane, count = sm.count[w];
+        if (at < count && (float)(32u * lane) * (float)n < (float)count * (float)(hi - lo))
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(sm.words[w] + at));
+    }
+    if (!kHybrid && g_mine <= g_last) {
+        const bool some0 = ex[0] != VGC_EXP_NONE, some1 = ex[1] != VGC_EXP_NONE;
+        const int e_max = __reduce_max_sync(0xffffffffu, max(some0 ? ex[0] : INT32_MIN, some1 ? ex[1] : INT32_MIN));
+        const int e_min = __reduce_min_sync(0xffffffffu, min(some0 ? ex[0] : INT32_MAX, some1 ? ex[1] : INT32_MAX));
+        if (lane == 0) {
+            int b = 0;                                           // (nothing was sent from this tensor)
+            bool fits = true;
+            if (e_max >= e_min) {
+                b = e_min - 7;                                   // the smallest value a word can stand for
+                // 2^base and every sum of multiples are normal numbers; with a power-of-two scale so are their products
+                fits = e_max - b + (32 - __clz((W - 1) | 1)) <= 22 && b >= -126 && b + 22 <= 127 &&
+                       (!pow2 || (b + s_exp >= -126 && b + 22 + s_exp <= 127));
+            }
+            // a tile takes elements of two tensors at most and begins at a multiple of four elements: a tensor of fewer
+            // than seven between two others would make it three
+            const uint32_t size = offs[g_mine + 1] - offs[g_mine];
+            if (!fits || (g_mine > g_first && g_mine < g_last && size > 0 && size < 7)) sm.unfit = 1;
+            sm.base[warp] = b;
+        }
+    }
+    __syncthreads();
+    if (sm.unfit) bad = ordered_range<kHybrid, kOverwrite>(sm, tile, W, offs, K, scale, tau, u, lo, hi, tile_elems);
+    else bad = exact_range<kHybrid, kOverwrite>(sm, tile, W, offs, g_first, scale, tau, u, lo, hi, tile_elems);
     if (bad) atomicOr(dev_status, VGC_DEV_RANGE);
 }
 
@@ -548,13 +780,29 @@ vgc_status decode_launch(bool hybrid, bool overwrite, const vgc_message_view *ms
             views.group_exp[w] = m.group_exp;
             views.max_words[w] = m.max_words;
         }
-        // one contiguous range per block, kBlocksPerSm blocks per SM, three or four tiles per range
+        const bool ow = overwrite && w0 == 0;                    // later groups of messages add to the first
+        size_t most_words = 0, longest = 0;
+        for (int w = 0; w < wb; ++w) {
+            most_words += views.max_words[w];
+            longest = longest > views.max_words[w] ? longest : views.max_words[w];
+        }
+        if (!ow && most_words * kSparseAdd < n) {                // whatever the counts on the device say
+            const size_t want = ((longest + kPiece - 1) / kPiece * wb + kFlatThreads / 32 - 1) / (kFlatThreads / 32);
+            const size_t most = (size_t)sm_count * kFlatBlocksPerSm;
+            const unsigned blocks = (unsigned)(want < 1 ? 1 : want < most ? want : most);
+            VGC_CUDA_OK(launch_kernel(hybrid ? decode_flat<true> : decode_flat<false>, dim3(blocks), dim3(kFlatThreads), 0, st, true,
+                                      views, wb, group_offsets, K, scale, tau, u, n, dev_status));
+            count_launch();
+            continue;
+        }
+        // one contiguous range per block, kBlocksPerSm blocks per SM, tiles of equal size; not less than 2048 elements
+        // each: a range costs its search
         size_t chunk = (n + (size_t)sm_count * kBlocksPerSm - 1) / ((size_t)sm_count * kBlocksPerSm);
+        chunk = chunk > 2048 ? chunk : 2048;
         chunk = (chunk + 3) / 4 * 4;
         const size_t tiles = (chunk + kTileMax - 1) / kTileMax;
         const uint32_t tile_elems = (uint32_t)(((chunk + tiles - 1) / tiles + 3) / 4 * 4);
         const unsigned blocks = (unsigned)((n + chunk - 1) / chunk);
-        const bool ow = overwrite && w0 == 0;                    // later groups of messages add to the first
         TilesFn fn = hybrid ? (ow ? decode_tiles<true, true> : decode_tiles<true, false>)
                             : (ow ? decode_tiles<false, true> : decode_tiles<false, false>);
         static TilesFn configured[4];
@@ -565,8 +813,8 @@ vgc_status decode_launch(bool hybrid, bool overwrite, const vgc_message_view *ms
             VGC_CUDA_OK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileMax * 4));
             if (n_configured < 4) configured[n_configured++] = fn;
         }
-        fn<<<blocks, kTileThreads, (size_t)kTileMax * 4, st>>>(views, wb, group_offsets, K, scale, tau, u, n, (uint32_t)chunk,
-                                                                 tile_elems, dev_status);
+        VGC_CUDA_OK(launch_kernel(fn, dim3(blocks), dim3(kTileThreads), (size_t)kTileMax * 4, st, true, views, wb, group_offsets, K,
+                                  scale, tau, u, n, (uint32_t)chunk, tile_elems, dev_status));
         count_launch();
     }
     VGC_CUDA_OK(cudaGetLastError());

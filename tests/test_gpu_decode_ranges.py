@@ -1,0 +1,70 @@
+"""The decoder at the sizes where its forms and ranges change: buffers around one block's least range (2048 elements),
+tiles that span two tensors, tensors too small or too many for the exact form, indices crowded at one end (the interpolating
+search has to fall back), and word counts on either side of the lines between flat, scatter and dense.  Values are powers of
+two within seven binades and the scale is one, so that every sum is exact in fp32: bit for bit, whatever the order."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_1802_06058_b200 as vgc
+from gpu_harness import Guarded, random_offsets
+from paper_1802_06058_b200 import workloads
+
+pytestmark = pytest.mark.gpu
+F32 = np.float32
+
+
+def _check(n, offs, msgs):
+    triples = [(w if w.numel() else torch.zeros(4, dtype=torch.int32, device="cuda"),
+                torch.tensor([w.numel()], dtype=torch.int32, device="cuda"), e) for w, e in msgs]
+    host = [(w.cpu().numpy().view(np.uint32), e.cpu().numpy()) for w, e in msgs]
+    for overwrite in (False, True):
+        gu = Guarded(n, fill=float("nan") if overwrite else 0.5)
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        vgc.vgc_decode_accumulate(triples, vgc.offsets_tensor(offs), 1.0, gu.t, st, overwrite=overwrite)
+        gu.check("u")
+        ref = np.zeros(n, F32) if overwrite else np.full(n, 0.5, F32)
+        oracle.decode_accumulate(host, offs, 1.0, ref)
+        assert int(st.item()) == 0
+        assert np.array_equal(gu.t.cpu().numpy().view(np.uint32), ref.view(np.uint32))
+
+
+def _message(n, offs, density, seed, lo=0.0, hi=1.0):
+    mask = torch.zeros(n, dtype=torch.bool, device="cuda")
+    a, b = int(n * lo), max(int(n * lo) + 1, int(n * hi))
+    gen = torch.Generator("cuda").manual_seed(seed)
+    mask[a:b] = torch.empty(b - a, device="cuda").uniform_(generator=gen) < density
+    words, exps = workloads.random_message(n, offs, density, seed + 1, "cuda", index_mask=mask)
+    return words, torch.full_like(exps, -1) - (exps & 1)
+
+
+@pytest.mark.parametrize("n", [1, 7, 2047, 2048, 2049, 4099, 2048 * 444 + 3])
+@pytest.mark.parametrize("density", [0.004, 0.3])
+@pytest.mark.parametrize("W", [1, 3, 9])
+def test_small_ranges(n, density, W):
+    offs = random_offsets(np.random.default_rng(n), n, min(n, 6))
+    _check(n, offs, [_message(n, offs, density, 10 * w + n) for w in range(W)])
+
+
+@pytest.mark.parametrize("sizes", [[100_000, 5, 900_000], [33_333, 3, 2, 1, 400_001, 17, 90_001], [64] * 3000, [0, 70_001, 0, 0, 1_500_002]])
+def test_tensor_borders_anywhere(sizes):
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint32)
+    n = int(offs[-1])
+    _check(n, offs, [_message(n, offs, 0.1, 50 + w) for w in range(8)])
+
+
+@pytest.mark.parametrize("W", [2, 20, 64])
+@pytest.mark.parametrize("density", [0.9, 0.02])
+def test_crowded_indices(W, density):
+    n = 3_000_001
+    offs = random_offsets(np.random.default_rng(W), n, 5)
+    msgs = [_message(n, offs, density, 70 + w, *((0.0, 0.02) if w % 2 else (0.97, 0.985))) for w in range(W)]
+    _check(n, offs, msgs)
+
+
+@pytest.mark.parametrize("n", [1_000_003, 5_000_003])
+@pytest.mark.parametrize("words_per_element", [1 / 17.5, 1 / 15, 1 / 8.6, 1 / 7.4])
+def test_either_side_of_the_lines(n, words_per_element):
+    offs = random_offsets(np.random.default_rng(4), n, 4)
+    _check(n, offs, [_message(n, offs, words_per_element / 3, 90 + w) for w in range(3)])
