@@ -10,6 +10,11 @@ vgc_status simt_sqgrad_linear(const float *x, const float *delta, int B, int in,
 vgc_status simt_sqgrad_conv(const float *x, const float *delta, int B, int C, int H, int W, int Cout,
                             int Kh, int Kw, int sh, int sw, int ph, int pw, int Ho, int Wo, float scale,
                             int accumulate, float *S, void *ws, size_t ws_bytes, cudaStream_t st);
+vgc_status dense_simt(const float *x, const float *delta, int B, int in, int out, float scale, int accumulate, float *S,
+                      cudaStream_t st);
+bool dense_supported(int B, int in, int out);
+vgc_status dense_sqgrad_linear(const float *x, const float *delta, int B, int in, int out, float scale, int accumulate,
+                               float *S, void *ws, cudaStream_t st);
 void tc_plan_hint(int concurrent_launches);
 bool tc_linear_supported(int B, int in, int out);
 bool tc_conv_supported(int B, int C, int H, int W, int Cout, int Kh, int Kw, int sh, int sw, int ph, int pw);
@@ -67,6 +72,17 @@ extern "C" vgc_status vgc_sqgrad_linear(const float *x, const float *delta, int 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (B == 0) return empty_batch(&S, 1, (size_t)in * out, accumulate, st);
     if (ws_bytes < vgc_sqgrad_linear_workspace_bytes(B, in, out) || !ws) return VGC_ERR_WORKSPACE;
+    // Up to 2^25 multiply-adds the CUDA cores are done before the tensor-core kernel has filled its pipeline (2.5 us against
+    // 5.0 at 2^20, equal near 2^25); beyond 512 examples the general tensor-core kernel takes over from the dense one, with
+    // a higher start (11 us).
+#ifndef VGC_LIMIT
+#define VGC_LIMIT (1ll << 25)
+#endif
+    const long long macs = (long long)in * out * B;
+    if (macs > VGC_LIMIT && dense_supported(B, in, out))
+        return dense_sqgrad_linear(x, delta, B, in, out, scale, accumulate, S, ws, st);
+    if (B <= 1024 && (macs <= (1ll << 27) || !tc_linear_supported(B, in, out)))
+        return dense_simt(x, delta, B, in, out, scale, accumulate, S, st);
     if (tc_linear_supported(B, in, out))
         return tc_sqgrad_linear(x, delta, B, in, out, scale, accumulate, S, ws, ws_bytes, st);
     return simt_sqgrad_linear(x, delta, B, in, out, scale, accumulate, S, static_cast<char *>(ws) + 256,

@@ -153,6 +153,161 @@ sqgrad_combine_splits(const float *__restrict__ partial, int splits, size_t mn, 
     S[i] = accumulate ? (float)((double)S[i] + res) : (float)res;
 }
 
+// ---- dense layers: few enough multiply-adds for the CUDA cores, or sizes the tensor-core kernels do not take ------------
+//
+// One block of 256 threads per kTile x kTile tile of S, 4 x 4 results per thread; 32 (64) examples at a time through shared
+// memory, squared on the way in, the next ones already in registers.  kTile = 64: one thread per result block.  kTile = 32
+// (where 64 x 64 tiles would leave SMs idle): four groups of 64 threads take every fourth example each and add up at the
+// end.  fp32 sums of at most 64 examples, fp64 above that.
+//
+// Bound: the launch and one round trip to memory for small layers, fp32 multiply-adds for large ones.  Measured (B200, one
+// call among others): 32 examples, 256 x 128: 11.2 us on the tensor-core kernel, 2.5 here; 128 examples, 1024 x 10: 10.5 us
+// on the kernel above, 4.6 here.
+constexpr int kDenseFlush = 2;                        // rounds per fp32 sum
+
+template <int kTile, bool kVec>                        // kVec: in and out are multiples of 4
+__global__ void __launch_bounds__(kSimtThreads)
+sqgrad_dense_simt(const float *__restrict__ x, const float *__restrict__ delta, int B, int in, int out, float scale,
+                  int accumulate, float *__restrict__ S)
+{
+    constexpr int kDenseK = kTile == 32 ? 64 : 32;                     // examples per round
+    constexpr int kThreadsPerTile = (kTile / 4) * (kTile / 4), kGroups = kSimtThreads / kThreadsPerTile;
+    constexpr int kVecs = kDenseK * kTile / 4 / kSimtThreads;          // float4 per thread, operand and round
+    __shared__ __align__(16) float As[kDenseK][kTile];
+    __shared__ __align__(16) float Bs[kDenseK][kTile];
+    const int tid = threadIdx.x, group = tid / kThreadsPerTile, t = tid % kThreadsPerTile;
+    const int tx = t % (kTile / 4), ty = t / (kTile / 4);
+    const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
+    grid_release();
+    grid_wait();
+    if (accumulate && kVec && tid < kTile && m0 + tid < out) {         // the old contents, needed at the end
+#pragma unroll
+        for (int j = 0; j < kTile; j += 32)
+            if (n0 + j < in) asm volatile("prefetch.global.L2 [%0];" ::"l"(S + (size_t)(m0 + tid) * in + n0 + j));
+    }
+    float4 a[kVecs], b[kVecs];
+    auto load4 = [&](const float *row, int at, int limit, bool valid) -> float4 {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!valid) return v;
+        if (kVec) {
+            if (at < limit) v = __ldg(reinterpret_cast<const float4 *>(row + at));
+        } else {
+            if (at < limit) v.x = __ldg(row + at);
+            if (at + 1 < limit) v.y = __ldg(row + at + 1);
+            if (at + 2 < limit) v.z = __ldg(row + at + 2);
+            if (at + 3 < limit) v.w = __ldg(row + at + 3);
+        }
+        return v;
+    };
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int i = 0; i < kVecs; ++i) {
+            const int e = tid + i * kSimtThreads, k = k0 + e / (kTile / 4), c = e % (kTile / 4) * 4;
+            a[i] = load4(delta + (size_t)k * out, m0 + c, out, k < B);
+            b[i] = load4(x + (size_t)k * in, n0 + c, in, k < B);
+        }
+    };
+    auto square = [](const float4 &v) {
+        return make_float4(__fmul_rn(v.x, v.x), __fmul_rn(v.y, v.y), __fmul_rn(v.z, v.z), __fmul_rn(v.w, v.w));
+    };
+    float acc[4][4];
+    double sum[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { acc[i][j] = 0.f; sum[i][j] = 0.0; }
+    fetch(0);
+    int rounds = 0;
+    for (int k0 = 0; k0 < B; k0 += kDenseK) {
+        if (k0) __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kVecs; ++i) {
+            const int e = tid + i * kSimtThreads, k = e / (kTile / 4), c = e % (kTile / 4) * 4;
+            *reinterpret_cast<float4 *>(&As[k][c]) = square(a[i]);
+            *reinterpret_cast<float4 *>(&Bs[k][c]) = square(b[i]);
+        }
+        __syncthreads();
+        if (k0 + kDenseK < B) fetch(k0 + kDenseK);
+        auto step = [&](int kk) {
+            const float4 a4 = *reinterpret_cast<const float4 *>(&As[kk][ty * 4]);
+            const float4 b4 = *reinterpret_cast<const float4 *>(&Bs[kk][tx * 4]);
+            const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        };
+        if (k0 + kDenseK <= B) {
+#pragma unroll 8
+            for (int kk = group; kk < kDenseK; kk += kGroups) step(kk);
+        } else {
+            for (int kk = group; kk < B - k0; kk += kGroups) step(kk);
+        }
+        if (++rounds == kDenseFlush) {
+            rounds = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { sum[i][j] += (double)acc[i][j]; acc[i][j] = 0.f; }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sum[i][j] += (double)acc[i][j];
+    if (kGroups > 1) {
+        __shared__ double part[kGroups > 1 ? kGroups - 1 : 1][kGroups > 1 ? 16 : 1][kThreadsPerTile];
+        if (group > 0) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) part[group - 1][i][t] = sum[i >> 2][i & 3];
+        }
+        __syncthreads();
+        if (group > 0) return;
+#pragma unroll
+        for (int g = 0; g < kGroups - 1; ++g)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sum[i >> 2][i & 3] += part[g][i][t];
+    }
+    const int n = n0 + tx * 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int m = m0 + ty * 4 + i;
+        if (m >= out || n >= in) continue;
+        float *dst = S + (size_t)m * in + n;
+        float res[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) res[j] = (float)((double)scale * sum[i][j]);
+        if (kVec) {
+            float4 v = make_float4(res[0], res[1], res[2], res[3]);
+            if (accumulate) {
+                const float4 old = *reinterpret_cast<const float4 *>(dst);
+                v.x = __fadd_rn(old.x, v.x); v.y = __fadd_rn(old.y, v.y);
+                v.z = __fadd_rn(old.z, v.z); v.w = __fadd_rn(old.w, v.w);
+            }
+            *reinterpret_cast<float4 *>(dst) = v;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (n + j < in) dst[j] = accumulate ? __fadd_rn(dst[j], res[j]) : res[j];
+        }
+    }
+}
+
+vgc_status dense_simt(const float *x, const float *delta, int B, int in, int out, float scale, int accumulate, float *S,
+                      cudaStream_t st)
+{
+    auto tiles = [&](int tile) { return (long long)((in + tile - 1) / tile) * ((out + tile - 1) / tile); };
+    const bool vec = in % 4 == 0 && out % 4 == 0, small = tiles(64) < 148;
+    const int tile = small ? 32 : 64;
+    const dim3 grid((in + tile - 1) / tile, (out + tile - 1) / tile);
+    if (grid.y > 65535u) return VGC_ERR_UNSUPPORTED;
+    auto fn = small ? (vec ? sqgrad_dense_simt<32, true> : sqgrad_dense_simt<32, false>)
+                    : (vec ? sqgrad_dense_simt<64, true> : sqgrad_dense_simt<64, false>);
+    VGC_CUDA_OK(launch_kernel(fn, grid, dim3(kSimtThreads), 0, st, true, x, delta, B, in, out, scale, accumulate, S));
+    count_launch();
+    return VGC_OK;
+}
+
 int simt_splits(int M, int N, int K)
 {
     const long tiles = (long)((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN);
