@@ -75,11 +75,8 @@ extern "C" vgc_status vgc_sqgrad_linear(const float *x, const float *delta, int 
     // Up to 2^25 multiply-adds the CUDA cores are done before the tensor-core kernel has filled its pipeline (2.5 us against
     // 5.0 at 2^20, equal near 2^25); beyond 512 examples the general tensor-core kernel takes over from the dense one, with
     // a higher start (11 us).
-#ifndef VGC_LIMIT
-#define VGC_LIMIT (1ll << 25)
-#endif
     const long long macs = (long long)in * out * B;
-    if (macs > VGC_LIMIT && dense_supported(B, in, out))
+    if (macs > (1ll << 25) && dense_supported(B, in, out))
         return dense_sqgrad_linear(x, delta, B, in, out, scale, accumulate, S, ws, st);
     if (B <= 1024 && (macs <= (1ll << 27) || !tc_linear_supported(B, in, out)))
         return dense_simt(x, delta, B, in, out, scale, accumulate, S, st);

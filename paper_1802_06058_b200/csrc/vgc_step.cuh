@@ -170,8 +170,7 @@ compress_step(const __grid_constant__ Args a)
     int k_first = 0, k_last = 0;
 
     const float tau_sq = __fmul_rn(a.tau, a.tau);
-
-        uint32_t run = 0;                                   // values staged by the block so far
+    uint32_t run = 0;                                   // values staged by the block so far
     int k_tile = 0;                                     // tensor of the tile's first parameter
     int k_held = 0;                                     // thread 0: the tensor whose maximum it holds
     uint32_t held_max = 0;
@@ -180,6 +179,7 @@ compress_step(const __grid_constant__ Args a)
     auto record = [&](int k, uint32_t most) {
         atomicMax(k == k_first ? sm_rec_max : k == k_last ? sm_rec_max + 1 : rec_max + k, most);
     };
+    grid_wait();
     uint32_t buf = 0;
     for (uint32_t base = lo; base < hi; base += a.tile, buf ^= 1) {
         const uint32_t end = hi - base < a.tile ? hi : base + a.tile;
@@ -557,7 +557,7 @@ vgc_status launch(Args a, void *records, cudaStream_t st)
     a.per_block = (uint32_t)per;
     a.tile = (uint32_t)round_up((per + tiles - 1) / tiles, 128);
     const dim3 grid((unsigned)((a.n + per - 1) / per));
-    VGC_CUDA_OK(launch_kernel(compress_step<kHasS, kAlgorithm>, grid, dim3(kThreads), 0, st, false, a));
+    VGC_CUDA_OK(launch_kernel(compress_step<kHasS, kAlgorithm>, grid, dim3(kThreads), 0, st, true, a));
     VGC_CUDA_OK(launch_kernel(encode_step<kAlgorithm == kBasic>, grid, dim3(kThreads), 0, st, true, a));
     count_launch(2);
     return VGC_OK;

@@ -1,0 +1,41 @@
+"""Dense layers on either side of the lines between the kernels (multiply-adds, examples, sizes TMA cannot address) and at
+the edges of their tiles: one example, one slice, the last slice of one and of two accumulators, one tile and several per
+block, ragged borders; written and added.  Reference: fp64 matmul of the squares.  Bound: 1e-5 relative (the library's own);
+written and added results agree to one fp32 addition exactly."""
+import pytest
+import torch
+
+import paper_1802_06058_b200 as vgc
+from gpu_harness import Guarded
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,n_in,n_out", [
+    (1, 8192, 8192), (9, 4100, 2052), (31, 2048, 1000), (33, 1028, 1092), (64, 4096, 4096), (64, 5000, 3004),   # one slice to many tiles
+    (255, 516, 516), (256, 512, 1000), (257, 512, 516), (512, 260, 516), (511, 2048, 132), (513, 512, 516),     # one and two accumulators
+    (1, 3, 5), (5, 32, 33), (64, 63, 129), (65, 64, 64), (129, 1000, 10), (200, 333, 257), (1024, 40, 36), (1025, 33, 65),
+    (128, 1031, 1009)])
+def test_dense(B, n_in, n_out):
+    gen = torch.Generator("cuda").manual_seed(B + n_in)
+    x = torch.randn(B, n_in, device="cuda", generator=gen).clamp_(min=0)
+    d = torch.randn(B, n_out, device="cuda", generator=gen) * 1e-3
+    x[:, 0] = 0
+    nb = max(256, vgc.vgc_sqgrad_linear_workspace_bytes(B, n_in, n_out))
+    scale = 1.0 / (B * B)
+    want = (d.double().square().t() @ x.double().square()).mul_(scale).reshape(-1)
+    S, T, ws = Guarded(n_in * n_out, fill=float("nan")), Guarded(n_in * n_out), Guarded(nb, torch.uint8, fill=0)
+    T.t.normal_(generator=gen).abs_().mul_(float(want.mean()))
+    old = T.t.clone()
+    for _ in range(2):                                           # again, right behind the first call
+        vgc.vgc_sqgrad_linear(x, d, scale, S.t, ws=ws.t)
+    vgc.vgc_sqgrad_linear(x, d, scale, T.t, accumulate=True, ws=ws.t)
+    assert int(ws.t[:4].view(torch.int32).item()) == 0
+    for g in (S, T, ws):
+        g.check()
+    assert bool(((S.t.double() - want).abs() <= 1e-5 * want).all())
+    if B > 1024:      # this kernel adds old and new in fp64 and rounds once: at most the rounding of S apart, 2^-24 of it, and
+        both = old.double() + S.t.double()                       # the rounding of either sum, 2^-24 each: 3 * 2^-24 in all
+        assert bool(((T.t.double() - both).abs() <= 3 * 2.0 ** -24 * both).all())
+    else:
+        assert torch.equal(T.t, old + S.t)
