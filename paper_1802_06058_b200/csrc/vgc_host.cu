@@ -1,10 +1,131 @@
 // vgc_step_host: one worker step driven from HOST buffers -- the end-to-end form of the path.
 // Copies each layer's x and delta (and the step's mean gradient g) from host memory into caller-provided
 // device buffers, runs the squared-gradient sums of every layer and one compressor step on the device,
-// and copies the message back to host memory.  Copies are one cudaMemcpyAsync per tensor on the
-// caller's stream; the call waits for the stream twice (the word count must be known on the host
-// before the words can be copied).
+// and copies the message back to host memory.
+//
+// Bound: the copies (PCIe).  They go back to back on a stream of the library's own, and a layer's kernels wait for that
+// layer's copies only, so that all but the last layer's run under the copies that follow (with everything on the caller's
+// stream every switch between copy and kernel cost 2 - 10 us besides; MLP 784-1024-1024-10, 128 examples, 9.5 MB:
+// @H@).  Layers whose staging buffers overlap take turns on the caller's stream.
+// The call waits for the stream twice (the word count must be known on the host before the words can be copied).
+#include <mutex>
+
 #include "vgc_common.cuh"
+
+namespace {
+
+// A stream for the copies and an event, kept between calls: a free list for all threads (one entry per call that runs at a
+// time), of kKept entries at most -- more are destroyed when their call ends, the kept ones when the process does.
+struct CopyLane {
+    int device = -1;
+    cudaStream_t stream = nullptr;
+    cudaEvent_t event = nullptr;
+};
+constexpr int kKept = 8;
+std::mutex g_lane_mutex;
+CopyLane g_lanes[kKept];
+int g_lanes_kept = 0;
+
+void destroy(CopyLane &lane)
+{
+    if (lane.event) cudaEventDestroy(lane.event);
+    if (lane.stream) cudaStreamDestroy(lane.stream);
+    lane = CopyLane();
+}
+
+bool acquire(CopyLane &lane)
+{
+    int device = -1;
+    if (cudaGetDevice(&device) != cudaSuccess) return false;
+    {
+        std::lock_guard<std::mutex> lock(g_lane_mutex);
+        for (int i = 0; i < g_lanes_kept; ++i)
+            if (g_lanes[i].device == device) {
+                lane = g_lanes[i];
+                g_lanes[i] = g_lanes[--g_lanes_kept];
+                return true;
+            }
+    }
+    lane.device = device;
+    if (cudaStreamCreateWithFlags(&lane.stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&lane.event, cudaEventDisableTiming) != cudaSuccess) {
+        destroy(lane);
+        return false;
+    }
+    return true;
+}
+
+void release(CopyLane &lane)
+{
+    {
+        std::lock_guard<std::mutex> lock(g_lane_mutex);
+        if (g_lanes_kept < kKept) {
+            g_lanes[g_lanes_kept++] = lane;
+            return;
+        }
+    }
+    destroy(lane);
+}
+
+// Copies of one call.  overlap() == false (staging shared between layers, or no stream to be had): all on the caller's stream.
+class Copies {
+public:
+    Copies(cudaStream_t caller, bool overlap) : caller_(caller), own_(overlap && acquire(lane_))
+    {
+        if (own_) ok_ = order(caller_, lane_.stream);            // after what the caller's stream holds already
+    }
+    ~Copies()
+    {
+        if (!own_) return;
+        if (pending_) arrived();                                 // (an error return: the caller's stream still covers the copies)
+        release(lane_);
+    }
+    bool in(void *dst, const void *src, size_t bytes)
+    {
+        pending_ = true;
+        return ok_ && cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, own_ ? lane_.stream : caller_) == cudaSuccess;
+    }
+    // what the caller's stream holds from here on comes after the copies so far
+    bool arrived()
+    {
+        pending_ = false;
+        return !own_ || order(lane_.stream, caller_);
+    }
+
+private:
+    // (a wait refers to the event's last record when it is enqueued, so one event serves all)
+    bool order(cudaStream_t first, cudaStream_t then)
+    {
+        return cudaEventRecord(lane_.event, first) == cudaSuccess && cudaStreamWaitEvent(then, lane_.event, 0) == cudaSuccess;
+    }
+    cudaStream_t caller_;
+    CopyLane lane_;
+    bool own_, ok_ = true, pending_ = false;
+};
+
+struct LayerSizes {
+    size_t n_x, n_d, n_w;
+};
+bool layer_sizes(const vgc_layer_host &L, LayerSizes &z)
+{
+    if (!L.x_host || !L.delta_host || !L.x_dev || !L.delta_dev) return false;
+    if (L.is_conv) {
+        if (L.H + 2 * L.pad_h < L.Kh || L.W + 2 * L.pad_w < L.Kw || L.stride_h < 1 || L.stride_w < 1) return false;
+        const size_t Ho = (L.H + 2 * L.pad_h - L.Kh) / L.stride_h + 1, Wo = (L.W + 2 * L.pad_w - L.Kw) / L.stride_w + 1;
+        z.n_x = (size_t)L.B * L.C * L.H * L.W;
+        z.n_d = (size_t)L.B * L.Cout * Ho * Wo;
+        z.n_w = (size_t)L.Cout * L.C * L.Kh * L.Kw;
+    } else {
+        z.n_x = (size_t)L.B * L.C;
+        z.n_d = (size_t)L.B * L.Cout;
+        z.n_w = (size_t)L.Cout * L.C;
+    }
+    return true;
+}
+
+bool overlapping(const float *a, size_t n_a, const float *b, size_t n_b) { return a < b + n_b && b < a + n_a; }
+
+}  // namespace
 
 extern "C" vgc_status vgc_step_host(const vgc_layer_host *layers, int n_layers, const float *g_host, float *g_dev,
                                     float *s_dev, float *r, float *v, size_t n, const uint32_t *group_offsets,
@@ -18,25 +139,34 @@ extern "C" vgc_status vgc_step_host(const vgc_layer_host *layers, int n_layers, 
     if (K != n_layers) return VGC_ERR_INVALID_ARG;        // one weight tensor (group) per layer, in order
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     size_t offset = 0;
+    bool shared = false;                                  // some layers' staging buffers (or g's) overlap
+    for (int l = 0; l < n_layers; ++l) {
+        LayerSizes z;
+        if (!layer_sizes(layers[l], z) || offset + z.n_w > n) return VGC_ERR_INVALID_ARG;
+        offset += z.n_w;
+        const float *const mine[2] = {layers[l].x_dev, layers[l].delta_dev};
+        const size_t len[2] = {z.n_x, z.n_d};
+        for (int i = 0; i < 2 && !shared; ++i) {
+            shared = overlapping(mine[i], len[i], g_dev, n);
+            for (int m = 0; m < l && !shared; ++m) {
+                LayerSizes y;
+                layer_sizes(layers[m], y);
+                shared = overlapping(mine[i], len[i], layers[m].x_dev, y.n_x) || overlapping(mine[i], len[i], layers[m].delta_dev, y.n_d);
+            }
+        }
+    }
+    if (offset != n) return VGC_ERR_INVALID_ARG;
+    Copies copies(st, !shared);
+    offset = 0;
     for (int l = 0; l < n_layers; ++l) {
         const vgc_layer_host &L = layers[l];
-        if (!L.x_host || !L.delta_host || !L.x_dev || !L.delta_dev) return VGC_ERR_INVALID_ARG;
-        size_t n_x, n_d, n_w;
-        if (L.is_conv) {
-            if (L.H + 2 * L.pad_h < L.Kh || L.W + 2 * L.pad_w < L.Kw || L.stride_h < 1 || L.stride_w < 1)
-                return VGC_ERR_INVALID_ARG;
-            const size_t Ho = (L.H + 2 * L.pad_h - L.Kh) / L.stride_h + 1, Wo = (L.W + 2 * L.pad_w - L.Kw) / L.stride_w + 1;
-            n_x = (size_t)L.B * L.C * L.H * L.W;
-            n_d = (size_t)L.B * L.Cout * Ho * Wo;
-            n_w = (size_t)L.Cout * L.C * L.Kh * L.Kw;
-        } else {
-            n_x = (size_t)L.B * L.C;
-            n_d = (size_t)L.B * L.Cout;
-            n_w = (size_t)L.Cout * L.C;
-        }
-        if (offset + n_w > n) return VGC_ERR_INVALID_ARG;
-        VGC_CUDA_OK(cudaMemcpyAsync(L.x_dev, L.x_host, n_x * sizeof(float), cudaMemcpyHostToDevice, st));
-        VGC_CUDA_OK(cudaMemcpyAsync(L.delta_dev, L.delta_host, n_d * sizeof(float), cudaMemcpyHostToDevice, st));
+        LayerSizes z;
+        layer_sizes(L, z);
+        if (!copies.in(L.x_dev, L.x_host, z.n_x * sizeof(float)) || !copies.in(L.delta_dev, L.delta_host, z.n_d * sizeof(float)) ||
+            !copies.arrived())
+            return VGC_ERR_CUDA;
+        // g under the last layer's kernels
+        if (!shared && l == n_layers - 1 && !copies.in(g_dev, g_host, n * sizeof(float))) return VGC_ERR_CUDA;
         vgc_status rc = L.is_conv
                             ? vgc_sqgrad_conv(L.x_dev, L.delta_dev, L.B, L.C, L.H, L.W, L.Cout, L.Kh, L.Kw, L.stride_h,
                                               L.stride_w, L.pad_h, L.pad_w, scale, 0, s_dev + offset, ws_sqgrad,
@@ -44,18 +174,22 @@ extern "C" vgc_status vgc_step_host(const vgc_layer_host *layers, int n_layers, 
                             : vgc_sqgrad_linear(L.x_dev, L.delta_dev, L.B, L.C, L.Cout, scale, 0, s_dev + offset,
                                                 ws_sqgrad, ws_sqgrad_bytes, stream);
         if (rc != VGC_OK) return rc;
-        offset += n_w;
+        offset += z.n_w;
     }
-    if (offset != n) return VGC_ERR_INVALID_ARG;
-    VGC_CUDA_OK(cudaMemcpyAsync(g_dev, g_host, n * sizeof(float), cudaMemcpyHostToDevice, st));
+    if ((shared || n_layers == 0) && !copies.in(g_dev, g_host, n * sizeof(float))) return VGC_ERR_CUDA;
+    if (!copies.arrived()) return VGC_ERR_CUDA;
     vgc_status rc = vgc_compress(g_dev, s_dev, r, v, n, group_offsets, K, alpha, zeta, out, ws_compress, ws_compress_bytes,
                                  stream);
     if (rc != VGC_OK) return rc;
-    // counters: nnz, n_criterion, n_dropped, dev_status
-    VGC_CUDA_OK(cudaMemcpyAsync(counters_host + 0, out->nnz, 4, cudaMemcpyDeviceToHost, st));
-    VGC_CUDA_OK(cudaMemcpyAsync(counters_host + 1, out->n_criterion, 4, cudaMemcpyDeviceToHost, st));
-    VGC_CUDA_OK(cudaMemcpyAsync(counters_host + 2, out->n_dropped, 4, cudaMemcpyDeviceToHost, st));
-    VGC_CUDA_OK(cudaMemcpyAsync(counters_host + 3, out->dev_status, 4, cudaMemcpyDeviceToHost, st));
+    // counters: nnz, n_criterion, n_dropped, dev_status -- one copy where they lie side by side
+    if (out->n_criterion == out->nnz + 1 && out->n_dropped == out->nnz + 2 && out->dev_status == out->nnz + 3) {
+        VGC_CUDA_OK(cudaMemcpyAsync(counters_host, out->nnz, 16, cudaMemcpyDeviceToHost, st));
+    } else {
+        VGC_CUDA_OK(cudaMemcpyAsync(counters_host + 0, out->nnz, 4, cudaMemcpyDeviceToHost, st));
+        VGC_CUDA_OK(cudaMemcpyAsync(counters_host + 1, out->n_criterion, 4, cudaMemcpyDeviceToHost, st));
+        VGC_CUDA_OK(cudaMemcpyAsync(counters_host + 2, out->n_dropped, 4, cudaMemcpyDeviceToHost, st));
+        VGC_CUDA_OK(cudaMemcpyAsync(counters_host + 3, out->dev_status, 4, cudaMemcpyDeviceToHost, st));
+    }
     VGC_CUDA_OK(cudaStreamSynchronize(st));
     const uint32_t kept = counters_host[0] < out->capacity ? counters_host[0] : out->capacity;
     if (kept) {

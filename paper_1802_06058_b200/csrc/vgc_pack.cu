@@ -11,8 +11,9 @@
 // side: one warp per run.
 //
 //   pack:   pack_count   every lane sizes 8 consecutive words of its warp's run; block totals are stored
-//           pack_emit    a block adds up the totals of the blocks before it (no waiting on other blocks), codes its words into
-//                        shared memory at the alignment they will have in the stream, and its bytes leave as whole words
+//           pack_emit    starts under pack_count with its words; a block adds up the totals of the blocks before it (no
+//                        waiting on other blocks), codes its words into shared memory at the alignment they will have in
+//                        the stream, and its bytes leave as whole words
 //   unpack: one kernel   a warp brings its run's bytes into shared memory, 4 at a time; a byte with a clear top bit ends a
 //                        number: a warp scan of their counts gives every end its place, every lane reads the 8 numbers
 //                        between its ends, and a second scan over the differences gives the indices
@@ -75,8 +76,8 @@ pack_count(const uint32_t *__restrict__ words, const uint32_t *__restrict__ nnz,
 {
     __shared__ uint32_t sm_tot[kPackWarps];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    grid_release();
     grid_wait();
+    grid_release();                                     // in this order: pack_emit reads the words before it waits for us
     const uint32_t n = min(*nnz, max_words);
     const uint32_t run = blockIdx.x * kPackWarps + warp;
     // the grid covers the buffer's capacity; blocks past the message's last run have nothing anyone reads
@@ -104,7 +105,6 @@ pack_emit(const uint32_t *__restrict__ words, const uint32_t *__restrict__ nnz, 
     __shared__ uint32_t sm_run[kPackWarps];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     grid_release();
-    grid_wait();
     const uint32_t n = min(*nnz, max_words);
     const uint32_t runs = (n + kPackRun - 1) / kPackRun;
     const size_t table_bytes = 4 * ((size_t)runs + 1);
@@ -112,9 +112,10 @@ pack_emit(const uint32_t *__restrict__ words, const uint32_t *__restrict__ nnz, 
     const uint32_t run = blockIdx.x * kPackWarps + warp;
     uint32_t v[kPerLane], mine;
     const uint32_t have = lane_numbers(words, n, run, lane, v, mine);
+    grid_wait();                                                        // pack_count's totals
     // payload bytes of all blocks before this one
     unsigned long long before = 0;
-    for (uint32_t b = threadIdx.x; b < blockIdx.x; b += kPackThreads) before += block_bytes[b];
+    for (uint32_t b = threadIdx.x; b < blockIdx.x; b += kPackThreads) before += __ldcg(block_bytes + b);
     before = warp_sum_u64(before);
     const uint32_t incl = warp_inclusive(mine, lane);
     if (lane == 31) sm_run[warp] = incl;

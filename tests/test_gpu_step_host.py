@@ -1,0 +1,103 @@
+"""vgc_step_host: staging buffers of their own (copies run beside the kernels), shared between the layers and with g (copies
+and kernels take turns), a message whose counters do not lie side by side, and calls from several threads on streams of
+their own.  All give what the device calls give, bit for bit."""
+import ctypes
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+import paper_1802_06058_b200 as vgc
+from paper_1802_06058_b200 import workloads
+
+pytestmark = pytest.mark.gpu
+B, SIZES = 64, [(1024, 512), (512, 256), (256, 12)]
+
+
+class Step:
+    def __init__(self, seed, staging):
+        specs = [workloads.LayerSpec(f"fc{i}", "fc", a, b) for i, (a, b) in enumerate(SIZES)]
+        offs = workloads.group_offsets(specs)
+        self.n, self.K = int(offs[-1]), len(specs)
+        self.offs = vgc.offsets_tensor(offs)
+        ins = [workloads.layer_inputs(sp, B, 1, 0, seed, i, "relu_normal", 1e-3, "cuda") for i, sp in enumerate(specs)]
+        g = torch.cat([workloads.mean_gradient(sp, x, d) for sp, (x, d) in zip(specs, ins)])
+        self.ws = torch.zeros(max(vgc.vgc_sqgrad_linear_workspace_bytes(B, sp.cin, sp.cout) for sp in specs) + 256,
+                              dtype=torch.uint8, device="cuda")
+        self.wc = torch.empty(vgc.vgc_compress_workspace_bytes(self.n, self.K), dtype=torch.uint8, device="cuda")
+        self.s, self.r, self.v = (torch.zeros(self.n, device="cuda") for _ in range(3))
+        for (x, d), lo, hi in zip(ins, offs[:-1].tolist(), offs[1:].tolist()):
+            vgc.vgc_sqgrad_linear(x, d, 1.0 / B ** 2, self.s[lo:hi], ws=self.ws)
+        out = vgc.MessageBuffers(self.n, self.K, self.n)
+        vgc.vgc_compress(g, self.s, self.r, self.v, self.offs, 2.0, 0.999, out, self.wc)
+        self.want = out.read()
+        self.g_dev = torch.empty(self.n, device="cuda")
+        room = self.g_dev if staging == "with g" else torch.empty(2 * B * 1024, device="cuda")
+        self.layers = []
+        for x, d in ins:
+            if staging == "own":
+                xd, dd = torch.empty_like(x), torch.empty_like(d)
+            else:
+                xd, dd = room[:x.numel()].view_as(x), room[x.numel():x.numel() + d.numel()].view_as(d)
+            self.layers.append({"is_conv": 0, "B": B, "C": x.shape[1], "Cout": d.shape[1], "x_host": x.cpu().pin_memory(),
+                                "delta_host": d.cpu().pin_memory(), "x_dev": xd, "delta_dev": dd})
+        self.g_host = g.cpu().pin_memory()
+        self.words, self.counters = torch.zeros(self.n, dtype=torch.int32), torch.zeros(4, dtype=torch.int32)
+
+    def check(self, out, stream=None):
+        s, r, v = torch.full_like(self.s, float("nan")), torch.zeros_like(self.r), torch.zeros_like(self.v)
+        torch.cuda.synchronize()
+        got = vgc.vgc_step_host(self.layers, self.g_host, self.g_dev, s, r, v, self.offs, 2.0, 0.999, 1.0 / B ** 2, out, self.words,
+                                self.counters, self.ws, self.wc, stream=stream)
+        w = self.want
+        assert got == (w["nnz"], w["n_criterion"], w["n_dropped"], 0)
+        assert np.array_equal(self.words[:got[0]].numpy().view(np.uint32), w["words"])
+        assert torch.equal(s, self.s) and torch.equal(r, self.r) and torch.equal(v, self.v)
+
+
+@pytest.mark.parametrize("staging", ["own", "shared", "with g"])
+def test_staging(staging):
+    step = Step(3, staging)
+    out = vgc.MessageBuffers(step.n, step.K, step.n)
+    for _ in range(3):
+        out.counters.zero_()
+        step.check(out)
+
+
+def test_counters_apart():
+    step = Step(4, "own")
+
+    class Apart(vgc.MessageBuffers):
+        def struct(self):
+            m, c = super().struct(), self.far.data_ptr()
+            m.nnz, m.n_criterion, m.n_dropped, m.dev_status = c, c + 64, c + 128, c + 192
+            return m
+
+    out = Apart(step.n, step.K, step.n)
+    out.far = torch.zeros(64, dtype=torch.int32, device="cuda")
+    assert isinstance(out.struct(), ctypes.Structure)
+    step.check(out)
+
+
+def test_threads():
+    steps = [Step(10 + i, "own") for i in range(3)]
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(step):
+        try:
+            stream = torch.cuda.Stream()
+            out = vgc.MessageBuffers(step.n, step.K, step.n)
+            for _ in range(5):
+                out.counters.zero_()
+                step.check(out, stream)
+        except BaseException as e:  # noqa: BLE001
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in steps]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed[0]
