@@ -6,7 +6,7 @@
 // Bound: the copies (PCIe).  They go back to back on a stream of the library's own, and a layer's kernels wait for that
 // layer's copies only, so that all but the last layer's run under the copies that follow (with everything on the caller's
 // stream every switch between copy and kernel cost 2 - 10 us besides; MLP 784-1024-1024-10, 128 examples, 9.5 MB:
-// @H@).  Layers whose staging buffers overlap take turns on the caller's stream.
+// 351 -> 261 us, of which the copies are 205).  Layers whose staging buffers overlap take turns on the caller's stream.
 // The call waits for the stream twice (the word count must be known on the host before the words can be copied).
 #include <mutex>
 

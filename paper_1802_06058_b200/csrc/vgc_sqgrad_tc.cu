@@ -34,7 +34,7 @@
 //                materialised.  With few output channels (Cout <= 64) the roles are swapped: the
 //                im2col rows become the 128-row A tile and the errors the narrow B tile.
 //
-// Warp roles (448 threads): 0 TMA producer, 1 MMA issuer + TMEM owner, 2-9 transform, 10-13 epilogue.
+// Warp roles (512 threads): 0 TMA producer, 1 MMA issuer + TMEM owner, 4-11 transform, 12-15 epilogue.
 // While the epilogue warps write a segment's tile out, the other roles are already working on the next one.
 // Every wait on an mbarrier is bounded; on expiry the block raises an abort flag, all roles fall
 // through to the common exit, outstanding TMA loads are waited for (bounded) and TMEM is freed.
@@ -68,7 +68,16 @@ constexpr int kGroups = VGC_TC_GROUPS;
 constexpr int kTransformWarps = 4 * kGroups;
 constexpr int kGatherThreads = 256;                                 // threads sharing a slice in the one-group forms
 constexpr int kEpilogueWarps = 4;
-constexpr int kThreadsTc = 32 * (2 + kTransformWarps + kEpilogueWarps);
+// Warps 0 and 1 are the producer and the issuer, 2 and 3 idle, so that the transform groups and the epilogue are warpgroups
+// and can be given different shares of the registers: the epilogue holds 128 sums per lane and spilled 1.4 KB of loads per
+// lane and chunk at the 128 registers that an even split leaves.
+constexpr int kFirstTransform = 4, kFirstEpilogue = kFirstTransform + kTransformWarps;
+constexpr int kThreadsTc = 32 * (kFirstEpilogue + kEpilogueWarps);
+constexpr int kRegsLaunch = 65536 / kThreadsTc, kRegsFew = 56, kRegsTransform = 112, kRegsEpilogue = 232;
+static_assert(kGroups == 2 && 128 * (kRegsFew + kGroups * kRegsTransform + kRegsEpilogue) <= kRegsLaunch * kThreadsTc,
+              "the shares come out of what the block was launched with");
+template <int kRegs> __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs)); }
+template <int kRegs> __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs)); }
 constexpr uint32_t kRawBytesA = kBM * kBK * 4;                      // 16 KB
 constexpr uint32_t kRawBytesB = kBN * kBK * 4;                      // 16 KB
 constexpr uint32_t kRawStageBytes = kRawBytesA + kRawBytesB;        // 32 KB: [A raw/hi][B raw/hi], same for lo
@@ -544,6 +553,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     uint64_t *acc_full = lo_empty + kLoSlotsAT, *acc_empty = acc_full + 2, *drain = acc_empty + 2;
     uint64_t *a_full = drain + 1, *a_empty = a_full + kNA;                 // split form: the A ring
 
+    grid_release();
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int i = 0; i < kNB; ++i) {
@@ -571,9 +581,11 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    grid_wait();
 
     // `it` below is the running number of a slice within this block (over all of its segments): ring slots and
     // barrier phases follow it, so the pipeline does not drain between segments.
+    if (warp < kFirstTransform) regs_dec<kRegsFew>();
     if (warp == 0) {
         // ================= TMA producer (one thread) =================
         if (lane == 0 && kAnyTma) {
@@ -733,9 +745,12 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 for (uint32_t t = 0; t < kWaitLimit && !mbar_try(smem_u32(drain), 0); ++t) {}
             }
         }
-    } else if (warp < 2 + kTransformWarps) {
+    } else if (warp < kFirstTransform) {
+        // nothing: the rest of the first warpgroup
+    } else if (warp < kFirstEpilogue) {
         // ================= transform warps: square and split into TF32 hi / lo =================
-        const int t = (int)threadIdx.x - 64;                               // 0 .. 128 * kGroups - 1
+        regs_dec<kRegsTransform>();
+        const int t = (int)threadIdx.x - 32 * kFirstTransform;                               // 0 .. 128 * kGroups - 1
         // With nothing to gather the warps work as groups of four that take consecutive slices in turn: the waits,
         // fences and tensor-memory stores of one slice then overlap the arithmetic of the others.  The same split
         // is used when the B tile is gathered several taps at a time next to a TMA-fed A tile.  The element-wise
@@ -786,7 +801,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 const uint8_t *arow = (kSplit ? smem_gen + (uint32_t)sa * kRawBytesA : hi) + m_local * 128;
 #pragma unroll
                 for (int hh = 0; hh < (kTwoGroups ? 2 : 1); ++hh) {
-                    const uint32_t h = kTwoGroups ? (uint32_t)hh : (warp - 2) >> 2;
+                    const uint32_t h = kTwoGroups ? (uint32_t)hh : (warp - kFirstTransform) >> 2;
                     float4 c4[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
@@ -932,6 +947,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         }
     } else {
         // ================= epilogue warps: drain chunks, accumulate in fp32 registers =================
+        regs_inc<kRegsEpilogue>();
         const uint32_t q = warp & 3;                                      // TMEM lane quarter of this warp
         const int r_local = (int)(q * 32u + lane);
         float acc[kBN];
@@ -1140,6 +1156,8 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
                   long long ld_m, long long ld_n)
 {
     __shared__ float patch[32][33];
+    grid_release();
+    grid_wait();
     const int tile = blockIdx.x >> 4, sub = blockIdx.x & 15;
     // the blocks that hold the tile's first and last unit: the first units_r blocks own units_q + 1 units each, the
     // others units_q
@@ -1213,6 +1231,50 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
             }
         }
     }
+}
+
+// The same for tiles that many blocks worked on: a thread block per 32 rows x 4 columns, the partial tiles dealt out to its
+// eight warps in turn and their sums added in the order of the warps (a fixed order as well).  A chain of 148 partial tiles
+// took 22 us in the kernel above.
+__global__ void __launch_bounds__(256)
+sqgrad_tc_combine_many(const float *__restrict__ partial, int units_q, int units_r, int units_per_tile,
+                       int tiles_x, int tiles_y, int M, int N, float scale, int accumulate, const ResultPtrs results,
+                       long long ld_m, long long ld_n)
+{
+    __shared__ float sums[8][4][32];
+    grid_release();
+    grid_wait();
+    const int tile = blockIdx.x >> 7, sub = blockIdx.x & 127;
+    const int t_lo = ((int)blockIdx.y * (tiles_x * tiles_y) + tile) * units_per_tile;
+    const int big = units_r * (units_q + 1);
+    auto block_of = [&](int u) -> int { return u < big ? u / (units_q + 1) : units_r + (u - big) / units_q; };
+    const int b_first = block_of(t_lo), b_last = block_of(t_lo + units_per_tile - 1);
+    if (b_first == b_last) return;
+    const int tx = tile % tiles_x, ty = tile / tiles_x;
+    const int r0 = (sub & 3) * 32, j0 = (sub >> 2) * 4;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (ty * kBM + r0 >= M || tx * kBN + j0 >= N) return;
+    const int lo_first = b_first * units_q + min(b_first, units_r);
+    const float *src = partial + (size_t)j0 * kBM + r0 + lane;
+    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int b = b_first + w; b <= b_last; b += 8) {
+        const float *at = src + (size_t)(2 * b + (b == b_first && lo_first < t_lo ? 1 : 0)) * (kBM * kBN);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sum[c] = __fadd_rn(sum[c], __ldcs(at + c * kBM));
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) sums[w][c][lane] = sum[c];
+    __syncthreads();
+    // thread: row `lane`, column `w`
+    const int m = ty * kBM + r0 + lane, n = tx * kBN + j0 + w;
+    if (w >= 4 || m >= M || n >= N) return;
+    float total = sums[0][w][lane];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) total = __fadd_rn(total, sums[i][w][lane]);
+    float *dst = results.S[blockIdx.y] + (size_t)m * ld_m + (size_t)n * ld_n;
+    const float res = __fmul_rn(scale, total);
+    *dst = accumulate ? __fadd_rn(*dst, res) : res;
 }
 
 // ---- host side --------------------------------------------------------------------------------
@@ -1322,6 +1384,9 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
     bool seen = false;
     for (int i = 0; i < n_configured; ++i) seen = seen || configured[i] == kernel;
     if (!seen) {
+        cudaFuncAttributes attr;
+        VGC_CUDA_OK(cudaFuncGetAttributes(&attr, kernel));
+        if (attr.numRegs != kRegsLaunch) return VGC_ERR_CUDA;        // the kernel's register shares assume this
         VGC_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
         if (n_configured < 32) configured[n_configured++] = kernel;
     }
@@ -1332,14 +1397,17 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
     prm.chunk = kChunk;
     prm.status = static_cast<uint32_t *>(ws);
     prm.partial = reinterpret_cast<float *>(static_cast<char *>(ws) + 256);
-    kernel<<<plan.blocks, kThreadsTc, kSmemBytes, st>>>(bt, prm);
+    VGC_CUDA_OK(launch_kernel(kernel, dim3((unsigned)plan.blocks), dim3(kThreadsTc), kSmemBytes, st, true, bt, prm));
     count_launch();
     if (plan.partials) {
         ResultPtrs results = {};
         for (int l = 0; l < n_layers; ++l) results.S[l] = bt.S[l];
-        sqgrad_tc_combine<<<dim3((unsigned)(plan.tiles_x * plan.tiles_y * 16), (unsigned)n_layers), 256, 0, st>>>(
-            prm.partial, prm.units_q, prm.units_r, plan.units_per_tile, plan.tiles_x, plan.tiles_y, M, N, prm.scale,
-            prm.accumulate, results, prm.ld_m, prm.ld_n);
+        // eight and more partial tiles per tile: the warps share the chain
+        const bool many = plan.units_per_tile >= 8 * (prm.units_q + 1);
+        const unsigned patches = (unsigned)(plan.tiles_x * plan.tiles_y) * (many ? 128u : 16u);
+        VGC_CUDA_OK(launch_kernel(many ? sqgrad_tc_combine_many : sqgrad_tc_combine, dim3(patches, (unsigned)n_layers), dim3(256), 0, st,
+                                  true, prm.partial, prm.units_q, prm.units_r, plan.units_per_tile, plan.tiles_x, plan.tiles_y, M, N,
+                                  prm.scale, prm.accumulate, results, prm.ld_m, prm.ld_n));
         count_launch();
     }
     VGC_CUDA_OK(cudaGetLastError());
@@ -1427,6 +1495,8 @@ __global__ void __launch_bounds__(256)
 sqgrad_repack(const __grid_constant__ RepackJobs jobs)
 {
     constexpr int kRows = 4, kCols = 2;
+    grid_release();
+    grid_wait();
     // blockIdx.y picks the tensor; its description is read once (a run-time index into kernel parameters
     // is expensive, so nothing below touches `jobs` again)
     const RepackJob job = jobs.job[blockIdx.y];
@@ -1552,7 +1622,7 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
             jobs.job[2 * l + 1] = RepackJob{delta[l], d_p, Cout, Ho * Wo, Wo, Wo4, Ho * Wo4, 1, 1, 0, Wo};
             xr[l] = x_p; dr[l] = d_p;
         }
-        sqgrad_repack<<<dim3(blocks_for((size_t)B * (C > Cout ? C : Cout)), 2 * n_layers), 256, 0, st>>>(jobs);
+        VGC_CUDA_OK(launch_kernel(sqgrad_repack, dim3(blocks_for((size_t)B * (C > Cout ? C : Cout)), 2 * n_layers), dim3(256), 0, st, true, jobs));
         count_launch();
         return conv_group(n_layers, xr, dr, S, B, C, H, Wx, Cout, Kh, Kw, sh, sw, ph, 1, Ho, Wo4, scale, accumulate, ws, inner, st);
     }
@@ -1575,7 +1645,7 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
             xr[l] = x_r;
             dr[l] = flat ? d_r : delta[l];
         }
-        sqgrad_repack<<<dim3(blocks_for((size_t)B * (flat && Cout > C ? Cout : C)), n_jobs), 256, 0, st>>>(jobs);
+        VGC_CUDA_OK(launch_kernel(sqgrad_repack, dim3(blocks_for((size_t)B * (flat && Cout > C ? Cout : C)), n_jobs), dim3(256), 0, st, true, jobs));
         count_launch();
         if (flat)
             return conv_group(n_layers, xr, dr, S, 1, C, B * P, 1, Cout, 1, 1, 1, 1, 0, 0, B * P, 1, scale, accumulate, ws,
