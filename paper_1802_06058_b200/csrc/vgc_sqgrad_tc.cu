@@ -74,7 +74,9 @@ constexpr int kEpilogueWarps = 4;
 constexpr int kFirstTransform = 4, kFirstEpilogue = kFirstTransform + kTransformWarps;
 constexpr int kThreadsTc = 32 * (kFirstEpilogue + kEpilogueWarps);
 constexpr int kRegsLaunch = 65536 / kThreadsTc, kRegsFew = 56, kRegsTransform = 112, kRegsEpilogue = 232;
-static_assert(kGroups == 2 && 128 * (kRegsFew + kGroups * kRegsTransform + kRegsEpilogue) <= kRegsLaunch * kThreadsTc,
+constexpr int kRegsTransformWide = 104, kRegsEpilogueWide = 248;
+static_assert(kGroups == 2 && 128 * (kRegsFew + kGroups * kRegsTransform + kRegsEpilogue) <= kRegsLaunch * kThreadsTc &&
+              128 * (kRegsFew + kGroups * kRegsTransformWide + kRegsEpilogueWide) <= kRegsLaunch * kThreadsTc,
               "the shares come out of what the block was launched with");
 template <int kRegs> __device__ __forceinline__ void regs_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs)); }
 template <int kRegs> __device__ __forceinline__ void regs_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs)); }
@@ -91,6 +93,12 @@ constexpr int kLoSlotsAT = 2 * kLoSlots;
 // early, and the 16-KB units this saves hold more B tiles: more slices in flight from the same shared memory.
 constexpr int kSplitA = 4, kSplitB = kGroups > 2 ? 6 : 7, kSplitLo = kGroups > 2 ? 4 : 3;   // 16-KB units: A raw, B raw/hi, B lo (+ A in TMEM)
 static_assert((kSplitA + kSplitB + kSplitLo) * kRawBytesA <= (kRawSlots + kLoSlots) * kRawStageBytes, "smem budget");
+// Wide form (the kernels that gather several taps at a time, tiles of 192 columns): the tensor core takes an N = 192
+// instruction in little more time than an N = 128 one, and 192 rows of the im2col view are 64 whole triples.  The raw A
+// tiles have a ring of two, the B tile and its lo part one of four, A in tensor memory two slots beside two accumulators.
+constexpr int kWideN = 192, kWideA = 2, kWideB = 4, kWideTmemA = 2;
+static_assert(kWideA * kRawBytesA + 2 * kWideB * kWideN * kBK * 4 <= (kRawSlots + kLoSlots) * kRawStageBytes, "smem budget");
+static_assert(2 * kWideN + kWideTmemA * 64 <= 512, "tensor memory");
 constexpr uint32_t kTmemColsA = 64;                                 // per slot: 32 columns hi + 32 columns lo
 constexpr uint32_t kTmemCols = 512;                                 // two accumulator buffers + the A operand ring
 
@@ -110,7 +118,8 @@ struct Params {
     int units_per_tile;      // k_slices / unit
     int units_total;         // layers * tiles * units_per_tile: the launch's work, cut evenly over the blocks:
     int units_q, units_r;    // block b owns units [b q + min(b, r), ...) with q = total / blocks, r = total % blocks
-    int tiles_x, tiles_y;    // 128-column / 128-row tiles of one layer's result
+    int tile_n;              // columns of a tile: 128, or 192 (wide form)
+    int tiles_x, tiles_y;    // tiles of one layer's result
     uint32_t tx_bytes;       // bytes the TMA loads of one slice deliver
     uint32_t tx_bytes_a;     // of which the A tile's
     float scale;
@@ -393,7 +402,7 @@ template <int kTriples> struct TapsOf<kGatherTaps7S2, kTriples> { typedef Gather
 // One interface over both gather forms: the registers of one slice, how they are loaded and where their
 // squared, split values go in a K-major swizzled tile.  row0 = t >> 3 and kq = t & 7 of transform thread t.
 // kHalf: the slice is shared by 128 threads instead of 256 (two transform groups on alternate slices)
-template <int kMode, bool kHalf = false, bool kTaps = IsTaps<kMode>::value>
+template <int kMode, bool kHalf = false, int kRows = kBM, bool kTaps = IsTaps<kMode>::value>
 struct Gatherer {
     struct Regs { float v[kRowsPerThread][4]; };
     GatherRows<kMode> g;
@@ -410,9 +419,10 @@ struct Gatherer {
             split_store<kSquare>(hi, lo, chunk_offset(row0 + 32 * i, kq), r.v[i][0], r.v[i][1], r.v[i][2], r.v[i][3]);
     }
 };
-template <int kMode, bool kHalf>
-struct Gatherer<kMode, kHalf, true> {
-    static constexpr int kTriples = kMode == kGatherTaps7S2 ? 2 : kHalf ? 3 : 2;      // tuples of rows per thread
+template <int kMode, bool kHalf, int kRows>
+struct Gatherer<kMode, kHalf, kRows, true> {
+    // tuples of rows per thread; with 192 rows (16 threads side by side) 64 whole triples, no remainder
+    static constexpr int kTriples = kMode == kGatherTaps7S2 ? 2 : kRows == kWideN ? 4 : kHalf ? 3 : 2;
     typedef typename TapsOf<kMode, kTriples>::type Impl;
     struct Regs { float v[kTriples][Impl::kSlots]; };
     Impl g;
@@ -426,7 +436,7 @@ struct Gatherer<kMode, kHalf, true> {
     {
 #pragma unroll
         for (int i = 0; i < kTriples; ++i) {
-            if (g.row_local[i] >= kBM || g.row_local[i] <= -Impl::kKw) continue;   // no row of this tuple in the tile
+            if (g.row_local[i] >= kRows || g.row_local[i] <= -Impl::kKw) continue;   // no row of this tuple in the tile
             // square and split every loaded element once; the three taps are views of the same parts
             uint32_t h[Impl::kSlots], l[Impl::kSlots];
 #pragma unroll
@@ -438,7 +448,7 @@ struct Gatherer<kMode, kHalf, true> {
 #pragma unroll
             for (int kw = 0; kw < Impl::kKw; ++kw) {
                 const int row = g.row_local[i] + kw;
-                if ((unsigned)row < (unsigned)kBM) {                 // kBM == kBN rows in either tile
+                if ((unsigned)row < (unsigned)kRows) {
                     const uint32_t off = chunk_offset(row, kq);
                     *reinterpret_cast<uint4 *>(hi + off) =
                         make_uint4(h[Impl::idx(kw, 0)], h[Impl::idx(kw, 1)], h[Impl::idx(kw, 2)], h[Impl::idx(kw, 3)]);
@@ -484,8 +494,8 @@ struct SegIter {
         const int rem = tile - sg.layer * tiles_layer;
         const int tile_m = rem / prm.tiles_x, tile_n = rem - tile_m * prm.tiles_x;
         sg.m0 = tile_m * kBM;
-        sg.n0 = tile_n * kBN;
-        sg.n_valid = min(kBN, prm.N - sg.n0);
+        sg.n0 = tile_n * prm.tile_n;
+        sg.n_valid = min(prm.tile_n, prm.N - sg.n0);
         sg.n_act = (sg.n_valid + 15) & ~15;
         sg.s_begin = u0 * prm.unit;
         sg.s_end = u1 * prm.unit;
@@ -505,7 +515,9 @@ struct SegIter {
 // tensor-pipe time of a tf32 product each; their rounding, 2^-9 relative on a term that is itself 2^-11 of the
 // product, stays below 2^-18 of the result).  A lo slot then holds [B hi as bf16][B lo as bf16], 8 KB each with
 // 64-byte rows, and an A slot in tensor memory [hi tf32: 32 columns][hi bf16: 16][lo bf16: 16].
-template <int kMajor, int kModeA, int kModeB, bool kATmem, bool kExact = false, bool kBf = false>
+// kN: columns of a tile, 128 or (wide form) 192.  The wide per-example form keeps the sum of squares in the epilogue's
+// registers: it takes layers whose examples fit one accumulator run (at most kChunk slices).
+template <int kMajor, int kModeA, int kModeB, bool kATmem, bool kExact = false, bool kBf = false, int kN = kBN>
 __global__ void __launch_bounds__(kThreadsTc, 1)
 sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
 {
@@ -514,21 +526,27 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     constexpr bool kGatherA = kModeA != kTma, kGatherB = kModeB != kTma;
     constexpr bool kAnyTma = !kGatherA || !kGatherB;
     constexpr bool kAnyGather = kGatherA || kGatherB;
-    constexpr bool kSplit = kATmem && !kAnyGather;                         // A raw tiles in a ring of their own
-    static_assert(!kBf || (kSplit && !kExact), "bf16 cross terms: the TMA-fed form with A in tensor memory");
-    constexpr int kNA = kSplitA;                                           // slots of the raw A ring (split form)
+    constexpr bool kWide = kN != kBN;
+    static_assert(!kWide || (kN == kWideN && kATmem && IsTaps<kModeB>::value), "wide tiles: several taps at a time");
+    constexpr bool kSplit = kATmem && (!kAnyGather || kWide);              // A raw tiles in a ring of their own
+    static_assert(!kBf || (kSplit && !kExact && !kWide), "bf16 cross terms: the TMA-fed form with A in tensor memory");
+    constexpr bool kTmaB = kSplit && !kGatherB;                            // split form: the B tile comes by TMA, too
+    constexpr int kNA = kWide ? kWideA : kSplitA;                                           // slots of the raw A ring (split form)
     // the transform warps work as two groups of four on alternate slices (else all eight on every slice)
     constexpr bool kTwoGroups = !kAnyGather || (IsTaps<kModeB>::value && kModeA == kTma);
-    constexpr int kNB = kSplit ? kSplitB : kRawSlots;                      // slots of the raw / hi ring
+    constexpr int kNB = kWide ? kWideB : kSplit ? kSplitB : kRawSlots;     // slots of the raw / hi ring
     // lo slots (and A slots in TMEM); the per-example form needs 128 TMEM columns for its sum of squares
-    constexpr int kLoN = (kExact && kATmem) ? 2 : kSplit ? kSplitLo : (kATmem ? kLoSlotsAT : kLoSlots);
+    constexpr int kLoN = kWide ? kWideB : (kExact && kATmem) ? 2 : kSplit ? kSplitLo : (kATmem ? kLoSlotsAT : kLoSlots);
+    constexpr int kAN = kWide ? kWideTmemA : kLoN;                         // A slots in tensor memory
+    constexpr uint32_t kBBytes = kN * kBK * 4;                             // bytes of a B tile
     constexpr uint32_t kSqCol = 2 * kBN + (kATmem ? 2 * kTmemColsA : 0);         // where that sum lives
     constexpr uint32_t kLoBytes = kATmem ? kRawBytesB : kRawStageBytes;  // bytes of one lo slot
     // byte offsets of slot s: the [A][B] pair of the raw / hi ring (split form: only its B half exists, the
     // offset points one A tile below it), the lo ring likewise, and the split form's A ring
-    auto pair_off = [](int s) -> uint32_t { return kSplit ? (uint32_t)(kSplitA + s - 1) * kRawBytesA : (uint32_t)s * kRawStageBytes; };
+    auto pair_off = [](int s) -> uint32_t { return kWide ? kWideA * kRawBytesA + (uint32_t)s * kBBytes - kRawBytesA : kSplit ? (uint32_t)(kSplitA + s - 1) * kRawBytesA : (uint32_t)s * kRawStageBytes; };
     auto lo_off = [](int s) -> uint32_t {
-        return kSplit ? (uint32_t)(kSplitA + kSplitB + s - 1) * kRawBytesA
+        return kWide ? kWideA * kRawBytesA + (uint32_t)(kWideB + s) * kBBytes - kRawBytesA
+               : kSplit ? (uint32_t)(kSplitA + kSplitB + s - 1) * kRawBytesA
                       : kLoBase + (uint32_t)s * kLoBytes - (kATmem ? kRawBytesA : 0u);
     };
     // bf16-cross form: where the B tile of raw slot s and the [hi bf16][lo bf16] tiles of lo slot s live
@@ -599,7 +617,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 for (int slice = sg.s_begin; slice < sg.s_end; ++slice, ++it) {
                     const int st = it % kNB;
                     const uint32_t ph = (uint32_t)(it / kNB) & 1u;
-                    if (!mbar_wait(smem_u32(&empty[st]), ph ^ 1u, &abort_flag, 64)) { ok = false; break; }
+                    if (!(kSplit && !kTmaB) && !mbar_wait(smem_u32(&empty[st]), ph ^ 1u, &abort_flag, 64)) { ok = false; break; }
                     const uint32_t full = smem_u32(&raw_full[st]);
                     const uint32_t dst_a = smem_base + pair_off(st), dst_b = dst_a + kRawBytesA;
                     if (kSplit) {
@@ -609,6 +627,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                         const int z = slice / prm.p_slices, p0 = (slice - z * prm.p_slices) * kBK;
                         mbar_expect_tx(full_a, prm.tx_bytes_a);
                         tma_load_3d(smem_base + (uint32_t)sa * kRawBytesA, map_a, full_a, p0, m0, z);
+                        if (!kTmaB) continue;
                         mbar_expect_tx(full, prm.tx_bytes - prm.tx_bytes_a);
                         if (kBf) tma_load_3d(smem_base + b_tile(st), map_b, full, p0, n0, z);
                         else tma_load_3d(dst_b, map_b, full, p0, n0, z);
@@ -631,7 +650,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             // on an abort: loads already issued (slices 0 .. it-1) must land before the block may exit
             if (abort_flag) {
                 const int issued = it;
-                const int first = issued > kNB ? issued - kNB : 0;
+                const int first = kSplit && !kTmaB ? issued : issued > kNB ? issued - kNB : 0;
                 for (int i = first; i < issued; ++i) {
                     const uint32_t bar = smem_u32(&raw_full[i % kNB]);
                     const uint32_t ph = (uint32_t)(i / kNB) & 1u;
@@ -666,7 +685,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             const uint32_t desc_bf_hi = (uint32_t)(smem_desc(0, 16u, 512u, 4u) >> 32);
             const uint32_t desc_bf_lo0 = (uint32_t)smem_desc(0, 16u, 512u, 4u);
             auto desc_bf = [&](uint32_t lo16) -> uint64_t { return ((uint64_t)desc_bf_hi << 32) | (desc_bf_lo0 + lo16); };
-            int st = 0, ls = 0;                          // the current slice's raw / hi slot and lo slot
+            int st = 0, ls = 0, as = 0;                  // the current slice's raw / hi slot, lo slot and A slot
             uint32_t st_phase = 0;
             int c = 0;                                   // running number of the chunk (accumulator buffer c & 1)
             bool ok = true;
@@ -688,7 +707,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                     ok = mbar_wait(smem_u32(&acc_empty[b]), ((uint32_t)(c >> 1) & 1u) ^ 1u, &abort_flag, 0);
                     if (!ok) break;
                     tc_fence_after();
-                    const uint32_t d_tmem = tmem_base + (uint32_t)b * kBN;
+                    const uint32_t d_tmem = tmem_base + (uint32_t)b * kN;
                     const int run = cc / cps, cq = cc - run * cps;              // run (example) and chunk inside it
                     const int chunk_end = run * seg_len + min(seg_len, (cq + 1) * prm.chunk);
                     for (bool first = true; i < chunk_end; ++i) {
@@ -697,7 +716,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                         tc_fence_after();
                         const uint32_t hi_a16 = (smem_base + pair_off(st)) >> 4, hi_b16 = hi_a16 + (kRawBytesA >> 4);
                         const uint32_t lo_a16 = (smem_base + lo_off(ls)) >> 4, lo_b16 = lo_a16 + (kRawBytesA >> 4);   // lo_a unused with A in TMEM
-                        const uint32_t ta_hi = tmem_base + 2 * kBN + ls * kTmemColsA, ta_lo = ta_hi + 32;
+                        const uint32_t ta_hi = tmem_base + 2 * kN + as * kTmemColsA, ta_lo = ta_hi + 32;
                         if (kBf) {
                             const uint32_t b16 = (smem_base + b_tile(st)) >> 4;
 #pragma unroll
@@ -736,6 +755,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                         tc_commit(smem_u32(&empty[st]));              // raw, lo and TMEM-A slots are free once these MMAs retire
                         if (++st == kNB) { st = 0; st_phase ^= 1u; }
                         if (++ls == kLoN) ls = 0;
+                        if (++as == kAN) as = 0;
                     }
                     if (ok) tc_commit(smem_u32(&acc_full[b]));
                 }
@@ -749,7 +769,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         // nothing: the rest of the first warpgroup
     } else if (warp < kFirstEpilogue) {
         // ================= transform warps: square and split into TF32 hi / lo =================
-        regs_dec<kRegsTransform>();
+        regs_dec<kWide ? kRegsTransformWide : kRegsTransform>();
         const int t = (int)threadIdx.x - 32 * kFirstTransform;                               // 0 .. 128 * kGroups - 1
         // With nothing to gather the warps work as groups of four that take consecutive slices in turn: the waits,
         // fences and tensor-memory stores of one slice then overlap the arithmetic of the others.  The same split
@@ -759,10 +779,12 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         const int group = kTwoGroups ? (t >> 7) : 0;
         const int tt = kTwoGroups ? (t & 127) : t;
         const int kq = tt & 7, row0 = tt >> 3;                             // gathered chunks: rows row0 + 32*i, k = 4*kq..4*kq+3
-        Gatherer<kModeA, kTwoGroups> rows_a;
-        Gatherer<kModeB, kTwoGroups> rows_b;
-        typedef typename Gatherer<kModeA, kTwoGroups>::Regs RegsA;
-        typedef typename Gatherer<kModeB, kTwoGroups>::Regs RegsB;
+        typedef Gatherer<kModeA, kTwoGroups> GatherA;
+        typedef Gatherer<kModeB, kTwoGroups, kN> GatherB;
+        GatherA rows_a;
+        GatherB rows_b;
+        typedef typename GatherA::Regs RegsA;
+        typedef typename GatherB::Regs RegsB;
         // where the current slice sits: example z, 32-wide block pblk of that example's output positions
         int z = 0, pblk = 0;
         auto advance = [&]() {
@@ -778,13 +800,13 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             const int st = i % kNB, ls = i % kLoN;
             const uint32_t ph = (uint32_t)(i / kNB) & 1u;
             const int sa = kSplit ? i % kNA : 0;
-            if (kSplit && !mbar_wait(smem_u32(&a_full[sa]), (uint32_t)(i / kNA) & 1u, &abort_flag)) return false;
+            if (kSplit && !kWide && !mbar_wait(smem_u32(&a_full[sa]), (uint32_t)(i / kNA) & 1u, &abort_flag)) return false;
             // a raw slot is ours once its TMA tiles landed (the producer waited for it to be empty), or, with
             // nothing coming by TMA, once the MMAs that last read it retired; likewise the lo slot
-            if (kAnyTma ? !mbar_wait(smem_u32(&raw_full[st]), ph, &abort_flag)
-                        : !mbar_wait(smem_u32(&empty[st]), ph ^ 1u, &abort_flag))
+            if (kAnyTma && !kWide ? !mbar_wait(smem_u32(&raw_full[st]), ph, &abort_flag)
+                                  : !mbar_wait(smem_u32(&empty[st]), ph ^ 1u, &abort_flag))
                 return false;
-            if (i >= kLoN) {      // the lo slot's previous user: slice i - kLoN
+            if (!kWide && i >= kLoN) {      // the lo slot's previous user: slice i - kLoN (wide: B and lo slots go together)
                 const int j = i - kLoN;
                 if (!mbar_wait(smem_u32(&empty[j % kNB]), (uint32_t)(j / kNB) & 1u, &abort_flag)) return false;
             }
@@ -792,6 +814,15 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             // lo tiles: [A lo][B lo], or the B tile alone when A lives in tensor memory (then `lo` points
             // one A tile below the slot so that the same chunk offsets address the B part)
             uint8_t *lo = smem_gen + lo_off(ls);
+            if (kWide) {
+                // the B tile first: only two A slots in tensor memory, so the A tile waits for slice i - 2 to retire
+                rows_b.template store<!kExact>(hi + kRawBytesA, lo + kRawBytesA, row0, kq, gb);
+                if (!mbar_wait(smem_u32(&a_full[sa]), (uint32_t)(i / kNA) & 1u, &abort_flag)) return false;
+                if (i >= kAN) {
+                    const int j = i - kAN;
+                    if (!mbar_wait(smem_u32(&empty[j % kNB]), (uint32_t)(j / kNB) & 1u, &abort_flag)) return false;
+                }
+            }
             if (kATmem) {
                 // A: this thread's row (TMEM lane) and 16 of the slice's 32 k at a time -> hi / lo straight into
                 // TMEM (a warp of the two-group form takes both halves, otherwise its group number picks one)
@@ -817,7 +848,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                             l16[4 * u + j] = __float_as_uint(__fsub_rn(sq, __uint_as_float(h16[4 * u + j])));
                         }
                     }
-                    const uint32_t taddr = tmem_base + ((q * 32u) << 16) + 2 * kBN + ls * kTmemColsA + 16 * h;
+                    const uint32_t taddr = tmem_base + ((q * 32u) << 16) + 2 * kN + (i % kAN) * kTmemColsA + 16 * h;
                     tc_st_32x16(taddr, h16);
                     if (kBf) {
                         uint32_t hb[8], lb[8];
@@ -876,7 +907,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                         x_first ? make_uint4(lx0, lx1, ly0, ly1) : make_uint4(ly0, ly1, lx0, lx1);
                 }
             } else
-            if (kAnyTma) {      // tiles that came by TMA: elementwise, in place, over their 16-byte chunks
+            if (kAnyTma && !kWide) {      // tiles that came by TMA: elementwise, in place, over their 16-byte chunks
                 constexpr uint32_t c_begin = (kGatherA || kATmem) ? kRawBytesA / 16 : 0;
                 constexpr uint32_t c_end = kGatherB ? kRawBytesA / 16 : kRawStageBytes / 16;
                 constexpr int kPerThread = c_end > c_begin ? (c_end - c_begin) / kTT : 1;
@@ -895,7 +926,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 }
             }
             if (kGatherA) rows_a.template store<!kExact>(hi, lo, row0, kq, ga);
-            if (kGatherB) rows_b.template store<!kExact>(hi + kRawBytesA, lo + kRawBytesA, row0, kq, gb);
+            if (kGatherB && !kWide) rows_b.template store<!kExact>(hi + kRawBytesA, lo + kRawBytesA, row0, kq, gb);
             if (kATmem) { tc_wait_st(); tc_fence_before(); }      // TMEM stores complete and ordered before the signal
             fence_async_smem();                                   // generic-proxy writes -> tensor core reads
             __syncwarp();
@@ -947,10 +978,10 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         }
     } else {
         // ================= epilogue warps: drain chunks, accumulate in fp32 registers =================
-        regs_inc<kRegsEpilogue>();
+        regs_inc<kWide ? kRegsEpilogueWide : kRegsEpilogue>();
         const uint32_t q = warp & 3;                                      // TMEM lane quarter of this warp
         const int r_local = (int)(q * 32u + lane);
-        float acc[kBN];
+        float acc[kN];
         const uint32_t sq_addr = tmem_base + ((q * 32u) << 16) + kSqCol;  // kExact: this warp's rows of the sum of squares
         int c = 0;                                                        // running number of the chunk
         bool ok = true;
@@ -958,13 +989,13 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         Seg sg;
         while (ok && iter.next(prm, sg)) {
 #pragma unroll
-            for (int j = 0; j < kBN; ++j) acc[j] = 0.f;
-            if (kExact) {
+            for (int j = 0; j < kN; ++j) acc[j] = 0.f;
+            if (kExact && !kWide) {
                 uint32_t zero[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j) zero[j] = 0u;
 #pragma unroll
-                for (int j0 = 0; j0 < kBN; j0 += 16) tc_st_32x16(sq_addr + j0, zero);
+                for (int j0 = 0; j0 < kN; j0 += 16) tc_st_32x16(sq_addr + j0, zero);
                 tc_wait_st();
             }
             const int n_act = sg.n_act, n_valid = sg.n_valid;
@@ -977,24 +1008,27 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 ok = mbar_wait(smem_u32(&acc_full[b]), (uint32_t)(c >> 1) & 1u, &abort_flag, 256);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t taddr = tmem_base + ((q * 32u) << 16) + (uint32_t)b * kBN;
+                const uint32_t taddr = tmem_base + ((q * 32u) << 16) + (uint32_t)b * kN;
 #pragma unroll
-                for (int j0 = 0; j0 < kBN; j0 += 32) {
+                for (int j0 = 0; j0 < kN; j0 += 32) {
                     if (j0 < n_act) {
                         uint32_t r[32];
                         tc_ld_32x32(taddr + j0, r);
                         tc_wait_ld();
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) acc[j0 + j] = __fadd_rn(acc[j0 + j], __uint_as_float(r[j]));
+                        for (int j = 0; j < 32; ++j) {
+                            const float d = __uint_as_float(r[j]);      // wide per-example form: the example's whole sum
+                            acc[j0 + j] = __fadd_rn(acc[j0 + j], kExact && kWide ? __fmul_rn(d, d) : d);
+                        }
                     }
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
-                if (kExact && (cc + 1) % cps == 0) {
+                if (kExact && !kWide && (cc + 1) % cps == 0) {
                     // end of an example: acc holds its sum over positions; add the squares to the running sum in TMEM
 #pragma unroll
-                    for (int j0 = 0; j0 < kBN; j0 += 32) {
+                    for (int j0 = 0; j0 < kN; j0 += 32) {
                         if (j0 < n_act) {
                             uint32_t r[32];
                             tc_ld_32x32(sq_addr + j0, r);
@@ -1011,13 +1045,13 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                     }
                     tc_wait_st();
 #pragma unroll
-                    for (int j = 0; j < kBN; ++j) acc[j] = 0.f;
+                    for (int j = 0; j < kN; ++j) acc[j] = 0.f;
                 }
             }
             if (!ok) break;
-            if (kExact) {        // the result is the sum of squares
+            if (kExact && !kWide) {        // the result is the sum of squares
 #pragma unroll
-                for (int j0 = 0; j0 < kBN; j0 += 32) {
+                for (int j0 = 0; j0 < kN; j0 += 32) {
                     uint32_t r[32];
                     tc_ld_32x32(sq_addr + j0, r);
                     tc_wait_ld();
@@ -1030,16 +1064,16 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             float *const S = bt.S[sg.layer];
             if (!sg.whole) {
                 // partial tile, column-major inside the tile: consecutive lanes -> consecutive addresses
-                float *dst = prm.partial + (size_t)sg.slot * (kBM * kBN) + r_local;
+                float *dst = prm.partial + (size_t)sg.slot * (kBM * kN) + r_local;
 #pragma unroll
-                for (int j = 0; j < kBN; ++j)
+                for (int j = 0; j < kN; ++j)
                     if (j < n_valid) dst[j * kBM] = acc[j];
             } else if (prm.ld_m == 1) {
                 // result is contiguous along m: lanes write neighbouring addresses directly
                 if (m < prm.M) {
                     float *col = S + (size_t)m + (size_t)sg.n0 * prm.ld_n;
 #pragma unroll
-                    for (int j0 = 0; j0 < kBN; j0 += 16) {        // old values sixteen at a time, all loads in flight
+                    for (int j0 = 0; j0 < kN; j0 += 16) {        // old values sixteen at a time, all loads in flight
                         float old[16];
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
@@ -1056,18 +1090,18 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 // result is contiguous along n, and this is the block's last segment: the pipeline stages are idle
                 // (the last accumulator was complete before we got here), so this warp's 32 x 128 block is transposed
                 // through shared memory and written row by row with consecutive lanes on consecutive addresses
-                float *tile = reinterpret_cast<float *>(smem_gen) + q * (32 * (kBN + 1));
+                float *tile = reinterpret_cast<float *>(smem_gen) + q * (32 * (kN + 1));
 #pragma unroll
-                for (int j = 0; j < kBN; ++j) tile[lane * (kBN + 1) + j] = __fmul_rn(prm.scale, acc[j]);
+                for (int j = 0; j < kN; ++j) tile[lane * (kN + 1) + j] = __fmul_rn(prm.scale, acc[j]);
                 __syncwarp();
                 for (int r0 = 0; r0 < 32; r0 += 8) {              // eight rows at a time, all loads in flight
-                    float old[8][kBN / 32];
+                    float old[8][kN / 32];
 #pragma unroll
                     for (int rr = 0; rr < 8; ++rr) {
                         const int mr = sg.m0 + (int)(q * 32u) + r0 + rr;
                         const float *src = S + (size_t)mr * prm.ld_m + sg.n0;
 #pragma unroll
-                        for (int cblk = 0; cblk < kBN / 32; ++cblk) {
+                        for (int cblk = 0; cblk < kN / 32; ++cblk) {
                             const int j = cblk * 32 + (int)lane;
                             old[rr][cblk] = (prm.accumulate && mr < prm.M && j < n_valid) ? src[j] : 0.f;
                         }
@@ -1077,10 +1111,10 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                         const int mr = sg.m0 + (int)(q * 32u) + r0 + rr;
                         float *dst = S + (size_t)mr * prm.ld_m + sg.n0;
 #pragma unroll
-                        for (int cblk = 0; cblk < kBN / 32; ++cblk) {
+                        for (int cblk = 0; cblk < kN / 32; ++cblk) {
                             const int j = cblk * 32 + (int)lane;
                             if (mr < prm.M && j < n_valid) {
-                                const float res = tile[(r0 + rr) * (kBN + 1) + j];
+                                const float res = tile[(r0 + rr) * (kN + 1) + j];
                                 dst[j] = prm.accumulate ? __fadd_rn(old[rr][cblk], res) : res;
                             }
                         }
@@ -1094,7 +1128,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 float *row = S + (size_t)m * prm.ld_m + sg.n0;
                 if ((prm.ld_m & 3) == 0) {
 #pragma unroll
-                    for (int j0 = 0; j0 < kBN; j0 += 16) {
+                    for (int j0 = 0; j0 < kN; j0 += 16) {
                         float4 old[4];
 #pragma unroll
                         for (int u = 0; u < 4; ++u)
@@ -1123,7 +1157,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                     }
                 } else {
 #pragma unroll
-                    for (int j = 0; j < kBN; ++j)
+                    for (int j = 0; j < kN; ++j)
                         if (j < n_valid) {
                             const float res = __fmul_rn(prm.scale, acc[j]);
                             row[j] = prm.accumulate ? __fadd_rn(row[j], res) : res;
@@ -1152,13 +1186,13 @@ struct ResultPtrs { float *S[kMaxBatch]; };
 
 __global__ void __launch_bounds__(256)
 sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, int units_per_tile,
-                  int tiles_x, int tiles_y, int M, int N, float scale, int accumulate, const ResultPtrs results,
+                  int tile_n, int tiles_x, int tiles_y, int M, int N, float scale, int accumulate, const ResultPtrs results,
                   long long ld_m, long long ld_n)
 {
     __shared__ float patch[32][33];
     grid_release();
     grid_wait();
-    const int tile = blockIdx.x >> 4, sub = blockIdx.x & 15;
+    const int tile = blockIdx.x / (tile_n >> 3), sub = blockIdx.x % (tile_n >> 3);
     // the blocks that hold the tile's first and last unit: the first units_r blocks own units_q + 1 units each, the
     // others units_q
     const int t_lo = ((int)blockIdx.y * (tiles_x * tiles_y) + tile) * units_per_tile;
@@ -1170,12 +1204,12 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
     const int tx = tile % tiles_x, ty = tile / tiles_x;
     const int r0 = (sub & 3) * 32, j0 = (sub >> 2) * 32;                  // patch origin inside the tile
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;              // lane -> row, warp -> four columns
-    if (ty * kBM + r0 >= M || tx * kBN + j0 >= N) return;
+    if (ty * kBM + r0 >= M || tx * tile_n + j0 >= N) return;
     // the first block's part of this tile is that block's last segment unless its range starts with the tile;
     // every later block's part is its first segment
     const int lo_first = b_first * units_q + min(b_first, units_r);
     const size_t within = (size_t)(j0 + 4 * w) * kBM + r0 + lane;
-    const float *src0 = partial + (size_t)(2 * b_first + (lo_first < t_lo ? 1 : 0)) * (kBM * kBN) + within;
+    const float *src0 = partial + (size_t)(2 * b_first + (lo_first < t_lo ? 1 : 0)) * (kBM * tile_n) + within;
     const float *src = partial + within;
     float sum[4];
 #pragma unroll
@@ -1186,7 +1220,7 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) v[u][c] = __ldcs(src + (size_t)(2 * (b + u)) * (kBM * kBN) + c * kBM);
+            for (int c = 0; c < 4; ++c) v[u][c] = __ldcs(src + (size_t)(2 * (b + u)) * (kBM * tile_n) + c * kBM);
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
@@ -1194,12 +1228,12 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
     }
     for (; b <= b_last; ++b)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) sum[c] = __fadd_rn(sum[c], __ldcs(src + (size_t)(2 * b) * (kBM * kBN) + c * kBM));
+        for (int c = 0; c < 4; ++c) sum[c] = __fadd_rn(sum[c], __ldcs(src + (size_t)(2 * b) * (kBM * tile_n) + c * kBM));
     if (ld_m == 1) {
         const int m = ty * kBM + r0 + lane;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const int n = tx * kBN + j0 + 4 * w + c;
+            const int n = tx * tile_n + j0 + 4 * w + c;
             if (m < M && n < N) {
                 float *dst = S + (size_t)m + (size_t)n * ld_n;
                 const float res = __fmul_rn(scale, sum[c]);
@@ -1213,7 +1247,7 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
     __syncthreads();
     {
         const int c0 = (threadIdx.x & 7) * 4, r = threadIdx.x >> 3;       // four consecutive columns of one row
-        const int m = ty * kBM + r0 + r, n = tx * kBN + j0 + c0;
+        const int m = ty * kBM + r0 + r, n = tx * tile_n + j0 + c0;
         if (m < M) {
             float *dst = S + (size_t)m * ld_m + n;
             if ((ld_m & 3) == 0 && n + 3 < N) {
@@ -1238,13 +1272,13 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
 // took 22 us in the kernel above.
 __global__ void __launch_bounds__(256)
 sqgrad_tc_combine_many(const float *__restrict__ partial, int units_q, int units_r, int units_per_tile,
-                       int tiles_x, int tiles_y, int M, int N, float scale, int accumulate, const ResultPtrs results,
+                       int tile_n, int tiles_x, int tiles_y, int M, int N, float scale, int accumulate, const ResultPtrs results,
                        long long ld_m, long long ld_n)
 {
     __shared__ float sums[8][4][32];
     grid_release();
     grid_wait();
-    const int tile = blockIdx.x >> 7, sub = blockIdx.x & 127;
+    const int tile = blockIdx.x / tile_n, sub = blockIdx.x % tile_n;
     const int t_lo = ((int)blockIdx.y * (tiles_x * tiles_y) + tile) * units_per_tile;
     const int big = units_r * (units_q + 1);
     auto block_of = [&](int u) -> int { return u < big ? u / (units_q + 1) : units_r + (u - big) / units_q; };
@@ -1253,13 +1287,13 @@ sqgrad_tc_combine_many(const float *__restrict__ partial, int units_q, int units
     const int tx = tile % tiles_x, ty = tile / tiles_x;
     const int r0 = (sub & 3) * 32, j0 = (sub >> 2) * 4;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (ty * kBM + r0 >= M || tx * kBN + j0 >= N) return;
+    if (ty * kBM + r0 >= M || tx * tile_n + j0 >= N) return;
     const int lo_first = b_first * units_q + min(b_first, units_r);
     const float *src = partial + (size_t)j0 * kBM + r0 + lane;
     float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
     for (int b = b_first + w; b <= b_last; b += 8) {
-        const float *at = src + (size_t)(2 * b + (b == b_first && lo_first < t_lo ? 1 : 0)) * (kBM * kBN);
+        const float *at = src + (size_t)(2 * b + (b == b_first && lo_first < t_lo ? 1 : 0)) * (kBM * tile_n);
 #pragma unroll
         for (int c = 0; c < 4; ++c) sum[c] = __fadd_rn(sum[c], __ldcs(at + c * kBM));
     }
@@ -1267,7 +1301,7 @@ sqgrad_tc_combine_many(const float *__restrict__ partial, int units_q, int units
     for (int c = 0; c < 4; ++c) sums[w][c][lane] = sum[c];
     __syncthreads();
     // thread: row `lane`, column `w`
-    const int m = ty * kBM + r0 + lane, n = tx * kBN + j0 + w;
+    const int m = ty * kBM + r0 + lane, n = tx * tile_n + j0 + w;
     if (w >= 4 || m >= M || n >= N) return;
     float total = sums[0][w][lane];
 #pragma unroll
@@ -1298,10 +1332,10 @@ struct Plan {
 // tile count allows), or an even cut of the slices over all SMs (tiles at the cuts are shared, their partial
 // sums combined by a second kernel).  Costs in slice times: a block's longest range, plus what the combine pass
 // adds to the call (its launch and the partial tiles' round trip, about 14 slices' worth).
-static Plan make_plan(int M, int N, int k_slices, int n_layers, int unit_min)
+static Plan make_plan(int M, int N, int k_slices, int n_layers, int unit_min, int tile_n)
 {
     Plan p;
-    p.tiles_x = (N + kBN - 1) / kBN;
+    p.tiles_x = (N + tile_n - 1) / tile_n;
     p.tiles_y = (M + kBM - 1) / kBM;
     const long long tiles = (long long)p.tiles_x * p.tiles_y * n_layers;
     const long long upt = k_slices / unit_min, units = tiles * upt;
@@ -1365,21 +1399,21 @@ bool tc_conv_supported(int B, int C, int H, int W, int Cout, int Kh, int Kw, int
            (long)B * ((P + kBK - 1) / kBK) < (1L << 30);
 }
 
-static size_t tc_workspace_bytes(int M, int N, int k_slices, int n_layers = 1, int unit = 1)
+static size_t tc_workspace_bytes(int M, int N, int k_slices, int n_layers = 1, int unit = 1, int tile_n = kBN)
 {
-    const Plan p = make_plan(M, N, k_slices, n_layers, unit);
+    const Plan p = make_plan(M, N, k_slices, n_layers, unit, tile_n);
     // status word (256 bytes) + two partial tiles per block (the first and the last segment of its range)
-    return 256 + (p.partials ? (size_t)2 * p.blocks * kBM * kBN * sizeof(float) : 0);
+    return 256 + (p.partials ? (size_t)2 * p.blocks * kBM * tile_n * sizeof(float) : 0);
 }
 
 typedef void (*KernelFn)(const Batch, const Params);
 
 static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Params prm, int M, int N,
-                            int k_slices, void *ws, size_t ws_bytes, cudaStream_t st, int unit = 1)
+                            int k_slices, void *ws, size_t ws_bytes, cudaStream_t st, int unit = 1, int tile_n = kBN)
 {
-    const Plan plan = make_plan(M, N, k_slices, n_layers, unit);
-    if (ws_bytes < tc_workspace_bytes(M, N, k_slices, n_layers, unit)) return VGC_ERR_WORKSPACE;
-    static KernelFn configured[32];
+    const Plan plan = make_plan(M, N, k_slices, n_layers, unit, tile_n);
+    if (ws_bytes < tc_workspace_bytes(M, N, k_slices, n_layers, unit, tile_n)) return VGC_ERR_WORKSPACE;
+    static KernelFn configured[64];
     static int n_configured = 0;
     bool seen = false;
     for (int i = 0; i < n_configured; ++i) seen = seen || configured[i] == kernel;
@@ -1388,12 +1422,12 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
         VGC_CUDA_OK(cudaFuncGetAttributes(&attr, kernel));
         if (attr.numRegs != kRegsLaunch) return VGC_ERR_CUDA;        // the kernel's register shares assume this
         VGC_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-        if (n_configured < 32) configured[n_configured++] = kernel;
+        if (n_configured < 64) configured[n_configured++] = kernel;
     }
     prm.M = M; prm.N = N; prm.k_slices = k_slices;
     prm.unit = plan.unit; prm.units_per_tile = plan.units_per_tile; prm.units_total = plan.units_total;
     prm.units_q = plan.units_total / plan.blocks; prm.units_r = plan.units_total % plan.blocks;
-    prm.tiles_x = plan.tiles_x; prm.tiles_y = plan.tiles_y;
+    prm.tile_n = tile_n; prm.tiles_x = plan.tiles_x; prm.tiles_y = plan.tiles_y;
     prm.chunk = kChunk;
     prm.status = static_cast<uint32_t *>(ws);
     prm.partial = reinterpret_cast<float *>(static_cast<char *>(ws) + 256);
@@ -1404,9 +1438,9 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
         for (int l = 0; l < n_layers; ++l) results.S[l] = bt.S[l];
         // eight and more partial tiles per tile: the warps share the chain
         const bool many = plan.units_per_tile >= 8 * (prm.units_q + 1);
-        const unsigned patches = (unsigned)(plan.tiles_x * plan.tiles_y) * (many ? 128u : 16u);
+        const unsigned patches = (unsigned)(plan.tiles_x * plan.tiles_y) * (unsigned)(many ? tile_n : tile_n / 8);
         VGC_CUDA_OK(launch_kernel(many ? sqgrad_tc_combine_many : sqgrad_tc_combine, dim3(patches, (unsigned)n_layers), dim3(256), 0, st,
-                                  true, prm.partial, prm.units_q, prm.units_r, plan.units_per_tile, plan.tiles_x, plan.tiles_y, M, N,
+                                  true, prm.partial, prm.units_q, prm.units_r, plan.units_per_tile, tile_n, plan.tiles_x, plan.tiles_y, M, N,
                                   prm.scale, prm.accumulate, results, prm.ld_m, prm.ld_n));
         count_launch();
     }
@@ -1552,8 +1586,11 @@ static size_t conv_workspace_plain(int n_layers, int B, int C, int Kh, int Kw, i
 {
     const int p_slices = (P + kBK - 1) / kBK, n_im2col = C * Kh * Kw, k_slices = B * p_slices;
     const int unit = t_exact ? p_slices : 1;
-    return conv_swapped(Cout, n_im2col) ? tc_workspace_bytes(n_im2col, Cout, k_slices, n_layers, unit)
-                                        : tc_workspace_bytes(Cout, n_im2col, k_slices, n_layers, unit);
+    // the wide and the narrow form of a layer that gathers several taps at a time: either can be chosen at call time
+    const size_t narrow = conv_swapped(Cout, n_im2col) ? tc_workspace_bytes(n_im2col, Cout, k_slices, n_layers, unit)
+                                                       : tc_workspace_bytes(Cout, n_im2col, k_slices, n_layers, unit);
+    const size_t wide = Kw > 1 ? tc_workspace_bytes(Cout, n_im2col, k_slices, n_layers, unit, kWideN) : 0;
+    return narrow > wide ? narrow : wide;
 }
 
 // Workspace of one launch over n_layers layers of this geometry (n_layers <= kMaxBatch).
@@ -1705,10 +1742,20 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
 #define VGC_TC_FN(A, B_, AT) (ex ? (KernelFn)sqgrad_tc<kMajorK, A, B_, AT, true> : (KernelFn)sqgrad_tc<kMajorK, A, B_, AT, false>)
     if (!swapped) {     // S[o][idx]: m = o, n = idx
         prm.ld_m = n_im2col; prm.ld_n = 1;
-        if (taps) fn = taps == 4 ? VGC_TC_FN(kTma, kGatherTaps4, true) : VGC_TC_FN(kTma, kGatherTaps2, true);
-        else if (taps_s2) fn = taps_s2 == 4 ? VGC_TC_FN(kTma, kGatherTaps4S2, true) : VGC_TC_FN(kTma, kGatherTaps2S2, true);
-        else if (taps7) fn = VGC_TC_FN(kTma, kGatherTaps7S2, true);
-        else if (tma_bf) fn = sqgrad_tc<kMajorK, kTma, kTma, true, false, true>;
+        // wide tiles where they are fewer than narrow ones (a slice of one takes about as long as a slice of the other)
+        const bool any_taps = taps || taps_s2 || taps7;
+        const bool wide = any_taps && (n_im2col + kWideN - 1) / kWideN < (n_im2col + kBN - 1) / kBN && (!ex || p_slices <= kChunk);
+#define VGC_TAPS_FN(B_) (wide ? (ex ? (KernelFn)sqgrad_tc<kMajorK, kTma, B_, true, true, false, kWideN>                          \
+                                    : (KernelFn)sqgrad_tc<kMajorK, kTma, B_, true, false, false, kWideN>)                        \
+                              : VGC_TC_FN(kTma, B_, true))
+        if (any_taps) {
+            if (taps) fn = taps == 4 ? VGC_TAPS_FN(kGatherTaps4) : VGC_TAPS_FN(kGatherTaps2);
+            else if (taps_s2) fn = taps_s2 == 4 ? VGC_TAPS_FN(kGatherTaps4S2) : VGC_TAPS_FN(kGatherTaps2S2);
+            else fn = VGC_TAPS_FN(kGatherTaps7S2);
+            return tc_launch(fn, bt, n_layers, prm, Cout, n_im2col, k_slices, ws, ws_bytes, st, unit, wide ? kWideN : kBN);
+        }
+#undef VGC_TAPS_FN
+        if (tma_bf) fn = sqgrad_tc<kMajorK, kTma, kTma, true, false, true>;
         else if (err_tma && in_tma) fn = sqgrad_tc<kMajorK, kTma, kTma, true, true>;
         else if (err_tma) fn = VGC_TC_FN(kTma, kGatherIm2col, true);
         else fn = VGC_TC_FN(kGatherErr, kGatherIm2col, false);
