@@ -796,7 +796,8 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             rows_b.load(prm, z, pbase, gb);
         };
         // transform of the block's slice number i; gathered elements come in registers, TMA tiles from the raw stage
-        auto process = [&](int i, const RegsA &ga, const RegsB &gb) -> bool {
+        // (`gathered`: called once the registers have been read)
+        auto process = [&](int i, const RegsA &ga, const RegsB &gb, auto gathered) -> bool {
             const int st = i % kNB, ls = i % kLoN;
             const uint32_t ph = (uint32_t)(i / kNB) & 1u;
             const int sa = kSplit ? i % kNA : 0;
@@ -817,6 +818,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             if (kWide) {
                 // the B tile first: only two A slots in tensor memory, so the A tile waits for slice i - 2 to retire
                 rows_b.template store<!kExact>(hi + kRawBytesA, lo + kRawBytesA, row0, kq, gb);
+                gathered();
                 if (!mbar_wait(smem_u32(&a_full[sa]), (uint32_t)(i / kNA) & 1u, &abort_flag)) return false;
                 if (i >= kAN) {
                     const int j = i - kAN;
@@ -830,6 +832,26 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 const uint32_t q = warp & 3;
                 const int m_local = (int)(q * 32 + lane);
                 const uint8_t *arow = (kSplit ? smem_gen + (uint32_t)sa * kRawBytesA : hi) + m_local * 128;
+                if (kWide) {         // 8 k at a time: the next slice's gathered values are held in registers meanwhile
+                    const uint32_t taddr = tmem_base + ((q * 32u) << 16) + 2 * kN + (i % kAN) * kTmemColsA;
+#pragma unroll
+                    for (int k8 = 0; k8 < kBK / 8; ++k8) {
+                        uint32_t h8[8], l8[8];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const float4 c = *reinterpret_cast<const float4 *>(arow + (((2 * k8 + u) ^ (m_local & 7)) << 4));
+                            const float e[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const float sq = kExact ? e[j] : __fmul_rn(e[j], e[j]);
+                                h8[4 * u + j] = to_tf32(sq);
+                                l8[4 * u + j] = __float_as_uint(__fsub_rn(sq, __uint_as_float(h8[4 * u + j])));
+                            }
+                        }
+                        tc_st_32x8(taddr + 8 * k8, h8);
+                        tc_st_32x8(taddr + 32 + 8 * k8, l8);
+                    }
+                } else
 #pragma unroll
                 for (int hh = 0; hh < (kTwoGroups ? 2 : 1); ++hh) {
                     const uint32_t h = kTwoGroups ? (uint32_t)hh : (warp - kFirstTransform) >> 2;
@@ -956,21 +978,31 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 const int i_first = (group - it0 % kGroups + kGroups) % kGroups;
                 if (kAnyGather)
                     for (int sk = 0; sk < i_first; ++sk) advance();
-                for (int i = i_first; i < n_slices; i += kGroups) {
-                    if (kAnyGather) gather(a0, b0);
-                    if (!process(it0 + i, a0, b0)) { ok = false; break; }
-                    if (kAnyGather)
-                        for (int sk = 0; sk < kGroups; ++sk) advance();
+                auto skip = [&]() {
+                    for (int sk = 0; sk < kGroups; ++sk) advance();
+                };
+                if (kWide) {
+                    // the registers are free as soon as the B tile is written: the next slice's loads go out there and are
+                    // on their way during the A tile, the signal and the wait for the next slot
+                    if (i_first < n_slices) gather(a0, b0);
+                    for (int i = i_first; i < n_slices; i += kGroups)
+                        if (!process(it0 + i, a0, b0, [&]() { if (i + kGroups < n_slices) { skip(); gather(a0, b0); } })) { ok = false; break; }
+                } else {
+                    for (int i = i_first; i < n_slices; i += kGroups) {
+                        if (kAnyGather) gather(a0, b0);
+                        if (!process(it0 + i, a0, b0, []() {})) { ok = false; break; }
+                        if (kAnyGather) skip();
+                    }
                 }
             } else {
                 // two register sets in turn: the loads of slice i+1 are in flight while slice i is transformed
                 if (kAnyGather) gather(a0, b0);
                 for (int i = 0; i < n_slices; i += 2) {
                     if (kAnyGather && i + 1 < n_slices) { advance(); gather(a1, b1); }
-                    if (!process(it0 + i, a0, b0)) { ok = false; break; }
+                    if (!process(it0 + i, a0, b0, []() {})) { ok = false; break; }
                     if (i + 1 < n_slices) {
                         if (kAnyGather && i + 2 < n_slices) { advance(); gather(a0, b0); }
-                        if (!process(it0 + i + 1, a1, b1)) { ok = false; break; }
+                        if (!process(it0 + i + 1, a1, b1, []() {})) { ok = false; break; }
                     }
                 }
             }
