@@ -73,8 +73,8 @@ constexpr int kEpilogueWarps = 4;
 // lane and chunk at the 128 registers that an even split leaves.
 constexpr int kFirstTransform = 4, kFirstEpilogue = kFirstTransform + kTransformWarps;
 constexpr int kThreadsTc = 32 * (kFirstEpilogue + kEpilogueWarps);
-constexpr int kRegsLaunch = 65536 / kThreadsTc, kRegsFew = 56, kRegsTransform = 112, kRegsEpilogue = 232;
-constexpr int kRegsTransformWide = 104, kRegsEpilogueWide = 248;
+constexpr int kRegsLaunch = 65536 / kThreadsTc, kRegsFew = 40, kRegsTransform = 112, kRegsEpilogue = 232;
+constexpr int kRegsTransformWide = 120, kRegsEpilogueWide = 232;
 static_assert(kGroups == 2 && 128 * (kRegsFew + kGroups * kRegsTransform + kRegsEpilogue) <= kRegsLaunch * kThreadsTc &&
               128 * (kRegsFew + kGroups * kRegsTransformWide + kRegsEpilogueWide) <= kRegsLaunch * kThreadsTc,
               "the shares come out of what the block was launched with");
@@ -188,7 +188,7 @@ struct GatherRows {
                 const bool pv = p < prm.P;
 #pragma unroll
                 for (int i = 0; i < kRowsPerThread; ++i) {
-                    const bool in = pv && ok[i] && (unsigned)(hs + dh[i]) < (unsigned)prm.H &&
+                    const bool in = pv && (unsigned)(hs + dh[i]) < (unsigned)prm.H &&
                                     (unsigned)(ws + dw[i]) < (unsigned)prm.W;
                     v[i][j] = in ? __ldg(xp + base[i]) : 0.f;
                 }
@@ -217,23 +217,23 @@ struct GatherTaps {
     static constexpr int kLoaded = kSpan == 4 ? 6 : 8;       // of which loaded
     // register that holds the input of tap kw for the j-th of the thread's four output positions
     __device__ __forceinline__ static constexpr int idx(int kw, int j) { return kSpan == 4 ? kw + j : (j >> 1) * 4 + (j & 1) + kw; }
-    int base[kTriples], dh[kTriples], row_local[kTriples];
-    bool ok[kTriples];
+    int base[kTriples], dh[kTriples], row0;      // dh: far outside where the tuple has no rows; row0: tile row of the first tuple
+    __device__ __forceinline__ int row(int i) const { return row0 + kKw * kStride * i; }
     const float *src;
 
     __device__ __forceinline__ void init(const Params &prm, const float *x, int tile_origin, int grp, int limit)
     {
         src = x;
         const int first_triple = tile_origin / 3;
+        row0 = 3 * (first_triple + grp) - tile_origin;               // (may be -2, -1)
 #pragma unroll
         for (int i = 0; i < kTriples; ++i) {
             const int T = first_triple + grp + kStride * i;          // triple = (c, kh)
-            ok[i] = 3 * T < limit;
-            const int tt = ok[i] ? T : 0;
+            const bool ok = 3 * T < limit;
+            const int tt = ok ? T : 0;
             const int c = tt / prm.Kh, kh = tt - c * prm.Kh;
-            dh[i] = kh - prm.ph;
-            base[i] = (c * prm.H + dh[i]) * prm.W;
-            row_local[i] = 3 * T - tile_origin;                      // tile row of the kw = 0 tap (may be -2, -1)
+            base[i] = (c * prm.H + kh - prm.ph) * prm.W;
+            dh[i] = ok ? kh - prm.ph : INT32_MIN / 2;
         }
     }
     // v[i][0..7]: kSpan = 4: {left, m0, m1, m2, m3, right, -, -} for positions pbase..pbase+3;
@@ -249,7 +249,7 @@ struct GatherTaps {
             const float *xp = xz + (ho * prm.W + wo);
 #pragma unroll
             for (int i = 0; i < kTriples; ++i) {
-                const bool in = pv && ok[i] && (unsigned)(ho + dh[i]) < (unsigned)prm.H;
+                const bool in = pv && (unsigned)(ho + dh[i]) < (unsigned)prm.H;
                 const float *q = xp + base[i];
                 float *o = &v[i][s * 4];
                 if (kSpan == 4) {
@@ -291,23 +291,23 @@ struct GatherTapsS2 {
     {
         return kSpan == 4 ? 2 * j + kw : (j >> 1) * 5 + 2 * (j & 1) + kw;
     }
-    int base[kTriples], dh[kTriples], row_local[kTriples];
-    bool ok[kTriples];
+    int base[kTriples], dh[kTriples], row0;      // dh: far outside where the tuple has no rows; row0: tile row of the first tuple
+    __device__ __forceinline__ int row(int i) const { return row0 + kKw * kStride * i; }
     const float *src;
 
     __device__ __forceinline__ void init(const Params &prm, const float *x, int tile_origin, int grp, int limit)
     {
         src = x;
         const int first_triple = tile_origin / 3;
+        row0 = 3 * (first_triple + grp) - tile_origin;               // (may be -2, -1)
 #pragma unroll
         for (int i = 0; i < kTriples; ++i) {
             const int T = first_triple + grp + kStride * i;          // triple = (c, kh)
-            ok[i] = 3 * T < limit;
-            const int tt = ok[i] ? T : 0;
+            const bool ok = 3 * T < limit;
+            const int tt = ok ? T : 0;
             const int c = tt / prm.Kh, kh = tt - c * prm.Kh;
-            dh[i] = kh - prm.ph;
-            base[i] = (c * prm.H + dh[i]) * prm.W;
-            row_local[i] = 3 * T - tile_origin;
+            base[i] = (c * prm.H + kh - prm.ph) * prm.W;
+            dh[i] = ok ? kh - prm.ph : INT32_MIN / 2;
         }
     }
     __device__ __forceinline__ void load(const Params &prm, int z, int pbase, float (&v)[kTriples][kSlots]) const
@@ -322,7 +322,7 @@ struct GatherTapsS2 {
             const float *xp = xz + (hs * prm.W + 2 * wo);
 #pragma unroll
             for (int i = 0; i < kTriples; ++i) {
-                const bool in = pv && ok[i] && (unsigned)(hs + dh[i]) < (unsigned)prm.H;
+                const bool in = pv && (unsigned)(hs + dh[i]) < (unsigned)prm.H;
                 const float *q = xp + base[i];
                 float *o = &v[i][s * kPerSpan];
                 const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -350,23 +350,23 @@ struct GatherTaps7S2 {
     static constexpr int kSlots = 16;
     static constexpr int kLoaded = 14;
     __device__ __forceinline__ static constexpr int idx(int kw, int j) { return 1 + 2 * j + kw; }
-    int base[kTuples], dh[kTuples], row_local[kTuples];
-    bool ok[kTuples];
+    int base[kTuples], dh[kTuples], row0;      // dh: far outside where the tuple has no rows; row0: tile row of the first tuple
+    __device__ __forceinline__ int row(int i) const { return row0 + kKw * kStride * i; }
     const float *src;
 
     __device__ __forceinline__ void init(const Params &prm, const float *x, int tile_origin, int grp, int limit)
     {
         src = x;
         const int first_tuple = tile_origin / 7;
+        row0 = 7 * (first_tuple + grp) - tile_origin;
 #pragma unroll
         for (int i = 0; i < kTuples; ++i) {
             const int T = first_tuple + grp + kStride * i;           // tuple = (c, kh)
-            ok[i] = 7 * T < limit;
-            const int tt = ok[i] ? T : 0;
+            const bool ok = 7 * T < limit;
+            const int tt = ok ? T : 0;
             const int c = tt / prm.Kh, kh = tt - c * prm.Kh;
-            dh[i] = kh - prm.ph;
-            base[i] = (c * prm.H + dh[i]) * prm.W;
-            row_local[i] = 7 * T - tile_origin;
+            base[i] = (c * prm.H + kh - prm.ph) * prm.W;
+            dh[i] = ok ? kh - prm.ph : INT32_MIN / 2;
         }
     }
     __device__ __forceinline__ void load(const Params &prm, int z, int pbase, float (&v)[kTuples][kSlots]) const
@@ -378,7 +378,7 @@ struct GatherTaps7S2 {
         const int col0 = 2 * wo - 4;
 #pragma unroll
         for (int i = 0; i < kTuples; ++i) {
-            const bool in = pv && ok[i] && (unsigned)(hs + dh[i]) < (unsigned)prm.H;
+            const bool in = pv && (unsigned)(hs + dh[i]) < (unsigned)prm.H;
             const float4 *q = reinterpret_cast<const float4 *>(xp + base[i]);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -436,7 +436,7 @@ struct Gatherer<kMode, kHalf, kRows, true> {
     {
 #pragma unroll
         for (int i = 0; i < kTriples; ++i) {
-            if (g.row_local[i] >= kRows || g.row_local[i] <= -Impl::kKw) continue;   // no row of this tuple in the tile
+            if (g.row(i) >= kRows || g.row(i) <= -Impl::kKw) continue;   // no row of this tuple in the tile
             // square and split every loaded element once; the three taps are views of the same parts
             uint32_t h[Impl::kSlots], l[Impl::kSlots];
 #pragma unroll
@@ -447,7 +447,7 @@ struct Gatherer<kMode, kHalf, kRows, true> {
             }
 #pragma unroll
             for (int kw = 0; kw < Impl::kKw; ++kw) {
-                const int row = g.row_local[i] + kw;
+                const int row = g.row(i) + kw;
                 if ((unsigned)row < (unsigned)kRows) {
                     const uint32_t off = chunk_offset(row, kq);
                     *reinterpret_cast<uint4 *>(hi + off) =
