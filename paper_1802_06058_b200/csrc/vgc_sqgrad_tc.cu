@@ -424,6 +424,9 @@ struct Gatherer<kMode, kHalf, kRows, true> {
     // tuples of rows per thread; with 192 rows (16 threads side by side) 64 whole triples, no remainder
     static constexpr int kTriples = kMode == kGatherTaps7S2 ? 2 : kRows == kWideN ? 4 : kHalf ? 3 : 2;
     typedef typename TapsOf<kMode, kTriples>::type Impl;
+    // the tile is whole tuples (192 rows of a three-tap kernel, its origin a multiple of 192): no row to test, and a
+    // thread's rows are 48 apart, so that their swizzled places differ by constants
+    static constexpr bool kWhole = Impl::kKw * Impl::kStride * kTriples == kRows;
     struct Regs { float v[kTriples][Impl::kSlots]; };
     Impl g;
     __device__ __forceinline__ void init(const Params &prm, const float *x, const float *, int origin, int row0, int limit)
@@ -436,7 +439,7 @@ struct Gatherer<kMode, kHalf, kRows, true> {
     {
 #pragma unroll
         for (int i = 0; i < kTriples; ++i) {
-            if (g.row(i) >= kRows || g.row(i) <= -Impl::kKw) continue;   // no row of this tuple in the tile
+            if (!kWhole && (g.row(i) >= kRows || g.row(i) <= -Impl::kKw)) continue;   // no row of this tuple in the tile
             // square and split every loaded element once; the three taps are views of the same parts
             uint32_t h[Impl::kSlots], l[Impl::kSlots];
 #pragma unroll
@@ -448,7 +451,7 @@ struct Gatherer<kMode, kHalf, kRows, true> {
 #pragma unroll
             for (int kw = 0; kw < Impl::kKw; ++kw) {
                 const int row = g.row(i) + kw;
-                if ((unsigned)row < (unsigned)kRows) {
+                if (kWhole || (unsigned)row < (unsigned)kRows) {
                     const uint32_t off = chunk_offset(row, kq);
                     *reinterpret_cast<uint4 *>(hi + off) =
                         make_uint4(h[Impl::idx(kw, 0)], h[Impl::idx(kw, 1)], h[Impl::idx(kw, 2)], h[Impl::idx(kw, 3)]);
