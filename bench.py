@@ -1049,7 +1049,7 @@ def main():
         sections["note"] = "section split measured in the unfused form (s written, then read by compress); ms_per_step is the fused step"
     traffic = ncu_traffic()
     compress_traffic = traffic.get("compress_bytes_per_param")
-    compress_roofline = {"kernel": "compress_phase_a + compress_count + compress_emit", "bound": "hbm",
+    compress_roofline = {"kernel": "compress_step + encode_step", "bound": "hbm",
                          "achieved": gbs(compress_bytes, co_ms), "peak": pk["hbm_gbs"], "unit": "GB/s",
                          "frac": gbs(compress_bytes, co_ms) / pk["hbm_gbs"],
                          "frac_of_8tbs": gbs(compress_bytes, co_ms) / HBM_NOMINAL_GBS,

@@ -94,7 +94,7 @@ constexpr int kLoSlotsAT = 2 * kLoSlots;
 constexpr int kSplitA = 4, kSplitB = kGroups > 2 ? 6 : 7, kSplitLo = kGroups > 2 ? 4 : 3;   // 16-KB units: A raw, B raw/hi, B lo (+ A in TMEM)
 static_assert((kSplitA + kSplitB + kSplitLo) * kRawBytesA <= (kRawSlots + kLoSlots) * kRawStageBytes, "smem budget");
 // Wide form (the kernels that gather several taps at a time, tiles of 192 columns): the tensor core takes an N = 192
-// instruction in little more time than an N = 128 one, and 192 rows of the im2col view are 64 whole triples.  The raw A
+// instruction in no more time than an N = 128 one (98 busy cycles by the counters, 110), and 192 rows of the im2col view are 64 whole triples.  The raw A
 // tiles have a ring of two, the B tile and its lo part one of four, A in tensor memory two slots beside two accumulators.
 constexpr int kWideN = 192, kWideA = 2, kWideB = 4, kWideTmemA = 2;
 static_assert(kWideA * kRawBytesA + 2 * kWideB * kWideN * kBK * 4 <= (kRawSlots + kLoSlots) * kRawStageBytes, "smem budget");
@@ -1777,7 +1777,9 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
 #define VGC_TC_FN(A, B_, AT) (ex ? (KernelFn)sqgrad_tc<kMajorK, A, B_, AT, true> : (KernelFn)sqgrad_tc<kMajorK, A, B_, AT, false>)
     if (!swapped) {     // S[o][idx]: m = o, n = idx
         prm.ld_m = n_im2col; prm.ld_n = 1;
-        // wide tiles where they are fewer than narrow ones (a slice of one takes about as long as a slice of the other)
+        // wide tiles where they are fewer than narrow ones: a slice of one takes about 1750 cycles, of the other 1390 - 1500,
+        // for 1.5 times the columns (B200, one call: 128 channels 28 x 28, batch 32: 47.9 -> 43.0 us; all of ResNet-50,
+        // batch 32: 2167 -> 2020 us).  The wide per-example form adds an example's sums up within one accumulator run.
         const bool any_taps = taps || taps_s2 || taps7;
         const bool wide = any_taps && (n_im2col + kWideN - 1) / kWideN < (n_im2col + kBN - 1) / kBN && (!ex || p_slices <= kChunk);
 #define VGC_TAPS_FN(B_) (wide ? (ex ? (KernelFn)sqgrad_tc<kMajorK, kTma, B_, true, true, false, kWideN>                          \
