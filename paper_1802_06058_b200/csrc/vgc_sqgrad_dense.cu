@@ -40,8 +40,9 @@ static_assert(kTmemCols == 512, "tensor memory");
 // Epilogue warps: with eight (two halves of the columns per lane quarter) a written tile leaves sooner (4096 x 4096, 16
 // examples: 15.0 us against 19.9); an added one needs the longer lead that four buffers per warp give its loads (25088 x
 // 4096, 64 examples: 178 us with four warps, 199 with eight).
-template <bool kAccumulate> struct Shape {
-    static constexpr int kHalves = kAccumulate ? 1 : 2, kEpilogueWarps = 4 * kHalves, kBoxes = kBN / 32 / kHalves;
+// kN: columns of a tile, 128 or (layers of few tiles) 64.
+template <bool kAccumulate, int kN> struct Shape {
+    static constexpr int kHalves = kAccumulate ? 1 : 2, kEpilogueWarps = 4 * kHalves, kBoxes = kN / 32 / kHalves;
     static constexpr int kThreads = 32 * (2 + kTransformWarps + kEpilogueWarps);
 };
 
@@ -61,12 +62,13 @@ template <int kLeft>
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kLeft) : "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-template <bool kAccumulate>
-__global__ void __launch_bounds__(Shape<kAccumulate>::kThreads, 1)
+template <bool kAccumulate, int kN>
+__global__ void __launch_bounds__(Shape<kAccumulate, kN>::kThreads, 1)
 sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
              const __grid_constant__ CUtensorMap map_s, const Params prm)
 {
-    constexpr int kEpilogueWarps = Shape<kAccumulate>::kEpilogueWarps, kBoxes = Shape<kAccumulate>::kBoxes;
+    constexpr int kEpilogueWarps = Shape<kAccumulate, kN>::kEpilogueWarps, kBoxes = Shape<kAccumulate, kN>::kBoxes;
+    constexpr uint32_t kBytesB = kN * kBK * 4;
     extern __shared__ uint8_t smem_raw_[];
     __shared__ __align__(8) uint64_t bars[3 * kRawSlots + 2 * kAccumulators + 1];
     __shared__ __align__(8) uint64_t box_full[kEpilogueWarps][kBoxes];
@@ -115,16 +117,16 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             int it = 0;
             bool ok = true;
             for (int t = first_tile; ok && t < prm.tiles; t += step) {
-                const int ty = t / prm.tiles_x, m0 = ty * kBM, n0 = (t - ty * prm.tiles_x) * kBN;
+                const int ty = t / prm.tiles_x, m0 = ty * kBM, n0 = (t - ty * prm.tiles_x) * kN;
                 for (int s = 0; s < k_slices; ++s, ++it) {
                     const int st = it % kRawSlots;
                     if (!mbar_wait(smem_u32(&empty[st]), ((uint32_t)(it / kRawSlots) & 1u) ^ 1u, &abort_flag, 32)) { ok = false; break; }
                     const uint32_t full = smem_u32(&raw_full[st]), dst = smem_base + (uint32_t)st * kStageBytes;
-                    mbar_expect_tx(full, kStageBytes);
+                    mbar_expect_tx(full, kTileBytes + kBytesB);
 #pragma unroll
                     for (int j = 0; j < 4; ++j) tma_load_2d(dst + j * 4096, &map_a, full, m0 + 32 * j, s * kBK);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) tma_load_2d(dst + kTileBytes + j * 4096, &map_b, full, n0 + 32 * j, s * kBK);
+                    for (int j = 0; j < kN / 32; ++j) tma_load_2d(dst + kTileBytes + j * 4096, &map_b, full, n0 + 32 * j, s * kBK);
                 }
             }
             if (abort_flag) {                            // loads already issued must land before the block may exit
@@ -139,7 +141,7 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             const uint32_t desc_hi = (uint32_t)(smem_desc(0, 4096u, 512u, 1u) >> 32);
             const uint32_t desc_lo0 = (uint32_t)smem_desc(0, 4096u, 512u, 1u);
             auto desc_at = [&](uint32_t lo16) -> uint64_t { return ((uint64_t)desc_hi << 32) | (desc_lo0 + lo16); };
-            const uint32_t idesc = instr_desc(kMajorK, kBN, kBM) | (1u << 16);        // A K-major (tensor memory), B MN-major
+            const uint32_t idesc = instr_desc(kMajorK, kN, kBM) | (1u << 16);        // A K-major (tensor memory), B MN-major
             int it = 0, c = 0;                           // running numbers of the slice and of the chunk
             bool ok = true;
             for (int t = first_tile; ok && t < prm.tiles; t += step) {
@@ -210,7 +212,7 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             }
             uint8_t *hi = smem_gen + (uint32_t)st * kStageBytes + kTileBytes, *lo = smem_gen + kLoBase + (uint32_t)ls * kTileBytes;
 #pragma unroll
-            for (int u0 = 0; u0 < (int)(kTileBytes / 16 / 128); u0 += 4) {
+            for (int u0 = 0; u0 < (int)(kBytesB / 16 / 128); u0 += 4) {
                 float4 v[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const float4 *>(hi + 16 * (tt + (u0 + u) * 128));
@@ -233,7 +235,7 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             const int ty = t / prm.tiles_x;
             const uint32_t full = smem_u32(&box_full[e][j]);
             mbar_expect_tx(full, kBoxBytes);
-            tma_load_2d(box0 + j * kBoxBytes, &map_s, full, (t - ty * prm.tiles_x) * kBN + (int)first_col + 32 * j, ty * kBM + 32 * (int)q);
+            tma_load_2d(box0 + j * kBoxBytes, &map_s, full, (t - ty * prm.tiles_x) * kN + (int)first_col + 32 * j, ty * kBM + 32 * (int)q);
         };
         int waited[kBoxes] = {};                         // loads of box j waited for (lane 0: for an abort)
         if (kAccumulate && lane == 0 && first_tile < prm.tiles)
@@ -242,7 +244,7 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
         int c = 0;                                       // running number of the tile
         bool ok = true;
         for (int t = first_tile; ok && t < prm.tiles; t += step, ++c) {
-            const int ty = t / prm.tiles_x, m0 = ty * kBM + 32 * (int)q, n0 = (t - ty * prm.tiles_x) * kBN + (int)first_col;
+            const int ty = t / prm.tiles_x, m0 = ty * kBM + 32 * (int)q, n0 = (t - ty * prm.tiles_x) * kN + (int)first_col;
             const int a0 = c * chunks, b = a0 % kAccumulators;
             for (int i = 0; ok && i < chunks; ++i)
                 ok = mbar_wait(smem_u32(&acc_full[(a0 + i) % kAccumulators]), (uint32_t)((a0 + i) / kAccumulators) & 1u, &abort_flag, 32);
@@ -341,25 +343,32 @@ vgc_status dense_sqgrad_linear(const float *x, const float *delta, int B, int in
         !make_map(&map_b, x, 2, dims_b, str_b, box, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B) ||
         !make_map(&map_s, S, 2, dims_s, str_b, box_s, CU_TENSOR_MAP_SWIZZLE_128B))
         return VGC_ERR_CUDA;
-    auto fn = accumulate ? sqgrad_dense<true> : sqgrad_dense<false>;
-    static bool configured[2][64];
+    // 64 columns where tiles of 128 leave half of the SMs idle: half of B's transform and of the result per block
+    // (128 examples, 1024 x 1024: 7.2 -> 6.4 us; from there on it is the slices one after another, twelve instructions of about
+    // 100 cycles whatever their columns: rings of twice the depth changed nothing)
+    const long long rows_m = (out + kBM - 1) / kBM;
+    const bool narrow = rows_m * ((in + kBN - 1) / kBN) <= 74;
+    const int tile_n = narrow ? 64 : kBN, form = (accumulate ? 1 : 0) + (narrow ? 2 : 0);
+    auto fn = accumulate ? (narrow ? sqgrad_dense<true, 64> : sqgrad_dense<true, kBN>)
+                         : (narrow ? sqgrad_dense<false, 64> : sqgrad_dense<false, kBN>);
+    static bool configured[4][64];
     int dev = -1;
     VGC_CUDA_OK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64 || !configured[accumulate ? 1 : 0][dev]) {
+    if (dev < 0 || dev >= 64 || !configured[form][dev]) {
         VGC_CUDA_OK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-        if (dev >= 0 && dev < 64) configured[accumulate ? 1 : 0][dev] = true;
+        if (dev >= 0 && dev < 64) configured[form][dev] = true;
     }
     Params prm;
     prm.k_slices = (B + kBK - 1) / kBK;
-    prm.tiles_x = (in + kBN - 1) / kBN;
-    const long long tiles = (long long)prm.tiles_x * ((out + kBM - 1) / kBM);
+    prm.tiles_x = (in + tile_n - 1) / tile_n;
+    const long long tiles = (long long)prm.tiles_x * rows_m;
     if (tiles >= (1LL << 26)) return VGC_ERR_UNSUPPORTED;
     prm.tiles = (int)tiles;
     prm.scale = scale;
     prm.status = static_cast<uint32_t *>(ws);
     // as few rounds as there have to be, of equal length
     const int rounds = (prm.tiles + 147) / 148, blocks = (prm.tiles + rounds - 1) / rounds;
-    const int threads = accumulate ? Shape<true>::kThreads : Shape<false>::kThreads;
+    const int threads = accumulate ? Shape<true, kBN>::kThreads : Shape<false, kBN>::kThreads;
     VGC_CUDA_OK(launch_kernel(fn, dim3((unsigned)blocks), dim3((unsigned)threads), kSmemBytes, st, true, map_a, map_b, map_s, prm));
     count_launch();
     return VGC_OK;

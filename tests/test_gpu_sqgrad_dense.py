@@ -14,6 +14,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,n_in,n_out", [
     (1, 8192, 8192), (9, 4100, 2052), (31, 2048, 1000), (33, 1028, 1092), (64, 4096, 4096), (64, 5000, 3004),   # one slice to many tiles
     (255, 516, 516), (256, 512, 1000), (257, 512, 516), (512, 260, 516), (511, 2048, 132), (513, 512, 516),     # one and two accumulators
+    (128, 1000, 1024), (70, 2364, 512), (300, 68, 1028), (130, 9472, 128), (130, 9476, 128),                   # 64 columns: at most 74 tiles of 128
     (1, 3, 5), (5, 32, 33), (64, 63, 129), (65, 64, 64), (129, 1000, 10), (200, 333, 257), (1024, 40, 36), (1025, 33, 65),
     (128, 1031, 1009)])
 def test_dense(B, n_in, n_out):
