@@ -91,23 +91,28 @@ __device__ __forceinline__ void add_flat(const Shared &sm, int W, const uint32_t
     longest = __reduce_max_sync(0xffffffffu, longest);
     const uint32_t pieces = (longest + kPiece - 1) / kPiece, units = pieces * (uint32_t)W;
     bool bad = false;
-    auto fetch = [&](uint32_t unit, const int32_t *&ge) -> uint32_t {
+    // this lane's word of a piece; `in`: the piece reaches this lane and the word's index lies inside u (in a buffer of 2^28
+    // elements no word could serve as filler: every index is an element)
+    auto fetch = [&](uint32_t unit, const int32_t *&ge, bool &in) -> uint32_t {
         const uint32_t piece = unit / (uint32_t)W, w = unit - piece * (uint32_t)W;
         const uint32_t c = sm.count[w], len = (c + pieces - 1) / pieces;          // at most kPiece
         const uint32_t p = piece * len + lane, end = min((piece + 1) * len, c);
         ge = kHybrid ? nullptr : sm.gexp[w];
-        const uint32_t word = p < end ? sm.words[w][p] : 0xFFFFFFFFu;
-        if (p < end && (word >> 4) >= n) bad = true;
+        const uint32_t word = p < end ? sm.words[w][p] : 0u;
+        in = p < end && (word >> 4) < n;
+        if (p < end && !in) bad = true;
         return word;
     };
     const int32_t *ge_next = nullptr;
-    uint32_t next = warp < units ? fetch(warp, ge_next) : 0u;
+    bool in_next = false;
+    uint32_t next = warp < units ? fetch(warp, ge_next, in_next) : 0u;
     int k = 0;
     for (uint32_t unit = warp; unit < units; unit += warps) {
         const int32_t *ge = ge_next;
-        const uint32_t word = next, idx = word >> 4;
-        if (unit + warps < units) next = fetch(unit + warps, ge_next);
-        if (idx < n) atomicAdd(u + idx, value_of<kHybrid>(word, ge, offs, K, scale, tau, k));    // (else filler, or outside u)
+        const bool in = in_next;
+        const uint32_t word = next;
+        if (unit + warps < units) next = fetch(unit + warps, ge_next, in_next);
+        if (in) atomicAdd(u + (word >> 4), value_of<kHybrid>(word, ge, offs, K, scale, tau, k));
     }
     if (bad) atomicOr(dev_status, VGC_DEV_RANGE);
 }
