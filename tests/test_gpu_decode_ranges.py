@@ -68,3 +68,40 @@ def test_crowded_indices(W, density):
 def test_either_side_of_the_lines(n, words_per_element):
     offs = random_offsets(np.random.default_rng(4), n, 4)
     _check(n, offs, [_message(n, offs, words_per_element / 3, 90 + w) for w in range(3)])
+
+
+@pytest.mark.parametrize("lengths", [[20_000] + [0] * 7, [30_000, 15_001, 15_000, 14_999, 1, 33], [5, 9_000, 0, 70_000, 2, 35_000] * 10, [31], [33, 16]])
+def test_flat_messages_of_unequal_lengths(lengths):
+    """Few words, added: the pieces of every message are taken once, whatever the lengths beside it."""
+    n, offs = 8_000_003, np.array([0, 5, 70_000, 8_000_003], np.uint32)
+    msgs = []
+    for w, c in enumerate(lengths):
+        words, exps = _message(n, offs, 1.3 * c / n + 1e-6, 300 + w)
+        msgs.append((words[:c].clone(), exps))
+    assert [m[0].numel() for m in msgs] == lengths
+    _check(n, offs, msgs)
+
+
+def test_flat_form_costs_what_the_words_cost():
+    """Seven short messages beside a long one must not cost what seven long ones would (every piece of a message that ran
+    out of words once took a warp's turn: 5 to 13 times the long message's own time)."""
+    n = 30_000_000
+    offs = np.array([0, n], np.uint32)
+
+    def time(lengths):
+        msgs = [_message(n, offs, c / n, 400 + w) for w, c in enumerate(lengths)]
+        triples = [(m, torch.tensor([m.numel()], dtype=torch.int32, device="cuda"), e) for m, e in msgs]
+        u, st, o = torch.zeros(n, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda"), vgc.offsets_tensor(offs)
+        best = float("inf")
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                vgc.vgc_decode_accumulate(triples, o, 1.0, u, st)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+
+    alone = time([1_500_000])
+    assert time([1_500_000] + [200] * 63) < 3.0 * alone
