@@ -46,9 +46,11 @@ inline void count_launch(unsigned k = 1) { g_launches += k; }
 
 // ---- launches that follow one another closely ---------------------------------------------------------------------
 // A kernel launched with `overlap` may start while the kernel before it on the stream is still running (programmatic
-// dependent launch): its blocks take the SMs as they become free, and everything before its grid_wait() -- which every
-// kernel launched that way executes before it touches memory another kernel writes -- hides under that kernel's end.
-// grid_wait() returns once the kernel before has finished and its writes are visible.
+// dependent launch): its blocks take the SMs as they become free, and everything before its grid_wait() hides under that
+// kernel's end.  grid_wait() returns once the kernel before has finished and its writes are visible.  Every kernel launched
+// that way executes it in all its threads, before it touches memory that work ahead of it on the stream may write -- every
+// array of the caller's, the tensor offsets too.  The one exception: the second kernel of a call may read what only the
+// caller writes, where the first one calls grid_release() after its own grid_wait().
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // lets the next kernel of the stream start now, where it was launched with `overlap`
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }

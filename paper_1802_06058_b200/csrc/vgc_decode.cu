@@ -165,9 +165,9 @@ decode_flat(const __grid_constant__ DecodeViews views, int W, const uint32_t *__
     __shared__ FlatShared sm;
     const uint32_t tid = threadIdx.x;
     const bool in_smem = !kHybrid && (K + 1) <= kDecOffsSmem;
+    grid_wait();
     if (in_smem)
         for (int i = tid; i <= K; i += kFlatThreads) sm_offs[i] = group_offsets[i];
-    grid_wait();
     if (tid < (uint32_t)W) {
         sm.words[tid] = views.words[tid];
         sm.gexp[tid] = views.group_exp[tid];
@@ -696,8 +696,6 @@ decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *_
 
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool in_smem = !kHybrid && (K + 1) <= kDecOffsSmem;
-    if (in_smem)
-        for (int i = tid; i <= K; i += kTileThreads) sm.offs[i] = group_offsets[i];
     const uint32_t *offs = in_smem ? sm.offs : group_offsets;
     if (tid == 0) sm.unfit = 0;
     if (tid < (uint32_t)W) {
@@ -705,6 +703,8 @@ decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *_
         sm.gexp[tid] = views.group_exp[tid];
     }
     grid_wait();
+    if (in_smem)
+        for (int i = tid; i <= K; i += kTileThreads) sm.offs[i] = group_offsets[i];
     if (tid < (uint32_t)W) {
         // never read past the buffer the caller says it has: a truncated message (VGC_DEV_CAPACITY at the sender)
         // carries the count that was needed, not the count that was written

@@ -155,7 +155,8 @@ compress_step(const __grid_constant__ Args a)
 
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x;
     const int K = a.K;
-    grid_release();
+    grid_wait();
+    grid_release();                                     // in this order: encode_step reads the offsets before it waits for us
     const bool offs_in_smem = kQuantise && (K + 1) <= kOffsSmem;
     if (offs_in_smem) {                                 // asynchronously: the first tile's loads go out before they arrive
         for (int i = tid; i <= K; i += kThreads)
@@ -179,7 +180,6 @@ compress_step(const __grid_constant__ Args a)
     auto record = [&](int k, uint32_t most) {
         atomicMax(k == k_first ? sm_rec_max : k == k_last ? sm_rec_max + 1 : rec_max + k, most);
     };
-    grid_wait();
     uint32_t buf = 0;
     for (uint32_t base = lo; base < hi; base += a.tile, buf ^= 1) {
         const uint32_t end = hi - base < a.tile ? hi : base + a.tile;
@@ -416,7 +416,8 @@ compress_step(const __grid_constant__ Args a)
     }
 }
 
-// The second kernel: same blocks, same ranges.
+// The second kernel: same blocks, same ranges.  Before its grid_wait() it reads the offsets only (from L2), which nothing
+// writes any more: it starts when every block of the first kernel has passed its own.
 template <bool kQuantise>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
 encode_step(const __grid_constant__ Args a)
@@ -431,7 +432,8 @@ encode_step(const __grid_constant__ Args a)
     const int K = a.K;
     const bool offs_in_smem = kQuantise && (K + 1) <= kOffsSmem;
     if (offs_in_smem)
-        for (int i = tid; i <= K; i += kThreads) sm_offs[i] = a.group_offsets[i];
+        for (int i = tid; i <= K; i += kThreads) sm_offs[i] = __ldcg(a.group_offsets + i);
+    else if (kQuantise) grid_wait();                    // read where they are, through L1
     const uint32_t *offs = offs_in_smem ? sm_offs : a.group_offsets;
     const uint32_t lo = b * a.per_block;
     const uint32_t hi = (uint32_t)((size_t)lo + a.per_block < a.n ? (size_t)lo + a.per_block : a.n);
