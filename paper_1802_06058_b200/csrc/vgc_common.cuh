@@ -51,6 +51,9 @@ inline void count_launch(unsigned k = 1) { g_launches += k; }
 // that way executes it in all its threads, before it touches memory that work ahead of it on the stream may write -- every
 // array of the caller's, the tensor offsets too.  The one exception: the second kernel of a call may read what only the
 // caller writes, where the first one calls grid_release() after its own grid_wait().
+// A kernel launched that way may be alive while the one ahead writes what it is going to read.  The non-coherent loads
+// (__ldg, const __restrict__ parameters) are defined only for data that nobody writes during the kernel's life, so these
+// kernels use ordinary ones.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // lets the next kernel of the stream start now, where it was launched with `overlap`
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }

@@ -158,8 +158,8 @@ __device__ __forceinline__ void add_flat(const Shared &sm, const FlatPlan &plan,
 
 template <bool kHybrid>
 __global__ void __launch_bounds__(kFlatThreads, kFlatBlocksPerSm)
-decode_flat(const __grid_constant__ DecodeViews views, int W, const uint32_t *__restrict__ group_offsets, int K, float scale,
-            float tau, float *__restrict__ u, size_t n, uint32_t *dev_status)
+decode_flat(const __grid_constant__ DecodeViews views, int W, const uint32_t *group_offsets, int K, float scale,
+            float tau, float *u, size_t n, uint32_t *dev_status)
 {
     __shared__ uint32_t sm_offs[kDecOffsSmem];
     __shared__ FlatShared sm;
@@ -279,7 +279,7 @@ constexpr uint32_t kScatterPiece = 32768;
 
 template <bool kHybrid>
 __device__ __forceinline__ bool scatter_range(TileShared &sm, int W, const uint32_t *offs, int K, float scale, float tau,
-                                              float *__restrict__ u, uint32_t lo, uint32_t hi)
+                                              float *u, uint32_t lo, uint32_t hi)
 {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     bool bad = false;
@@ -324,7 +324,7 @@ __device__ __forceinline__ bool scatter_range(TileShared &sm, int W, const uint3
 // Returns whether a word was out of place.
 template <bool kHybrid, bool kOverwrite>
 __device__ __forceinline__ bool ordered_range(TileShared &sm, float *tile, int W, const uint32_t *offs, int K, float scale, float tau,
-                                              float *__restrict__ u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
+                                              float *u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
 {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t *const cur = sm.cur, *const end = sm.end;
@@ -441,7 +441,7 @@ __device__ __forceinline__ bool ordered_range(TileShared &sm, float *tile, int W
 // Returns whether a word was out of place.
 template <bool kHybrid, bool kOverwrite>
 __device__ __forceinline__ bool exact_range(TileShared &sm, float *tile, int W, const uint32_t *offs, int g_first, float scale,
-                                            float tau, float *__restrict__ u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
+                                            float tau, float *u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
 {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t tile_addr = (uint32_t)__cvta_generic_to_shared(tile);
@@ -687,8 +687,8 @@ __device__ __forceinline__ bool exact_range(TileShared &sm, float *tile, int W, 
 // tiles that may span two tensors, tables made once per tensor, and the sparse forms.
 template <bool kHybrid, bool kOverwrite>
 __global__ void __launch_bounds__(kTileThreads, kBlocksPerSm)
-decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *__restrict__ group_offsets, int K,
-             float scale, float tau, float *__restrict__ u, size_t n, uint32_t chunk_elems, uint32_t tile_elems,
+decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *group_offsets, int K,
+             float scale, float tau, float *u, size_t n, uint32_t chunk_elems, uint32_t tile_elems,
              uint32_t *dev_status)
 {
     extern __shared__ __align__(16) float tile[];                // kTileMax floats

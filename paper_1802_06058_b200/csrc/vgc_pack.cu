@@ -35,7 +35,7 @@ __device__ __forceinline__ uint32_t code_length(uint32_t v)
 }
 
 // the numbers of this lane's 8 words of run `run` and how many of them exist; `bytes`: what they take
-__device__ __forceinline__ uint32_t lane_numbers(const uint32_t *__restrict__ words, uint32_t n, uint32_t run, uint32_t lane,
+__device__ __forceinline__ uint32_t lane_numbers(const uint32_t *words, uint32_t n, uint32_t run, uint32_t lane,
                                                  uint32_t (&v)[kPerLane], uint32_t &bytes)
 {
     const uint32_t first = run * kPackRun + lane * kPerLane;
@@ -71,8 +71,7 @@ __device__ __forceinline__ uint32_t warp_inclusive(uint32_t x, uint32_t lane)
 }
 
 __global__ void __launch_bounds__(kPackThreads)
-pack_count(const uint32_t *__restrict__ words, const uint32_t *__restrict__ nnz, uint32_t max_words,
-           uint32_t *__restrict__ block_bytes)
+pack_count(const uint32_t *words, const uint32_t *nnz, uint32_t max_words, uint32_t *block_bytes)
 {
     __shared__ uint32_t sm_tot[kPackWarps];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -96,9 +95,8 @@ pack_count(const uint32_t *__restrict__ words, const uint32_t *__restrict__ nnz,
 }
 
 __global__ void __launch_bounds__(kPackThreads)
-pack_emit(const uint32_t *__restrict__ words, const uint32_t *__restrict__ nnz, uint32_t max_words,
-          const uint32_t *__restrict__ block_bytes, uint8_t *__restrict__ packed, size_t capacity,
-          uint32_t *__restrict__ packed_bytes, uint32_t *dev_status)
+pack_emit(const uint32_t *words, const uint32_t *nnz, uint32_t max_words,
+          const uint32_t *block_bytes, uint8_t *packed, size_t capacity, uint32_t *packed_bytes, uint32_t *dev_status)
 {
     __shared__ __align__(16) uint8_t sm_bytes[kPackWarps * kRunBytesMax + 16];
     __shared__ unsigned long long sm_part[kPackWarps];
@@ -171,8 +169,7 @@ pack_emit(const uint32_t *__restrict__ words, const uint32_t *__restrict__ nnz, 
 }
 
 __global__ void __launch_bounds__(kPackThreads)
-unpack_runs(const uint8_t *__restrict__ packed, const uint32_t *__restrict__ nnz, uint32_t max_words,
-            uint32_t *__restrict__ words, uint32_t *dev_status)
+unpack_runs(const uint8_t *packed, const uint32_t *nnz, uint32_t max_words, uint32_t *words, uint32_t *dev_status)
 {
     constexpr int kWordsMax = kRunBytesMax / 4 + 4;                     // a run's bytes at any alignment, and a word to read past
     __shared__ uint32_t sm_words[kPackWarps][kWordsMax];

@@ -167,8 +167,7 @@ constexpr int kDenseFlush = 2;                        // rounds per fp32 sum
 
 template <int kTile, bool kVec>                        // kVec: in and out are multiples of 4
 __global__ void __launch_bounds__(kSimtThreads)
-sqgrad_dense_simt(const float *__restrict__ x, const float *__restrict__ delta, int B, int in, int out, float scale,
-                  int accumulate, float *__restrict__ S)
+sqgrad_dense_simt(const float *x, const float *delta, int B, int in, int out, float scale, int accumulate, float *S)
 {
     constexpr int kDenseK = kTile == 32 ? 64 : 32;                     // examples per round
     constexpr int kThreadsPerTile = (kTile / 4) * (kTile / 4), kGroups = kSimtThreads / kThreadsPerTile;
@@ -190,12 +189,12 @@ sqgrad_dense_simt(const float *__restrict__ x, const float *__restrict__ delta, 
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (!valid) return v;
         if (kVec) {
-            if (at < limit) v = __ldg(reinterpret_cast<const float4 *>(row + at));
+            if (at < limit) v = *reinterpret_cast<const float4 *>(row + at);
         } else {
-            if (at < limit) v.x = __ldg(row + at);
-            if (at + 1 < limit) v.y = __ldg(row + at + 1);
-            if (at + 2 < limit) v.z = __ldg(row + at + 2);
-            if (at + 3 < limit) v.w = __ldg(row + at + 3);
+            if (at < limit) v.x = row[at];
+            if (at + 1 < limit) v.y = row[at + 1];
+            if (at + 2 < limit) v.z = row[at + 2];
+            if (at + 3 < limit) v.w = row[at + 3];
         }
         return v;
     };

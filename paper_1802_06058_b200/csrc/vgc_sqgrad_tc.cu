@@ -190,7 +190,7 @@ struct GatherRows {
                 for (int i = 0; i < kRowsPerThread; ++i) {
                     const bool in = pv && (unsigned)(hs + dh[i]) < (unsigned)prm.H &&
                                     (unsigned)(ws + dw[i]) < (unsigned)prm.W;
-                    v[i][j] = in ? __ldg(xp + base[i]) : 0.f;
+                    v[i][j] = in ? xp[base[i]] : 0.f;
                 }
             }
         } else if (kMode == kGatherErr) {
@@ -198,7 +198,7 @@ struct GatherRows {
 #pragma unroll
             for (int i = 0; i < kRowsPerThread; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) v[i][j] = (ok[i] && pbase + j < prm.P) ? __ldg(dz + (base[i] + j)) : 0.f;
+                for (int j = 0; j < 4; ++j) v[i][j] = (ok[i] && pbase + j < prm.P) ? dz[base[i] + j] : 0.f;
         }
     }
 };
@@ -253,15 +253,15 @@ struct GatherTaps {
                 const float *q = xp + base[i];
                 float *o = &v[i][s * 4];
                 if (kSpan == 4) {
-                    const float4 m = in ? __ldg(reinterpret_cast<const float4 *>(q)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    o[0] = (in && wo > 0) ? __ldg(q - 1) : 0.f;
+                    const float4 m = in ? *reinterpret_cast<const float4 *>(q) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    o[0] = (in && wo > 0) ? q[-1] : 0.f;
                     o[1] = m.x; o[2] = m.y; o[3] = m.z; o[4] = m.w;
-                    o[5] = (in && wo + 4 < prm.W) ? __ldg(q + 4) : 0.f;
+                    o[5] = (in && wo + 4 < prm.W) ? q[4] : 0.f;
                 } else {
-                    const float2 m = in ? __ldg(reinterpret_cast<const float2 *>(q)) : make_float2(0.f, 0.f);
-                    o[0] = (in && wo > 0) ? __ldg(q - 1) : 0.f;
+                    const float2 m = in ? *reinterpret_cast<const float2 *>(q) : make_float2(0.f, 0.f);
+                    o[0] = (in && wo > 0) ? q[-1] : 0.f;
                     o[1] = m.x; o[2] = m.y;
-                    o[3] = (in && wo + 2 < prm.W) ? __ldg(q + 2) : 0.f;
+                    o[3] = (in && wo + 2 < prm.W) ? q[2] : 0.f;
                 }
             }
         }
@@ -326,11 +326,11 @@ struct GatherTapsS2 {
                 const float *q = xp + base[i];
                 float *o = &v[i][s * kPerSpan];
                 const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 m0 = in ? __ldg(reinterpret_cast<const float4 *>(q)) : zero;
-                o[0] = (in && wo > 0) ? __ldg(q - 1) : 0.f;
+                const float4 m0 = in ? *reinterpret_cast<const float4 *>(q) : zero;
+                o[0] = (in && wo > 0) ? q[-1] : 0.f;
                 o[1] = m0.x; o[2] = m0.y; o[3] = m0.z; o[4] = m0.w;
                 if (kSpan == 4) {
-                    const float4 m1 = in ? __ldg(reinterpret_cast<const float4 *>(q) + 1) : zero;
+                    const float4 m1 = in ? reinterpret_cast<const float4 *>(q)[1] : zero;
                     o[5] = m1.x; o[6] = m1.y; o[7] = m1.z; o[8] = m1.w;
                 }
             }
@@ -383,7 +383,7 @@ struct GatherTaps7S2 {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const bool inside = in && (unsigned)(col0 + 4 * u) < (unsigned)prm.W;
-                const float4 m = inside ? __ldg(q + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 m = inside ? q[u] : make_float4(0.f, 0.f, 0.f, 0.f);
                 v[i][4 * u] = m.x; v[i][4 * u + 1] = m.y; v[i][4 * u + 2] = m.z; v[i][4 * u + 3] = m.w;
             }
         }
@@ -1220,7 +1220,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
 struct ResultPtrs { float *S[kMaxBatch]; };
 
 __global__ void __launch_bounds__(256)
-sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, int units_per_tile,
+sqgrad_tc_combine(const float *partial, int units_q, int units_r, int units_per_tile,
                   int tile_n, int tiles_x, int tiles_y, int M, int N, float scale, int accumulate, const ResultPtrs results,
                   long long ld_m, long long ld_n)
 {
@@ -1235,7 +1235,7 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
     auto block_of = [&](int u) -> int { return u < big ? u / (units_q + 1) : units_r + (u - big) / units_q; };
     const int b_first = block_of(t_lo), b_last = block_of(t_lo + units_per_tile - 1);
     if (b_first == b_last) return;
-    float *__restrict__ S = results.S[blockIdx.y];                         // blockIdx.y: layer of the batch
+    float *S = results.S[blockIdx.y];                                      // blockIdx.y: layer of the batch
     const int tx = tile % tiles_x, ty = tile / tiles_x;
     const int r0 = (sub & 3) * 32, j0 = (sub >> 2) * 32;                  // patch origin inside the tile
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;              // lane -> row, warp -> four columns
@@ -1306,7 +1306,7 @@ sqgrad_tc_combine(const float *__restrict__ partial, int units_q, int units_r, i
 // eight warps in turn and their sums added in the order of the warps (a fixed order as well).  A chain of 148 partial tiles
 // took 22 us in the kernel above.
 __global__ void __launch_bounds__(256)
-sqgrad_tc_combine_many(const float *__restrict__ partial, int units_q, int units_r, int units_per_tile,
+sqgrad_tc_combine_many(const float *partial, int units_q, int units_r, int units_per_tile,
                        int tile_n, int tiles_x, int tiles_y, int M, int N, float scale, int accumulate, const ResultPtrs results,
                        long long ld_m, long long ld_n)
 {
@@ -1596,7 +1596,7 @@ sqgrad_repack(const __grid_constant__ RepackJobs jobs)
             for (int u = 0; u < kRepackRun / 32; ++u) {
                 const uint32_t i = lane + 32u * u, q = p0 + i;
                 const uint32_t dr = by_P(q), dc = by_B(z0 + dr), plane = (z0 + dr - dc * B) * job.C + (c0 + dc);
-                v[u] = i < left ? __ldg(job.in + ((size_t)plane * P + (q - dr * P))) : 0.f;
+                v[u] = i < left ? job.in[(size_t)plane * P + (q - dr * P)] : 0.f;
             }
         } else
 #pragma unroll
@@ -1610,7 +1610,7 @@ sqgrad_repack(const __grid_constant__ RepackJobs jobs)
             } else plane = row0 + dr;
             const uint32_t ho = by_Wo(p), wo = p - ho * job.Wo;
             // columns wo >= wo_valid are zero padding
-            v[u] = i < left && wo < (uint32_t)job.wo_valid ? __ldg(job.in + plane * job.HW + (ho * row_step + wo * job.sw)) : 0.f;
+            v[u] = i < left && wo < (uint32_t)job.wo_valid ? job.in[plane * job.HW + (ho * row_step + wo * job.sw)] : 0.f;
         }
 #pragma unroll
         for (int u = 0; u < kRepackRun / 32; ++u)

@@ -79,3 +79,68 @@ def test_offsets_written_just_ahead(n, K):
         # (where two words meet in an element, the order of their additions is free in the sparse forms)
         assert all(torch.allclose(x, y, rtol=2.0 ** -22, atol=1e-8) for x, y in zip(b[3], ref[3]))
     assert int(written.status.item()) == 0
+
+
+def _alternate(call, inputs, results):
+    """call(input, result) for the inputs one after another without a pause, against the same with the stream idle before each."""
+    want = []
+    for i in inputs:
+        torch.cuda.synchronize()
+        call(i, results[0])
+        torch.cuda.synchronize()
+        want.append(results[0].clone())
+    for _ in range(4):
+        for i, r in zip(inputs, results):
+            call(i, r)
+        for w, r in zip(want, results):
+            assert torch.equal(w, r)
+
+
+# padded planes (7 x 7, pitch 196 bytes) with stride 1 and 2, subsampled planes, planes merged channel by channel, gathered rows
+@pytest.mark.parametrize("C,H,Cout,k,stride,pad,exact", [(64, 7, 96, 3, 1, 1, False), (64, 7, 96, 3, 1, 1, True), (32, 14, 64, 3, 2, 1, False),
+                                                         (128, 28, 96, 1, 2, 0, False), (256, 7, 96, 1, 1, 0, False),
+                                                         (48, 9, 40, 5, 1, 2, False), (64, 28, 64, 3, 1, 1, False)])
+def test_layers_change_between_calls_on_one_workspace(C, H, Cout, k, stride, pad, exact):
+    B, Ho = 16, (H + 2 * pad - k) // stride + 1
+    geo = (B, C, H, H, Cout, k, k, stride, stride, pad, pad)
+    need = (vgc.vgc_sqgrad_conv_exact_workspace_bytes if exact else vgc.vgc_sqgrad_conv_workspace_bytes)(*geo)
+    ws = torch.zeros(need, dtype=torch.uint8, device="cuda")
+    inputs = [(torch.randn(B, C, H, H, device="cuda"), torch.randn(B, Cout, Ho, Ho, device="cuda")) for _ in range(4)]
+    fn = vgc.vgc_sqgrad_conv_exact if exact else vgc.vgc_sqgrad_conv
+    _alternate(lambda i, S: fn(*i, (k, k), (stride, stride), (pad, pad), 1.0, S, ws=ws), inputs,
+               [torch.empty(Cout * C * k * k, device="cuda") for _ in inputs])
+    assert int(ws[:4].view(torch.int32).item()) == 0
+
+
+@pytest.mark.parametrize("B,n_in,n_out", [(32, 64, 40), (16, 1024, 4096), (600, 96, 64)])
+def test_layer_input_written_just_ahead(B, n_in, n_out):
+    """x of a layer is the result of the call ahead (CUDA cores, tensor cores, long reductions)."""
+    ws = torch.zeros(max(vgc.vgc_sqgrad_linear_workspace_bytes(8, n_in, B), vgc.vgc_sqgrad_linear_workspace_bytes(B, n_in, n_out)),
+                     dtype=torch.uint8, device="cuda")
+    x, d = torch.empty(B * n_in, device="cuda"), torch.randn(B, n_out, device="cuda")
+    inputs = [(torch.randn(8, n_in, device="cuda"), torch.randn(8, B, device="cuda")) for _ in range(4)]
+
+    def call(i, S):
+        vgc.vgc_sqgrad_linear(*i, 1.0, x, ws=ws)
+        vgc.vgc_sqgrad_linear(x.view(B, n_in), d, 1.0, S, ws=ws)
+
+    _alternate(call, inputs, [torch.empty(n_in * n_out, device="cuda") for _ in inputs])
+
+
+def test_stream_packed_just_ahead():
+    n = 300_000
+    status, ws = torch.zeros(1, dtype=torch.int32, device="cuda"), torch.zeros(vgc.vgc_pack_workspace_bytes(n), dtype=torch.uint8, device="cuda")
+    packed, nbytes = torch.zeros(vgc.vgc_pack_bound_bytes(n), dtype=torch.uint8, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    inputs = []
+    for seed in range(4):
+        words, _ = workloads.random_message(4 * n, np.array([0, 4 * n], np.uint32), 0.2, seed, "cuda")
+        inputs.append((words[:n].clone(), torch.tensor([min(n, words.numel())], dtype=torch.int32, device="cuda")))
+
+    def call(i, back):
+        back.zero_()
+        vgc.vgc_pack_indices(*i, packed, nbytes, status, ws)
+        vgc.vgc_unpack_indices(packed, i[1], back, status)
+
+    back = [torch.zeros(n, dtype=torch.int32, device="cuda") for _ in inputs]
+    _alternate(call, inputs, back)
+    assert all(torch.equal(b[:i[0].numel()], i[0]) for b, i in zip(back, inputs)) and int(status.item()) == 0
