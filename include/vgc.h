@@ -40,7 +40,8 @@ typedef enum {
     VGC_ERR_INVALID_ARG = 1, /* null / misaligned pointer, negative size, n > 2^28, bad alpha or zeta */
     VGC_ERR_UNSUPPORTED = 2, /* shape outside what the kernels cover                               */
     VGC_ERR_WORKSPACE = 3,   /* workspace smaller than the matching *_workspace_bytes()             */
-    VGC_ERR_CUDA = 4         /* a CUDA call failed; cudaGetLastError() has the detail               */
+    VGC_ERR_CUDA = 4         /* a CUDA call failed (VGC_DEBUG=1 in the environment names it on stderr), or a
+                                kernel was not compiled to the registers that its code shares out    */
 } vgc_status;
 
 /* bits OR-ed into *dev_status by kernels */

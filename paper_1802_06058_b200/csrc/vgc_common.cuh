@@ -8,6 +8,7 @@
 #include <cstdlib>
 
 #include "vgc.h"
+#include "vgc_once.cuh"
 
 #ifndef __CUDA_ARCH__
 #define VGC_HOST_ONLY 1
@@ -16,6 +17,7 @@
 namespace vgc {
 
 constexpr int kWarp = 32;
+constexpr int kSmCount = 148;       // SMs of a B200: work is cut by this number, so that results do not depend on the device
 
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -75,6 +77,25 @@ cudaError_t launch_kernel(void (*fn)(Params...), dim3 grid, dim3 block, size_t s
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, fn, static_cast<Params>(given)...);
+}
+
+// Lets a kernel use `bytes` of dynamic shared memory on the current device.  regs > 0: it has to have been compiled to that
+// many registers (its code shares them out); cudaErrorInvalidKernelImage where it was not.
+inline cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes, int regs = 0)
+{
+    static OncePerDevice once;
+    int device = -1;
+    const cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)once(kernel, device, [&]() -> int {
+        if (regs > 0) {
+            cudaFuncAttributes attr;
+            const cudaError_t a = cudaFuncGetAttributes(&attr, kernel);
+            if (a != cudaSuccess) return (int)a;
+            if (attr.numRegs != regs) return (int)cudaErrorInvalidKernelImage;
+        }
+        return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    });
 }
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }

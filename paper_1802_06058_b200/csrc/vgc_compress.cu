@@ -1,6 +1,8 @@
 // C ABI of the compressor: one step of Algorithm 1 ("Basic") over the flat parameter buffer followed by Encode() -- the
 // 4-bit quantiser of Sec. 4.2 in the bit-level form of Sec. 4.4 and the 32-bit (value, index) word.  The kernel is in
 // vgc_step.cuh.
+#include <atomic>
+
 #include "vgc_step.cuh"
 
 using namespace vgc;
@@ -87,16 +89,15 @@ extern "C" vgc_status vgc_compress_static(const float *g, const float *s, float 
     // Host code sees g_compress_scratch only as a stand-in for the device array: the address a kernel can
     // use has to be asked for, once per device, with that device current.
     constexpr int kMaxDevices = 64;
-    static void *scratch_of_device[kMaxDevices] = {};
+    static std::atomic<void *> scratch_of_device[kMaxDevices] = {};
     int dev = -1;
     VGC_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevices) return VGC_ERR_UNSUPPORTED;
-    if (!scratch_of_device[dev]) {
-        void *p = nullptr;
-        VGC_CUDA_OK(cudaGetSymbolAddress(&p, g_compress_scratch));
-        if (!p) return VGC_ERR_CUDA;
-        scratch_of_device[dev] = p;
+    void *scratch = scratch_of_device[dev];
+    if (!scratch) {
+        VGC_CUDA_OK(cudaGetSymbolAddress(&scratch, g_compress_scratch));
+        if (!scratch) return VGC_ERR_CUDA;
+        scratch_of_device[dev] = scratch;
     }
-    return vgc_compress(g, s, r, v, n, group_offsets, K, alpha, zeta, out, scratch_of_device[dev], kStaticScratchBytes,
-                        stream);
+    return vgc_compress(g, s, r, v, n, group_offsets, K, alpha, zeta, out, scratch, kStaticScratchBytes, stream);
 }

@@ -809,13 +809,6 @@ typedef void (*TilesFn)(const DecodeViews, int, const uint32_t *, int, float, fl
 vgc_status decode_launch(bool hybrid, bool overwrite, const vgc_message_view *msgs, int W, const uint32_t *group_offsets,
                          int K, float scale, float tau, float *u, size_t n, uint32_t *dev_status, cudaStream_t st)
 {
-    static int sm_count = 0;
-    if (sm_count == 0) {
-        int dev = 0, c = 0;
-        VGC_CUDA_OK(cudaGetDevice(&dev));
-        VGC_CUDA_OK(cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev));
-        sm_count = c > 0 ? c : 148;
-    }
     if (W == 0) {                                                // vgc_decode_sum of nothing
         VGC_CUDA_OK(cudaMemsetAsync(u, 0, n * sizeof(float), st));
         return VGC_OK;
@@ -838,7 +831,7 @@ vgc_status decode_launch(bool hybrid, bool overwrite, const vgc_message_view *ms
         }
         if (!ow && most_words * kSparseAdd < n) {                // whatever the counts on the device say
             const size_t want = ((longest + kPiece - 1) / kPiece * wb + kFlatThreads / 32 - 1) / (kFlatThreads / 32);
-            const size_t most = (size_t)sm_count * kFlatBlocksPerSm;
+            const size_t most = (size_t)kSmCount * kFlatBlocksPerSm;
             const unsigned blocks = (unsigned)(want < 1 ? 1 : want < most ? want : most);
             VGC_CUDA_OK(launch_kernel(hybrid ? decode_flat<true> : decode_flat<false>, dim3(blocks), dim3(kFlatThreads), 0, st, true,
                                       views, wb, group_offsets, K, scale, tau, u, n, dev_status));
@@ -847,7 +840,7 @@ vgc_status decode_launch(bool hybrid, bool overwrite, const vgc_message_view *ms
         }
         // one contiguous range per block, kBlocksPerSm blocks per SM, tiles of equal size; not less than 2048 elements
         // each: a range costs its search
-        size_t chunk = (n + (size_t)sm_count * kBlocksPerSm - 1) / ((size_t)sm_count * kBlocksPerSm);
+        size_t chunk = (n + (size_t)kSmCount * kBlocksPerSm - 1) / ((size_t)kSmCount * kBlocksPerSm);
         chunk = chunk > 2048 ? chunk : 2048;
         chunk = (chunk + 3) / 4 * 4;
         const size_t tiles = (chunk + kTileMax - 1) / kTileMax;
@@ -855,14 +848,7 @@ vgc_status decode_launch(bool hybrid, bool overwrite, const vgc_message_view *ms
         const unsigned blocks = (unsigned)((n + chunk - 1) / chunk);
         TilesFn fn = hybrid ? (ow ? decode_tiles<true, true> : decode_tiles<true, false>)
                             : (ow ? decode_tiles<false, true> : decode_tiles<false, false>);
-        static TilesFn configured[4];
-        static int n_configured = 0;
-        bool seen = false;
-        for (int i = 0; i < n_configured; ++i) seen = seen || configured[i] == fn;
-        if (!seen) {
-            VGC_CUDA_OK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileMax * 4));
-            if (n_configured < 4) configured[n_configured++] = fn;
-        }
+        VGC_CUDA_OK(allow_dynamic_smem(reinterpret_cast<const void *>(fn), (size_t)kTileMax * 4));
         VGC_CUDA_OK(launch_kernel(fn, dim3(blocks), dim3(kTileThreads), (size_t)kTileMax * 4, st, true, views, wb, group_offsets, K,
                                   scale, tau, u, n, (uint32_t)chunk, tile_elems, dev_status));
         count_launch();

@@ -348,16 +348,10 @@ vgc_status dense_sqgrad_linear(const float *x, const float *delta, int B, int in
     // 100 cycles whatever their columns: rings of twice the depth changed nothing)
     const long long rows_m = (out + kBM - 1) / kBM;
     const bool narrow = rows_m * ((in + kBN - 1) / kBN) <= 74;
-    const int tile_n = narrow ? 64 : kBN, form = (accumulate ? 1 : 0) + (narrow ? 2 : 0);
+    const int tile_n = narrow ? 64 : kBN;
     auto fn = accumulate ? (narrow ? sqgrad_dense<true, 64> : sqgrad_dense<true, kBN>)
                          : (narrow ? sqgrad_dense<false, 64> : sqgrad_dense<false, kBN>);
-    static bool configured[4][64];
-    int dev = -1;
-    VGC_CUDA_OK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64 || !configured[form][dev]) {
-        VGC_CUDA_OK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-        if (dev >= 0 && dev < 64) configured[form][dev] = true;
-    }
+    VGC_CUDA_OK(allow_dynamic_smem(reinterpret_cast<const void *>(fn), kSmemBytes));
     Params prm;
     prm.k_slices = (B + kBK - 1) / kBK;
     prm.tiles_x = (in + tile_n - 1) / tile_n;

@@ -1351,7 +1351,6 @@ sqgrad_tc_combine_many(const float *partial, int units_q, int units_r, int units
 // sum per instruction), so an accumulator is handed to the round-to-nearest register sums after at most 8 slices
 // (96 instructions): results then sit 1 - 3e-6 below the exact sum, against the 1e-5 bound.
 constexpr int kChunk = 8;
-constexpr int kSmCount = 148;            // SMs of a B200
 // how many sqgrad launches the caller keeps in flight side by side (vgc_sqgrad_plan_hint)
 static int g_concurrent = 1;
 
@@ -1448,17 +1447,7 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
 {
     const Plan plan = make_plan(M, N, k_slices, n_layers, unit, tile_n);
     if (ws_bytes < tc_workspace_bytes(M, N, k_slices, n_layers, unit, tile_n)) return VGC_ERR_WORKSPACE;
-    static KernelFn configured[64];
-    static int n_configured = 0;
-    bool seen = false;
-    for (int i = 0; i < n_configured; ++i) seen = seen || configured[i] == kernel;
-    if (!seen) {
-        cudaFuncAttributes attr;
-        VGC_CUDA_OK(cudaFuncGetAttributes(&attr, kernel));
-        if (attr.numRegs != kRegsLaunch) return VGC_ERR_CUDA;        // the kernel's register shares assume this
-        VGC_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-        if (n_configured < 64) configured[n_configured++] = kernel;
-    }
+    VGC_CUDA_OK(allow_dynamic_smem(reinterpret_cast<const void *>(kernel), kSmemBytes, kRegsLaunch));
     prm.M = M; prm.N = N; prm.k_slices = k_slices;
     prm.unit = plan.unit; prm.units_per_tile = plan.units_per_tile; prm.units_total = plan.units_total;
     prm.units_q = plan.units_total / plan.blocks; prm.units_r = plan.units_total % plan.blocks;
