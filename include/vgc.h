@@ -14,7 +14,7 @@
  * General rules
  *   - Every pointer is a DEVICE pointer owned by the caller unless a parameter says "host".
  *     The library allocates nothing, keeps no state between calls and never synchronises:
- *     each call only enqueues work on `stream` and returns.
+ *     each call only enqueues work on `stream` and returns.  (vgc_step_host is the exception, see there.)
  *   - Pointers to fp32 / u32 arrays must be 16-byte aligned (whole allocations are).
  *   - Return value: a vgc_status detected on the host before anything is enqueued, or
  *     VGC_ERR_CUDA when a launch failed.  Conditions found on the device are OR-ed into the
@@ -281,6 +281,12 @@ vgc_status vgc_decode_sum(const vgc_message_view *msgs, int W, const uint32_t *g
  * first min(nnz, capacity) words into words_host.  Host buffers should be pinned.  Unlike the other
  * entry points this one WAITS for the stream (twice: the word count has to reach the host before the
  * words can be copied).  `out` holds device pointers as for vgc_compress; r, v are device state.
+ *
+ * The results are those of this order.  The copies themselves run ahead, on a stream of the library's own behind
+ * what `stream` holds at the call: a layer's kernels wait for that layer's copies only, and g arrives under the last
+ * layer's kernels.  Where x_dev, delta_dev and g_dev of the layers overlap one another, s_dev or ws_sqgrad, copies and
+ * kernels take turns on `stream` instead.  The first call of a thread that finds none free creates a stream and an
+ * event; up to eight such pairs are kept until the process ends (cudaDeviceReset with pairs kept is not supported).
  * ------------------------------------------------------------------------------------------- */
 typedef struct {
     int is_conv;                 /* 0: dense layer (C = in, Cout = out; H, W, K*, stride, pad ignored) */

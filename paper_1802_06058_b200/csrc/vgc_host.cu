@@ -6,7 +6,8 @@
 // Bound: the copies (PCIe).  They go back to back on a stream of the library's own, and a layer's kernels wait for that
 // layer's copies only, so that all but the last layer's run under the copies that follow (with everything on the caller's
 // stream every switch between copy and kernel cost 2 - 10 us besides; MLP 784-1024-1024-10, 128 examples, 9.5 MB:
-// 351 -> 261 us, of which the copies are 205).  Layers whose staging buffers overlap take turns on the caller's stream.
+// 351 -> 261 us, of which the copies are 205).  Where a staging buffer lies over another one or over memory that an earlier
+// layer's kernels write, copies and kernels take turns on the caller's stream.
 // The call waits for the stream twice (the word count must be known on the host before the words can be copied).
 #include <mutex>
 
@@ -67,7 +68,7 @@ void release(CopyLane &lane)
     destroy(lane);
 }
 
-// Copies of one call.  overlap() == false (staging shared between layers, or no stream to be had): all on the caller's stream.
+// Copies of one call.  Not `overlap`, or no stream to be had: all on the caller's stream.
 class Copies {
 public:
     Copies(cudaStream_t caller, bool overlap) : caller_(caller), own_(overlap && acquire(lane_))
@@ -123,7 +124,32 @@ bool layer_sizes(const vgc_layer_host &L, LayerSizes &z)
     return true;
 }
 
-bool overlapping(const float *a, size_t n_a, const float *b, size_t n_b) { return a < b + n_b && b < a + n_a; }
+struct Span {
+    uintptr_t begin, end;
+    Span(const void *p, size_t bytes) : begin(reinterpret_cast<uintptr_t>(p)), end(begin + bytes) {}
+    bool meets(const Span &o) const { return begin < o.end && o.begin < end; }
+};
+
+// Copies may run beside the kernels of the layers before: no two of the copies' destinations overlap, and none lies over what
+// those kernels write (the squared sums, the workspace).
+bool copies_may_overlap(const vgc_layer_host *layers, int n_layers, const float *g_dev, size_t n, const float *s_dev, const void *ws,
+                        size_t ws_bytes)
+{
+    // 0: sums, 1: workspace, 2: g, then x and delta of every layer
+    auto span = [&](int i) {
+        if (i == 0) return Span(s_dev, n * sizeof(float));
+        if (i == 1) return Span(ws, ws_bytes);
+        if (i == 2) return Span(g_dev, n * sizeof(float));
+        const vgc_layer_host &L = layers[(i - 3) / 2];
+        LayerSizes z;
+        layer_sizes(L, z);
+        return i % 2 ? Span(L.x_dev, z.n_x * sizeof(float)) : Span(L.delta_dev, z.n_d * sizeof(float));
+    };
+    for (int i = 2; i < 3 + 2 * n_layers; ++i)
+        for (int j = 0; j < i; ++j)
+            if (span(i).meets(span(j))) return false;
+    return true;
+}
 
 }  // namespace
 
@@ -139,24 +165,14 @@ extern "C" vgc_status vgc_step_host(const vgc_layer_host *layers, int n_layers, 
     if (K != n_layers) return VGC_ERR_INVALID_ARG;        // one weight tensor (group) per layer, in order
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     size_t offset = 0;
-    bool shared = false;                                  // some layers' staging buffers (or g's) overlap
     for (int l = 0; l < n_layers; ++l) {
         LayerSizes z;
         if (!layer_sizes(layers[l], z) || offset + z.n_w > n) return VGC_ERR_INVALID_ARG;
         offset += z.n_w;
-        const float *const mine[2] = {layers[l].x_dev, layers[l].delta_dev};
-        const size_t len[2] = {z.n_x, z.n_d};
-        for (int i = 0; i < 2 && !shared; ++i) {
-            shared = overlapping(mine[i], len[i], g_dev, n);
-            for (int m = 0; m < l && !shared; ++m) {
-                LayerSizes y;
-                layer_sizes(layers[m], y);
-                shared = overlapping(mine[i], len[i], layers[m].x_dev, y.n_x) || overlapping(mine[i], len[i], layers[m].delta_dev, y.n_d);
-            }
-        }
     }
     if (offset != n) return VGC_ERR_INVALID_ARG;
-    Copies copies(st, !shared);
+    const bool beside = copies_may_overlap(layers, n_layers, g_dev, n, s_dev, ws_sqgrad, ws_sqgrad_bytes);
+    Copies copies(st, beside);
     offset = 0;
     for (int l = 0; l < n_layers; ++l) {
         const vgc_layer_host &L = layers[l];
@@ -166,7 +182,7 @@ extern "C" vgc_status vgc_step_host(const vgc_layer_host *layers, int n_layers, 
             !copies.arrived())
             return VGC_ERR_CUDA;
         // g under the last layer's kernels
-        if (!shared && l == n_layers - 1 && !copies.in(g_dev, g_host, n * sizeof(float))) return VGC_ERR_CUDA;
+        if (beside && l == n_layers - 1 && !copies.in(g_dev, g_host, n * sizeof(float))) return VGC_ERR_CUDA;
         vgc_status rc = L.is_conv
                             ? vgc_sqgrad_conv(L.x_dev, L.delta_dev, L.B, L.C, L.H, L.W, L.Cout, L.Kh, L.Kw, L.stride_h,
                                               L.stride_w, L.pad_h, L.pad_w, scale, 0, s_dev + offset, ws_sqgrad,
@@ -176,7 +192,7 @@ extern "C" vgc_status vgc_step_host(const vgc_layer_host *layers, int n_layers, 
         if (rc != VGC_OK) return rc;
         offset += z.n_w;
     }
-    if ((shared || n_layers == 0) && !copies.in(g_dev, g_host, n * sizeof(float))) return VGC_ERR_CUDA;
+    if ((!beside || n_layers == 0) && !copies.in(g_dev, g_host, n * sizeof(float))) return VGC_ERR_CUDA;
     if (!copies.arrived()) return VGC_ERR_CUDA;
     vgc_status rc = vgc_compress(g_dev, s_dev, r, v, n, group_offsets, K, alpha, zeta, out, ws_compress, ws_compress_bytes,
                                  stream);

@@ -1,6 +1,6 @@
 """vgc_step_host: staging buffers of their own (copies run beside the kernels), shared between the layers and with g (copies
 and kernels take turns), a message whose counters do not lie side by side, and calls from several threads on streams of
-their own.  All give what the device calls give, bit for bit."""
+their own; staging in memory that the kernels of earlier layers write.  All give what the device calls give, bit for bit."""
 import ctypes
 import threading
 
@@ -16,7 +16,7 @@ B, SIZES = 64, [(1024, 512), (512, 256), (256, 12)]
 
 
 class Step:
-    def __init__(self, seed, staging):
+    def __init__(self, seed, staging, B=B):
         specs = [workloads.LayerSpec(f"fc{i}", "fc", a, b) for i, (a, b) in enumerate(SIZES)]
         offs = workloads.group_offsets(specs)
         self.n, self.K = int(offs[-1]), len(specs)
@@ -32,11 +32,17 @@ class Step:
         out = vgc.MessageBuffers(self.n, self.K, self.n)
         vgc.vgc_compress(g, self.s, self.r, self.v, self.offs, 2.0, 0.999, out, self.wc)
         self.want = out.read()
+        self.B = B
         self.g_dev = torch.empty(self.n, device="cuda")
+        in_ws = self.ws[1 << 20:self.ws.numel() // 4 * 4].view(torch.float32)     # past the status word and what small layers need
+        if staging == "g in the workspace":
+            self.g_dev = in_ws[:self.n]
         room = self.g_dev if staging == "with g" else torch.empty(2 * B * 1024, device="cuda")
         self.layers = []
         for x, d in ins:
-            if staging == "own":
+            if staging == "last layer in the workspace" and d.shape[1] == SIZES[-1][1]:
+                xd, dd = in_ws[:x.numel()].view_as(x), in_ws[x.numel():x.numel() + d.numel()].view_as(d)
+            elif staging not in ("shared", "with g"):
                 xd, dd = torch.empty_like(x), torch.empty_like(d)
             else:
                 xd, dd = room[:x.numel()].view_as(x), room[x.numel():x.numel() + d.numel()].view_as(d)
@@ -48,7 +54,7 @@ class Step:
     def check(self, out, stream=None):
         s, r, v = torch.full_like(self.s, float("nan")), torch.zeros_like(self.r), torch.zeros_like(self.v)
         torch.cuda.synchronize()
-        got = vgc.vgc_step_host(self.layers, self.g_host, self.g_dev, s, r, v, self.offs, 2.0, 0.999, 1.0 / B ** 2, out, self.words,
+        got = vgc.vgc_step_host(self.layers, self.g_host, self.g_dev, s, r, v, self.offs, 2.0, 0.999, 1.0 / self.B ** 2, out, self.words,
                                 self.counters, self.ws, self.wc, stream=stream)
         w = self.want
         assert got == (w["nnz"], w["n_criterion"], w["n_dropped"], 0)
@@ -61,6 +67,18 @@ def test_staging(staging):
     step = Step(3, staging)
     out = vgc.MessageBuffers(step.n, step.K, step.n)
     for _ in range(3):
+        out.counters.zero_()
+        step.check(out)
+
+
+@pytest.mark.parametrize("staging", ["g in the workspace", "last layer in the workspace"])
+def test_staging_over_memory_that_earlier_kernels_write(staging):
+    """The first layers (1100 examples) leave partial tiles all over the workspace; what is copied there for a later use
+    must not arrive before they are done."""
+    step = Step(5, staging, B=1100)
+    assert step.ws.numel() > (1 << 20) + 4 * step.n
+    out = vgc.MessageBuffers(step.n, step.K, step.n)
+    for _ in range(5):
         out.counters.zero_()
         step.check(out)
 
