@@ -12,7 +12,8 @@
 //   scatter   few words, u written: a block owns a range of u, writes zeros piece by piece and adds the piece's words while
 //             it is still in L2 (scatter_range);
 //   dense     a block owns a range of u and walks it in tiles held in shared memory; u is read and written once, coalesced:
-//             exact_range where every word is a multiple of one power of two, ordered_range otherwise.
+//             exact_range where every word of a tensor is a multiple of one power of two, ordered_range where no tensor's
+//             are, many_range where some are and some are not, or where the tensors are many.
 // kOverwrite: the range starts from zero instead of the old contents of u (u = scale * sum of the messages).
 // kHybrid: messages of the hybrid algorithm (Algorithm 2) -- every word stands for +-tau, no exponents.
 #include <type_traits>
@@ -43,7 +44,7 @@ constexpr int kTileThreads = 256;
 constexpr int kBlocksPerSm = 3;
 constexpr int kTileWarps = kTileThreads / 32;
 constexpr int kTileMax = 15360;                  // elements per tile: three tiles and the tables fit in shared memory
-constexpr int kTensors = kTileWarps;             // weight tensors of a range that takes the exact form
+constexpr int kTensors = kTileWarps;             // weight tensors of a range that exact_range takes
 constexpr int kTilePre = 8;                      // ordered form: words per thread in one batch
 
 __device__ __forceinline__ void cp_async_16(void *smem, const void *gmem)
@@ -56,6 +57,11 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
+__device__ __forceinline__ float value_at(uint32_t word, int32_t tensor_exp, float scale)
+{
+    const int32_t e = tensor_exp - (int32_t)(word & 7u);
+    return __fmul_rn(scale, __uint_as_float(((uint32_t)(e + 127) << 23) | ((word & 8u) << 28)));
+}
 template <bool kHybrid>
 __device__ __forceinline__ float value_of(uint32_t word, const int32_t *gexp, const uint32_t *offs, int K, float scale, float tau,
                                           int &k)
@@ -63,8 +69,7 @@ __device__ __forceinline__ float value_of(uint32_t word, const int32_t *gexp, co
     if (kHybrid) return __fmul_rn(scale, (word & 8u) ? -tau : tau);
     const uint32_t idx = word >> 4;
     if (idx < offs[k] || idx >= offs[k + 1]) k = group_of(offs, K, idx);
-    const int32_t e = gexp[k] - (int32_t)(word & 7u);
-    return __fmul_rn(scale, __uint_as_float(((uint32_t)(e + 127) << 23) | ((word & 8u) << 28)));
+    return value_at(word, gexp[k], scale);
 }
 
 // ---- flat -----------------------------------------------------------------------------------------------------------
@@ -192,8 +197,9 @@ struct TileShared {
     const int32_t *gexp[kMaxViews];
     int32_t base[kTensors];                                      // exact form: 2^base is the unit of the range's tensors
     float lut[2][kMaxViews * 16];                                // values of the words of two tensors, 16 per message
-    uint32_t unfit;                                              // something rules the exact form out
+    uint32_t unfit;                                              // what the range's tensors are like: kOrdered, ...
 };
+enum : uint32_t { kOrdered = 1, kCrowded = 2, kSomeUnfit = 4, kSomeFit = 8 };
 
 // Where every message's run enters the range: sm.cur[w] becomes the first position of message w whose index is >= bound
 // (its count if none).  Warp j looks after the messages j, j + 8, ...; lane i holds the state of the i-th of them.
@@ -322,10 +328,14 @@ __device__ __forceinline__ bool scatter_range(TileShared &sm, int W, const uint3
 // batch's loads in flight (indices inside a message are distinct, so plain read-modify-writes, a block barrier between
 // messages): an element receives its additions in message order, the fp32 sequence of a sequential sum.
 // Returns whether a word was out of place.
+// This and many_range are functions of their own, given shared-memory addresses: inlined, their registers make the other forms
+// spill (messages that are not aligned, K = 1, W = 64, added to 25.5 M elements: 294 -> 324 us).
 template <bool kHybrid, bool kOverwrite>
-__device__ __forceinline__ bool ordered_range(TileShared &sm, float *tile, int W, const uint32_t *offs, int K, float scale, float tau,
-                                              float *u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
+__device__ __noinline__ bool ordered_range(uint32_t sm_addr, uint32_t tile_addr, int W, const uint32_t *offs, int K, float scale,
+                                           float tau, float *u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
 {
+    TileShared &sm = *static_cast<TileShared *>(__cvta_shared_to_generic(sm_addr));
+    float *const tile = static_cast<float *>(__cvta_shared_to_generic(tile_addr));
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t *const cur = sm.cur, *const end = sm.end;
     bool bad = false;
@@ -333,13 +343,19 @@ __device__ __forceinline__ bool ordered_range(TileShared &sm, float *tile, int W
     for (uint32_t t0 = lo; t0 < hi; t0 += t_len) {
         t_len = min(hi - t0, tile_elems);
         int tile_group = kHybrid ? 0 : -1;                          // weight tensor of the tile, -1 if it spans several
+        int g0 = -1;                                                // its first tensor, where the exponents of all fit into exps
+        int32_t *const exps = reinterpret_cast<int32_t *>(sm.lut);  // [tensor of the tile][message]
         if (!kHybrid) {
-            // a tile ends with its weight tensor when that keeps the next one on a 16-byte boundary and leaves no sliver:
-            // inside one tensor a word's value is one look-up
             const int g = group_of(offs, K, t0);
             const uint32_t rem = offs[g + 1] - t0;
-            if (rem < t_len && (rem & 3u) == 0u && rem >= 2048u) t_len = rem;
             if (rem >= t_len) tile_group = g;
+            else {
+                const int all = (group_of(offs, K, t0 + t_len - 1) - g + 1) * W;
+                if (all <= (int)(sizeof(sm.lut) / sizeof(int32_t))) {
+                    g0 = g;
+                    for (int i = tid; i < all; i += kTileThreads) exps[i] = sm.gexp[i % W][g + i / W];
+                }
+            }
         }
         const uint32_t t_hi = t0 + t_len;
         const uint32_t n_vec = t_len / 4;                           // t0 is a multiple of 4 elements
@@ -406,7 +422,12 @@ __device__ __forceinline__ bool ordered_range(TileShared &sm, float *tile, int W
                 if (first + j * kTileThreads >= e) continue;
                 // a word of a sorted message lies inside the tile; one that does not (the message is not sorted) is skipped
                 if (at >= t_len) { bad = true; continue; }
-                const float v = tile_group >= 0 ? lut[word & 15u] : value_of<kHybrid>(word, gexp, offs, K, scale, tau, k);
+                float v;
+                if (tile_group >= 0) v = lut[word & 15u];
+                else if (g0 >= 0) {
+                    if ((word >> 4) < offs[k] || (word >> 4) >= offs[k + 1]) k = group_of(offs, K, word >> 4);
+                    v = value_at(word, exps[(k - g0) * W + w], scale);
+                } else v = value_of<kHybrid>(word, gexp, offs, K, scale, tau, k);
                 tile[at] = __fadd_rn(tile[at], v);
             }
             if (w2 != w) __syncthreads();                            // the next message may hit the same elements
@@ -429,6 +450,112 @@ __device__ __forceinline__ bool ordered_range(TileShared &sm, float *tile, int W
     return bad;
 }
 
+// ---- dense, the exact form's words --------------------------------------------------------------------------------------
+// Warps stream the messages' words from their cursors.  Message m is shared by the warps m, m + W, ... (W < 8) in turns of
+// 256 words -- or a warp takes the messages warp, warp + 8, ... -- and a warp stops at its first turn that reaches past the
+// tile (or the message's end); the words it found inside are added to the message's count (sm.taken), which moves the cursor
+// once all warps are done.
+// A word minus t0 << 4 keeps its low four bits and turns its index into the offset inside the tile; one unsigned comparison
+// then says "inside the tile" (a word behind the tile wraps around to a huge number, and so does the filler 0xFFFFFFFF,
+// because the range ends before 2^28).  add(word, message, count) makes that comparison, adds the word and counts it.
+template <class Add>
+__device__ __forceinline__ void stream_tile(TileShared &sm, int W, uint32_t t0, uint32_t t_len, bool &bad, Add add)
+{
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t t0s = t0 << 4, t_len16 = t_len << 4;
+    const int sharers = W < kTileWarps ? kTileWarps / W : 1;       // warps per message
+    for (int m = (int)warp % W; m < W; m += kTileWarps) {
+        if (W < kTileWarps && (int)warp >= sharers * W) break;     // warps left over when W does not divide the warps
+        const uint32_t turn0 = W < kTileWarps ? warp / (uint32_t)W : 0u;
+        const uint32_t *words = sm.words[m];
+        const uint32_t c = sm.cur[m], cnt = sm.count[m];
+        const uint32_t a = c & ~3u;                                // 16-byte loads: start at the boundary before the cursor
+        uint32_t inside = 0, n_in = 0;                             // words up to the tile's end; words added
+        // a turn is 256 consecutive words, two 16-byte loads per lane; the next turn's loads are issued before
+        // this turn's words are looked at, so the latency of one turn hides under the work of the other
+        constexpr int kVecs = 2, kAhead = 4;
+        constexpr uint32_t kTurnWords = 128u * kVecs;
+        uint4 nxt[kVecs];
+        auto fetch = [&](uint32_t turn, uint4 (&dst)[kVecs]) {
+            const uint32_t p0 = a + turn * kTurnWords + 4u * lane;
+            if (a + (turn + 1u) * kTurnWords <= cnt) {             // warp-uniform: the whole turn lies inside the message
+#pragma unroll
+                for (int v = 0; v < kVecs; ++v) dst[v] = *reinterpret_cast<const uint4 *>(words + p0 + 128u * v);
+            } else {
+#pragma unroll
+                for (int v = 0; v < kVecs; ++v) {
+                    const uint32_t p = p0 + 128u * v;
+                    dst[v].x = p < cnt ? words[p] : 0xFFFFFFFFu;
+                    dst[v].y = p + 1u < cnt ? words[p + 1] : 0xFFFFFFFFu;
+                    dst[v].z = p + 2u < cnt ? words[p + 2] : 0xFFFFFFFFu;
+                    dst[v].w = p + 3u < cnt ? words[p + 3] : 0xFFFFFFFFu;
+                }
+            }
+            // ... and the turns after it are asked into L2 (no registers held): a turn's loads then find their lines there
+            const uint32_t ahead = a + (turn + (uint32_t)(kAhead * sharers)) * kTurnWords + 32u * lane;
+            if (lane < kTurnWords / 32u && ahead < cnt) asm volatile("prefetch.global.L2 [%0];" ::"l"(words + ahead));
+        };
+        fetch(turn0, nxt);
+        for (uint32_t turn = turn0;; turn += (uint32_t)sharers) {
+            uint4 wd[kVecs];
+#pragma unroll
+            for (int v = 0; v < kVecs; ++v) wd[v] = nxt[v];
+            fetch(turn + (uint32_t)sharers, nxt);
+#pragma unroll
+            for (int v = 0; v < kVecs; ++v) {
+                add(wd[v].x, (uint32_t)m, n_in); add(wd[v].y, (uint32_t)m, n_in);
+                add(wd[v].z, (uint32_t)m, n_in); add(wd[v].w, (uint32_t)m, n_in);
+            }
+            // sorted words: the turn lies inside the tile when its last word does (and the message goes on)
+            const uint32_t turn_end = a + (turn + 1u) * kTurnWords;
+            const bool last_in = wd[kVecs - 1].w - t0s < t_len16;
+            if (turn_end <= cnt && (__ballot_sync(0xffffffffu, last_in) >> 31)) {
+                inside += kTurnWords - (turn == 0u ? c - a : 0u);
+                continue;
+            }
+            // the last turn of this warp: count the words from the cursor on that lie before the tile's end
+            uint32_t mine = 0;
+            const uint32_t p0 = a + turn * kTurnWords + 4u * lane, t_hi = t0 + t_len;
+#pragma unroll
+            for (int v = 0; v < kVecs; ++v) {
+                const uint32_t p = p0 + 128u * v;
+                const uint32_t x[4] = {wd[v].x, wd[v].y, wd[v].z, wd[v].w};
+#pragma unroll
+                for (uint32_t i = 0; i < 4; ++i) mine += (p + i >= c && p + i < cnt && (x[i] >> 4) < t_hi) ? 1u : 0u;
+            }
+            inside += __reduce_add_sync(0xffffffffu, mine);
+            break;
+        }
+        // a word before the tile's end that was not added lies behind the tile: the message is not sorted
+        if (__reduce_add_sync(0xffffffffu, n_in) != inside) bad = true;
+        if (lane == 0 && inside) atomicAdd(&sm.taken[m], inside);
+    }
+}
+
+constexpr int32_t kUnfit = INT32_MIN;
+
+// Unit of a tensor whose exponents (of this lane's two messages: ex[0], ex[1]) lie close enough together; else kUnfit.
+// With a scale that is a power of two 2^s_exp (pow2) the result is the sequential sum's, bit for bit.
+__device__ __forceinline__ int32_t unit_of_tensor(const int32_t (&ex)[2], int W, bool pow2, int s_exp)
+{
+    const bool some0 = ex[0] != VGC_EXP_NONE, some1 = ex[1] != VGC_EXP_NONE;
+    const int e_max = __reduce_max_sync(0xffffffffu, max(some0 ? ex[0] : INT32_MIN, some1 ? ex[1] : INT32_MIN));
+    const int e_min = __reduce_min_sync(0xffffffffu, min(some0 ? ex[0] : INT32_MAX, some1 ? ex[1] : INT32_MAX));
+    if (e_max < e_min) return 0;                                 // (nothing was sent from this tensor)
+    const int b = e_min - 7;                                     // the smallest value a word can stand for
+    // 2^base and every sum of multiples are normal numbers; with a power-of-two scale so are their products
+    const bool fits = e_max - b + (32 - __clz((W - 1) | 1)) <= 22 && b >= -126 && b + 22 <= 127 &&
+                      (!pow2 || (b + s_exp >= -126 && b + 22 + s_exp <= 127));
+    return fits ? b : kUnfit;
+}
+// A sum of multiples (at most 2^22 either way, so 1.5 * 2^23 plus it is a float whose bits are 0x4B400000 plus it) times
+// the unit (exact).
+__device__ __forceinline__ float times_unit(int mult, float unit)
+{
+    return __fmul_rn(__fsub_rn(__int_as_float(0x4B400000 + mult), 12582912.f), unit);
+}
+__device__ __forceinline__ float power_of_two(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
+
 // ---- dense, exact form ----------------------------------------------------------------------------------------------------
 // When the exponents of all messages for a tensor lie close enough together, every word is an integer multiple of one power
 // of two, 2^base, and every partial sum of up to W of them stays within 2^22 multiples: all of them are exact fp32 numbers,
@@ -437,15 +564,15 @@ __device__ __forceinline__ bool ordered_range(TileShared &sm, float *tile, int W
 // per message, and vgc_decode_accumulate adds the scaled sum to u in one addition).  A tile is then accumulated as int32
 // multiples of 2^base with shared-memory integer atomics, in any order: no barrier between messages, no search for the
 // runs' ends -- the warps stream every message's words from its cursor until the indices leave the tile -- and one
-// conversion at the end.  Same bits, much less waiting.  A block takes this form when it applies to all tensors of its range.
+// conversion at the end.  Same bits, much less waiting.  exact_range is for ranges of few tensors, all of which fit: its tiles
+// hold two at most, and a word's multiple is one look-up.
 // Returns whether a word was out of place.
 template <bool kHybrid, bool kOverwrite>
 __device__ __forceinline__ bool exact_range(TileShared &sm, float *tile, int W, const uint32_t *offs, int g_first, float scale,
                                             float tau, float *u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
 {
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t tid = threadIdx.x;
     const uint32_t tile_addr = (uint32_t)__cvta_generic_to_shared(tile);
-    const int sharers = W < kTileWarps ? kTileWarps / W : 1;       // warps per message
     bool bad = false;
     int g = g_first, made = -1;        // tensor of the tile's first element; the last tensor whose table was made
     int slot = 1;                      // the table of the tile's first tensor
@@ -490,127 +617,57 @@ __device__ __forceinline__ bool exact_range(TileShared &sm, float *tile, int W, 
         if (tid < (uint32_t)W) sm.taken[tid] = 0;
         __syncthreads();
 
-        // ---- warps stream the messages' words from their cursors.  Message m is shared by the warps m, m + W, ...
-        // (W < 8) in turns of 256 words -- or a warp takes the messages warp, warp + 8, ... -- and a warp stops at its
-        // first turn that reaches past the tile (or the message's end); the words it found inside are added to the
-        // message's count, which moves the cursor once all warps are done.
-        // A word minus t0 << 4 keeps its low four bits and turns its index into the offset inside the tile; one unsigned
-        // comparison then says "inside the tile" (a word behind the tile wraps around to a huge number, and so does the
-        // filler 0xFFFFFFFF, because the range ends before 2^28).
         const uint32_t t0s = t0 << 4, t_len16 = t_len << 4, split16 = split << 4;
         auto stream = [&](auto two) {
             constexpr bool kTwo = decltype(two)::value;             // the tile has elements of two tensors
             const uint32_t lut_addr = (uint32_t)__cvta_generic_to_shared(sm.lut[slot]);
             const uint32_t lut_other = (uint32_t)__cvta_generic_to_shared(sm.lut[slot ^ 1]) - lut_addr;
-            for (int m = (int)warp % W; m < W; m += kTileWarps) {
-                if (W < kTileWarps && (int)warp >= sharers * W) break;   // warps left over when W does not divide the warps
-                const uint32_t turn0 = W < kTileWarps ? warp / (uint32_t)W : 0u;
-                const uint32_t *words = sm.words[m];
-                const uint32_t c = sm.cur[m], cnt = sm.count[m];
-                const uint32_t a = c & ~3u;                          // 16-byte loads: start at the boundary before the cursor
-                const uint32_t lut_m = lut_addr + 64u * (uint32_t)m;
-                uint32_t inside = 0, n_in = 0;                       // words up to the tile's end; words added
-                // a turn is 256 consecutive words, two 16-byte loads per lane; the next turn's loads are issued before
-                // this turn's words are looked at, so the latency of one turn hides under the work of the other
-                constexpr int kVecs = 2, kAhead = 4;
-                constexpr uint32_t kTurnWords = 128u * kVecs;
-                uint4 nxt[kVecs];
-                auto fetch = [&](uint32_t turn, uint4 (&dst)[kVecs]) {
-                    const uint32_t p0 = a + turn * kTurnWords + 4u * lane;
-                    if (a + (turn + 1u) * kTurnWords <= cnt) {          // warp-uniform: the whole turn lies inside the message
-#pragma unroll
-                        for (int v = 0; v < kVecs; ++v) dst[v] = *reinterpret_cast<const uint4 *>(words + p0 + 128u * v);
-                    } else {
-#pragma unroll
-                        for (int v = 0; v < kVecs; ++v) {
-                            const uint32_t p = p0 + 128u * v;
-                            dst[v].x = p < cnt ? words[p] : 0xFFFFFFFFu;
-                            dst[v].y = p + 1u < cnt ? words[p + 1] : 0xFFFFFFFFu;
-                            dst[v].z = p + 2u < cnt ? words[p + 2] : 0xFFFFFFFFu;
-                            dst[v].w = p + 3u < cnt ? words[p + 3] : 0xFFFFFFFFu;
-                        }
-                    }
-                    // ... and the turns after it are asked into L2 (no registers held): a turn's loads then find their lines there
-                    const uint32_t ahead = a + (turn + (uint32_t)(kAhead * sharers)) * kTurnWords + 32u * lane;
-                    if (lane < kTurnWords / 32u && ahead < cnt) asm volatile("prefetch.global.L2 [%0];" ::"l"(words + ahead));
-                };
-                // one word: inside the tile -> look its multiple up and add it; all of it predicated, no branch
-                auto add = [&](uint32_t word) {
-                    if (kTwo)
-                        asm volatile("{\n\t"
-                                     ".reg .pred p, second;\n\t"
-                                     ".reg .s32 iv;\n\t"
-                                     ".reg .u32 o, at, l;\n\t"
-                                     "sub.u32 o, %1, %2;\n\t"
-                                     "setp.lt.u32 p, o, %3;\n\t"
-                                     "setp.ge.u32 second, o, %6;\n\t"
-                                     "and.b32 l, %1, 15;\n\t"
-                                     "shl.b32 l, l, 2;\n\t"
-                                     "add.u32 l, l, %4;\n\t"
-                                     "@second add.u32 l, l, %7;\n\t"
-                                     "shr.u32 at, o, 2;\n\t"
-                                     "and.b32 at, at, 0xFFFFFFFC;\n\t"
-                                     "add.u32 at, at, %5;\n\t"
-                                     "@p ld.shared.s32 iv, [l];\n\t"
-                                     "@p red.shared.add.s32 [at], iv;\n\t"
-                                     "@p add.u32 %0, %0, 1;\n\t"
-                                     "}"
-                                     : "+r"(n_in)
-                                     : "r"(word), "r"(t0s), "r"(t_len16), "r"(lut_m), "r"(tile_addr), "r"(split16), "r"(lut_other)
-                                     : "memory");
-                    else
-                        asm volatile("{\n\t"
-                                     ".reg .pred p;\n\t"
-                                     ".reg .s32 iv;\n\t"
-                                     ".reg .u32 o, at, l;\n\t"
-                                     "sub.u32 o, %1, %2;\n\t"
-                                     "setp.lt.u32 p, o, %3;\n\t"
-                                     "and.b32 l, %1, 15;\n\t"
-                                     "shl.b32 l, l, 2;\n\t"
-                                     "add.u32 l, l, %4;\n\t"
-                                     "shr.u32 at, o, 2;\n\t"
-                                     "and.b32 at, at, 0xFFFFFFFC;\n\t"
-                                     "add.u32 at, at, %5;\n\t"
-                                     "@p ld.shared.s32 iv, [l];\n\t"
-                                     "@p red.shared.add.s32 [at], iv;\n\t"
-                                     "@p add.u32 %0, %0, 1;\n\t"
-                                     "}"
-                                     : "+r"(n_in)
-                                     : "r"(word), "r"(t0s), "r"(t_len16), "r"(lut_m), "r"(tile_addr)
-                                     : "memory");
-                };
-                fetch(turn0, nxt);
-                for (uint32_t turn = turn0;; turn += (uint32_t)sharers) {
-                    uint4 wd[kVecs];
-#pragma unroll
-                    for (int v = 0; v < kVecs; ++v) wd[v] = nxt[v];
-                    fetch(turn + (uint32_t)sharers, nxt);
-#pragma unroll
-                    for (int v = 0; v < kVecs; ++v) { add(wd[v].x); add(wd[v].y); add(wd[v].z); add(wd[v].w); }
-                    // sorted words: the turn lies inside the tile when its last word does (and the message goes on)
-                    const uint32_t turn_end = a + (turn + 1u) * kTurnWords;
-                    const bool last_in = wd[kVecs - 1].w - t0s < t_len16;
-                    if (turn_end <= cnt && (__ballot_sync(0xffffffffu, last_in) >> 31)) {
-                        inside += kTurnWords - (turn == 0u ? c - a : 0u);
-                        continue;
-                    }
-                    // the last turn of this warp: count the words from the cursor on that lie before the tile's end
-                    uint32_t mine = 0;
-                    const uint32_t p0 = a + turn * kTurnWords + 4u * lane, t_hi = t0 + t_len;
-#pragma unroll
-                    for (int v = 0; v < kVecs; ++v) {
-                        const uint32_t p = p0 + 128u * v;
-                        const uint32_t x[4] = {wd[v].x, wd[v].y, wd[v].z, wd[v].w};
-#pragma unroll
-                        for (uint32_t i = 0; i < 4; ++i) mine += (p + i >= c && p + i < cnt && (x[i] >> 4) < t_hi) ? 1u : 0u;
-                    }
-                    inside += __reduce_add_sync(0xffffffffu, mine);
-                    break;
-                }
-                // a word before the tile's end that was not added lies behind the tile: the message is not sorted
-                if (__reduce_add_sync(0xffffffffu, n_in) != inside) bad = true;
-                if (lane == 0 && inside) atomicAdd(&sm.taken[m], inside);
-            }
+            // one word: inside the tile -> look its multiple up and add it; all of it predicated, no branch
+            stream_tile(sm, W, t0, t_len, bad, [&](uint32_t word, uint32_t m, uint32_t &n_in) {
+                const uint32_t lut_m = lut_addr + 64u * m;
+                if (kTwo)
+                    asm volatile("{\n\t"
+                                 ".reg .pred p, second;\n\t"
+                                 ".reg .s32 iv;\n\t"
+                                 ".reg .u32 o, at, l;\n\t"
+                                 "sub.u32 o, %1, %2;\n\t"
+                                 "setp.lt.u32 p, o, %3;\n\t"
+                                 "setp.ge.u32 second, o, %6;\n\t"
+                                 "and.b32 l, %1, 15;\n\t"
+                                 "shl.b32 l, l, 2;\n\t"
+                                 "add.u32 l, l, %4;\n\t"
+                                 "@second add.u32 l, l, %7;\n\t"
+                                 "shr.u32 at, o, 2;\n\t"
+                                 "and.b32 at, at, 0xFFFFFFFC;\n\t"
+                                 "add.u32 at, at, %5;\n\t"
+                                 "@p ld.shared.s32 iv, [l];\n\t"
+                                 "@p red.shared.add.s32 [at], iv;\n\t"
+                                 "@p add.u32 %0, %0, 1;\n\t"
+                                 "}"
+                                 : "+r"(n_in)
+                                 : "r"(word), "r"(t0s), "r"(t_len16), "r"(lut_m), "r"(tile_addr), "r"(split16), "r"(lut_other)
+                                 : "memory");
+                else
+                    asm volatile("{\n\t"
+                                 ".reg .pred p;\n\t"
+                                 ".reg .s32 iv;\n\t"
+                                 ".reg .u32 o, at, l;\n\t"
+                                 "sub.u32 o, %1, %2;\n\t"
+                                 "setp.lt.u32 p, o, %3;\n\t"
+                                 "and.b32 l, %1, 15;\n\t"
+                                 "shl.b32 l, l, 2;\n\t"
+                                 "add.u32 l, l, %4;\n\t"
+                                 "shr.u32 at, o, 2;\n\t"
+                                 "and.b32 at, at, 0xFFFFFFFC;\n\t"
+                                 "add.u32 at, at, %5;\n\t"
+                                 "@p ld.shared.s32 iv, [l];\n\t"
+                                 "@p red.shared.add.s32 [at], iv;\n\t"
+                                 "@p add.u32 %0, %0, 1;\n\t"
+                                 "}"
+                                 : "+r"(n_in)
+                                 : "r"(word), "r"(t0s), "r"(t_len16), "r"(lut_m), "r"(tile_addr)
+                                 : "memory");
+            });
         };
         if (split < t_len) stream(std::true_type());
         else stream(std::false_type());
@@ -621,11 +678,11 @@ __device__ __forceinline__ bool exact_range(TileShared &sm, float *tile, int W, 
         // whose bits are 0x4B400000 plus it), times 2^base (exact), times the scale: one rounding, none when the scale is a
         // power of two.  vgc_decode_accumulate adds the result to u; an element no word points at keeps its bits.
         auto unit_of = [&](int k) {
-            return kHybrid ? __fmul_rn(scale, tau) : __uint_as_float((uint32_t)(sm.base[k - g_first] + 127) << 23);
+            return kHybrid ? __fmul_rn(scale, tau) : power_of_two(sm.base[k - g_first]);
         };
         const float unit_a = unit_of(g), unit_b = unit_of(next);
         auto value = [&](int mult, float unit) {
-            const float m = __fmul_rn(__fsub_rn(__int_as_float(0x4B400000 + mult), 12582912.f), unit);
+            const float m = times_unit(mult, unit);
             return kHybrid ? m : __fmul_rn(m, scale);           // hybrid: a word is worth scale * tau, rounded once
         };
         // vector q of the tile: the units of its elements (they differ inside the one vector that holds the border)
@@ -678,6 +735,188 @@ __device__ __forceinline__ bool exact_range(TileShared &sm, float *tile, int W, 
         if (next != g) { g = next; slot ^= 1; }
     }
     return bad;
+}
+
+// ---- dense, many tensors ----------------------------------------------------------------------------------------------------
+// Tiles of any number of tensors, each in its own form: words of a tensor whose exponents fit are added as multiples of its
+// unit, in any order, in one pass over all messages; then, where a tensor of the tile does not fit, the words of such
+// tensors are added message after message, a block barrier between messages.  Both share the tile: an element belongs to
+// one tensor.  A word's tensor is searched among the tile's (kept from word to word: neighbours mostly share it), its
+// multiple made from the exponent's distance to the tensor's unit.
+// Measured (B200, ResNet-50 with its normalisation vectors: 161 tensors, 25.6 M elements, written): 8 messages of density
+// 0.05 47 us, 64 of 0.01 99 us; with the range in the ordered form 103 and 472, with tiles in it 81 and 315.
+// What a tile needs to know about its tensors; in the place of the exact form's tables.
+constexpr int kMany = 511, kAbove = 4096;
+struct ManyTensors {
+    uint8_t above[kAbove];                       // [tensor][message]: exponent above the unit's; kNothing: nothing was sent
+    uint32_t begin[kMany + 1];                   // first element, counted from the tile's; [tensors]: behind the last one
+    int32_t base[kMany + 1];                     // 2^base is the unit; kUnfit: the tensor is added in message order
+};
+static_assert(sizeof(ManyTensors) <= sizeof(TileShared::lut), "in the place of the tables");
+constexpr uint8_t kNothing = 255;
+
+// Walks [lo, hi) from lo on.  Returns where it stopped -- hi, but where more tensors than a tile has room for begin within
+// four elements (the ordered form does the rest) -- and whether a word was out of place (kBad).
+constexpr uint32_t kBad = 1u << 31;
+template <bool kOverwrite>
+__device__ __noinline__ uint32_t many_range(uint32_t sm_addr, uint32_t tile_addr, int W, const uint32_t *offs, int K, float scale, bool pow2,
+                                            int s_exp, float *u, uint32_t lo, uint32_t hi, uint32_t tile_elems)
+{
+    TileShared &sm = *static_cast<TileShared *>(__cvta_shared_to_generic(sm_addr));
+    float *const tile = static_cast<float *>(__cvta_shared_to_generic(tile_addr));
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    ManyTensors &mt = *reinterpret_cast<ManyTensors *>(sm.lut);
+    const int room = min(kMany, kAbove / W);
+    int *const sums = reinterpret_cast<int *>(tile);
+    bool bad = false;
+    int g = group_of(offs, K, lo);                                  // tensor of the tile's first element
+    uint32_t t0 = lo, t_len = 0;
+    for (; t0 < hi; t0 += t_len) {
+        t_len = min(hi - t0, tile_elems);
+        for (int j = tid; j <= room; j += kTileThreads) mt.begin[j] = j == 0 ? 0u : g + j <= K ? offs[g + j] - t0 : 0xFFFFFFFFu;
+        if (tid == 0) sm.unfit = 0;
+        if (tid < (uint32_t)W) sm.taken[tid] = 0;
+        __syncthreads();
+        // last of the first `last + 1` tensors that begins at or before element i
+        auto tensor_at = [&](uint32_t i, int last) -> int {
+            int a = 0, b = last + 1;
+            while (b - a > 1) {
+                const int mid = (a + b) >> 1;
+                if (mt.begin[mid] <= i) a = mid; else b = mid;
+            }
+            return a;
+        };
+        if (mt.begin[room] < t_len) t_len = mt.begin[room] & ~3u;
+        if (t_len == 0) { __syncthreads(); break; }
+        const int T = tensor_at(t_len - 1, room - 1) + 1;
+        // units and exponents, four tensors per warp at a time
+        for (int j0 = warp; j0 < T; j0 += 4 * kTileWarps) {
+            int32_t ex[4][2];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = j0 + q * kTileWarps;
+                ex[q][0] = j < T && lane < (uint32_t)W ? sm.gexp[lane][g + j] : VGC_EXP_NONE;
+                ex[q][1] = j < T && lane + 32u < (uint32_t)W ? sm.gexp[lane + 32][g + j] : VGC_EXP_NONE;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = j0 + q * kTileWarps;
+                if (j >= T) break;
+                const int32_t b = unit_of_tensor(ex[q], W, pow2, s_exp);
+                if (lane == 0) {
+                    mt.base[j] = b;
+                    if (b == kUnfit) sm.unfit = 1;
+                }
+                if (lane < (uint32_t)W) mt.above[j * W + lane] = ex[q][0] == VGC_EXP_NONE ? kNothing : (uint8_t)(ex[q][0] - b);
+                if (lane + 32u < (uint32_t)W) mt.above[j * W + lane + 32] = ex[q][1] == VGC_EXP_NONE ? kNothing : (uint8_t)(ex[q][1] - b);
+            }
+        }
+        __syncthreads();
+        const bool unfit = sm.unfit;
+        if (!kOverwrite) {                                          // u is read at the tile's end: ask it into L2 now
+            for (uint32_t line = tid; line < (t_len + 31u) / 32u; line += kTileThreads)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(u + t0 + 32u * line));
+        }
+        int j = 0;                                                  // tensor of the word looked at last, its elements
+        uint32_t from = 0, len = T > 1 ? mt.begin[1] : t_len;
+        auto look_up = [&](uint32_t at) {
+            if (at - from >= len) {
+                j = tensor_at(at, T - 1);
+                from = mt.begin[j];
+                len = mt.begin[j + 1] - from;
+            }
+        };
+        if (!kOverwrite && unfit) {                                 // the old content that is added to in message order
+            for (uint32_t i = 4 * tid; i < t_len; i += 4 * kTileThreads) {
+                look_up(i);
+                if (i + 4 <= t_len && i + 3 - from < len) {
+                    if (mt.base[j] == kUnfit) cp_async_16(tile + i, u + t0 + i);
+                } else {
+                    for (uint32_t c = i; c < min(i + 4, t_len); ++c) {
+                        look_up(c);
+                        if (mt.base[j] == kUnfit) tile[c] = u[t0 + c];
+                    }
+                }
+            }
+            cp_async_wait_all();                                    // (before the barrier behind the words that fit)
+        }
+        stream_tile(sm, W, t0, t_len, bad, [&](uint32_t word, uint32_t m, uint32_t &n_in) {
+            const uint32_t at = (word - (t0 << 4)) >> 4;
+            if (at >= t_len) return;
+            ++n_in;
+            look_up(at);
+            const uint32_t above = mt.above[j * W + (int)m];
+            if (mt.base[j] == kUnfit || above == kNothing) return;
+            const int mult = 1 << (above - (word & 7u));
+            atomicAdd(sums + at, (word & 8u) ? -mult : mult);
+        });
+        __syncthreads();
+        if (unfit) {
+            for (int w = 0; w < W; ++w) {
+                const uint32_t words = sm.taken[w], *run = sm.words[w] + sm.cur[w];
+                if (words == 0) continue;
+                const int32_t *gexp = sm.gexp[w] + g;
+                for (uint32_t i = tid; i < words; i += kTileThreads) {
+                    const uint32_t word = run[i], at = (word >> 4) - t0;
+                    if (at >= t_len) continue;                      // (counted as out of place above)
+                    look_up(at);
+                    if (mt.base[j] != kUnfit) continue;
+                    tile[at] = __fadd_rn(tile[at], value_at(word, gexp[j], scale));
+                }
+                __syncthreads();                                    // the next message may hit the same elements
+            }
+        }
+        if (tid < (uint32_t)W) sm.cur[tid] += sm.taken[tid];
+
+        // ---- the tile leaves, zeros stay behind
+        auto result = [&](int mult, int jj, float old) -> float {
+            const int32_t b = mt.base[jj];
+            if (b == kUnfit) return __int_as_float(mult);
+            if (!kOverwrite && mult == 0) return old;
+            const float v = __fmul_rn(times_unit(mult, power_of_two(b)), scale);
+            return kOverwrite ? v : __fadd_rn(old, v);
+        };
+        float *const dst = u + t0;
+        constexpr int kHeld = 4;                                    // vectors of u per thread in flight
+        const uint32_t n_vec = t_len / 4;
+        for (uint32_t q0 = tid; q0 < n_vec; q0 += kHeld * kTileThreads) {
+            float4 o[kHeld];
+#pragma unroll
+            for (int h = 0; h < kHeld; ++h) {
+                o[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (!kOverwrite && q0 + h * kTileThreads < n_vec) o[h] = *reinterpret_cast<const float4 *>(dst + 4 * (q0 + h * kTileThreads));
+            }
+#pragma unroll
+            for (int h = 0; h < kHeld; ++h) {
+                const uint32_t q = q0 + h * kTileThreads;
+                if (q >= n_vec) break;
+                const int4 mlt = reinterpret_cast<const int4 *>(sums)[q];
+                reinterpret_cast<int4 *>(sums)[q] = make_int4(0, 0, 0, 0);
+                float4 v;
+                look_up(4 * q);
+                v.x = result(mlt.x, j, o[h].x);
+                if (4 * q + 3 - from < len) {
+                    v.y = result(mlt.y, j, o[h].y);
+                    v.z = result(mlt.z, j, o[h].z);
+                    v.w = result(mlt.w, j, o[h].w);
+                } else {                                            // a border inside the vector
+                    look_up(4 * q + 1); v.y = result(mlt.y, j, o[h].y);
+                    look_up(4 * q + 2); v.z = result(mlt.z, j, o[h].z);
+                    look_up(4 * q + 3); v.w = result(mlt.w, j, o[h].w);
+                }
+                *reinterpret_cast<float4 *>(dst + 4 * q) = v;
+            }
+        }
+        if (tid < t_len - 4 * n_vec) {                              // the buffer's last elements
+            const uint32_t i = 4 * n_vec + tid;
+            look_up(i);
+            dst[i] = result(sums[i], j, kOverwrite ? 0.f : dst[i]);
+            sums[i] = 0;
+        }
+        g += tensor_at(t_len, room);
+        __syncthreads();                                            // cursors, tensors, and the tile's zeros
+    }
+    return t0 | (bad ? kBad : 0u);
 }
 
 // Bound: HBM for the dense forms (4 B per word, 4 or 8 B per element), DRAM accesses for the sparse ones, latency for small
@@ -750,9 +989,10 @@ decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *g
     const bool pow2 = (__float_as_uint(scale) & 0x807FFFFFu) == 0u && s_exp > -127 && s_exp < 128;
     const int g_first = kHybrid ? 0 : group_of(offs, K, lo);
     const int g_last = kHybrid ? 0 : hi <= offs[g_first + 1] ? g_first : group_of(offs, K, hi - 1);
-    if (tid < (uint32_t)W && (reinterpret_cast<uintptr_t>(sm.words[tid]) & 15u)) sm.unfit = 1;      // read 16 bytes at a time
-    // a scale that is not finite; the filler's index would be an element; more tensors than there is room for
-    if (tid == 0 && (s_exp >= 128 || hi == (1u << 28) || g_last - g_first >= kTensors)) sm.unfit = 1;
+    // kOrdered: read 16 bytes at a time; a scale that is not finite; the filler's index would be an element
+    if (tid < (uint32_t)W && (reinterpret_cast<uintptr_t>(sm.words[tid]) & 15u)) atomicOr(&sm.unfit, kOrdered);
+    if (tid == 0 && (s_exp >= 128 || hi == (1u << 28))) atomicOr(&sm.unfit, kOrdered);
+    if (tid == 0 && g_last - g_first >= kTensors) atomicOr(&sm.unfit, kCrowded);
     int32_t ex[2] = {VGC_EXP_NONE, VGC_EXP_NONE};                // warp j looks at the range's j-th tensor
     const int g_mine = g_first + (int)warp;
     if (!kHybrid && g_mine <= g_last) {                          // on their way during the search
@@ -773,28 +1013,34 @@ decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *g
             asm volatile("prefetch.global.L2 [%0];" ::"l"(sm.words[w] + at));
     }
     if (!kHybrid && g_mine <= g_last) {
-        const bool some0 = ex[0] != VGC_EXP_NONE, some1 = ex[1] != VGC_EXP_NONE;
-        const int e_max = __reduce_max_sync(0xffffffffu, max(some0 ? ex[0] : INT32_MIN, some1 ? ex[1] : INT32_MIN));
-        const int e_min = __reduce_min_sync(0xffffffffu, min(some0 ? ex[0] : INT32_MAX, some1 ? ex[1] : INT32_MAX));
+        const int32_t b = unit_of_tensor(ex, W, pow2, s_exp);
         if (lane == 0) {
-            int b = 0;                                           // (nothing was sent from this tensor)
-            bool fits = true;
-            if (e_max >= e_min) {
-                b = e_min - 7;                                   // the smallest value a word can stand for
-                // 2^base and every sum of multiples are normal numbers; with a power-of-two scale so are their products
-                fits = e_max - b + (32 - __clz((W - 1) | 1)) <= 22 && b >= -126 && b + 22 <= 127 &&
-                       (!pow2 || (b + s_exp >= -126 && b + 22 + s_exp <= 127));
-            }
-            // a tile takes elements of two tensors at most and begins at a multiple of four elements: a tensor of fewer
-            // than seven between two others would make it three
+            // a tile of exact_range takes elements of two tensors at most and begins at a multiple of four elements: a
+            // tensor of fewer than seven between two others would make it three
             const uint32_t size = offs[g_mine + 1] - offs[g_mine];
-            if (!fits || (g_mine > g_first && g_mine < g_last && size > 0 && size < 7)) sm.unfit = 1;
+            uint32_t about = b == kUnfit ? kSomeUnfit : kSomeFit;
+            if (g_mine > g_first && g_mine < g_last && size > 0 && size < 7) about |= kCrowded;
+            atomicOr(&sm.unfit, about);
             sm.base[warp] = b;
         }
     }
     __syncthreads();
-    if (sm.unfit) bad = ordered_range<kHybrid, kOverwrite>(sm, tile, W, offs, K, scale, tau, u, lo, hi, tile_elems);
-    else bad = exact_range<kHybrid, kOverwrite>(sm, tile, W, offs, g_first, scale, tau, u, lo, hi, tile_elems);
+    const uint32_t about = sm.unfit;
+    const uint32_t sm_addr = (uint32_t)__cvta_generic_to_shared(&sm), tile_addr = (uint32_t)__cvta_generic_to_shared(tile);
+    uint32_t from = lo;                                          // what is left to the ordered form
+    bad = false;
+    if (!(about & (kOrdered | kCrowded | kSomeUnfit))) {
+        bad = exact_range<kHybrid, kOverwrite>(sm, tile, W, offs, g_first, scale, tau, u, lo, hi, tile_elems);
+        from = hi;
+    } else if constexpr (!kHybrid) {
+        if (!(about & kOrdered) && (about & (kCrowded | kSomeFit))) {
+            __syncthreads();                                     // (everybody has read sm.unfit)
+            const uint32_t end = many_range<kOverwrite>(sm_addr, tile_addr, W, offs, K, scale, pow2, s_exp, u, lo, hi, tile_elems);
+            from = end & ~kBad;
+            bad = (end & kBad) != 0;
+        }
+    }
+    if (from < hi) bad |= ordered_range<kHybrid, kOverwrite>(sm_addr, tile_addr, W, offs, K, scale, tau, u, from, hi, tile_elems);
     if (bad) atomicOr(dev_status, VGC_DEV_RANGE);
 }
 

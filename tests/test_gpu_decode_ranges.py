@@ -47,7 +47,8 @@ def test_small_ranges(n, density, W):
     _check(n, offs, [_message(n, offs, density, 10 * w + n) for w in range(W)])
 
 
-@pytest.mark.parametrize("sizes", [[100_000, 5, 900_000], [33_333, 3, 2, 1, 400_001, 17, 90_001], [64] * 3000, [0, 70_001, 0, 0, 1_500_002]])
+@pytest.mark.parametrize("sizes", [[100_000, 5, 900_000], [33_333, 3, 2, 1, 400_001, 17, 90_001], [64] * 3000, [0, 70_001, 0, 0, 1_500_002],
+                                   [0] * 600 + [40_000, 2] + [0] * 900 + [1, 30_000, 0, 5, 0]])
 def test_tensor_borders_anywhere(sizes):
     offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint32)
     n = int(offs[-1])
@@ -105,3 +106,40 @@ def test_flat_form_costs_what_the_words_cost():
 
     alone = time([1_500_000])
     assert time([1_500_000] + [200] * 63) < 3.0 * alone
+
+
+@pytest.mark.parametrize("sizes", [[50_000] + [64, 64] * 40 + [300_000], [1] * 2000 + [70_000], [0] * 50 + [40_000] + [0] * 55 + [3, 0, 0, 5] * 200 + [9_001],
+                                   list(range(1, 900)) + [200_003], [500] * 1200 + [7]])
+@pytest.mark.parametrize("W", [3, 8, 40, 64])
+def test_form_is_chosen_tensor_by_tensor(sizes, W):
+    """More tensors in a block's range and in a tile than any fixed number, with a scale that is no power of two.  A tensor
+    whose exponents lie close together is scale * the exact sum, its neighbour whose exponents do not is the sequential sum:
+    both bit for bit."""
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint32)
+    n, K, scale = int(offs[-1]), len(sizes), np.float32(1.0 / 7)
+    apart = np.random.default_rng(K).random(K) < 0.3                       # tensors that take the ordered form
+    host, dev = [], []
+    for w in range(W):
+        words, exps = _message(n, offs, 1.2 / W, 500 + w)
+        exps = np.where(apart, -5 - 25 * (w % 2), exps.cpu().numpy()).astype(np.int32)
+        host.append((words.cpu().numpy().view(np.uint32), exps))
+        dev.append((words, torch.tensor([words.numel()], dtype=torch.int32, device="cuda"), torch.from_numpy(exps).cuda()))
+    ordered = np.repeat(apart, sizes)
+    for overwrite in (False, True):
+        u0 = np.zeros(n, F32) if overwrite else np.random.default_rng(1).standard_normal(n).astype(F32)
+        gu = Guarded(n)
+        gu.t.copy_(torch.from_numpy(u0))
+        st = torch.zeros(1, dtype=torch.int32, device="cuda")
+        vgc.vgc_decode_accumulate(dev, vgc.offsets_tensor(offs), float(scale), gu.t, st, overwrite=overwrite)
+        gu.check("u")
+        sequential, exact = u0.copy(), np.zeros(n, F32)
+        oracle.decode_accumulate(host, offs, float(scale), sequential)
+        oracle.decode_accumulate([(m, np.where(apart, 0, e).astype(np.int32)) for m, e in host], offs, 1.0, exact)
+        touched = np.zeros(n, bool)
+        for m, _ in host:
+            touched[m >> 4] = True
+        scaled = np.where(touched & (exact != 0), u0 + exact * scale, u0)   # (float32: each operation rounded once)
+        want = np.where(ordered, sequential, scaled).astype(F32)
+        assert int(st.item()) == 0
+        got = gu.t.cpu().numpy()
+        assert np.array_equal(got, want), (np.flatnonzero(got != want)[:5], got[got != want][:5], want[got != want][:5])
