@@ -114,3 +114,24 @@ def test_packed_message_decodes_to_the_same_update():
     ref = np.zeros(n, np.float32)
     oracle.decode_accumulate([(oracle.unpack_indices(packed[:nbytes].cpu().numpy(), msg["nnz"]), msg["group_exp"])], offs, 1.0, ref)
     assert np.array_equal(u1.cpu().numpy(), ref)
+
+
+def test_more_chunks_than_blocks():
+    """Message and buffer lengths on either side of what the blocks take in one turn (9472 x 2048 words), messages much shorter
+    than their buffer, a stream cut short."""
+    n = 1 << 25
+    words, _ = workloads.random_message(n, np.array([0, n], np.uint32), 0.9, seed=11, device="cuda")
+    host, turn = words.cpu().numpy().view(np.uint32), 9472 * 2048
+    for m in (0, 5000, turn - 1, turn, turn + 1, host.size):
+        want = oracle.pack_indices(host[:m])
+        for capacity in (None, want.size - 3) if m else (None,):
+            packed, nbytes, status, count = gpu_pack(words, m, capacity)
+            kept = want.size if capacity is None else capacity
+            assert nbytes == want.size and status == (0 if capacity is None else vgc.VGC_DEV_CAPACITY), m
+            assert np.array_equal(packed[:kept].cpu().numpy(), want[:kept]), m
+            if capacity is None:
+                back = torch.full((host.size,), -1, dtype=torch.int32, device="cuda")
+                st = torch.zeros(1, dtype=torch.int32, device="cuda")
+                vgc.vgc_unpack_indices(packed, count, back, st)
+                assert int(st.item()) == 0 and np.array_equal(back[:m].cpu().numpy().view(np.uint32), host[:m]), m
+                assert bool((back[m:] == -1).all()), m
