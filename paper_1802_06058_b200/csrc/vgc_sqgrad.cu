@@ -12,6 +12,7 @@ vgc_status simt_sqgrad_conv(const float *x, const float *delta, int B, int C, in
                             int accumulate, float *S, void *ws, size_t ws_bytes, cudaStream_t st);
 vgc_status dense_simt(const float *x, const float *delta, int B, int in, int out, float scale, int accumulate, float *S,
                       cudaStream_t st);
+bool dense_simt_better(int B, int in, int out, bool tensor_cores);
 bool dense_supported(int B, int in, int out);
 vgc_status dense_sqgrad_linear(const float *x, const float *delta, int B, int in, int out, float scale, int accumulate,
                                float *S, void *ws, cudaStream_t st);
@@ -73,14 +74,15 @@ extern "C" vgc_status vgc_sqgrad_linear(const float *x, const float *delta, int 
     if (B == 0) return empty_batch(&S, 1, (size_t)in * out, accumulate, st);
     if (ws_bytes < vgc_sqgrad_linear_workspace_bytes(B, in, out) || !ws) return VGC_ERR_WORKSPACE;
     // Up to 2^25 multiply-adds the CUDA cores are done before the tensor-core kernel has filled its pipeline (2.5 us against
-    // 5.0 at 2^20, equal near 2^25); beyond 512 examples the general tensor-core kernel takes over from the dense one, with
-    // a higher start (11 us).
-    const long long macs = (long long)in * out * B;
-    if (macs > (1ll << 25) && dense_supported(B, in, out))
-        return dense_sqgrad_linear(x, delta, B, in, out, scale, accumulate, S, ws, st);
-    if (B <= 1024 && (macs <= (1ll << 27) || !tc_linear_supported(B, in, out)))
+    // 5.0 at 2^20, equal near 2^25); where that kernel does not reach (beyond 512 examples, sizes TMA cannot address) it is
+    // the CUDA cores in one launch or a kernel with a higher start (11 us).
+    const bool tc = tc_linear_supported(B, in, out);
+    if (dense_supported(B, in, out)) {
+        if ((long long)in * out * B > (1ll << 25)) return dense_sqgrad_linear(x, delta, B, in, out, scale, accumulate, S, ws, st);
         return dense_simt(x, delta, B, in, out, scale, accumulate, S, st);
-    if (tc_linear_supported(B, in, out))
+    }
+    if (dense_simt_better(B, in, out, tc)) return dense_simt(x, delta, B, in, out, scale, accumulate, S, st);
+    if (tc)
         return tc_sqgrad_linear(x, delta, B, in, out, scale, accumulate, S, ws, ws_bytes, st);
     return simt_sqgrad_linear(x, delta, B, in, out, scale, accumulate, S, static_cast<char *>(ws) + 256,
                               ws_bytes - 256, st);

@@ -136,7 +136,7 @@ sqgrad_simt(const Ops ops, int M, int N, int K, int k_per_split, float scale, in
             } else {
                 const size_t at = (size_t)m * N + n;
                 const double res = (double)scale * sum;
-                S[at] = accumulate ? (float)((double)S[at] + res) : (float)res;
+                S[at] = accumulate ? __fadd_rn(S[at], (float)res) : (float)res;      // one fp32 addition, as everywhere
             }
         }
 }
@@ -150,7 +150,7 @@ sqgrad_combine_splits(const float *__restrict__ partial, int splits, size_t mn, 
     double sum = 0.0;
     for (int z = 0; z < splits; ++z) sum += (double)partial[(size_t)z * mn + i];
     const double res = (double)scale * sum;
-    S[i] = accumulate ? (float)((double)S[i] + res) : (float)res;
+    S[i] = accumulate ? __fadd_rn(S[i], (float)res) : (float)res;
 }
 
 // ---- dense layers: few enough multiply-adds for the CUDA cores, or sizes the tensor-core kernels do not take ------------
@@ -179,7 +179,7 @@ sqgrad_dense_simt(const float *x, const float *delta, int B, int in, int out, fl
     const int m0 = blockIdx.y * kTile, n0 = blockIdx.x * kTile;
     grid_release();
     grid_wait();
-    if (accumulate && kVec && tid < kTile && m0 + tid < out) {         // the old contents, needed at the end
+    if (accumulate && tid < kTile && m0 + tid < out) {                 // the old contents, needed at the end
 #pragma unroll
         for (int j = 0; j < kTile; j += 32)
             if (n0 + j < in) asm volatile("prefetch.global.L2 [%0];" ::"l"(S + (size_t)(m0 + tid) * in + n0 + j));
@@ -225,8 +225,8 @@ sqgrad_dense_simt(const float *x, const float *delta, int B, int in, int out, fl
             *reinterpret_cast<float4 *>(&As[k][c]) = square(a[i]);
             *reinterpret_cast<float4 *>(&Bs[k][c]) = square(b[i]);
         }
+        if (k0 + kDenseK < B) fetch(k0 + kDenseK);                      // (before the barrier: ordinary loads stay behind it)
         __syncthreads();
-        if (k0 + kDenseK < B) fetch(k0 + kDenseK);
         auto step = [&](int kk) {
             const float4 a4 = *reinterpret_cast<const float4 *>(&As[kk][ty * 4]);
             const float4 b4 = *reinterpret_cast<const float4 *>(&Bs[kk][tx * 4]);
@@ -268,6 +268,19 @@ sqgrad_dense_simt(const float *x, const float *delta, int B, int in, int out, fl
             for (int i = 0; i < 16; ++i) sum[i >> 2][i & 3] += part[g][i][t];
     }
     const int n = n0 + tx * 4;
+    float old[4][4];                                                    // all of it asked for before the first store
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int m = m0 + ty * 4 + i;
+        const float *src = S + (size_t)m * in + n;
+        if (kVec) {
+            const float4 o = accumulate && m < out && n < in ? *reinterpret_cast<const float4 *>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+            old[i][0] = o.x; old[i][1] = o.y; old[i][2] = o.z; old[i][3] = o.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) old[i][j] = accumulate && m < out && n + j < in ? src[j] : 0.f;
+        }
+    }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int m = m0 + ty * 4 + i;
@@ -275,21 +288,33 @@ sqgrad_dense_simt(const float *x, const float *delta, int B, int in, int out, fl
         float *dst = S + (size_t)m * in + n;
         float res[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) res[j] = (float)((double)scale * sum[i][j]);
+        for (int j = 0; j < 4; ++j) {
+            res[j] = (float)((double)scale * sum[i][j]);
+            if (accumulate) res[j] = __fadd_rn(old[i][j], res[j]);
+        }
         if (kVec) {
-            float4 v = make_float4(res[0], res[1], res[2], res[3]);
-            if (accumulate) {
-                const float4 old = *reinterpret_cast<const float4 *>(dst);
-                v.x = __fadd_rn(old.x, v.x); v.y = __fadd_rn(old.y, v.y);
-                v.z = __fadd_rn(old.z, v.z); v.w = __fadd_rn(old.w, v.w);
-            }
-            *reinterpret_cast<float4 *>(dst) = v;
+            *reinterpret_cast<float4 *>(dst) = make_float4(res[0], res[1], res[2], res[3]);
         } else {
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (n + j < in) dst[j] = accumulate ? __fadd_rn(dst[j], res[j]) : res[j];
+                if (n + j < in) dst[j] = res[j];
         }
     }
+}
+
+// Whether the kernel above is faster than what else takes the layer; tensor_cores: that is the general tensor-core kernel
+// (sqgrad_tc), else sqgrad_simt with its split reduction.  Measured on both sides (B200, one call among others, us above / else):
+//   sqgrad_tc, up to 2^27 multiply-adds: 640 examples 500 x 256 15.9 / 17.8, 768 18.6 / 19.7, 896 21.3 / 20.0, 1024 24.1 / 21.2
+//   sqgrad_simt: 149 to 296 tiles leave SMs with one or two blocks that nothing hides behind: 1031 x 1009, 64 examples faster
+//   above, 128 17.4 / 16.8, 256 31.9 / 27.8, 1024 119 / 93; more tiles are as fast above (2049 x 1023, 1024 examples: 171 / 174);
+//   fewer: 333 x 257, 768 examples 20.5 / 23.0, 896 23.7 / 21.0; less than half of the other kernel's tile used: 1024
+//   examples, 1000 x 10: 20.3 / 22.9
+bool dense_simt_better(int B, int in, int out, bool tensor_cores)
+{
+    if (tensor_cores) return B <= 768 && (long long)in * out * B <= (1ll << 27);
+    const long long tiles = (long long)((in + 63) / 64) * ((out + 63) / 64);
+    if (tiles > 148 && tiles <= 296) return B < 128;
+    return B <= 768 || (B <= 1024 && (tiles > 296 || in < 32 || out < 32));
 }
 
 vgc_status dense_simt(const float *x, const float *delta, int B, int in, int out, float scale, int accumulate, float *S,

@@ -1323,6 +1323,13 @@ sqgrad_tc_combine_many(const float *partial, int units_q, int units_r, int units
     const int r0 = (sub & 3) * 32, j0 = (sub >> 2) * 4;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (ty * kBM + r0 >= M || tx * tile_n + j0 >= N) return;
+    // thread of the first four warps: one element of the patch, lanes along whichever of m / n has unit stride; its old
+    // content is on its way during the sums
+    const int row = ld_m == 1 ? lane : 8 * w + (lane >> 2), col = ld_m == 1 ? w : lane & 3;
+    const int m = ty * kBM + r0 + row, n = tx * tile_n + j0 + col;
+    const bool mine = w < 4 && m < M && n < N;
+    float *const dst = results.S[blockIdx.y] + (size_t)m * ld_m + (size_t)n * ld_n;
+    const float old = accumulate && mine ? *dst : 0.f;
     const int lo_first = b_first * units_q + min(b_first, units_r);
     const float *src = partial + (size_t)j0 * kBM + r0 + lane;
     float sum[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1335,15 +1342,12 @@ sqgrad_tc_combine_many(const float *partial, int units_q, int units_r, int units
 #pragma unroll
     for (int c = 0; c < 4; ++c) sums[w][c][lane] = sum[c];
     __syncthreads();
-    // thread: row `lane`, column `w`
-    const int m = ty * kBM + r0 + lane, n = tx * tile_n + j0 + w;
-    if (w >= 4 || m >= M || n >= N) return;
-    float total = sums[0][w][lane];
+    if (!mine) return;
+    float total = sums[0][col][row];
 #pragma unroll
-    for (int i = 1; i < 8; ++i) total = __fadd_rn(total, sums[i][w][lane]);
-    float *dst = results.S[blockIdx.y] + (size_t)m * ld_m + (size_t)n * ld_n;
+    for (int i = 1; i < 8; ++i) total = __fadd_rn(total, sums[i][col][row]);
     const float res = __fmul_rn(scale, total);
-    *dst = accumulate ? __fadd_rn(*dst, res) : res;
+    *dst = accumulate ? __fadd_rn(old, res) : res;
 }
 
 // ---- host side --------------------------------------------------------------------------------

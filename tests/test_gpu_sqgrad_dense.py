@@ -40,3 +40,23 @@ def test_dense(B, n_in, n_out):
         assert bool(((T.t.double() - both).abs() <= 3 * 2.0 ** -24 * both).all())
     else:
         assert torch.equal(T.t, old + S.t)
+
+
+@pytest.mark.parametrize("B,n_in,n_out", [
+    (127, 1031, 1009), (640, 901, 901), (768, 333, 257), (769, 333, 257), (769, 500, 256), (768, 500, 256), (1024, 20, 300),
+    (900, 1301, 1301), (1024, 701, 701),                                                        # CUDA cores: one launch or a split reduction
+    (576, 512, 512), (1024, 512, 512), (2048, 64, 64), (5000, 260, 36)])                        # many partial tiles per tile
+def test_long_reductions(B, n_in, n_out):
+    test_dense(B, n_in, n_out)
+
+
+@pytest.mark.parametrize("B,n_in,n_out", [(1100, 333, 257), (1300, 33, 35), (640, 901, 901), (3000, 512, 512)])
+def test_added_is_one_fp32_addition(B, n_in, n_out):
+    """Long reductions, too: what is added is the written result, rounded once (a compressor step with s in v counts on it)."""
+    x, d = torch.randn(B, n_in, device="cuda"), torch.randn(B, n_out, device="cuda")
+    ws = torch.zeros(vgc.vgc_sqgrad_linear_workspace_bytes(B, n_in, n_out), dtype=torch.uint8, device="cuda")
+    S, T = torch.empty(n_in * n_out, device="cuda"), torch.rand(n_in * n_out, device="cuda")
+    vgc.vgc_sqgrad_linear(x, d, 1.0 / B, S, ws=ws)
+    want = T + S
+    vgc.vgc_sqgrad_linear(x, d, 1.0 / B, T, accumulate=True, ws=ws)
+    assert torch.equal(T, want)
