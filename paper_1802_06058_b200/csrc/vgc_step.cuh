@@ -42,7 +42,7 @@ constexpr int kOffsSmem = 1024;                      // group offsets cached in 
 constexpr uint32_t kStagedCopy = 2048;
 // a staged value: position in the block's range << 10 | sign << 9 | (rounded exponent + 127)
 constexpr uint32_t kPosShift = 10;
-constexpr size_t kMostPerBlock = 1u << (32 - kPosShift);
+static_assert(((size_t)VGC_MAX_PARAMS + kMaxGrid - 1) / kMaxGrid + 128 <= (size_t)1 << (32 - kPosShift), "a block's range");
 
 enum { kBasic = 0, kHybridBefore = 1, kHybridAfter = 2 };     // the hybrid's correction uses |r| from before / after r -= Sign(r) tau
 
@@ -299,6 +299,8 @@ compress_step(const __grid_constant__ Args a)
         }
         const uint32_t total = __shfl_sync(0xffffffffu, pincl, 31);
         const uint32_t pexcl = pincl - part;
+        int k_mine = k_tile;
+        uint32_t mine_max = 0;
 #pragma unroll
         for (int j = 0; j < kRowsA; ++j) {
             const uint32_t row_base = __shfl_sync(0xffffffffu, pexcl, j * kWarps + warp);
@@ -316,10 +318,17 @@ compress_step(const __grid_constant__ Args a)
                         a.stage[lo + at] = staged;
                         if (kQuantise && at < kStagedCopy) sm_staged[at] = staged;
                         ++at;
-                        if (kQuantise && grp < 0) record(group_of(offs, K, e + q), bits & 0x7FFFFFFFu);
+                        if (kQuantise && grp < 0) {      // (a thread's values mostly share a tensor: one search, one maximum)
+                            if (e + q < offs[k_mine] || e + q >= offs[k_mine + 1]) {
+                                if (mine_max) record(k_mine, mine_max);
+                                k_mine = group_of(offs, K, e + q); mine_max = 0;
+                            }
+                            mine_max = max(mine_max, bits & 0x7FFFFFFFu);
+                        }
                     }
             }
         }
+        if (kQuantise && mine_max) record(k_mine, mine_max);
         if (kQuantise && tid == 0 && grp >= 0 && total) {
             if (grp != k_held) {
                 if (held_max) record(k_held, held_max);
@@ -343,6 +352,7 @@ compress_step(const __grid_constant__ Args a)
         const int own_first = (int)(sm_rec_max[0] >> 23), own_last = (int)(sm_rec_max[1] >> 23);         // biased
         constexpr uint32_t kBatch = 8, kRound = 3 * kBatch * kThreads;
         uint32_t sums = 0;                               // thread j of the first kCounts: entry j
+        int k_in = -1, own_in = 0;                       // the tensor looked at last of those between the first and the last one
         for (uint32_t i0 = 0; i0 < run; i0 += kRound) {  // block-uniform
             unsigned long long of_first = 0, of_last = 0;
             uint32_t inside = 0;
@@ -366,8 +376,11 @@ compress_step(const __grid_constant__ Args a)
                         const int level = e - own_last + 7;
                         if (level >= 0) of_last += 1ull << (7 * level);
                     } else {                             // a tensor wholly inside: E_k is this block's
-                        const int own = (int)(__ldcg(rec_max + group_of(offs, K, idx)) >> 23);
-                        inside += e >= own - 7 ? 1u : 0u;
+                        if (k_in < 0 || idx < offs[k_in] || idx >= offs[k_in + 1]) {
+                            k_in = group_of(offs, K, idx);
+                            own_in = (int)(__ldcg(rec_max + k_in) >> 23);
+                        }
+                        inside += e >= own_in - 7 ? 1u : 0u;
                     }
                 }
             }
