@@ -82,11 +82,12 @@ void workspace(PyObject *o, void **p, size_t *bytes)
     *bytes = (size_t)t.numel() * t.element_size();
 }
 
+// whatever float() takes
 double number(PyObject *o)
 {
-    const double v = PyFloat_AsDouble(o);
-    if (v == -1.0 && PyErr_Occurred()) throw Raised{};
-    return v;
+    if (PyFloat_CheckExact(o)) return PyFloat_AS_DOUBLE(o);
+    Ref f(PyNumber_Float(o));
+    return PyFloat_AS_DOUBLE(f.p);
 }
 long long integer(PyObject *o)
 {
@@ -464,17 +465,16 @@ PyObject *unpack_indices(Args a)
     VGC_CALL(vgc_unpack_indices(packed, nnz, max_words, words, status, st));
 }
 
-// value of a layer's key; `missing` < 0: the key has to be there
-long long layer_int(PyObject *layer, const char *key, long long missing = -1)
+long long layer_int(PyObject *layer, const char *key)
 {
-    PyObject *v = PyMapping_GetItemString(layer, key);
-    if (!v) {
-        if (missing < 0 || !PyErr_ExceptionMatches(PyExc_KeyError)) throw Raised{};
-        PyErr_Clear();
-        return missing;
-    }
-    Ref r(v);
-    return integer(r.p);
+    Ref v(PyMapping_GetItemString(layer, key));
+    return integer(v.p);
+}
+// layer.get(key, missing)
+long long layer_int(PyObject *layer, const char *key, int missing)
+{
+    Ref v(PyObject_CallMethod(layer, "get", "si", key, missing));
+    return integer(v.p);
 }
 
 // layers, g_host, g_dev, s_dev, r, v, group_offsets, alpha, zeta, scale, out, words_host, counters_host, ws_sqgrad,
@@ -487,7 +487,9 @@ PyObject *step_host(Args a)
     for (Py_ssize_t k = 0; k < n_layers; ++k) {
         PyObject *L = PySequence_Fast_GET_ITEM(seq.p, k);
         vgc_layer_host &o = layers[(size_t)k];
-        o.is_conv = layer_int(L, "is_conv") != 0;
+        Ref conv(PyMapping_GetItemString(L, "is_conv"));
+        Ref conv_number(PyNumber_Long(conv.p));                          // (whatever int() takes)
+        o.is_conv = truth(conv_number.p);
         o.B = (int)layer_int(L, "B");
         o.C = (int)layer_int(L, "C");
         o.H = (int)layer_int(L, "H", 1);
