@@ -22,6 +22,7 @@ OBJ_DIR = os.path.join(PKG_DIR, "build")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE]
+NATIVE_FLAGS = ["-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden"]
 
 
 def _sources():
@@ -61,20 +62,32 @@ def _compile(nvcc: str, src: str, verbose: bool) -> str:
     return obj
 
 
+def _native_tag() -> str:
+    """What the extension module depends on beside its source: the interpreter, torch's version (its C++ ABI) and the flags."""
+    import importlib.metadata
+    return " ".join([sysconfig.get_config_var("SOABI") or "", importlib.metadata.version("torch"), *NATIVE_FLAGS])
+
+
 def _build_native(force: bool) -> None:
     """The extension module that marshals the Python calls: compiled against torch's headers, linked to libvgc.so."""
+    stamp = os.path.join(OBJ_DIR, "native.tag")
     if not force and os.path.exists(NATIVE_PATH) and os.path.getmtime(NATIVE_PATH) >= _newest([NATIVE_SRC] + _headers()):
-        return
+        # (no stamp: the module came without its build folder, as on a machine that only runs it)
+        if not os.path.exists(stamp) or open(stamp).read() == _native_tag():
+            return
     torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
     torch_inc, torch_lib = os.path.join(torch_dir, "include"), os.path.join(torch_dir, "lib")
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     tmp = NATIVE_PATH + ".tmp.%d" % os.getpid()
-    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+    subprocess.run([os.environ.get("CXX", "g++"), *NATIVE_FLAGS,
                     "-I", INCLUDE, "-isystem", torch_inc, "-isystem", os.path.join(torch_inc, "torch", "csrc", "api", "include"),
                     "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), NATIVE_SRC, "-o", tmp,
                     "-L", torch_lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-L", PKG_DIR, "-lvgc",
                     "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + torch_lib], check=True)
     os.replace(tmp, NATIVE_PATH)
+    os.makedirs(OBJ_DIR, exist_ok=True)
+    with open(stamp, "w") as f:
+        f.write(_native_tag())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
