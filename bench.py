@@ -65,9 +65,11 @@ def peaks():
 
 def ncu_traffic():
     """DRAM traffic figures read off ncu captures (profiles/ncu_traffic.json names the captures and the library
-    version they were taken on); None where the file has no figure."""
+    version they were taken on); nothing where that is not this library's version, None where the file has no figure."""
+    import paper_1802_06058_b200 as vgc
     path = os.path.join(ROOT, "profiles", "ncu_traffic.json")
-    return json.load(open(path)) if os.path.exists(path) else {}
+    traffic = json.load(open(path)) if os.path.exists(path) else {}
+    return traffic if traffic.get("library_version") == vgc.vgc_version() else {}
 
 
 def measure_tf32_peak(sustain_s: float = 2.0):
