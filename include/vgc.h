@@ -173,8 +173,8 @@ vgc_status vgc_sqgrad_conv_batch(int n_layers, const float *const *x, const floa
  *   r, v          [n] fp32 state, updated in place (all zeros before the first step)
  *   group_offsets [K+1] u32 on the device, offsets[0] = 0, offsets[K] = n, non-decreasing
  *   out           HOST struct of device pointers, see below
- *   ws            at least vgc_compress_workspace_bytes(n, K) (about 8 bytes per parameter: every
- *                 tile of the buffer owns a staging segment that could hold all of its elements)
+ *   ws            at least vgc_compress_workspace_bytes(n, K): about 8 bytes per parameter, of which a call
+ *                 touches 4 for every element it selects, beside some tens of KB of records
  *
  * n == 0: no-op, OK (counters are not written).  n > VGC_MAX_PARAMS, alpha < 0, non-finite alpha or
  * zeta, K < 1, null or misaligned pointers: VGC_ERR_INVALID_ARG.  When the word buffer is too small
@@ -214,8 +214,8 @@ vgc_status vgc_compress(const float *g, const float *s, float *r, float *v, size
  *   - The call itself performs no allocation of any kind.  The first call on each device looks up
  *     the device address of the array (one cudaGetSymbolAddress, with that device current); make that
  *     first call before any stream capture starts.
- *   - All calls on a device share the one array and it keeps whatever the previous call left in it
- *     (the call clears the part that must start at zero).  Two calls that overlap on the GPU -- other
+ *   - All calls on a device share the one array and it keeps whatever the previous call left in it (a
+ *     call reads nothing there that it has not written).  Two calls that overlap on the GPU -- other
  *     streams, other host threads -- race on it: serialise them, or use vgc_compress with separate
  *     workspaces.
  */
@@ -237,8 +237,8 @@ vgc_status vgc_compress_static(const float *g, const float *s, float *r, float *
  *   u      [n] fp32, accumulated in place (the caller zeroes it when a fresh sum is wanted)
  *
  * Arithmetic.  Every result is a deterministic function of the inputs' bits when the messages together hold at
- * least one word per eight elements (u then moves through shared memory, tensor by tensor), so every worker that
- * decodes the same messages gets the same bits.  Two forms, chosen per weight tensor:
+ * least one word per eight elements (u then moves through shared memory), so every worker that decodes the same
+ * messages gets the same bits.  Two forms, chosen per weight tensor:
  *   exact    taken when all messages start on 16-byte boundaries and, for the tensor, the messages' exponents lie
  *            close together (E_max - E_min + 7 + ceil(log2 W) <= 22).  The words of an element are then integer
  *            multiples of one power of two and are summed exactly; the element becomes scale * sum (vgc_decode_sum)
@@ -246,7 +246,9 @@ vgc_status vgc_compress_static(const float *g, const float *s, float *r, float *
  *            power of two nothing is rounded before the final addition, and vgc_decode_sum returns the bits of the
  *            sum taken message by message in fp32.  Elements no word points at keep their bits (accumulate).
  *   ordered  otherwise: u[idx] += scale * value, rounded per word, in message order (w = 0, 1, ...) -- the fp32
- *            sequence of a sequential loop.
+ *            sequence of a sequential loop.  (Also what follows, in its block's range, a place where more than
+ *            4096 / W tensors, empty ones counted, begin within four elements; and the last range of a buffer of
+ *            2^28 elements.)
  *   The two differ by at most the roundings of the sequential loop: (W + 2) half-ulps of |u| + sum |scale * value|.
  * Sparser calls add scale * value with fp32 atomics, in any order: an element hit by three or more messages may
  * then differ from the sequential sum in the last bit.

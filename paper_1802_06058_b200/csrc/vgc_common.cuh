@@ -98,26 +98,7 @@ inline cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes, int regs
     });
 }
 
-__device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
-
-__device__ __forceinline__ uint64_t ld_volatile_u64(const uint64_t *p)
-{
-    uint64_t v;
-    asm volatile("ld.volatile.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_volatile_u64(uint64_t *p, uint64_t v)
-{
-    asm volatile("st.volatile.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t ld_volatile_u32(const uint32_t *p)
-{
-    uint32_t v;
-    asm volatile("ld.volatile.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Streaming (evict-first) 128-bit accesses for data touched once per call.
+// Streaming (evict-first) 128-bit load for data touched once per call.
 __device__ __forceinline__ float4 ld_stream_f4(const float *p)
 {
     float4 v;
@@ -126,12 +107,6 @@ __device__ __forceinline__ float4 ld_stream_f4(const float *p)
                  : "l"(p));
     return v;
 }
-__device__ __forceinline__ void st_stream_f4(float *p, float4 v)
-{
-    asm volatile("st.global.cs.v4.f32 [%0], {%1,%2,%3,%4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
-                 : "memory");
-}
-
 // Index of the weight tensor holding flat index i: the k with offs[k] <= i < offs[k+1].
 // offs has K+1 non-decreasing entries, offs[0] = 0; empty tensors are skipped.
 __device__ __forceinline__ int group_of(const uint32_t *offs, int K, uint32_t i)

@@ -34,8 +34,11 @@ struct DecodeViews {
 
 // Below one word per this many elements (all messages together) a call is not dense.  Added: an atomic costs two DRAM
 // accesses, a dense pass reads and writes all of u (n = 138 M, one word per 16: 172 us flat, 330 us dense; per 6: 250 us
-// dense).  Written: a buffer whose zeros are still in L2 when the words come takes scatter up to one word per eight
-// (n = 1.86 M, one per 12: 5.5 us against 7.5), larger ones up to one per 16 (n = 25.5 M: 29 us dense, 37 scatter).
+// dense).  Written: small buffers take scatter up to one word per eight, larger ones up to one per 16.  Measured just below /
+// above the line (4 messages; 32 messages), us: around one per 8, n = 1.86 M 5.6 / 7.0 and 8.1 / 12.9, n = 4 M 8.3 / 8.3 and
+// 10.3 / 13.6; around one per 16, n = 12 M 16.5 / 13.6 and 16.0 / 21.9, n = 25.5 M 43.4 / 23.7 and 34.0 / 37.7, n = 138 M 238 / 120
+// and 219 / 183.  (Between 4 and 12 M elements many messages would gain from scatter beyond one per 16: 8 M, 32 messages,
+// 12.4 / 20.2.)
 constexpr size_t kSparseAdd = 8;
 __host__ __device__ constexpr size_t sparse_write(size_t n) { return n <= ((size_t)4 << 20) ? 8 : 16; }
 

@@ -91,7 +91,7 @@ constexpr int kLoSlotsAT = 2 * kLoSlots;
 // Pure TMA form with A in tensor memory ("split rings"): the raw A tile is dead as soon as the transform has
 // read it, long before the MMAs of its slice retire.  It therefore gets a ring of its own that is freed
 // early, and the 16-KB units this saves hold more B tiles: more slices in flight from the same shared memory.
-constexpr int kSplitA = 4, kSplitB = kGroups > 2 ? 6 : 7, kSplitLo = kGroups > 2 ? 4 : 3;   // 16-KB units: A raw, B raw/hi, B lo (+ A in TMEM)
+constexpr int kSplitA = 4, kSplitB = 7, kSplitLo = 3;   // 16-KB units: A raw, B raw/hi, B lo (+ A in TMEM)
 static_assert((kSplitA + kSplitB + kSplitLo) * kRawBytesA <= (kRawSlots + kLoSlots) * kRawStageBytes, "smem budget");
 // Wide form (the kernels that gather several taps at a time, tiles of 192 columns): the tensor core takes an N = 192
 // instruction in no more time than an N = 128 one (98 busy cycles by the counters, 110), and 192 rows of the im2col view are 64 whole triples.  The raw A
@@ -558,7 +558,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     constexpr uint32_t kBTile = kRawBytesB;
 
     extern __shared__ uint8_t smem_raw_[];
-    __shared__ __align__(8) uint64_t bars[3 * kSplitB + kLoSlotsAT + 5 + 2 * kSplitA];
+    __shared__ __align__(8) uint64_t bars[3 * kSplitB + 5 + 2 * kSplitA];
     __shared__ uint32_t tmem_base_slot;
     __shared__ volatile uint32_t abort_flag;
 
@@ -570,8 +570,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     // a lo slot (and its A slot in tensor memory) is free when the MMAs of the slice that used it last have
     // retired, which is what that slice's `empty` barrier says: no barrier of its own, one commit per slice
     uint64_t *raw_full = bars, *op_full = bars + kNB, *empty = bars + 2 * kNB;
-    uint64_t *lo_empty = bars + 3 * kNB;
-    uint64_t *acc_full = lo_empty + kLoSlotsAT, *acc_empty = acc_full + 2, *drain = acc_empty + 2;
+    uint64_t *acc_full = bars + 3 * kNB, *acc_empty = acc_full + 2, *drain = acc_empty + 2;
     uint64_t *a_full = drain + 1, *a_empty = a_full + kNA;                 // split form: the A ring
 
     grid_release();
@@ -587,7 +586,6 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 mbar_init(smem_u32(&a_full[i]), 1);
                 mbar_init(smem_u32(&a_empty[i]), 4);
             }
-        for (int i = 0; i < kLoSlotsAT; ++i) mbar_init(smem_u32(&lo_empty[i]), 1);      // unused, kept initialised
         for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&acc_full[i]), 1); mbar_init(smem_u32(&acc_empty[i]), kEpilogueWarps); }
         mbar_init(smem_u32(drain), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1369,7 +1367,8 @@ struct Plan {
 // Two candidates: whole tiles per block (no scratch, no second kernel, but the blocks' loads are as even as the
 // tile count allows), or an even cut of the slices over all SMs (tiles at the cuts are shared, their partial
 // sums combined by a second kernel).  Costs in slice times: a block's longest range, plus what the combine pass
-// adds to the call (its launch and the partial tiles' round trip, about 14 slices' worth).
+// adds to the call (its launch and the partial tiles' round trip, about 14 slices' worth: measured with tiles of 128 columns
+// and before launches overlapped; not measured again for the wide form and for chains that several warps share).
 static Plan make_plan(int M, int N, int k_slices, int n_layers, int unit_min, int tile_n)
 {
     Plan p;
