@@ -17,7 +17,9 @@
 // Bound: the pipeline's round trip per slice, shared-memory bandwidth (416 KB a tile of 64 examples) and HBM: 8 bytes per
 // weight when S is added to, 4 when it is written.  Measured (B200, one call among others): 64 examples, 25088 x 4096 added
 // to: 741 -> 178 us (822 MB, 0.70 of the measured copy rate); 4096 x 4096 written: 81 -> 19.8; 128 examples, 1024 x 1024:
-// 14.5 -> 7.7; 512 examples, 2048 x 2048: 43 -> 29.
+// 14.5 -> 6.4; 512 examples, 2048 x 2048: 43 -> 29.
+#include <type_traits>
+
 #include "vgc_tc.cuh"
 
 namespace vgc {
@@ -50,6 +52,8 @@ struct Params {
     int k_slices, tiles, tiles_x;
     float scale;
     uint32_t *status;
+    const float *x, *delta;
+    int examples, in, out;
 };
 
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1)
@@ -62,7 +66,8 @@ template <int kLeft>
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kLeft) : "memory"); }
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-template <bool kAccumulate, int kN>
+// kFew: fewer than 32 examples (see the epilogue; the check costs an added layer 6 %, so it is compiled for these only)
+template <bool kAccumulate, int kN, bool kFew>
 __global__ void __launch_bounds__(Shape<kAccumulate, kN>::kThreads, 1)
 sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
              const __grid_constant__ CUtensorMap map_s, const Params prm)
@@ -271,6 +276,33 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
 #pragma unroll
                     for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__fadd_rn(__uint_as_float(r[i]), __uint_as_float(r2[i])));
                 }
+                // Fewer examples than the general tensor-core kernel takes: a layer is infinite where a square or a sum is, as
+                // on the CUDA cores.  The three products make NaN of that (infinity times a zero low part, infinity minus
+                // infinity), so what comes out NaN is summed again in plain fp32.
+                uint32_t top = 0;                        // (sums of squares: NaN is what lies above infinity's bits)
+                if (kFew) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) top = max(top, r[i]);
+                }
+                if (kFew && top > 0x7F800000u) {
+                    uint32_t nan = 0;
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) nan |= (__uint_as_float(r[i]) != __uint_as_float(r[i]) ? 1u : 0u) << i;
+                    const int m = m0 + (int)lane;
+                    while (nan) {
+                        const int at = __ffs(nan) - 1, n = n0 + 32 * j + at;
+                        nan &= nan - 1u;
+                        float sum = 0.f;
+                        for (int z = 0; z < prm.examples && m < prm.out && n < prm.in; ++z) {
+                            const float d = prm.delta[(size_t)z * prm.out + m], v = prm.x[(size_t)z * prm.in + n];
+                            sum = fmaf(__fmul_rn(d, d), __fmul_rn(v, v), sum);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if (i == at) r[i] = __float_as_uint(sum);
+                    }
+                }
+                if (kFew) __syncwarp();
                 uint8_t *const row = box_gen + j * kBoxBytes + lane * 128;
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -349,8 +381,12 @@ vgc_status dense_sqgrad_linear(const float *x, const float *delta, int B, int in
     const long long rows_m = (out + kBM - 1) / kBM;
     const bool narrow = rows_m * ((in + kBN - 1) / kBN) <= 74;
     const int tile_n = narrow ? 64 : kBN;
-    auto fn = accumulate ? (narrow ? sqgrad_dense<true, 64> : sqgrad_dense<true, kBN>)
-                         : (narrow ? sqgrad_dense<false, 64> : sqgrad_dense<false, kBN>);
+    auto pick = [&](auto few) {
+        constexpr bool kFew = decltype(few)::value;
+        return accumulate ? (narrow ? sqgrad_dense<true, 64, kFew> : sqgrad_dense<true, kBN, kFew>)
+                          : (narrow ? sqgrad_dense<false, 64, kFew> : sqgrad_dense<false, kBN, kFew>);
+    };
+    auto fn = B < 32 ? pick(std::true_type()) : pick(std::false_type());
     VGC_CUDA_OK(allow_dynamic_smem(reinterpret_cast<const void *>(fn), kSmemBytes));
     Params prm;
     prm.k_slices = (B + kBK - 1) / kBK;
@@ -360,6 +396,7 @@ vgc_status dense_sqgrad_linear(const float *x, const float *delta, int B, int in
     prm.tiles = (int)tiles;
     prm.scale = scale;
     prm.status = static_cast<uint32_t *>(ws);
+    prm.x = x; prm.delta = delta; prm.examples = B; prm.in = in; prm.out = out;
     // as few rounds as there have to be, of equal length
     const int rounds = (prm.tiles + 147) / 148, blocks = (prm.tiles + rounds - 1) / rounds;
     const int threads = accumulate ? Shape<true, kBN>::kThreads : Shape<false, kBN>::kThreads;
