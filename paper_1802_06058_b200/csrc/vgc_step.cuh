@@ -299,8 +299,6 @@ compress_step(const __grid_constant__ Args a)
         }
         const uint32_t total = __shfl_sync(0xffffffffu, pincl, 31);
         const uint32_t pexcl = pincl - part;
-        int k_mine = k_tile;
-        uint32_t mine_max = 0;
 #pragma unroll
         for (int j = 0; j < kRowsA; ++j) {
             const uint32_t row_base = __shfl_sync(0xffffffffu, pexcl, j * kWarps + warp);
@@ -318,17 +316,29 @@ compress_step(const __grid_constant__ Args a)
                         a.stage[lo + at] = staged;
                         if (kQuantise && at < kStagedCopy) sm_staged[at] = staged;
                         ++at;
-                        if (kQuantise && grp < 0) {      // (a thread's values mostly share a tensor: one search, one maximum)
-                            if (e + q < offs[k_mine] || e + q >= offs[k_mine + 1]) {
-                                if (mine_max) record(k_mine, mine_max);
-                                k_mine = group_of(offs, K, e + q); mine_max = 0;
-                            }
-                            mine_max = max(mine_max, bits & 0x7FFFFFFFu);
-                        }
                     }
             }
         }
-        if (kQuantise && mine_max) record(k_mine, mine_max);
+        if (kQuantise && grp < 0 && send_bits) {         // a thread's values mostly share a tensor: one search, one maximum
+            int k_mine = k_tile;
+            uint32_t mine_max = 0;
+#pragma unroll 1
+            for (uint32_t left = send_bits; left; left &= left - 1u) {
+                const uint32_t c = (uint32_t)__ffs(left) - 1u, i = base + ((c >> 2) * kThreads + tid) * 4 + (c & 3u);
+                uint32_t bits = 0;
+#pragma unroll
+                for (int j = 0; j < kRowsA; ++j)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (c == (uint32_t)(4 * j + q)) bits = __float_as_uint(reinterpret_cast<const float *>(&G[j])[q]) & 0x7FFFFFFFu;
+                if (i < offs[k_mine] || i >= offs[k_mine + 1]) {
+                    if (mine_max) record(k_mine, mine_max);
+                    k_mine = group_of(offs, K, i); mine_max = 0;
+                }
+                mine_max = max(mine_max, bits);
+            }
+            record(k_mine, mine_max);
+        }
         if (kQuantise && tid == 0 && grp >= 0 && total) {
             if (grp != k_held) {
                 if (held_max) record(k_held, held_max);
