@@ -128,7 +128,7 @@ struct Params {
     int chw;                 // C*H*W
     unsigned wo_magic;       // floor(2^32 / Wo) + 1: p / Wo == umulhi(p, wo_magic) for p * Wo < 2^32
     long long ld_m, ld_n;    // result: element (m, n) lives at S[m*ld_m + n*ld_n]; one of the two is 1
-    float *partial;          // scratch for partial tiles [2 * block + (0: a block's first segment, 1: its last)][column][row]
+    float *partial;          // scratch for partial tiles [2 * block + (0: a block's first segment, 1: its last)][column / 4][row][column % 4]
     uint32_t *status;        // device word; VGC_DEV_TIMEOUT is OR-ed in if a wait expired
 };
 
@@ -600,19 +600,24 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
-    grid_wait();
 
+    // Every role works its first segment out (divisions, cold instructions: 2 us) before it waits for the work ahead, as it
+    // does with all else that follows from the parameters alone.
     // `it` below is the running number of a slice within this block (over all of its segments): ring slots and
     // barrier phases follow it, so the pipeline does not drain between segments.
     if (warp < kFirstTransform) regs_dec<kRegsFew>();
     if (warp == 0) {
         // ================= TMA producer (one thread) =================
         if (lane == 0 && kAnyTma) {
-            int it = 0;
-            bool ok = true;
             SegIter iter(prm);
             Seg sg;
-            while (ok && iter.next(prm, sg)) {
+            bool more = iter.next(prm, sg);
+            if (!kGatherA) prefetch_map(&bt.a[sg.layer]);
+            if (!kGatherB) prefetch_map(&bt.b[sg.layer]);
+            grid_wait();
+            int it = 0;
+            bool ok = true;
+            for (; ok && more; more = iter.next(prm, sg)) {
                 const CUtensorMap *map_a = &bt.a[sg.layer], *map_b = &bt.b[sg.layer];
                 const int m0 = sg.m0, n0 = sg.n0;
                 for (int slice = sg.s_begin; slice < sg.s_end; ++slice, ++it) {
@@ -692,7 +697,8 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             bool ok = true;
             SegIter iter(prm);
             Seg sg;
-            while (ok && iter.next(prm, sg)) {
+            bool more = iter.next(prm, sg);
+            for (; ok && more; more = iter.next(prm, sg)) {
                 const uint32_t idesc = instr_desc(kMajor, sg.n_act, kBM);
                 const uint32_t idesc_bf = instr_desc_bf16(sg.n_act, kBM);
                 // an accumulator is drained every prm.chunk slices, and (kExact) at the end of every example: the
@@ -961,10 +967,11 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         RegsB b0, b1;
         int it0 = 0;                                 // block-wide number of the segment's first slice
         bool ok = true;
+        if (!kTwoGroups && t >= kGatherThreads) ok = false;
         SegIter iter(prm);
         Seg sg;
-        if (!kTwoGroups && t >= kGatherThreads) ok = false;
-        while (ok && iter.next(prm, sg)) {
+        bool more = iter.next(prm, sg);
+        for (; ok && more; more = iter.next(prm, sg)) {
             const int n_slices = sg.s_end - sg.s_begin;
             if (kAnyGather) {
                 rows_a.init(prm, bt.x[sg.layer], bt.delta[sg.layer], sg.m0, row0, prm.M);
@@ -972,6 +979,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 z = sg.s_begin / prm.p_slices;
                 pblk = sg.s_begin - z * prm.p_slices;
             }
+            grid_wait();                             // (returns at once from the second segment on)
             if (kTwoGroups) {
                 // this group's slices: those whose block-wide number is the group's modulo kGroups.  With a gathered
                 // tile: one register set per thread -- the other groups' work covers this group's load latency
@@ -1020,7 +1028,9 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         bool ok = true;
         SegIter iter(prm);
         Seg sg;
-        while (ok && iter.next(prm, sg)) {
+        bool more = iter.next(prm, sg);
+        grid_wait();
+        for (; ok && more; more = iter.next(prm, sg)) {
 #pragma unroll
             for (int j = 0; j < kN; ++j) acc[j] = 0.f;
             if (kExact && !kWide) {
@@ -1096,11 +1106,13 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             const int m = sg.m0 + r_local;
             float *const S = bt.S[sg.layer];
             if (!sg.whole) {
-                // partial tile, column-major inside the tile: consecutive lanes -> consecutive addresses
-                float *dst = prm.partial + (size_t)sg.slot * (kBM * kN) + r_local;
+                // partial tile, [four columns][row][column]: a lane's four columns in one store, lanes side by side; rows past
+                // the result's end (few output channels) are nobody's
+                float *dst = prm.partial + (size_t)sg.slot * (kBM * kN) + 4 * r_local;
+                if (sg.m0 + (int)(q * 32u) < prm.M)
 #pragma unroll
-                for (int j = 0; j < kN; ++j)
-                    if (j < n_valid) dst[j * kBM] = acc[j];
+                    for (int j = 0; j < kN; j += 4)
+                        if (j < n_valid) *reinterpret_cast<float4 *>(dst + j * kBM) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
             } else if (prm.ld_m == 1) {
                 // result is contiguous along m: lanes write neighbouring addresses directly
                 if (m < prm.M) {
@@ -1201,6 +1213,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     }
 
     // ---- common exit ----
+    grid_wait();                                          // (the threads without a role that touches memory)
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -1212,10 +1225,34 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
 
 // Adds the partial tiles of every tile that more than one block worked on, in the order of the blocks (a fixed
 // order: the result does not depend on scheduling).  One thread block per 32 x 32 patch of a tile: a warp takes
-// four columns, a lane one row -- partials are read along rows (their unit stride), four independent sums per
-// thread -- and the result is written along whichever of m / n has unit stride.  Tiles that one block covered
-// alone were written by that block; their patches return at once.
+// four columns, a lane one row of them -- 16 bytes per lane and partial tile, four sums -- and the result is written along
+// whichever of m / n has unit stride.  Tiles that one block covered alone were written by that block; their patches return
+// at once.  Which partial tiles they are is worked out before the wait for the kernel that writes them.
 struct ResultPtrs { float *S[kMaxBatch]; };
+
+// What both combine kernels need to know about a tile of the launch.
+struct TileParts {
+    int b_first, b_last;     // the blocks that hold the tile's first and last unit
+    int tx, ty;
+    bool first_is_last;      // the first block's part of this tile is that block's last segment (slot 1), not its first;
+                             // every later block's part is its first segment
+    __device__ __forceinline__ TileParts(int units_q, int units_r, int units_per_tile, int tiles_x, int tiles_y, int layer, int tile)
+    {
+        // the first units_r blocks own units_q + 1 units each, the others units_q
+        const int t_lo = (layer * (tiles_x * tiles_y) + tile) * units_per_tile, t_hi = t_lo + units_per_tile - 1;
+        const int big = units_r * (units_q + 1);
+        auto block_of = [&](int u) -> int { return u < big ? u / (units_q + 1) : units_r + (u - big) / units_q; };
+        b_first = block_of(t_lo);
+        b_last = block_of(t_hi);
+        first_is_last = b_first * units_q + min(b_first, units_r) < t_lo;
+        ty = tile / tiles_x;
+        tx = tile - ty * tiles_x;
+    }
+};
+__device__ __forceinline__ float4 add4(const float4 &a, const float4 &b)
+{
+    return make_float4(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z), __fadd_rn(a.w, b.w));
+}
 
 __global__ void __launch_bounds__(256)
 sqgrad_tc_combine(const float *partial, int units_q, int units_r, int units_per_tile,
@@ -1224,44 +1261,37 @@ sqgrad_tc_combine(const float *partial, int units_q, int units_r, int units_per_
 {
     __shared__ float patch[32][33];
     grid_release();
-    grid_wait();
-    const int tile = blockIdx.x / (tile_n >> 3), sub = blockIdx.x % (tile_n >> 3);
-    // the blocks that hold the tile's first and last unit: the first units_r blocks own units_q + 1 units each, the
-    // others units_q
-    const int t_lo = ((int)blockIdx.y * (tiles_x * tiles_y) + tile) * units_per_tile;
-    const int big = units_r * (units_q + 1);
-    auto block_of = [&](int u) -> int { return u < big ? u / (units_q + 1) : units_r + (u - big) / units_q; };
-    const int b_first = block_of(t_lo), b_last = block_of(t_lo + units_per_tile - 1);
-    if (b_first == b_last) return;
+    const int tile = blockIdx.x / (tile_n >> 3), sub = blockIdx.x - tile * (tile_n >> 3);
+    const TileParts parts(units_q, units_r, units_per_tile, tiles_x, tiles_y, (int)blockIdx.y, tile);
+    const int tx = parts.tx, ty = parts.ty;
     float *S = results.S[blockIdx.y];                                      // blockIdx.y: layer of the batch
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
     const int r0 = (sub & 3) * 32, j0 = (sub >> 2) * 32;                  // patch origin inside the tile
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;              // lane -> row, warp -> four columns
-    if (ty * kBM + r0 >= M || tx * tile_n + j0 >= N) return;
-    // the first block's part of this tile is that block's last segment unless its range starts with the tile;
-    // every later block's part is its first segment
-    const int lo_first = b_first * units_q + min(b_first, units_r);
-    const size_t within = (size_t)(j0 + 4 * w) * kBM + r0 + lane;
-    const float *src0 = partial + (size_t)(2 * b_first + (lo_first < t_lo ? 1 : 0)) * (kBM * tile_n) + within;
-    const float *src = partial + within;
-    float sum[4];
+    const size_t step = (size_t)2 * kBM * tile_n;                         // from a block's first segment to the next block's
+    const float *src = partial + ((size_t)(j0 / 4 + w) * kBM + r0 + lane) * 4 + (size_t)parts.b_first * step;
+    const float *src0 = src + (parts.first_is_last ? step / 2 : 0);
+    grid_wait();
+    if (parts.b_first == parts.b_last || ty * kBM + r0 >= M || tx * tile_n + j0 >= N) return;
+    float4 sum = __ldcs(reinterpret_cast<const float4 *>(src0));
+    const int n = parts.b_last - parts.b_first;
+    int b = 1;
+    for (; b + 4 <= n + 1; b += 4) {                     // four loads in flight, summed in block order
+        float4 v[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) sum[c] = __ldcs(src0 + c * kBM);
-    int b = b_first + 1;
-    for (; b + 2 <= b_last + 1; b += 2) {                // eight loads in flight, summed in block order
-        float v[2][4];
+        for (int u = 0; u < 4; ++u) v[u] = __ldcs(reinterpret_cast<const float4 *>(src + (size_t)(b + u) * step));
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v[u][c] = __ldcs(src + (size_t)(2 * (b + u)) * (kBM * tile_n) + c * kBM);
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) sum[c] = __fadd_rn(sum[c], v[u][c]);
+        for (int u = 0; u < 4; ++u) sum = add4(sum, v[u]);
     }
-    for (; b <= b_last; ++b)
+    {
+        float4 v[3];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) sum[c] = __fadd_rn(sum[c], __ldcs(src + (size_t)(2 * b) * (kBM * tile_n) + c * kBM));
+        for (int u = 0; u < 3; ++u)
+            if (b + u <= n) v[u] = __ldcs(reinterpret_cast<const float4 *>(src + (size_t)(b + u) * step));
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            if (b + u <= n) sum = add4(sum, v[u]);
+    }
+    const float sums[4] = {sum.x, sum.y, sum.z, sum.w};
     if (ld_m == 1) {
         const int m = ty * kBM + r0 + lane;
 #pragma unroll
@@ -1269,14 +1299,14 @@ sqgrad_tc_combine(const float *partial, int units_q, int units_r, int units_per_
             const int n = tx * tile_n + j0 + 4 * w + c;
             if (m < M && n < N) {
                 float *dst = S + (size_t)m + (size_t)n * ld_n;
-                const float res = __fmul_rn(scale, sum[c]);
+                const float res = __fmul_rn(scale, sums[c]);
                 *dst = accumulate ? __fadd_rn(*dst, res) : res;
             }
         }
         return;
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) patch[4 * w + c][lane] = __fmul_rn(scale, sum[c]);      // patch[column][row]
+    for (int c = 0; c < 4; ++c) patch[4 * w + c][lane] = __fmul_rn(scale, sums[c]);      // patch[column][row]
     __syncthreads();
     {
         const int c0 = (threadIdx.x & 7) * 4, r = threadIdx.x >> 3;       // four consecutive columns of one row
@@ -1285,11 +1315,7 @@ sqgrad_tc_combine(const float *partial, int units_q, int units_r, int units_per_
             float *dst = S + (size_t)m * ld_m + n;
             if ((ld_m & 3) == 0 && n + 3 < N) {
                 float4 out = make_float4(patch[c0][r], patch[c0 + 1][r], patch[c0 + 2][r], patch[c0 + 3][r]);
-                if (accumulate) {
-                    const float4 old = *reinterpret_cast<const float4 *>(dst);
-                    out.x = __fadd_rn(old.x, out.x); out.y = __fadd_rn(old.y, out.y);
-                    out.z = __fadd_rn(old.z, out.z); out.w = __fadd_rn(old.w, out.w);
-                }
+                if (accumulate) out = add4(*reinterpret_cast<const float4 *>(dst), out);
                 *reinterpret_cast<float4 *>(dst) = out;
             } else {
 #pragma unroll
@@ -1310,35 +1336,27 @@ sqgrad_tc_combine_many(const float *partial, int units_q, int units_r, int units
 {
     __shared__ float sums[8][4][32];
     grid_release();
-    grid_wait();
-    const int tile = blockIdx.x / tile_n, sub = blockIdx.x % tile_n;
-    const int t_lo = ((int)blockIdx.y * (tiles_x * tiles_y) + tile) * units_per_tile;
-    const int big = units_r * (units_q + 1);
-    auto block_of = [&](int u) -> int { return u < big ? u / (units_q + 1) : units_r + (u - big) / units_q; };
-    const int b_first = block_of(t_lo), b_last = block_of(t_lo + units_per_tile - 1);
-    if (b_first == b_last) return;
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
+    const int tile = blockIdx.x / tile_n, sub = blockIdx.x - tile * tile_n;
+    const TileParts parts(units_q, units_r, units_per_tile, tiles_x, tiles_y, (int)blockIdx.y, tile);
     const int r0 = (sub & 3) * 32, j0 = (sub >> 2) * 4;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (ty * kBM + r0 >= M || tx * tile_n + j0 >= N) return;
     // thread of the first four warps: one element of the patch, lanes along whichever of m / n has unit stride; its old
     // content is on its way during the sums
     const int row = ld_m == 1 ? lane : 8 * w + (lane >> 2), col = ld_m == 1 ? w : lane & 3;
-    const int m = ty * kBM + r0 + row, n = tx * tile_n + j0 + col;
+    const int m = parts.ty * kBM + r0 + row, n = parts.tx * tile_n + j0 + col;
     const bool mine = w < 4 && m < M && n < N;
     float *const dst = results.S[blockIdx.y] + (size_t)m * ld_m + (size_t)n * ld_n;
+    const size_t step = (size_t)2 * kBM * tile_n;
+    const float *src = partial + ((size_t)(j0 / 4) * kBM + r0 + lane) * 4 + (size_t)parts.b_first * step;
+    grid_wait();
+    if (parts.b_first == parts.b_last || parts.ty * kBM + r0 >= M || parts.tx * tile_n + j0 >= N) return;
     const float old = accumulate && mine ? *dst : 0.f;
-    const int lo_first = b_first * units_q + min(b_first, units_r);
-    const float *src = partial + (size_t)j0 * kBM + r0 + lane;
-    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int last = parts.b_last - parts.b_first;
 #pragma unroll 4
-    for (int b = b_first + w; b <= b_last; b += 8) {
-        const float *at = src + (size_t)(2 * b + (b == b_first && lo_first < t_lo ? 1 : 0)) * (kBM * tile_n);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) sum[c] = __fadd_rn(sum[c], __ldcs(at + c * kBM));
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) sums[w][c][lane] = sum[c];
+    for (int b = w; b <= last; b += 8)
+        sum = add4(sum, __ldcs(reinterpret_cast<const float4 *>(src + (size_t)b * step + (b == 0 && parts.first_is_last ? step / 2 : 0))));
+    sums[w][0][lane] = sum.x; sums[w][1][lane] = sum.y; sums[w][2][lane] = sum.z; sums[w][3][lane] = sum.w;
     __syncthreads();
     if (!mine) return;
     float total = sums[0][col][row];
