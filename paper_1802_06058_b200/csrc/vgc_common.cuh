@@ -98,6 +98,20 @@ inline cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes, int regs
     });
 }
 
+// Asks for `percent` of an SM's on-chip memory to be shared memory while this kernel runs there, the rest L1.  A kernel that
+// starts under the end of the one ahead otherwise runs with what that one left: behind a kernel that takes all the shared
+// memory, 28 KB of L1, too little for the loads that a streaming kernel keeps in flight.
+inline cudaError_t prefer_carveout(const void *kernel, int percent)
+{
+    static OncePerDevice once;
+    int device = -1;
+    const cudaError_t e = cudaGetDevice(&device);
+    if (e != cudaSuccess) return e;
+    return (cudaError_t)once(kernel, device, [&]() -> int {
+        return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent);
+    });
+}
+
 // Streaming (evict-first) 128-bit load for data touched once per call.
 __device__ __forceinline__ float4 ld_stream_f4(const float *p)
 {

@@ -1484,7 +1484,11 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
         // eight and more partial tiles per tile: the warps share the chain
         const bool many = plan.units_per_tile >= 8 * (prm.units_q + 1);
         const unsigned patches = (unsigned)(plan.tiles_x * plan.tiles_y) * (unsigned)(many ? tile_n : tile_n / 8);
-        VGC_CUDA_OK(launch_kernel(many ? sqgrad_tc_combine_many : sqgrad_tc_combine, dim3(patches, (unsigned)n_layers), dim3(256), 0, st,
+        const auto combine = many ? sqgrad_tc_combine_many : sqgrad_tc_combine;
+        // L1 for the loads of eight blocks (34 KB of shared memory) behind the kernel above, which takes all shared memory;
+        // with the same for sqgrad_repack, a pass over ResNet-50, batch 32, takes 1853 us instead of 1880
+        VGC_CUDA_OK(prefer_carveout(reinterpret_cast<const void *>(combine), 18));
+        VGC_CUDA_OK(launch_kernel(combine, dim3(patches, (unsigned)n_layers), dim3(256), 0, st,
                                   true, prm.partial, prm.units_q, prm.units_r, plan.units_per_tile, tile_n, plan.tiles_x, plan.tiles_y, M, N,
                                   prm.scale, prm.accumulate, results, prm.ld_m, prm.ld_n));
         count_launch();
@@ -1687,6 +1691,7 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
 {
     const int P = Ho * Wo, n_im2col = C * Kh * Kw;
     const int mode = repack_mode(B, C, Cout, Kh, Kw, sh, sw, ph, pw, P, W, Ho, Wo);
+    if (mode != kRepackNone) VGC_CUDA_OK(prefer_carveout(reinterpret_cast<const void *>(sqgrad_repack), 5));      // no shared memory: all L1
     // one run of the output per warp; more when there are many
     auto blocks_for = [](size_t values) { const size_t b = (values + 8 * kRepackRun - 1) / (8 * kRepackRun); return (unsigned)(b < 1 ? 1 : (b > 148 * 32 ? 148 * 32 : b)); };
     if (mode == kRepackPadW) {

@@ -582,6 +582,10 @@ vgc_status launch(Args a, void *records, cudaStream_t st)
     a.per_block = (uint32_t)per;
     a.tile = (uint32_t)round_up((per + tiles - 1) / tiles, 128);
     const dim3 grid((unsigned)((a.n + per - 1) / per));
+    // Two blocks' 26 KB, the rest L1: 1024 threads with eight 16-byte loads each.  Behind a dense layer's kernel without it (119.6 M
+    // parameters, B200): 531 us for this kernel, 383 with it.  Not the hybrid, which asks for next to no shared memory and would
+    // rather start under a decoder (25 M, 8 messages: 129.7 us a step, 131.1 with it).
+    if (kAlgorithm == kBasic) VGC_CUDA_OK(prefer_carveout(reinterpret_cast<const void *>(compress_step<kHasS, kAlgorithm>), 15));
     VGC_CUDA_OK(launch_kernel(compress_step<kHasS, kAlgorithm>, grid, dim3(kThreads), 0, st, true, a));
     VGC_CUDA_OK(launch_kernel(encode_step<kAlgorithm == kBasic>, grid, dim3(kThreads), 0, st, true, a));
     count_launch(2);
