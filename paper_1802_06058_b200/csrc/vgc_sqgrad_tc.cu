@@ -11,9 +11,11 @@
 //      and in place (hi overwrites the raw tile, lo goes beside it), so both inherit the swizzled
 //      layout the tensor core wants,
 //   3. issues three tcgen05.mma per 8-deep step -- hi*hi, hi*lo, lo*hi -- into a TMEM
-//      accumulator (the dropped lo*lo term is 2^-22 relative).  In the TMA-fed K-major form the two
-//      cross terms use bf16 copies of hi and lo instead (kind::f16, 16 deep per instruction): a
-//      cross term is 2^-11 of the product, so 8-bit operands leave an error below 2^-18 of it.
+//      accumulator (the dropped lo*lo term is 2^-22 relative).  In the TMA-fed K-major form and the
+//      wide form the two cross terms use bf16 copies of hi and lo instead (kind::f16, 16 deep per
+//      instruction): a cross term is 2^-11 of the product, so 8-bit operands leave an error below
+//      2^-18 of it, of either sign -- less than the third of the instructions saves of the
+//      accumulator's truncation bias (largest error of 3x3 layers 2.9e-6 -> 2.4e-6).
 // The tensor core's fp32 accumulation is not trusted over long reductions: every kChunk k slices
 // the accumulator is drained by four epilogue warps (tcgen05.ld) and added, round-to-nearest, to
 // fp32 registers while the next chunk accumulates into the second TMEM buffer.
@@ -142,6 +144,12 @@ struct Batch {
 
 // One 16-byte chunk (4 consecutive k of one row) of a K-major 128-byte-swizzled tile.
 __device__ __forceinline__ uint32_t chunk_offset(int row, int kq) { return (uint32_t)row * 128u + (uint32_t)((kq ^ (row & 7)) << 4); }
+
+// Four consecutive k of one row of a K-major tile of bf16: 64-byte rows, 64-byte swizzle.
+__device__ __forceinline__ uint32_t bf_offset(int row, int kq)
+{
+    return (uint32_t)row * 64u + (uint32_t)((((kq >> 1) ^ (row >> 1)) & 3) << 4) + (uint32_t)((kq & 1) << 3);
+}
 
 constexpr int kRowsPerThread = kBM * 8 / kGatherThreads;        // 4 gathered chunks per thread per tile
 
@@ -434,7 +442,8 @@ struct Gatherer<kMode, kHalf, kRows, true> {
         g.init(prm, x, origin, row0, limit);
     }
     __device__ __forceinline__ void load(const Params &prm, int z, int pbase, Regs &r) const { g.load(prm, z, pbase, r.v); }
-    template <bool kSquare>
+    // kBf: `lo` takes hi and lo as bf16, tiles of 64-byte rows one behind the other; a thread's four k are half of a 16-byte chunk
+    template <bool kSquare, bool kBf = false>
     __device__ __forceinline__ void store(uint8_t *hi, uint8_t *lo, int, int kq, const Regs &r) const
     {
 #pragma unroll
@@ -455,6 +464,14 @@ struct Gatherer<kMode, kHalf, kRows, true> {
                     const uint32_t off = chunk_offset(row, kq);
                     *reinterpret_cast<uint4 *>(hi + off) =
                         make_uint4(h[Impl::idx(kw, 0)], h[Impl::idx(kw, 1)], h[Impl::idx(kw, 2)], h[Impl::idx(kw, 3)]);
+                    if (kBf) {
+                        auto pair = [&](const uint32_t (&v)[Impl::kSlots], int j) {
+                            return pack_bf16(__uint_as_float(v[Impl::idx(kw, j)]), __uint_as_float(v[Impl::idx(kw, j + 1)]));
+                        };
+                        uint8_t *const at = lo + bf_offset(row, kq);
+                        *reinterpret_cast<uint2 *>(at) = make_uint2(pair(h, 0), pair(h, 2));
+                        *reinterpret_cast<uint2 *>(at + kRows * 64) = make_uint2(pair(l, 0), pair(l, 2));
+                    } else
                     *reinterpret_cast<uint4 *>(lo + off) =
                         make_uint4(l[Impl::idx(kw, 0)], l[Impl::idx(kw, 1)], l[Impl::idx(kw, 2)], l[Impl::idx(kw, 3)]);
                 }
@@ -518,6 +535,10 @@ struct SegIter {
 // tensor-pipe time of a tf32 product each; their rounding, 2^-9 relative on a term that is itself 2^-11 of the
 // product, stays below 2^-18 of the result).  A lo slot then holds [B hi as bf16][B lo as bf16], 8 KB each with
 // 64-byte rows, and an A slot in tensor memory [hi tf32: 32 columns][hi bf16: 16][lo bf16: 16].
+// The wide form's B tile is split as it is gathered: a thread's four k are 16 bytes of the tf32 tile and 8 of each bf16 tile
+// (12 KB each, in the same lo slot); five conversions of pairs serve three taps.  Twelve instructions a slice were what the
+// tensor pipe and the power cap allowed (1290 cycles a slice at 1.6 GHz); with eight, 128 channels 28 x 28, batch 32, take
+// 41.6 -> 38.6 us a call, the ResNet-50 pass 1920 -> 1871.
 // kN: columns of a tile, 128 or (wide form) 192.  The wide per-example form keeps the sum of squares in the epilogue's
 // registers: it takes layers whose examples fit one accumulator run (at most kChunk slices).
 template <int kMajor, int kModeA, int kModeB, bool kATmem, bool kExact = false, bool kBf = false, int kN = kBN>
@@ -532,7 +553,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     constexpr bool kWide = kN != kBN;
     static_assert(!kWide || (kN == kWideN && kATmem && IsTaps<kModeB>::value), "wide tiles: several taps at a time");
     constexpr bool kSplit = kATmem && (!kAnyGather || kWide);              // A raw tiles in a ring of their own
-    static_assert(!kBf || (kSplit && !kExact && !kWide), "bf16 cross terms: the TMA-fed form with A in tensor memory");
+    static_assert(!kBf || (kSplit && !kExact), "bf16 cross terms: A in tensor memory, sums of squares");
     constexpr bool kTmaB = kSplit && !kGatherB;                            // split form: the B tile comes by TMA, too
     constexpr int kNA = kWide ? kWideA : kSplitA;                                           // slots of the raw A ring (split form)
     // the transform warps work as two groups of four on alternate slices (else all eight on every slice)
@@ -555,7 +576,6 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     // bf16-cross form: where the B tile of raw slot s and the [hi bf16][lo bf16] tiles of lo slot s live
     auto b_tile = [&](int s) -> uint32_t { return pair_off(s) + kRawBytesA; };
     auto bf_tile = [&](int s) -> uint32_t { return lo_off(s) + kRawBytesA; };
-    constexpr uint32_t kBTile = kRawBytesB;
 
     extern __shared__ uint8_t smem_raw_[];
     __shared__ __align__(8) uint64_t bars[3 * kSplitB + 5 + 2 * kSplitA];
@@ -733,7 +753,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                                 else tc_mma_tf32_ts_acc(d_tmem, ta_hi + kk * 8, db_hi, idesc);
                             }
                             // cross terms, 16 k (32 bytes of a 64-byte row, 8 columns of tensor memory) per instruction
-                            const uint32_t bf_hi16 = (smem_base + bf_tile(ls)) >> 4, bf_lo16 = bf_hi16 + (kBTile >> 5);
+                            const uint32_t bf_hi16 = (smem_base + bf_tile(ls)) >> 4, bf_lo16 = bf_hi16 + (kBBytes >> 5);
 #pragma unroll
                             for (int kk = 0; kk < kBK / 16; ++kk) {
                                 tc_mma_bf16_ts_acc(d_tmem, ta_hi + 32 + kk * 8, desc_bf(bf_lo16 + kk * 2), idesc_bf);
@@ -822,9 +842,9 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             // lo tiles: [A lo][B lo], or the B tile alone when A lives in tensor memory (then `lo` points
             // one A tile below the slot so that the same chunk offsets address the B part)
             uint8_t *lo = smem_gen + lo_off(ls);
-            if (kWide) {
+            if constexpr (kWide) {
                 // the B tile first: only two A slots in tensor memory, so the A tile waits for slice i - 2 to retire
-                rows_b.template store<!kExact>(hi + kRawBytesA, lo + kRawBytesA, row0, kq, gb);
+                rows_b.template store<!kExact, kBf>(hi + kRawBytesA, lo + kRawBytesA, row0, kq, gb);
                 gathered();
                 if (!mbar_wait(smem_u32(&a_full[sa]), (uint32_t)(i / kNA) & 1u, &abort_flag)) return false;
                 if (i >= kAN) {
@@ -856,6 +876,16 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                             }
                         }
                         tc_st_32x8(taddr + 8 * k8, h8);
+                        if (kBf) {
+                            uint32_t hb[4], lb[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                hb[j] = pack_bf16(__uint_as_float(h8[2 * j]), __uint_as_float(h8[2 * j + 1]));
+                                lb[j] = pack_bf16(__uint_as_float(l8[2 * j]), __uint_as_float(l8[2 * j + 1]));
+                            }
+                            tc_st_32x4(taddr + 32 + 4 * k8, hb);
+                            tc_st_32x4(taddr + 48 + 4 * k8, lb);
+                        } else
                         tc_st_32x8(taddr + 32 + 8 * k8, l8);
                     }
                 } else
@@ -897,16 +927,16 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                     if (lane == 0) mbar_arrive(smem_u32(&a_empty[sa]));
                 }
             }
-            if (kBf) {
+            if (kBf && !kWide) {
                 // B tile: a thread takes pairs of adjacent 16-byte chunks (8 consecutive k of one row: the 128-byte
                 // swizzle permutes the two chunks of a pair only among themselves).  hi goes back in place as tf32;
                 // hi and lo as bf16 make one 16-byte chunk each, and under the 64-byte swizzle that chunk's place in
                 // its tile is the pair's place in the raw tile.  Half of each quarter-warp reads the second chunk of
                 // its pair first, which keeps the 16-byte accesses free of bank conflicts.
-                uint8_t *braw = smem_gen + b_tile(st), *bf_hi = smem_gen + bf_tile(ls), *bf_lo = bf_hi + kBTile / 2;
+                uint8_t *braw = smem_gen + b_tile(st), *bf_hi = smem_gen + bf_tile(ls), *bf_lo = bf_hi + kBBytes / 2;
                 const uint32_t s1 = (lane >> 2) & 1u;
 #pragma unroll
-                for (int u = 0; u < (int)(kBTile / 32) / kTT; ++u) {
+                for (int u = 0; u < (int)(kBBytes / 32) / kTT; ++u) {
                     const uint32_t p = (uint32_t)tt + (uint32_t)u * kTT;          // pair index = 4 * row + pair of the row
                     const uint32_t offx = 32 * p + 16 * s1, offy = 32 * p + 16 * (s1 ^ 1u);
                     const float4 x4 = *reinterpret_cast<const float4 *>(braw + offx);
@@ -1799,7 +1829,7 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
         const bool any_taps = taps || taps_s2 || taps7;
         const bool wide = any_taps && (n_im2col + kWideN - 1) / kWideN < (n_im2col + kBN - 1) / kBN && (!ex || p_slices <= kChunk);
 #define VGC_TAPS_FN(B_) (wide ? (ex ? (KernelFn)sqgrad_tc<kMajorK, kTma, B_, true, true, false, kWideN>                          \
-                                    : (KernelFn)sqgrad_tc<kMajorK, kTma, B_, true, false, false, kWideN>)                        \
+                                    : (KernelFn)sqgrad_tc<kMajorK, kTma, B_, true, false, true, kWideN>)                         \
                               : VGC_TC_FN(kTma, B_, true))
         if (any_taps) {
             if (taps) fn = taps == 4 ? VGC_TAPS_FN(kGatherTaps4) : VGC_TAPS_FN(kGatherTaps2);

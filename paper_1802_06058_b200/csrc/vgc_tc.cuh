@@ -136,7 +136,12 @@ __device__ __forceinline__ void tc_mma_bf16_ts_acc(uint32_t d_tmem, uint32_t a_t
         ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc)
         : "memory");
 }
-// 32 lanes x 8 columns
+// 32 lanes x 4 columns, x 8 columns
+__device__ __forceinline__ void tc_st_32x4(uint32_t taddr, const uint32_t (&r)[4])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
 __device__ __forceinline__ void tc_st_32x8(uint32_t taddr, const uint32_t (&r)[8])
 {
     asm volatile(
