@@ -151,6 +151,46 @@ sqgrad_tc_combine_many(const float *partial, int units_q, int units_r, int units
     *dst = accumulate ? __fadd_rn(old, res) : res;
 }
 
+// Examples cut into parts: S = scale * sum_z (sum of the example's parts)^2.  A thread block per 32 rows x 4 columns of a tile, its
+// eight warps take the examples in turn; their sums are added in the order of the warps.
+__global__ void __launch_bounds__(256)
+sqgrad_tc_combine_examples(const float *partial, int examples, int n_parts, int tile_n, int slot_n, int tiles_x, int tiles_y, int M, int N,
+                           float scale, int accumulate, const ResultPtrs results, long long ld_m, long long ld_n)
+{
+    __shared__ float sums[8][4][32];
+    grid_release();
+    const int tile = blockIdx.x / slot_n, sub = blockIdx.x - tile * slot_n;
+    const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
+    const int r0 = (sub & 3) * 32, j0 = (sub >> 2) * 4;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int row = ld_m == 1 ? lane : 8 * w + (lane >> 2), col = ld_m == 1 ? w : lane & 3;
+    const int m = ty * kBM + r0 + row, n = tx * tile_n + j0 + col;
+    const bool mine = w < 4 && m < M && n < min(N, (tx + 1) * tile_n);
+    float *const dst = results.S[blockIdx.y] + (size_t)m * ld_m + (size_t)n * ld_n;
+    const size_t slot = (size_t)kBM * slot_n;
+    const float *src = partial + ((size_t)blockIdx.y * tiles_x * tiles_y + tile) * examples * n_parts * slot +
+                       ((size_t)(j0 / 4) * kBM + r0 + lane) * 4;
+    grid_wait();
+    if (ty * kBM + r0 >= M || tx * tile_n + j0 >= N) return;
+    const float old = accumulate && mine ? *dst : 0.f;
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int z = w; z < examples; z += 8) {
+        const float *at = src + (size_t)z * n_parts * slot;
+        float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int i = 0; i < n_parts; ++i) d = add4(d, __ldcs(reinterpret_cast<const float4 *>(at + (size_t)i * slot)));
+        sum = add4(sum, make_float4(__fmul_rn(d.x, d.x), __fmul_rn(d.y, d.y), __fmul_rn(d.z, d.z), __fmul_rn(d.w, d.w)));
+    }
+    sums[w][0][lane] = sum.x; sums[w][1][lane] = sum.y; sums[w][2][lane] = sum.z; sums[w][3][lane] = sum.w;
+    __syncthreads();
+    if (!mine) return;
+    float total = sums[0][col][row];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) total = __fadd_rn(total, sums[i][col][row]);
+    const float res = __fmul_rn(scale, total);
+    *dst = accumulate ? __fadd_rn(old, res) : res;
+}
+
 // ---- host side --------------------------------------------------------------------------------
 // Slices per accumulator drain.  The tensor core's fp32 accumulation truncates (a one-sided bias of about 1.3e-8 of the
 // sum per instruction), so an accumulator is handed to the round-to-nearest register sums after at most 8 slices
@@ -162,6 +202,7 @@ static int g_concurrent = 1;
 struct Plan {
     int unit, units_per_tile, blocks, tiles_x, tiles_y;
     int units_total;
+    int parts, part_slices;  // examples cut up: parts of each (0: not), slices of a part
     bool partials;           // some tile is shared by several blocks: partial tiles go through the scratch
 };
 
@@ -202,6 +243,27 @@ static Plan make_plan(int M, int N, int k_slices, int n_layers, int unit_min, in
         const long long cost_b = ((units + blocks_b - 1) / blocks_b) * unit_min + 14;
         even = cost_b < cost_a;
         blocks = even ? blocks_b : blocks_a;
+    }
+    p.parts = p.part_slices = 0;
+    if (unit_min > 1 && g_concurrent == 1) {
+        // Few long examples, which the form that adds up an example's products before it squares them keeps whole, leave SMs
+        // idle: parts of an example, a block each, at most two waves of them; costs as above, a wave's start about 5 slices.
+        const long long waves_now = even ? (units + blocks - 1) / blocks : ((tiles + blocks - 1) / blocks) * upt;
+        long long best = waves_now * unit_min + (even ? 14 : 0);
+        for (int q = 1; q < unit_min; ++q) {
+            const long long n_parts = (unit_min + q - 1) / q, n = units * n_parts;
+            if (n > 2 * kSmCount) continue;
+            const long long cost = ((n + kSmCount - 1) / kSmCount) * (q + 5) + 14;
+            if (cost < best) { best = cost; p.parts = (int)n_parts; p.part_slices = q; }
+        }
+        if (p.parts) {
+            p.unit = p.part_slices;
+            p.units_per_tile = (int)(upt * p.parts);
+            p.units_total = (int)(units * p.parts);
+            p.blocks = p.units_total;
+            p.partials = true;
+            return p;
+        }
     }
     if (even && units >= (1LL << 31)) {          // unit positions are 32-bit in the kernel: whole tiles then
         even = false;
@@ -246,7 +308,7 @@ static size_t tc_workspace_bytes(int M, int N, int k_slices, int n_layers = 1, i
 {
     const Plan p = make_plan(M, N, k_slices, n_layers, unit, tile_n);
     // status word (256 bytes) + two partial tiles per block (the first and the last segment of its range)
-    return 256 + (p.partials ? (size_t)2 * p.blocks * kBM * slot_columns(tile_n) * sizeof(float) : 0);
+    return 256 + (p.partials ? (size_t)(p.parts ? 1 : 2) * p.blocks * kBM * slot_columns(tile_n) * sizeof(float) : 0);
 }
 
 static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Params prm, int M, int N,
@@ -258,6 +320,7 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
     prm.M = M; prm.N = N; prm.k_slices = k_slices;
     prm.unit = plan.unit; prm.units_per_tile = plan.units_per_tile; prm.units_total = plan.units_total;
     prm.units_q = plan.units_total / plan.blocks; prm.units_r = plan.units_total % plan.blocks;
+    prm.parts = plan.parts; prm.part_slices = plan.part_slices;
     prm.tile_n = tile_n; prm.tiles_x = plan.tiles_x; prm.tiles_y = plan.tiles_y;
     prm.chunk = kChunk;
     prm.status = static_cast<uint32_t *>(ws);
@@ -267,6 +330,16 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
     if (plan.partials) {
         ResultPtrs results = {};
         for (int l = 0; l < n_layers; ++l) results.S[l] = bt.S[l];
+        if (plan.parts) {
+            const int slot_n = slot_columns(tile_n);
+            VGC_CUDA_OK(prefer_carveout(reinterpret_cast<const void *>(sqgrad_tc_combine_examples), 18));
+            VGC_CUDA_OK(launch_kernel(sqgrad_tc_combine_examples, dim3((unsigned)(plan.tiles_x * plan.tiles_y * slot_n), (unsigned)n_layers), dim3(256), 0,
+                                      st, true, prm.partial, k_slices / prm.p_slices, plan.parts, tile_n, slot_n, plan.tiles_x, plan.tiles_y, M, N,
+                                      prm.scale, prm.accumulate, results, prm.ld_m, prm.ld_n));
+            count_launch();
+            VGC_CUDA_OK(cudaGetLastError());
+            return VGC_OK;
+        }
         // eight and more partial tiles per tile: the warps share the chain
         const bool many = plan.units_per_tile >= 8 * (prm.units_q + 1);
         const int slot_n = slot_columns(tile_n);
@@ -547,9 +620,13 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
     const bool taps7 = !in_tma && err_tma && Kw == 7 && sw == 2 && pw == 3 && W == 2 * Wo && Wo % 4 == 0;
     // with few output channels the roles are swapped -- except in the three-tap form, where keeping the errors as
     // the A operand (in tensor memory, half of its rows unused) measures faster than both operands in shared memory
-    // a square kernel that keeps the width: its input rows by TMA (the per-example form where an example fits one accumulator run)
+    // a square kernel that keeps the width: its input rows by TMA (the per-example form where it can take wide tiles)
+    // (wide tiles of the per-example form: an example fits one accumulator run, or parts of examples leave as plain sums)
+    auto short_runs = [&](int tile_n) {
+        return !t_exact || p_slices <= kChunk || make_plan(Cout, n_im2col, k_slices, n_layers, p_slices, tile_n).parts > 0;
+    };
     const bool halo = !in_tma && err_tma && (Kw == 5 || Kw == 7) && Kh == Kw && sh == 1 && sw == 1 && 2 * pw == Kw - 1 &&
-                      Wo == W && W % 2 == 0 && H * W % 4 == 0 && (!t_exact || p_slices <= kChunk);
+                      Wo == W && W % 2 == 0 && H * W % 4 == 0 && short_runs(kWideN / Kw * Kw);
     const bool swapped = conv_swapped(Cout, n_im2col) && !taps && !taps_s2 && !taps7 && !halo;
     // both tiles by TMA: A in tensor memory, cross terms in bf16 (the per-example form keeps tf32 cross terms)
     const bool tma_bf = err_tma && in_tma && !t_exact;
@@ -605,7 +682,7 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
             // 16 x 16 to 958, 81 columns: 25.0 us narrow, 28.7 wide).  The wide per-example form adds an example's sums up within
             // one accumulator run.
             const int mode = taps ? (taps == 4 ? kGatherTaps4 : kGatherTaps2) : taps_s2 ? (taps_s2 == 4 ? kGatherTaps4S2 : kGatherTaps2S2) : kGatherTaps7S2;
-            const bool wide = (n_im2col + kWideN - 1) / kWideN < (n_im2col + kBN - 1) / kBN && (!ex || p_slices <= kChunk);
+            const bool wide = (n_im2col + kWideN - 1) / kWideN < (n_im2col + kBN - 1) / kBN && short_runs(kWideN);
             fn = wide ? wide_taps_kernel(mode, ex) : narrow_taps_kernel(mode, ex);
             return tc_launch(fn, bt, n_layers, prm, Cout, n_im2col, k_slices, ws, ws_bytes, st, unit, wide ? kWideN : kBN);
         }

@@ -125,6 +125,7 @@ struct Params {
     int chunk;               // slices per accumulator drain
     int unit;                // slices that stay in one block: the reduction is cut between units only
     int units_per_tile;      // k_slices / unit
+    int parts, part_slices;  // per-example form, examples cut up: parts of an example (0: whole examples), slices of one; a block each
     int units_total;         // layers * tiles * units_per_tile: the launch's work, cut evenly over the blocks:
     int units_q, units_r;    // block b owns units [b q + min(b, r), ...) with q = total / blocks, r = total % blocks
     int tile_n;              // columns of a tile: 128, or 192 (wide form)
@@ -592,6 +593,7 @@ struct Seg {
 
 // The launch's work is the sequence (layer, tile, unit of the tile's reduction), units_total long; block b owns
 // units [b U / G, (b + 1) U / G).  Every role of a block walks the same segments with an iterator of its own.
+template <bool kPerExample>
 struct SegIter {
     int pos, end;
     int index;
@@ -610,6 +612,7 @@ struct SegIter {
         const int u0 = pos - tile * upt;
         const int u1 = min(end - tile * upt, upt);
         const int tiles_layer = prm.tiles_x * prm.tiles_y;
+        const bool cut = kPerExample && prm.parts > 0;
         sg.layer = tile / tiles_layer;
         const int rem = tile - sg.layer * tiles_layer;
         const int tile_m = rem / prm.tiles_x, tile_n = rem - tile_m * prm.tiles_x;
@@ -617,10 +620,17 @@ struct SegIter {
         sg.n0 = tile_n * prm.tile_n;
         sg.n_valid = min(prm.tile_n, prm.N - sg.n0);
         sg.n_act = (sg.n_valid + 15) & ~15;
-        sg.s_begin = u0 * prm.unit;
-        sg.s_end = u1 * prm.unit;
-        sg.whole = u0 == 0 && u1 == upt;
-        sg.slot = 2 * (int)blockIdx.x + (index > 0 ? 1 : 0);     // a block's partial segments: its first and / or its last
+        if (cut) {                                               // one part of one example
+            const int z = u0 / prm.parts, part = u0 - z * prm.parts;
+            sg.s_begin = z * prm.p_slices + part * prm.part_slices;
+            sg.s_end = min(sg.s_begin + prm.part_slices, (z + 1) * prm.p_slices);
+        } else {
+            sg.s_begin = u0 * prm.unit;
+            sg.s_end = u1 * prm.unit;
+        }
+        sg.whole = !cut && u0 == 0 && u1 == upt;
+        // a block's partial segments: its first and / or its last; with parts of examples its only one
+        sg.slot = cut ? (int)blockIdx.x : 2 * (int)blockIdx.x + (index > 0 ? 1 : 0);
         pos += u1 - u0;
         ++index;
         return true;
@@ -641,6 +651,8 @@ struct SegIter {
 // 41.6 -> 38.6 us a call, the ResNet-50 pass 1920 -> 1871.
 // kN: columns of a tile, 128 or (wide form) 192.  The wide per-example form keeps the sum of squares in the epilogue's
 // registers: it takes layers whose examples fit one accumulator run (at most kChunk slices).
+// Where examples are cut into parts (Params::parts), kExact writes a part's plain sums and a kernel of its own adds an example's
+// parts up, squares and adds.
 template <int kMajor, int kModeA, int kModeB, bool kATmem, bool kExact = false, bool kBf = false, int kN = kBN>
 __global__ void __launch_bounds__(kThreadsTc, 1)
 sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
@@ -740,7 +752,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
     if (warp == 0) {
         // ================= TMA producer (one thread) =================
         if (lane == 0 && kAnyTma) {
-            SegIter iter(prm);
+            SegIter<kExact> iter(prm);
             Seg sg;
             bool more = iter.next(prm, sg);
             if (!kGatherA) prefetch_map(&bt.a[sg.layer]);
@@ -826,7 +838,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             uint32_t st_phase = 0;
             int c = 0;                                   // running number of the chunk (accumulator buffer c & 1)
             bool ok = true;
-            SegIter iter(prm);
+            SegIter<kExact> iter(prm);
             Seg sg;
             bool more = iter.next(prm, sg);
             for (; ok && more; more = iter.next(prm, sg)) {
@@ -836,7 +848,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 // segment's slices are runs of seg_len slices (whole examples -- the work is cut that way), each cut
                 // into cps chunks
                 const int n_slices = sg.s_end - sg.s_begin;
-                const int seg_len = kExact ? prm.p_slices : n_slices;
+                const int seg_len = kExact && prm.parts == 0 ? prm.p_slices : n_slices;
                 const int cps = (seg_len + prm.chunk - 1) / prm.chunk;
                 const int n_chunks = (n_slices / seg_len) * cps;
                 int i = 0;                               // slice within the segment
@@ -908,7 +920,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         if (lane == 0) {
             int it = 0;
             bool ok = true;
-            SegIter iter(prm);
+            SegIter<kExact> iter(prm);
             Seg sg;
             bool more = iter.next(prm, sg);
             prefetch_map(&bt.b[sg.layer]);
@@ -1156,7 +1168,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         int it0 = 0;                                 // block-wide number of the segment's first slice
         bool ok = true;
         if (!kTwoGroups && t >= kGatherThreads) ok = false;
-        SegIter iter(prm);
+        SegIter<kExact> iter(prm);
         Seg sg;
         bool more = iter.next(prm, sg);
         for (; ok && more; more = iter.next(prm, sg)) {
@@ -1215,14 +1227,15 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
         const uint32_t sq_addr = tmem_base + ((q * 32u) << 16) + kSqCol;  // kExact: this warp's rows of the sum of squares
         int c = 0;                                                        // running number of the chunk
         bool ok = true;
-        SegIter iter(prm);
+        SegIter<kExact> iter(prm);
         Seg sg;
         bool more = iter.next(prm, sg);
         grid_wait();
         for (; ok && more; more = iter.next(prm, sg)) {
 #pragma unroll
             for (int j = 0; j < kN; ++j) acc[j] = 0.f;
-            if (kExact && !kWide) {
+            const bool square = kExact && prm.parts == 0;
+            if (kExact && !kWide && square) {
                 uint32_t zero[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j) zero[j] = 0u;
@@ -1232,7 +1245,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
             }
             const int n_act = sg.n_act, n_valid = sg.n_valid;
             const int n_slices = sg.s_end - sg.s_begin;
-            const int seg_len = kExact ? prm.p_slices : n_slices;
+            const int seg_len = kExact && prm.parts == 0 ? prm.p_slices : n_slices;
             const int cps = (seg_len + prm.chunk - 1) / prm.chunk;
             const int n_chunks = (n_slices / seg_len) * cps;
             for (int cc = 0; cc < n_chunks && ok; ++cc, ++c) {
@@ -1247,17 +1260,19 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                         uint32_t r[32];
                         tc_ld_32x32(taddr + j0, r);
                         tc_wait_ld();
+                        if (kExact && kWide && square) {                // the example's whole sum
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float d = __uint_as_float(r[j]);      // wide per-example form: the example's whole sum
-                            acc[j0 + j] = __fadd_rn(acc[j0 + j], kExact && kWide ? __fmul_rn(d, d) : d);
+                            for (int j = 0; j < 32; ++j) acc[j0 + j] = __fadd_rn(acc[j0 + j], __fmul_rn(__uint_as_float(r[j]), __uint_as_float(r[j])));
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) acc[j0 + j] = __fadd_rn(acc[j0 + j], __uint_as_float(r[j]));
                         }
                     }
                 }
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
-                if (kExact && !kWide && (cc + 1) % cps == 0) {
+                if (kExact && !kWide && square && (cc + 1) % cps == 0) {
                     // end of an example: acc holds its sum over positions; add the squares to the running sum in TMEM
 #pragma unroll
                     for (int j0 = 0; j0 < kN; j0 += 32) {
@@ -1281,7 +1296,7 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
                 }
             }
             if (!ok) break;
-            if (kExact && !kWide) {        // the result is the sum of squares
+            if (kExact && !kWide && square) {        // the result is the sum of squares
 #pragma unroll
                 for (int j0 = 0; j0 < kN; j0 += 32) {
                     uint32_t r[32];
