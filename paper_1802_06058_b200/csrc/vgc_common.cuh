@@ -6,6 +6,7 @@
 
 #include <cstdio>
 #include <cstdlib>
+#include <utility>
 
 #include "vgc.h"
 #include "vgc_once.cuh"
@@ -60,8 +61,13 @@ __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;
 // lets the next kernel of the stream start now, where it was launched with `overlap`
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;"); }
 
+// carveout >= 0: percent of an SM's on-chip memory that shall be shared memory while the kernel runs there, the rest L1.  A kernel
+// that starts under the end of the one ahead otherwise runs with what that one left: behind a kernel that takes all the shared
+// memory, 28 KB of L1, too little for the loads that a streaming kernel keeps in flight.  (It costs small kernels some of the
+// overlap, since an SM changes over only when nothing runs there.)
+struct Carveout { int percent; };
 template <class... Params, class... Given>
-cudaError_t launch_kernel(void (*fn)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap,
+cudaError_t launch_kernel(Carveout carveout, void (*fn)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap,
                           Given &&...given)
 {
     cudaLaunchConfig_t cfg = {};
@@ -69,14 +75,25 @@ cudaError_t launch_kernel(void (*fn)(Params...), dim3 grid, dim3 block, size_t s
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    if (overlap) {
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-    }
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = overlap ? 1 : 0;
+    cfg.numAttrs = 0;
+    if (overlap) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (carveout.percent >= 0) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        attr[cfg.numAttrs++].val.sharedMemCarveout = (unsigned)carveout.percent;
+    }
     return cudaLaunchKernelEx(&cfg, fn, static_cast<Params>(given)...);
+}
+
+template <class... Params, class... Given>
+cudaError_t launch_kernel(void (*fn)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap,
+                          Given &&...given)
+{
+    return launch_kernel(Carveout{-1}, fn, grid, block, smem, st, overlap, std::forward<Given>(given)...);
 }
 
 // Lets a kernel use `bytes` of dynamic shared memory on the current device.  regs > 0: it has to have been compiled to that
@@ -95,20 +112,6 @@ inline cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes, int regs
             if (attr.numRegs != regs) return (int)cudaErrorInvalidKernelImage;
         }
         return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    });
-}
-
-// Asks for `percent` of an SM's on-chip memory to be shared memory while this kernel runs there, the rest L1.  A kernel that
-// starts under the end of the one ahead otherwise runs with what that one left: behind a kernel that takes all the shared
-// memory, 28 KB of L1, too little for the loads that a streaming kernel keeps in flight.
-inline cudaError_t prefer_carveout(const void *kernel, int percent)
-{
-    static OncePerDevice once;
-    int device = -1;
-    const cudaError_t e = cudaGetDevice(&device);
-    if (e != cudaSuccess) return e;
-    return (cudaError_t)once(kernel, device, [&]() -> int {
-        return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent);
     });
 }
 

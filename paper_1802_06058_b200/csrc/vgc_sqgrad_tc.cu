@@ -332,8 +332,7 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
         for (int l = 0; l < n_layers; ++l) results.S[l] = bt.S[l];
         if (plan.parts) {
             const int slot_n = slot_columns(tile_n);
-            VGC_CUDA_OK(prefer_carveout(reinterpret_cast<const void *>(sqgrad_tc_combine_examples), 18));
-            VGC_CUDA_OK(launch_kernel(sqgrad_tc_combine_examples, dim3((unsigned)(plan.tiles_x * plan.tiles_y * slot_n), (unsigned)n_layers), dim3(256), 0,
+            VGC_CUDA_OK(launch_kernel(Carveout{18}, sqgrad_tc_combine_examples, dim3((unsigned)(plan.tiles_x * plan.tiles_y * slot_n), (unsigned)n_layers), dim3(256), 0,
                                       st, true, prm.partial, k_slices / prm.p_slices, plan.parts, tile_n, slot_n, plan.tiles_x, plan.tiles_y, M, N,
                                       prm.scale, prm.accumulate, results, prm.ld_m, prm.ld_n));
             count_launch();
@@ -347,8 +346,7 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
         const auto combine = many ? sqgrad_tc_combine_many : sqgrad_tc_combine;
         // L1 for the loads of eight blocks (34 KB of shared memory) behind the kernel above, which takes all shared memory;
         // with the same for sqgrad_repack, a pass over ResNet-50, batch 32, takes 1853 us instead of 1880
-        VGC_CUDA_OK(prefer_carveout(reinterpret_cast<const void *>(combine), 18));
-        VGC_CUDA_OK(launch_kernel(combine, dim3(patches, (unsigned)n_layers), dim3(256), 0, st,
+        VGC_CUDA_OK(launch_kernel(Carveout{18}, combine, dim3(patches, (unsigned)n_layers), dim3(256), 0, st,
                                   true, prm.partial, prm.units_q, prm.units_r, plan.units_per_tile, tile_n, slot_n, plan.tiles_x, plan.tiles_y, M, N,
                                   prm.scale, prm.accumulate, results, prm.ld_m, prm.ld_n));
         count_launch();
@@ -418,6 +416,8 @@ static int repack_mode(int B, int C, int Cout, int Kh, int Kw, int sh, int sw, i
     if (t_exact) return kRepackNone;                 // the flat form merges the examples' positions
     return (flat >= kBK && flat % 4 == 0 && flat < (1L << 30)) ? kRepackFlat : kRepackNone;
 }
+
+constexpr Carveout kAllL1{5};       // sqgrad_repack has no shared memory
 
 // One tensor to repack: out[a][b][p] = in[z][c][(p / Wo) sh W + (p % Wo) sw], zero where p % Wo >= wo_valid, with
 // (a, b) = (z, c), or (c, z) when channel_major.  All tensors of a layer group go into one launch.
@@ -555,7 +555,6 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
 {
     const int P = Ho * Wo, n_im2col = C * Kh * Kw;
     const int mode = repack_mode(B, C, Cout, Kh, Kw, sh, sw, ph, pw, P, W, Ho, Wo);
-    if (mode != kRepackNone) VGC_CUDA_OK(prefer_carveout(reinterpret_cast<const void *>(sqgrad_repack), 5));      // no shared memory: all L1
     // one run of the output per warp; more when there are many
     auto blocks_for = [](size_t values) { const size_t b = (values + 8 * kRepackRun - 1) / (8 * kRepackRun); return (unsigned)(b < 1 ? 1 : (b > 148 * 32 ? 148 * 32 : b)); };
     if (mode == kRepackPadW) {
@@ -574,7 +573,7 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
             jobs.job[2 * l + 1] = RepackJob{delta[l], d_p, Cout, Ho * Wo, Wo, Wo4, Ho * Wo4, 1, 1, 0, Wo};
             xr[l] = x_p; dr[l] = d_p;
         }
-        VGC_CUDA_OK(launch_kernel(sqgrad_repack, dim3(blocks_for((size_t)B * ((size_t)C * H * Wx > (size_t)Cout * Ho * Wo4 ? (size_t)C * H * Wx : (size_t)Cout * Ho * Wo4)), 2 * n_layers), dim3(256), 0, st, true, jobs));
+        VGC_CUDA_OK(launch_kernel(kAllL1, sqgrad_repack, dim3(blocks_for((size_t)B * ((size_t)C * H * Wx > (size_t)Cout * Ho * Wo4 ? (size_t)C * H * Wx : (size_t)Cout * Ho * Wo4)), 2 * n_layers), dim3(256), 0, st, true, jobs));
         count_launch();
         return conv_group(n_layers, xr, dr, S, B, C, H, Wx, Cout, Kh, Kw, sh, sw, ph, 1, Ho, Wo4, scale, accumulate, ws, inner, st);
     }
@@ -597,7 +596,7 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
             xr[l] = x_r;
             dr[l] = flat ? d_r : delta[l];
         }
-        VGC_CUDA_OK(launch_kernel(sqgrad_repack, dim3(blocks_for((size_t)B * (flat && Cout > C ? Cout : C) * P), n_jobs), dim3(256), 0, st, true, jobs));
+        VGC_CUDA_OK(launch_kernel(kAllL1, sqgrad_repack, dim3(blocks_for((size_t)B * (flat && Cout > C ? Cout : C) * P), n_jobs), dim3(256), 0, st, true, jobs));
         count_launch();
         if (flat)
             return conv_group(n_layers, xr, dr, S, 1, C, B * P, 1, Cout, 1, 1, 1, 1, 0, 0, B * P, 1, scale, accumulate, ws,

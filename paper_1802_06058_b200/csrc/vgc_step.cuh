@@ -568,6 +568,10 @@ encode_step(const __grid_constant__ Args a)
     }
 }
 
+// Buffers from which on the streaming kernel asks for L1.  Steps of one dense layer, 60 examples, without / with, us: 131 thousand
+// parameters 12.9 / 13.9, 262 and 524 thousand the same, 1.05 M 19.4 / 19.0 (added to v 19.4 / 19.6), 2.1 M 25.4 / 23.6, 8.4 M 69.0 / 58.8.
+constexpr size_t kCarveLeast = 1 << 20;
+
 // Enqueues one step.  a: everything but the ranges; records: kRecordBytes, 16-byte aligned.
 template <bool kHasS, int kAlgorithm>
 vgc_status launch(Args a, void *records, cudaStream_t st)
@@ -585,8 +589,8 @@ vgc_status launch(Args a, void *records, cudaStream_t st)
     // Two blocks' 26 KB, the rest L1: 1024 threads with eight 16-byte loads each.  Behind a dense layer's kernel without it (119.6 M
     // parameters, B200): 531 us for this kernel, 383 with it.  Not the hybrid, which asks for next to no shared memory and would
     // rather start under a decoder (25 M, 8 messages: 129.7 us a step, 131.1 with it).
-    if (kAlgorithm == kBasic) VGC_CUDA_OK(prefer_carveout(reinterpret_cast<const void *>(compress_step<kHasS, kAlgorithm>), 15));
-    VGC_CUDA_OK(launch_kernel(compress_step<kHasS, kAlgorithm>, grid, dim3(kThreads), 0, st, true, a));
+    const Carveout carveout{kAlgorithm == kBasic && a.n >= kCarveLeast ? 15 : -1};
+    VGC_CUDA_OK(launch_kernel(carveout, compress_step<kHasS, kAlgorithm>, grid, dim3(kThreads), 0, st, true, a));
     VGC_CUDA_OK(launch_kernel(encode_step<kAlgorithm == kBasic>, grid, dim3(kThreads), 0, st, true, a));
     count_launch(2);
     return VGC_OK;
