@@ -6,9 +6,10 @@
 // (64 KB more to read when it is added to what is there).  The general kernel drains a tile through registers into
 // row-by-row accesses of global memory, 17 us a tile for 64 examples; here the tile leaves (and the old one arrives) by TMA:
 //   warp 0       one thread: TMA loads of the operand slices (A plain, B MN-major with the 128-byte swizzle of 32-byte units)
-//   warp 1       one thread: 12 tcgen05.mma per slice (3xTF32: hi hi + hi lo + lo hi, A from tensor memory)
+//   warp 1       one thread: 12 tcgen05.mma per slice (3xTF32: hi hi + hi lo + lo hi, A from tensor memory), or 8 (hi lo and lo hi
+//                with bf16 copies)
 //   warps 2-9    square and split, two groups of four on alternate slices: A into tensor memory (a lane per row: 32 loads of
-//                neighbouring floats), B in place with its lo part beside it
+//                neighbouring floats), B in place with its lo part (or bf16 copies of both parts) beside it
 //   the others   epilogue: 32 x 32 boxes, one accumulator row per lane, through a shared-memory buffer of their own; the
 //                box's old contents were loaded by TMA while the tile before was written, the result is stored by TMA
 // An accumulator takes at most 8 slices (96 instructions: the bias of the tensor core's truncating accumulation is about
@@ -31,12 +32,13 @@ constexpr int kRawSlots = 3, kLoSlots = 4;           // [A raw][B raw / hi]; [B 
 constexpr int kTransformWarps = 8;
 constexpr uint32_t kTileBytes = kBM * kBK * 4;                      // 16 KB: one operand of one slice
 constexpr uint32_t kStageBytes = 2 * kTileBytes;
+constexpr uint32_t kBfBytes = kTileBytes / 2;                       // a bf16 copy of B; a lo slot takes two, [hi][lo]
 constexpr uint32_t kLoBase = kRawSlots * kStageBytes;
 constexpr uint32_t kBoxBase = kLoBase + kLoSlots * kTileBytes;
 constexpr uint32_t kBoxBytes = 32 * 32 * 4;
 constexpr uint32_t kSmemBytes = kBoxBase + kBM * kBN * 4 + 1024 /*align*/;
 constexpr int kAccumulators = 2, kChunk = 8;                         // slices per accumulator
-constexpr uint32_t kTmemA = kAccumulators * kBN, kTmemColsA = 64;    // A slots: 32 columns hi, 32 columns lo
+constexpr uint32_t kTmemA = kAccumulators * kBN, kTmemColsA = 64;    // A slots: 32 columns hi, 32 columns lo (16 hi as bf16, 16 lo as bf16)
 constexpr uint32_t kTmemCols = kTmemA + kLoSlots * kTmemColsA;
 static_assert(kTmemCols == 512, "tensor memory");
 // Epilogue warps: with eight (two halves of the columns per lane quarter) a written tile leaves sooner (4096 x 4096, 16
@@ -47,6 +49,14 @@ template <bool kAccumulate, int kN> struct Shape {
     static constexpr int kHalves = kAccumulate ? 1 : 2, kEpilogueWarps = 4 * kHalves, kBoxes = kN / 32 / kHalves;
     static constexpr int kThreads = 32 * (2 + kTransformWarps + kEpilogueWarps);
 };
+
+// Where the bf16 copy of the raw tile's i-th 16 bytes goes.  Raw: boxes of 32 columns, 128 bytes a row k, whose 32-byte units were put
+// in place unit ^ (k & 3).  Copy: blocks of 64 columns, 128 bytes a row, 16-byte units in place unit ^ (k & 7).
+__device__ __forceinline__ uint32_t bf_place(uint32_t i)
+{
+    const uint32_t k = (i >> 3) & 31u, n = 32 * (i >> 8) + 8 * (((i >> 1) ^ k) & 3u) + 4 * (i & 1u);
+    return (n >> 6) * 4096u + k * 128u + (((n >> 3) ^ k) & 7u) * 16u + (n & 4u) * 2u;
+}
 
 struct Params {
     int k_slices, tiles, tiles_x;
@@ -67,7 +77,12 @@ __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.w
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // kFew: fewer than 32 examples (see the epilogue; the check costs an added layer 6 %, so it is compiled for these only)
-template <bool kAccumulate, int kN, bool kFew>
+// kBf: the two cross terms take bf16 copies of hi and lo, 16 deep an instruction: a third fewer instructions and so less of the
+// accumulator's bias, but their rounding shows in sums of few terms (largest error of 1024 x 1024 sums, 64 examples: 1.7e-6 in
+// tf32, 2.9e-6 with bf16; 192: 3.4e-6, 3.3e-6; 512: 3.6e-6, 3.0e-6), hence from kBfLeast examples on (512 examples, 2048 x 2048:
+// 27.9 -> 26.0 us; 256 examples, 1024 x 1024: 9.4 -> 8.7).
+constexpr int kBfLeast = 192;
+template <bool kAccumulate, int kN, bool kFew, bool kBf>
 __global__ void __launch_bounds__(Shape<kAccumulate, kN>::kThreads, 1)
 sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
              const __grid_constant__ CUtensorMap map_s, const Params prm)
@@ -113,6 +128,7 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_slot;
+    if (threadIdx.x == 0) { prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_s); }
     grid_wait();
 
     const int k_slices = prm.k_slices, step = (int)gridDim.x, first_tile = (int)blockIdx.x;
@@ -147,6 +163,10 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
             const uint32_t desc_lo0 = (uint32_t)smem_desc(0, 4096u, 512u, 1u);
             auto desc_at = [&](uint32_t lo16) -> uint64_t { return ((uint64_t)desc_hi << 32) | (desc_lo0 + lo16); };
             const uint32_t idesc = instr_desc(kMajorK, kN, kBM) | (1u << 16);        // A K-major (tensor memory), B MN-major
+            // the bf16 copies: 64-wide column blocks 4096 B apart (LBO), 8-deep k groups 1024 B apart (SBO), 128-byte swizzle
+            const uint32_t bf_hi = (uint32_t)(smem_desc(0, 4096u, 1024u, 2u) >> 32), bf_lo0 = (uint32_t)smem_desc(0, 4096u, 1024u, 2u);
+            auto desc_bf = [&](uint32_t lo16) -> uint64_t { return ((uint64_t)bf_hi << 32) | (bf_lo0 + lo16); };
+            const uint32_t idesc_bf = instr_desc_bf16(kN, kBM) | (1u << 16);
             int it = 0, c = 0;                           // running numbers of the slice and of the chunk
             bool ok = true;
             for (int t = first_tile; ok && t < prm.tiles; t += step) {
@@ -170,8 +190,14 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                             const uint64_t db_hi = desc_at(hi_b + kk * 64), db_lo = desc_at(lo_b + kk * 64);
                             if (kk == 0) tc_mma_tf32_ts(d_tmem, ta, db_hi, idesc, s == s0 ? 0u : 1u);
                             else tc_mma_tf32_ts_acc(d_tmem, ta + kk * 8, db_hi, idesc);
+                            if (kBf) continue;
                             tc_mma_tf32_ts_acc(d_tmem, ta + kk * 8, db_lo, idesc);
                             tc_mma_tf32_ts_acc(d_tmem, ta + 32 + kk * 8, db_hi, idesc);
+                        }
+#pragma unroll
+                        for (int kk = 0; kk < (kBf ? kBK / 16 : 0); ++kk) {
+                            tc_mma_bf16_ts_acc(d_tmem, ta + 32 + kk * 8, desc_bf(lo_b + (kBfBytes >> 4) + kk * 128), idesc_bf);
+                            tc_mma_bf16_ts_acc(d_tmem, ta + 48 + kk * 8, desc_bf(lo_b + kk * 128), idesc_bf);
                         }
                         tc_commit(smem_u32(&empty[st]));
                     }
@@ -213,7 +239,15 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                     l[k] = __float_as_uint(__fsub_rn(sq, __uint_as_float(h[k])));
                 }
                 tc_st_32x16(ta + k0, h);
-                tc_st_32x16(ta + 32 + k0, l);
+                if (!kBf) { tc_st_32x16(ta + 32 + k0, l); continue; }
+                uint32_t hb[8], lb[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    hb[k] = pack_bf16(__uint_as_float(h[2 * k]), __uint_as_float(h[2 * k + 1]));
+                    lb[k] = pack_bf16(__uint_as_float(l[2 * k]), __uint_as_float(l[2 * k + 1]));
+                }
+                tc_st_32x8(ta + 32 + k0 / 2, hb);
+                tc_st_32x8(ta + 48 + k0 / 2, lb);
             }
             uint8_t *hi = smem_gen + (uint32_t)st * kStageBytes + kTileBytes, *lo = smem_gen + kLoBase + (uint32_t)ls * kTileBytes;
 #pragma unroll
@@ -222,7 +256,22 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
 #pragma unroll
                 for (int u = 0; u < 4; ++u) v[u] = *reinterpret_cast<const float4 *>(hi + 16 * (tt + (u0 + u) * 128));
 #pragma unroll
-                for (int u = 0; u < 4; ++u) split_store<true>(hi, lo, 16 * (uint32_t)(tt + (u0 + u) * 128), v[u].x, v[u].y, v[u].z, v[u].w);
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t i = (uint32_t)(tt + (u0 + u) * 128);
+                    if (!kBf) { split_store<true>(hi, lo, 16 * i, v[u].x, v[u].y, v[u].z, v[u].w); continue; }
+                    const float e[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+                    uint32_t h[4], l[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float sq = __fmul_rn(e[j], e[j]);
+                        h[j] = to_tf32(sq);
+                        l[j] = __float_as_uint(__fsub_rn(sq, __uint_as_float(h[j])));
+                    }
+                    *reinterpret_cast<uint4 *>(hi + 16 * i) = make_uint4(h[0], h[1], h[2], h[3]);
+                    uint8_t *const bf = lo + bf_place(i);
+                    *reinterpret_cast<uint2 *>(bf) = make_uint2(pack_bf16(__uint_as_float(h[0]), __uint_as_float(h[1])), pack_bf16(__uint_as_float(h[2]), __uint_as_float(h[3])));
+                    *reinterpret_cast<uint2 *>(bf + kBfBytes) = make_uint2(pack_bf16(__uint_as_float(l[0]), __uint_as_float(l[1])), pack_bf16(__uint_as_float(l[2]), __uint_as_float(l[3])));
+                }
             }
             tc_wait_st();
             tc_fence_before();
@@ -381,12 +430,14 @@ vgc_status dense_sqgrad_linear(const float *x, const float *delta, int B, int in
     const long long rows_m = (out + kBM - 1) / kBM;
     const bool narrow = rows_m * ((in + kBN - 1) / kBN) <= 74;
     const int tile_n = narrow ? 64 : kBN;
-    auto pick = [&](auto few) {
-        constexpr bool kFew = decltype(few)::value;
-        return accumulate ? (narrow ? sqgrad_dense<true, 64, kFew> : sqgrad_dense<true, kBN, kFew>)
-                          : (narrow ? sqgrad_dense<false, 64, kFew> : sqgrad_dense<false, kBN, kFew>);
+    auto pick = [&](auto few, auto bf) {
+        constexpr bool kFew = decltype(few)::value, kBf = decltype(bf)::value;
+        return accumulate ? (narrow ? sqgrad_dense<true, 64, kFew, kBf> : sqgrad_dense<true, kBN, kFew, kBf>)
+                          : (narrow ? sqgrad_dense<false, 64, kFew, kBf> : sqgrad_dense<false, kBN, kFew, kBf>);
     };
-    auto fn = B < 32 ? pick(std::true_type()) : pick(std::false_type());
+    const std::true_type yes;
+    const std::false_type no;
+    auto fn = B < 32 ? pick(yes, no) : B < kBfLeast ? pick(no, no) : pick(no, yes);
     VGC_CUDA_OK(allow_dynamic_smem(reinterpret_cast<const void *>(fn), kSmemBytes));
     Params prm;
     prm.k_slices = (B + kBK - 1) / kBK;

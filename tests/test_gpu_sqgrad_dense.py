@@ -60,3 +60,21 @@ def test_added_is_one_fp32_addition(B, n_in, n_out):
     want = T + S
     vgc.vgc_sqgrad_linear(x, d, 1.0 / B, T, accumulate=True, ws=ws)
     assert torch.equal(T, want)
+
+
+@pytest.mark.parametrize("B", [191, 192, 193, 224, 257, 512])
+@pytest.mark.parametrize("n_in,n_out", [(1024, 1024), (1000, 132), (4096, 1300), (132, 2052)])
+def test_cross_terms_in_bf16(B, n_in, n_out):
+    """Around the number of examples from which the two cross terms take bf16 copies (each a 2^-11 of the product, the copies good
+    to 2^-9 of it): narrow and full tiles, edges of tiles and slices.  Bound 1e-5 of every entry, all of whose terms are positive."""
+    gen = torch.Generator("cuda").manual_seed(B + n_in)
+    x = torch.randn(B, n_in, device="cuda", generator=gen)
+    d = torch.randn(B, n_out, device="cuda", generator=gen) * 1e-3
+    ws = torch.zeros(max(256, vgc.vgc_sqgrad_linear_workspace_bytes(B, n_in, n_out)), dtype=torch.uint8, device="cuda")
+    want = (d.double().square().t() @ x.double().square()) * 0.5
+    for accumulate in (False, True):
+        S = torch.rand(n_out, n_in, device="cuda", generator=gen) * 1e-4 if accumulate else torch.full((n_out, n_in), -1.0, device="cuda")
+        full = want + S.double() if accumulate else want
+        vgc.vgc_sqgrad_linear(x, d, 0.5, S, accumulate, ws)
+        assert int(ws[:4].view(torch.int32)) == 0
+        assert float(((S.double() - full).abs() / full).max()) < 1e-5
