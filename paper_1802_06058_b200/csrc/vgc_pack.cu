@@ -11,14 +11,15 @@
 // side: one warp per run.
 //
 //   pack:   pack_count   every lane sizes 8 consecutive words of its warp's run; the totals of chunks of 8 runs are stored
-//           pack_emit    starts under pack_count with its words; a block adds up the totals of the chunks before its own (no
-//                        waiting on other blocks), codes its words into shared memory at the alignment they will have in
-//                        the stream, and its bytes leave as whole words
+//           pack_emit    starts under pack_count and codes its words into shared memory; then a block adds up the totals of the
+//                        chunks before its own (no waiting on other blocks), and its bytes leave as whole words, shifted to the
+//                        alignment they have in the stream
 //   unpack: one kernel   a warp brings its run's bytes into shared memory, 4 at a time; a byte with a clear top bit ends a
 //                        number: a warp scan of their counts gives every end its place, every lane reads the 8 numbers
 //                        between its ends, and a second scan over the differences gives the indices
 // Bound: latency (launch, the counter, the table, the bytes follow one another).  Measured (B200, 765 thousand words, 2 bytes
-// each): pack and unpack together 28.7 us byte by byte (31 M warp instructions), 15.2 now.
+// each): pack and unpack together 28.7 us byte by byte (31 M warp instructions), 13.6 with whole words, 12.9 with the code written
+// before the wait.
 #include "vgc_common.cuh"
 
 namespace vgc {
@@ -98,7 +99,7 @@ __global__ void __launch_bounds__(kPackThreads, 6)
 pack_emit(const uint32_t *words, const uint32_t *nnz, uint32_t max_words,
           const uint32_t *chunk_bytes, uint8_t *packed, size_t capacity, uint32_t *packed_bytes, uint32_t *dev_status)
 {
-    __shared__ __align__(16) uint8_t sm_bytes[kPackWarps * kRunBytesMax + 16];
+    __shared__ uint32_t sm_code[kPackWarps * kRunBytesMax / 4 + 1];     // (and a word to read past)
     __shared__ unsigned long long sm_part[kPackWarps];
     __shared__ uint32_t sm_run[kPackWarps];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -106,48 +107,21 @@ pack_emit(const uint32_t *words, const uint32_t *nnz, uint32_t max_words,
     const uint32_t n = min(*nnz, max_words);
     const uint32_t runs = (n + kPackRun - 1) / kPackRun;
     const size_t table_bytes = 4 * ((size_t)runs + 1);
-    uint32_t v[kPerLane], mine = 0, have = 0;
-    if (blockIdx.x * kPackWarps <= runs) have = lane_numbers(words, n, blockIdx.x * kPackWarps + warp, lane, v, mine);
-    grid_wait();                                                        // pack_count's totals
-    unsigned long long before = 0;                                      // payload bytes of all chunks before this one
-    uint32_t summed = 0;                                                // chunks summed so far
-    // one chunk more than the runs need: the warp that writes table[runs]
-    for (uint32_t chunk = blockIdx.x; chunk * kPackWarps <= runs; chunk += gridDim.x) {
-        if (chunk != blockIdx.x) {
-            __syncthreads();                                            // the chunk before has left shared memory
-            have = lane_numbers(words, n, chunk * kPackWarps + warp, lane, v, mine);
-        }
-        unsigned long long more = 0;
-        for (uint32_t b = summed + threadIdx.x; b < chunk; b += kPackThreads) more += __ldcg(chunk_bytes + b);
-        summed = chunk;
-        more = warp_sum_u64(more);
-        const uint32_t run = chunk * kPackWarps + warp;
+    // a chunk's code in shared memory, from its first byte on: all of it before the wait where the chunk is the block's first
+    uint32_t in_chunk = 0, chunk_total = 0;
+    auto code = [&](uint32_t chunk) {
+        uint32_t v[kPerLane], mine;
+        const uint32_t have = lane_numbers(words, n, chunk * kPackWarps + warp, lane, v, mine);
         const uint32_t incl = warp_inclusive(mine, lane);
         if (lane == 31) sm_run[warp] = incl;
-        if (lane == 0) sm_part[warp] = more;
         __syncthreads();
-        uint32_t in_chunk = 0, chunk_total = 0;
+        in_chunk = chunk_total = 0;
 #pragma unroll
         for (int w = 0; w < kPackWarps; ++w) {
-            before += sm_part[w];
             in_chunk += (uint32_t)w < warp ? sm_run[w] : 0u;
             chunk_total += sm_run[w];
         }
-        const unsigned long long run_off = before + in_chunk;           // this run's first byte inside the payload
-        if (run <= runs && lane < 4) {                                  // table[run]
-            const size_t at = 4 * (size_t)run + lane;
-            if (at < capacity) packed[at] = (uint8_t)((uint32_t)run_off >> (8 * lane));
-        }
-        if (run == runs && lane == 0) {
-            // table[runs] is the payload length: written by the warp whose run number is `runs` (its offset is the total)
-            const unsigned long long total = table_bytes + run_off;
-            *packed_bytes = (uint32_t)total;
-            if (total > capacity) atomicOr(dev_status, VGC_DEV_CAPACITY);
-        }
-        // the chunk's bytes in shared memory, at the alignment they will have in the stream
-        const size_t dst0 = table_bytes + before;                       // of the chunk's first byte
-        const uint32_t skew = (uint32_t)((reinterpret_cast<uintptr_t>(packed) + dst0) & 3u);
-        uint8_t *at = sm_bytes + skew + in_chunk + (incl - mine);
+        uint8_t *at = reinterpret_cast<uint8_t *>(sm_code) + in_chunk + (incl - mine);
 #pragma unroll
         for (int j = 0; j < kPerLane; ++j) {
             if ((uint32_t)j < have) {
@@ -160,16 +134,49 @@ pack_emit(const uint32_t *words, const uint32_t *nnz, uint32_t max_words,
                 at += len;
             }
         }
+    };
+    if (blockIdx.x * kPackWarps <= runs) code(blockIdx.x);
+    grid_wait();                                                        // pack_count's totals
+    unsigned long long before = 0;                                      // payload bytes of all chunks before this one
+    uint32_t summed = 0;                                                // chunks summed so far
+    // one chunk more than the runs need: the warp that writes table[runs]
+    for (uint32_t chunk = blockIdx.x; chunk * kPackWarps <= runs; chunk += gridDim.x) {
+        if (chunk != blockIdx.x) {
+            __syncthreads();                                            // the chunk before has left shared memory
+            code(chunk);
+        }
+        unsigned long long more = 0;
+        for (uint32_t b = summed + threadIdx.x; b < chunk; b += kPackThreads) more += __ldcg(chunk_bytes + b);
+        summed = chunk;
+        more = warp_sum_u64(more);
+        const uint32_t run = chunk * kPackWarps + warp;
+        if (lane == 0) sm_part[warp] = more;
         __syncthreads();
-        // whole words of the stream; the first and last one, which neighbouring chunks share, byte by byte
-        const uint32_t span = skew + chunk_total;
+#pragma unroll
+        for (int w = 0; w < kPackWarps; ++w) before += sm_part[w];
+        const unsigned long long run_off = before + in_chunk;           // this run's first byte inside the payload
+        if (run <= runs && lane < 4) {                                  // table[run]
+            const size_t at = 4 * (size_t)run + lane;
+            if (at < capacity) packed[at] = (uint8_t)((uint32_t)run_off >> (8 * lane));
+        }
+        if (run == runs && lane == 0) {
+            // table[runs] is the payload length: written by the warp whose run number is `runs` (its offset is the total)
+            const unsigned long long total = table_bytes + run_off;
+            *packed_bytes = (uint32_t)total;
+            if (total > capacity) atomicOr(dev_status, VGC_DEV_CAPACITY);
+        }
+        // whole words of the stream, each out of two of the chunk's; the first and last one, which neighbouring chunks share,
+        // byte by byte
+        const size_t dst0 = table_bytes + before;                       // of the chunk's first byte
+        const uint32_t skew = (uint32_t)((reinterpret_cast<uintptr_t>(packed) + dst0) & 3u), span = skew + chunk_total;
         uint8_t *const base = packed + dst0 - skew;                     // 4-byte aligned
         for (uint32_t i = 4 * threadIdx.x; i < span; i += 4 * kPackThreads) {
             if (i >= skew && i + 4 <= span && dst0 - skew + i + 4 <= capacity) {
-                *reinterpret_cast<uint32_t *>(base + i) = *reinterpret_cast<const uint32_t *>(sm_bytes + i);
+                const uint32_t *const from = sm_code + ((i - skew) >> 2);
+                *reinterpret_cast<uint32_t *>(base + i) = __funnelshift_r(from[0], from[1], 8 * ((i - skew) & 3u));
             } else {
                 for (uint32_t b = i < skew ? skew : i; b < i + 4 && b < span; ++b)
-                    if (dst0 - skew + b < capacity) base[b] = sm_bytes[b];
+                    if (dst0 - skew + b < capacity) base[b] = reinterpret_cast<const uint8_t *>(sm_code)[b - skew];
             }
         }
     }

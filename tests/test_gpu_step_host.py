@@ -119,3 +119,35 @@ def test_threads():
     for t in threads:
         t.join()
     assert not failed, failed[0]
+
+
+@pytest.mark.parametrize("sizes,pinned,shift", [([(1024, 512), (256, 12)], "both", 0), ([(1024, 512), (256, 12)], "both", 1),
+                                                ([(1024, 512), (256, 12)], "words", 0), ([(2048, 1024), (64, 12)], "both", 0)])
+def test_message_goes_home_by_a_kernel_or_by_copies(sizes, pinned, shift):
+    """Page-locked results (written by a kernel up to 2^18 words), at an odd place, the counters in ordinary memory, a longer message."""
+    specs = [workloads.LayerSpec(f"fc{i}", "fc", a, b) for i, (a, b) in enumerate(sizes)]
+    offs = workloads.group_offsets(specs)
+    n, K = int(offs[-1]), len(specs)
+    ins = [workloads.layer_inputs(sp, B, 1, 0, 5, i, "relu_normal", 1e-3, "cuda") for i, sp in enumerate(specs)]
+    g = torch.cat([workloads.mean_gradient(sp, x, d) for sp, (x, d) in zip(specs, ins)])
+    ws = torch.zeros(max(vgc.vgc_sqgrad_linear_workspace_bytes(B, sp.cin, sp.cout) for sp in specs) + 256, dtype=torch.uint8, device="cuda")
+    wc = torch.empty(vgc.vgc_compress_workspace_bytes(n, K), dtype=torch.uint8, device="cuda")
+    s, r, v = (torch.zeros(n, device="cuda") for _ in range(3))
+    for (x, d), lo, hi in zip(ins, offs[:-1].tolist(), offs[1:].tolist()):
+        vgc.vgc_sqgrad_linear(x, d, 1.0 / B ** 2, s[lo:hi], ws=ws)
+    out = vgc.MessageBuffers(n, K, n)
+    vgc.vgc_compress(g, s, r, v, vgc.offsets_tensor(offs), 2.0, 0.999, out, wc)
+    want = out.read()
+    assert (want["nnz"] > 1 << 18) == (sizes[0][0] == 2048)
+    layers = [{"is_conv": 0, "B": B, "C": x.shape[1], "Cout": d.shape[1], "x_host": x.cpu().pin_memory(), "delta_host": d.cpu().pin_memory(),
+               "x_dev": torch.empty_like(x), "delta_dev": torch.empty_like(d)} for x, d in ins]
+    words = torch.full((n + 8,), -1, dtype=torch.int32).pin_memory()[shift:]
+    counters = torch.zeros(4, dtype=torch.int32)
+    if pinned == "both":
+        counters = counters.pin_memory()
+    out2 = vgc.MessageBuffers(n, K, n)
+    got = vgc.vgc_step_host(layers, g.cpu().pin_memory(), torch.empty_like(g), torch.empty_like(s), torch.zeros_like(r), torch.zeros_like(v),
+                            vgc.offsets_tensor(offs), 2.0, 0.999, 1.0 / B ** 2, out2, words, counters, ws, wc)
+    assert got == (want["nnz"], want["n_criterion"], want["n_dropped"], 0)
+    assert np.array_equal(words[:want["nnz"]].numpy().view(np.uint32), want["words"])
+    assert bool((words[want["nnz"]:] == -1).all())
