@@ -194,10 +194,12 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                             tc_mma_tf32_ts_acc(d_tmem, ta + kk * 8, db_lo, idesc);
                             tc_mma_tf32_ts_acc(d_tmem, ta + 32 + kk * 8, db_hi, idesc);
                         }
+                        if constexpr (kBf) {
 #pragma unroll
-                        for (int kk = 0; kk < (kBf ? kBK / 16 : 0); ++kk) {
-                            tc_mma_bf16_ts_acc(d_tmem, ta + 32 + kk * 8, desc_bf(lo_b + (kBfBytes >> 4) + kk * 128), idesc_bf);
-                            tc_mma_bf16_ts_acc(d_tmem, ta + 48 + kk * 8, desc_bf(lo_b + kk * 128), idesc_bf);
+                            for (int kk = 0; kk < kBK / 16; ++kk) {
+                                tc_mma_bf16_ts_acc(d_tmem, ta + 32 + kk * 8, desc_bf(lo_b + (kBfBytes >> 4) + kk * 128), idesc_bf);
+                                tc_mma_bf16_ts_acc(d_tmem, ta + 48 + kk * 8, desc_bf(lo_b + kk * 128), idesc_bf);
+                            }
                         }
                         tc_commit(smem_u32(&empty[st]));
                     }
@@ -239,15 +241,18 @@ sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ 
                     l[k] = __float_as_uint(__fsub_rn(sq, __uint_as_float(h[k])));
                 }
                 tc_st_32x16(ta + k0, h);
-                if (!kBf) { tc_st_32x16(ta + 32 + k0, l); continue; }
-                uint32_t hb[8], lb[8];
+                if constexpr (kBf) {
+                    uint32_t hb[8], lb[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    hb[k] = pack_bf16(__uint_as_float(h[2 * k]), __uint_as_float(h[2 * k + 1]));
-                    lb[k] = pack_bf16(__uint_as_float(l[2 * k]), __uint_as_float(l[2 * k + 1]));
+                    for (int k = 0; k < 8; ++k) {
+                        hb[k] = pack_bf16(__uint_as_float(h[2 * k]), __uint_as_float(h[2 * k + 1]));
+                        lb[k] = pack_bf16(__uint_as_float(l[2 * k]), __uint_as_float(l[2 * k + 1]));
+                    }
+                    tc_st_32x8(ta + 32 + k0 / 2, hb);
+                    tc_st_32x8(ta + 48 + k0 / 2, lb);
+                } else {
+                    tc_st_32x16(ta + 32 + k0, l);
                 }
-                tc_st_32x8(ta + 32 + k0 / 2, hb);
-                tc_st_32x8(ta + 48 + k0 / 2, lb);
             }
             uint8_t *hi = smem_gen + (uint32_t)st * kStageBytes + kTileBytes, *lo = smem_gen + kLoBase + (uint32_t)ls * kTileBytes;
 #pragma unroll
