@@ -82,15 +82,28 @@ __device__ __forceinline__ float value_of(uint32_t word, const int32_t *gexp, co
 // lies in one stretch of u: DRAM pages are opened once for the words of all of them.  Shorter messages make groups of their
 // own, so that a piece is at least about half full whatever the lengths (one group for all took 4.5 ms for 64
 // messages into 138 M elements, one of 6.9 M words and the others empty; now 127 us).
-// Two blocks per SM: with four the stretch doubles, and 8.9 M words into 138 M elements take 267 us instead of 172.
-constexpr int kFlatThreads = 256, kFlatBlocksPerSm = 2, kPiece = 32;
+// Warps: one block's per SM where there is less than one word per 40 elements of a large buffer, but words enough that what they
+// touch does not stay in L2 (16 M elements, 0.35 M words: 11.7 us with one block per SM, 7.3 with two; 138 M, 0.22 M words: 6.4, 4.6; 68 M,
+// 1.5 M: 51.9, 50.0; 100 M, 1.9 M: 69.0, 72.2; 138 M, 0.9 M: 40.7, 43.1), two and a half blocks' otherwise -- DRAM is what
+// bounds it (a touched 64 bytes is read, and read again and written when its half-filled line leaves L2), more in flight only
+// widens the stretch.  138 M elements, us, with 1 / 2 / 2.5 / 3 / 4 blocks per SM: 64 messages, 2.7 M words 95 / 103 / 103 / 103 / 102,
+// 8.9 M words 230 / 173 / 172 / 223 / 271; 4 messages, 11 M words 272 / 189 / 175 / 170 / 200; 32 M elements, 7 messages, 2 M words
+// 55 / 41 / 39 / 40 / 40.
+constexpr int kFlatThreads = 256, kPiece = 32, kFlatFewest = kSmCount, kFlatMost = kSmCount * 5 / 2;
+constexpr uint32_t kFlatThin = 40;
+constexpr uint32_t kFlatMany = 1u << 19;             // words
+constexpr size_t kFlatLarge = (size_t)3 << 25;       // elements
+__device__ __forceinline__ uint32_t flat_blocks(uint32_t words, size_t n)
+{
+    return n >= kFlatLarge && words >= kFlatMany && (size_t)words * kFlatThin < n ? kFlatFewest : kFlatMost;
+}
 
 struct FlatGroup {
     uint32_t first, members, pieces, end;                        // place in order[]; messages; pieces of each; end of its units
 };
 struct FlatPlan {
     FlatGroup group[32];                                         // (a message has less than 2^29 words)
-    uint32_t units;
+    uint32_t units, words;                                       // all pieces, all words
     uint8_t order[kMaxViews];                                    // messages, longest group first
 };
 struct FlatShared {
@@ -124,7 +137,8 @@ __device__ __forceinline__ void plan_flat(FlatPlan &plan, const uint32_t *count,
         if (lane == 0) plan.group[g] = FlatGroup{first, members, pieces, units};
         first += members;
     }
-    if (lane == 0) plan.units = units;
+    const uint32_t words = __reduce_add_sync(0xffffffffu, c0 + c1);       // (fewer than one per eight elements)
+    if (lane == 0) { plan.units = units; plan.words = words; }
 }
 
 template <bool kHybrid, class Shared>
@@ -165,7 +179,7 @@ __device__ __forceinline__ void add_flat(const Shared &sm, const FlatPlan &plan,
 }
 
 template <bool kHybrid>
-__global__ void __launch_bounds__(kFlatThreads, kFlatBlocksPerSm)
+__global__ void __launch_bounds__(kFlatThreads, 3)
 decode_flat(const __grid_constant__ DecodeViews views, int W, const uint32_t *group_offsets, int K, float scale,
             float tau, float *u, size_t n, uint32_t *dev_status)
 {
@@ -186,8 +200,10 @@ decode_flat(const __grid_constant__ DecodeViews views, int W, const uint32_t *gr
     __syncthreads();
     if (tid < 32) plan_flat(sm.plan, sm.count, W);
     __syncthreads();
-    add_flat<kHybrid>(sm, sm.plan, in_smem ? sm_offs : group_offsets, K, scale, tau, u, n, dev_status,
-                      blockIdx.x * (kFlatThreads / 32) + (tid >> 5), gridDim.x * (kFlatThreads / 32));
+    const uint32_t blocks = min(gridDim.x, flat_blocks(sm.plan.words, n));
+    if (blockIdx.x < blocks)
+        add_flat<kHybrid>(sm, sm.plan, in_smem ? sm_offs : group_offsets, K, scale, tau, u, n, dev_status,
+                          blockIdx.x * (kFlatThreads / 32) + (tid >> 5), blocks * (kFlatThreads / 32));
 }
 
 // ---- a block's range --------------------------------------------------------------------------------------------------
@@ -981,7 +997,9 @@ decode_tiles(const __grid_constant__ DecodeViews views, int W, const uint32_t *g
             static_assert(sizeof(FlatPlan) <= sizeof(sm.lut) && alignof(FlatPlan) <= alignof(float), "the plan takes the tables' place");
             if (warp == 0) plan_flat(plan, sm.count, W);
             __syncthreads();
-            add_flat<kHybrid>(sm, plan, offs, K, scale, tau, u, n, dev_status, blockIdx.x * kTileWarps + warp, gridDim.x * kTileWarps);
+            const uint32_t blocks = min(gridDim.x, flat_blocks(plan.words, n));
+            if (blockIdx.x < blocks)
+                add_flat<kHybrid>(sm, plan, offs, K, scale, tau, u, n, dev_status, blockIdx.x * kTileWarps + warp, blocks * kTileWarps);
         }
         return;
     }
@@ -1080,8 +1098,7 @@ vgc_status decode_launch(bool hybrid, bool overwrite, const vgc_message_view *ms
         }
         if (!ow && most_words * kSparseAdd < n) {                // whatever the counts on the device say
             const size_t want = ((longest + kPiece - 1) / kPiece * wb + kFlatThreads / 32 - 1) / (kFlatThreads / 32);
-            const size_t most = (size_t)kSmCount * kFlatBlocksPerSm;
-            const unsigned blocks = (unsigned)(want < 1 ? 1 : want < most ? want : most);
+            const unsigned blocks = (unsigned)(want < 1 ? 1 : want < (size_t)kFlatMost ? want : (size_t)kFlatMost);
             VGC_CUDA_OK(launch_kernel(hybrid ? decode_flat<true> : decode_flat<false>, dim3(blocks), dim3(kFlatThreads), 0, st, true,
                                       views, wb, group_offsets, K, scale, tau, u, n, dev_status));
             count_launch();
