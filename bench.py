@@ -225,9 +225,9 @@ class HotPath:
             for li, spec in enumerate(self.layers):
                 M, N, K = spec.gemm_mnk(B)
                 self.flops_useful += 2 * M * N * K
-                # fp32 accuracy costs three TF32 products per algorithmic one; the TMA-fed form (all 1x1 convs) takes
-                # its two cross terms in bf16, at half the TF32 cost each
-                bf16_cross = spec.kind == "conv" and spec.k == 1 and not exact_conv
+                # fp32 accuracy costs three TF32 products per algorithmic one; the TMA-fed form (1x1 convs) and tiles of 192
+                # columns (the 3x3 and 7x7 convs) take their two cross terms in bf16, at half the TF32 cost each
+                bf16_cross = spec.kind == "conv" and not exact_conv
                 self.flops_issued += 2 * M * N * K * (2.0 if bf16_cross else 3.0)
             for g in self.groups:
                 spec = self.layers[g[0]]
@@ -1070,7 +1070,7 @@ def main():
     # dominant kernel of the step
     if sq_ms >= co_ms + de_ms and hp.flops_useful:
         # The contraction must be fp32-accurate (1e-5): three tensor-core products per algorithmic product (hi*hi in
-        # TF32 plus two cross terms -- TF32, or bf16 at half the TF32 cost in the TMA-fed form).  issue_factor is their
+        # TF32 plus two cross terms -- TF32, or bf16 at half the TF32 cost in the conv layers).  issue_factor is their
         # flop-weighted cost in TF32 products; issued = issue_factor x algorithmic is what the tensor pipe is asked to
         # do, and frac = issued / TF32 peak is the load on the pipe.
         issue_factor = hp.flops_issued / hp.flops_useful
