@@ -211,8 +211,11 @@ struct Plan {
 // Two candidates: whole tiles per block (no scratch, no second kernel, but the blocks' loads are as even as the
 // tile count allows), or an even cut of the slices over all SMs (tiles at the cuts are shared, their partial
 // sums combined by a second kernel).  Costs in slice times: a block's longest range, plus what the combine pass
-// adds to the call (its launch and the partial tiles' round trip, about 14 slices' worth: measured with tiles of 128 columns
-// and before launches overlapped; not measured again for the wide form and for chains that several warps share).
+// adds to the call: its launch and the partial tiles' round trip, kCombineSlices.  Measured over 40 convolutions and small
+// networks (B200): 6 is 5 % faster than 14 (which held before launches overlapped and partial tiles left in 16-byte
+// stores), up to 1.6 times (9 examples, 544 channels 14 x 14 to 48, 3x3 stride 2: 31.5 -> 19.3 us), none slower by more than the runs of
+// one side differ; 10 is 2 % faster than 14, 4 as fast as 6 but for small networks (ResNet-50, 128 x 128, 3 examples: 378 -> 367).
+constexpr int kCombineSlices = 4;
 static Plan make_plan(int M, int N, int k_slices, int n_layers, int unit_min, int tile_n)
 {
     Plan p;
@@ -234,13 +237,12 @@ static Plan make_plan(int M, int N, int k_slices, int n_layers, int unit_min, in
         blocks = tiles * parts;
     } else {
         // Alone, the launch is one block per SM at most.  Two candidates, costs in slice times: whole tiles per block
-        // (a block's longest range), or an even cut of all slices (plus what the combine pass adds to the call: its
-        // launch and the partial tiles' round trip, about 14 slices' worth).
+        // (a block's longest range), or an even cut of all slices (plus what the combine pass adds to the call).
         const long long waves = (tiles + kSmCount - 1) / kSmCount;
         const long long blocks_a = (tiles + waves - 1) / waves;
         const long long cost_a = ((tiles + blocks_a - 1) / blocks_a) * k_slices;
         const long long blocks_b = units < kSmCount ? units : kSmCount;
-        const long long cost_b = ((units + blocks_b - 1) / blocks_b) * unit_min + 14;
+        const long long cost_b = ((units + blocks_b - 1) / blocks_b) * unit_min + kCombineSlices;
         even = cost_b < cost_a;
         blocks = even ? blocks_b : blocks_a;
     }
