@@ -666,7 +666,11 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
     prm.C = C; prm.H = H; prm.W = W; prm.Cout = Cout; prm.Kh = Kh; prm.Kw = Kw; prm.sh = sh; prm.sw = sw;
     prm.ph = ph; prm.pw = pw; prm.Wo = Wo; prm.P = P;
     prm.chw = C * H * W;
-    prm.wo_magic = (unsigned)(0x100000000ull / (unsigned)Wo) + 1u;
+    if (Wo > 1) {
+        const RowDivisor by_wo = row_divisor((uint32_t)Wo);
+        prm.wo_magic = by_wo.magic;
+        prm.wo_shift = by_wo.shift;
+    }
     const bool ex = t_exact;
     const int unit = ex ? p_slices : 1;
     KernelFn fn = nullptr;

@@ -42,6 +42,7 @@
 // through to the common exit, outstanding TMA loads are waited for (bounded) and TMEM is freed.
 #pragma once
 
+#include "vgc_rows.cuh"
 #include "vgc_tc.cuh"
 
 namespace vgc {
@@ -136,7 +137,8 @@ struct Params {
     int accumulate;
     int C, H, W, Cout, Kh, Kw, sh, sw, ph, pw, Wo, P;     // conv geometry (gathered tiles)
     int chw;                 // C*H*W
-    unsigned wo_magic;       // floor(2^32 / Wo) + 1: p / Wo == umulhi(p, wo_magic) for p * Wo < 2^32
+    unsigned wo_magic;       // p / Wo == row_of(p, wo_magic, wo_shift); Wo >= 2
+    int wo_shift;
     long long ld_m, ld_n;    // result: element (m, n) lives at S[m*ld_m + n*ld_n]; one of the two is 1
     float *partial;          // scratch for partial tiles [2 * block + (0: a block's first segment, 1: its last)][column / 4][row][column % 4]
     uint32_t *status;        // device word; VGC_DEV_TIMEOUT is OR-ed in if a wait expired
@@ -198,7 +200,7 @@ struct GatherRows {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int p = pbase + j;
-                const int ho = prm.Wo == 1 ? p : (int)__umulhi((unsigned)p, prm.wo_magic), wo = p - ho * prm.Wo;
+                const int ho = prm.Wo == 1 ? p : (int)row_of((unsigned)p, prm.wo_magic, prm.wo_shift), wo = p - ho * prm.Wo;
                 const int hs = ho * prm.sh, ws = wo * prm.sw;
                 const float *xp = xz + (hs * prm.W + ws);
                 const bool pv = p < prm.P;
@@ -260,7 +262,7 @@ struct GatherTaps {
 #pragma unroll
         for (int s = 0; s < 4 / kSpan; ++s) {
             const int p = pbase + s * kSpan;
-            const int ho = (int)__umulhi((unsigned)p, prm.wo_magic), wo = p - ho * prm.Wo;
+            const int ho = (int)row_of((unsigned)p, prm.wo_magic, prm.wo_shift), wo = p - ho * prm.Wo;
             const bool pv = p < prm.P;
             const float *xp = xz + (ho * prm.W + wo);
 #pragma unroll
@@ -332,7 +334,7 @@ struct GatherTapsS2 {
 #pragma unroll
         for (int s = 0; s < 4 / kSpan; ++s) {
             const int p = pbase + s * kSpan;
-            const int ho = (int)__umulhi((unsigned)p, prm.wo_magic), wo = p - ho * prm.Wo;
+            const int ho = (int)row_of((unsigned)p, prm.wo_magic, prm.wo_shift), wo = p - ho * prm.Wo;
             const bool pv = p < prm.P;
             const int hs = ho * prm.sh;
             const float *xp = xz + (hs * prm.W + 2 * wo);
@@ -387,7 +389,7 @@ struct GatherTaps7S2 {
     }
     __device__ __forceinline__ void load(const Params &prm, int z, int pbase, float (&v)[kTuples][kSlots]) const
     {
-        const int ho = (int)__umulhi((unsigned)pbase, prm.wo_magic), wo = pbase - ho * prm.Wo;
+        const int ho = (int)row_of((unsigned)pbase, prm.wo_magic, prm.wo_shift), wo = pbase - ho * prm.Wo;
         const int hs = ho * prm.sh;
         const bool pv = pbase < prm.P;
         const float *xp = src + (size_t)z * prm.chw + (hs * prm.W + 2 * wo - 4);
@@ -463,7 +465,7 @@ struct Halo {
 #pragma unroll
         for (int s = 0; s < 4 / kSpan; ++s) {
             const int p = pbase + s * kSpan;
-            const int ho = (int)__umulhi((unsigned)p, prm.wo_magic), wo = p - ho * prm.Wo;
+            const int ho = (int)row_of((unsigned)p, prm.wo_magic, prm.wo_shift), wo = p - ho * prm.Wo;
 #pragma unroll
             for (int i = 0; i < kSpan + kKw - 1; ++i)
                 bits |= ((i >= kPad && i < kSpan + kPad) || (unsigned)(wo + i - kPad) < (unsigned)prm.W ? 1u : 0u) << (s * (kKw + 1) + i);
