@@ -3,7 +3,6 @@
 #pragma once
 
 #include <cuda.h>
-#include <cuda_bf16.h>
 
 #include "vgc_common.cuh"
 
@@ -149,11 +148,14 @@ __device__ __forceinline__ void tc_st_32x8(uint32_t taddr, const uint32_t (&r)[8
         ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
         : "memory");
 }
-// two consecutive k as one 32-bit word of bf16 (round to nearest even): k in the low half, k + 1 in the high half
+// two consecutive k as one 32-bit word of bf16 (round to nearest even): k in the low half, k + 1 in the high half.  What would round
+// to infinity (finite numbers from 3.3962e38 on) becomes the largest finite number, 2^-8 off at most: squares that are finite in tf32
+// stay finite in their bf16 copies, where infinity times a small or zero part made the whole sum infinite or NaN.
 __device__ __forceinline__ uint32_t pack_bf16(float k0, float k1)
 {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(k0, k1);
-    return *reinterpret_cast<const uint32_t *>(&v);
+    uint32_t v;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(v) : "f"(k1), "f"(k0));
+    return v;
 }
 // 32 lanes x 16 columns: each thread stores 16 registers into its lane's row
 __device__ __forceinline__ void tc_st_32x16(uint32_t taddr, const uint32_t (&r)[16])
