@@ -1,5 +1,6 @@
 // Squared per-example gradient sums on the tensor cores: the pass that adds partial tiles, the repacking pre-pass, planning and
 // launches.  The kernel is in vgc_sqgrad_tc.cuh.
+#include <atomic>
 #include <cstdlib>
 
 #include "vgc_sqgrad_tc.cuh"
@@ -197,9 +198,18 @@ sqgrad_tc_combine_examples(const float *partial, int examples, int n_parts, int 
 // (96 instructions): results then sit 1 - 3e-6 below the exact sum, against the 1e-5 bound.
 constexpr int kChunk = 8;
 // how many sqgrad launches the caller keeps in flight side by side (vgc_sqgrad_plan_hint)
-static int g_concurrent = 1;
+static std::atomic<int> g_concurrent{1};
+
+// What one call of the library goes by from its beginning to its end: plans, workspace and the kernel's form have to agree, and
+// another thread may change the hint meanwhile.
+struct Call {
+    bool exact;              // the per-example statistic
+    int concurrent;
+    explicit Call(bool per_example) : exact(per_example), concurrent(g_concurrent.load(std::memory_order_relaxed)) {}
+};
 
 struct Plan {
+    int M, N, k_slices, n_layers, tile_n;
     int unit, units_per_tile, blocks, tiles_x, tiles_y;
     int units_total;
     int parts, part_slices;  // examples cut up: parts of each (0: not), slices of a part
@@ -216,16 +226,17 @@ struct Plan {
 // stores), up to 1.6 times (9 examples, 544 channels 14 x 14 to 48, 3x3 stride 2: 31.5 -> 19.3 us), none slower by more than the runs of
 // one side differ; 10 is 2 % faster than 14, 4 as fast as 6 but for small networks (ResNet-50, 128 x 128, 3 examples: 378 -> 367).
 constexpr int kCombineSlices = 4;
-static Plan make_plan(int M, int N, int k_slices, int n_layers, int unit_min, int tile_n)
+static Plan make_plan(const Call &call, int M, int N, int k_slices, int n_layers, int unit_min, int tile_n)
 {
     Plan p;
+    p.M = M; p.N = N; p.k_slices = k_slices; p.n_layers = n_layers; p.tile_n = tile_n;
     p.tiles_x = (N + tile_n - 1) / tile_n;
     p.tiles_y = (M + kBM - 1) / kBM;
     const long long tiles = (long long)p.tiles_x * p.tiles_y * n_layers;
     const long long upt = k_slices / unit_min, units = tiles * upt;
     bool even;
     long long blocks;
-    if (g_concurrent > 1) {
+    if (call.concurrent > 1) {
         // Next to other launches the hardware's block scheduler does the balancing: blocks of all launches in flight
         // queue for the SMs and a partly filled wave costs nothing (the neighbours' blocks take the idle SMs).  Each
         // tile's reduction is cut into as many parts as make about half a wave of blocks per launch: shorter blocks
@@ -247,7 +258,7 @@ static Plan make_plan(int M, int N, int k_slices, int n_layers, int unit_min, in
         blocks = even ? blocks_b : blocks_a;
     }
     p.parts = p.part_slices = 0;
-    if (unit_min > 1 && g_concurrent == 1) {
+    if (unit_min > 1 && call.concurrent == 1) {
         // Few long examples, which the form that adds up an example's products before it squares them keeps whole, leave SMs
         // idle: parts of an example, a block each, at most two waves of them; costs as above, a wave's start about 5 slices.
         const long long waves_now = even ? (units + blocks - 1) / blocks : ((tiles + blocks - 1) / blocks) * upt;
@@ -287,7 +298,7 @@ using namespace tc;
 
 void tc_plan_hint(int concurrent_launches)
 {
-    g_concurrent = concurrent_launches > 1 ? concurrent_launches : 1;
+    g_concurrent.store(concurrent_launches > 1 ? concurrent_launches : 1, std::memory_order_relaxed);
 }
 
 bool tc_linear_supported(int B, int in, int out)
@@ -306,20 +317,18 @@ bool tc_conv_supported(int B, int C, int H, int W, int Cout, int Kh, int Kw, int
 // columns of an accumulator and of a partial tile, whatever part of them a tile uses
 static int slot_columns(int tile_n) { return tile_n > kBN ? kWideN : kBN; }
 
-static size_t tc_workspace_bytes(int M, int N, int k_slices, int n_layers = 1, int unit = 1, int tile_n = kBN)
+static size_t tc_workspace_bytes(const Plan &p)
 {
-    const Plan p = make_plan(M, N, k_slices, n_layers, unit, tile_n);
     // status word (256 bytes) + two partial tiles per block (the first and the last segment of its range)
-    return 256 + (p.partials ? (size_t)(p.parts ? 1 : 2) * p.blocks * kBM * slot_columns(tile_n) * sizeof(float) : 0);
+    return 256 + (p.partials ? (size_t)(p.parts ? 1 : 2) * p.blocks * kBM * slot_columns(p.tile_n) * sizeof(float) : 0);
 }
 
-static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Params prm, int M, int N,
-                            int k_slices, void *ws, size_t ws_bytes, cudaStream_t st, int unit = 1, int tile_n = kBN)
+static vgc_status tc_launch(KernelFn kernel, const Batch &bt, const Plan &plan, Params prm, void *ws, size_t ws_bytes, cudaStream_t st)
 {
-    const Plan plan = make_plan(M, N, k_slices, n_layers, unit, tile_n);
-    if (ws_bytes < tc_workspace_bytes(M, N, k_slices, n_layers, unit, tile_n)) return VGC_ERR_WORKSPACE;
+    const int M = plan.M, N = plan.N, n_layers = plan.n_layers, tile_n = plan.tile_n;
+    if (ws_bytes < tc_workspace_bytes(plan)) return VGC_ERR_WORKSPACE;
     VGC_CUDA_OK(allow_dynamic_smem(reinterpret_cast<const void *>(kernel), kSmemBytes, kRegsLaunch));
-    prm.M = M; prm.N = N; prm.k_slices = k_slices;
+    prm.M = M; prm.N = N; prm.k_slices = plan.k_slices;
     prm.unit = plan.unit; prm.units_per_tile = plan.units_per_tile; prm.units_total = plan.units_total;
     prm.units_q = plan.units_total / plan.blocks; prm.units_r = plan.units_total % plan.blocks;
     prm.parts = plan.parts; prm.part_slices = plan.part_slices;
@@ -335,7 +344,7 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
         if (plan.parts) {
             const int slot_n = slot_columns(tile_n);
             VGC_CUDA_OK(launch_kernel(Carveout{18}, sqgrad_tc_combine_examples, dim3((unsigned)(plan.tiles_x * plan.tiles_y * slot_n), (unsigned)n_layers), dim3(256), 0,
-                                      st, true, prm.partial, k_slices / prm.p_slices, plan.parts, tile_n, slot_n, plan.tiles_x, plan.tiles_y, M, N,
+                                      st, true, prm.partial, plan.k_slices / prm.p_slices, plan.parts, tile_n, slot_n, plan.tiles_x, plan.tiles_y, M, N,
                                       prm.scale, prm.accumulate, results, prm.ld_m, prm.ld_n));
             count_launch();
             VGC_CUDA_OK(cudaGetLastError());
@@ -357,7 +366,9 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, int n_layers, Para
     return VGC_OK;
 }
 
-size_t tc_linear_workspace_bytes(int B, int in, int out) { return tc_workspace_bytes(out, in, (B + kBK - 1) / kBK); }
+static Plan linear_plan(int B, int in, int out) { return make_plan(Call(false), out, in, (B + kBK - 1) / kBK, 1, 1, kBN); }
+
+size_t tc_linear_workspace_bytes(int B, int in, int out) { return tc_workspace_bytes(linear_plan(B, in, out)); }
 
 vgc_status tc_sqgrad_linear(const float *x, const float *delta, int B, int in, int out, float scale, int accumulate,
                             float *S, void *ws, size_t ws_bytes, cudaStream_t st)
@@ -374,16 +385,8 @@ vgc_status tc_sqgrad_linear(const float *x, const float *delta, int B, int in, i
     prm.p_slices = 1; prm.tx_bytes = kRawStageBytes; prm.tx_bytes_a = kRawBytesA; prm.scale = scale;
     prm.accumulate = accumulate;
     prm.ld_m = in; prm.ld_n = 1;
-    return tc_launch(sqgrad_tc<kMajorMN, kTma, kTma, false>, bt, 1, prm, out, in, (B + kBK - 1) / kBK, ws, ws_bytes, st);
+    return tc_launch(sqgrad_tc<kMajorMN, kTma, kTma, false>, bt, linear_plan(B, in, out), prm, ws, ws_bytes, st);
 }
-
-// Set for the duration of a per-example (exact) call: planning, repacking and kernel choice consult it.
-static thread_local bool t_exact = false;
-struct ExactScope {
-    bool saved;
-    explicit ExactScope(bool on) : saved(t_exact) { t_exact = on; }
-    ~ExactScope() { t_exact = saved; }
-};
 
 // Cout <= 64: the im2col rows take the 128-row A tile and the errors the narrow B tile
 static bool conv_swapped(int Cout, int n_im2col) { return Cout <= 64 && n_im2col > Cout; }
@@ -404,7 +407,7 @@ static bool conv_swapped(int Cout, int n_im2col) { return Cout <= 64 && n_im2col
 //                   the padded layer has TMA-able error planes and takes the three-tap gather
 enum { kRepackNone = 0, kRepackPlanes = 1, kRepackFlat = 2, kRepackPadW = 3 };
 
-static int repack_mode(int B, int C, int Cout, int Kh, int Kw, int sh, int sw, int ph, int pw, int P, int W = 0, int Ho = 0,
+static int repack_mode(const Call &call, int B, int C, int Cout, int Kh, int Kw, int sh, int sw, int ph, int pw, int P, int W = 0, int Ho = 0,
                        int Wo = 0)
 {
     if ((long)B * C >= (1L << 31) || (long)B * Cout >= (1L << 31)) return kRepackNone;      // 32-bit row index
@@ -415,7 +418,7 @@ static int repack_mode(int B, int C, int Cout, int Kh, int Kw, int sh, int sw, i
     const bool planes_ok = P >= kBK && P % 4 == 0;
     if (planes_ok) return (sh > 1 || sw > 1) ? kRepackPlanes : kRepackNone;
     const long flat = (long)B * P;
-    if (t_exact) return kRepackNone;                 // the flat form merges the examples' positions
+    if (call.exact) return kRepackNone;                 // the flat form merges the examples' positions
     return (flat >= kBK && flat % 4 == 0 && flat < (1L << 30)) ? kRepackFlat : kRepackNone;
 }
 
@@ -494,41 +497,42 @@ sqgrad_repack(const __grid_constant__ RepackJobs jobs)
     }
 }
 
-static size_t conv_workspace_plain(int n_layers, int B, int C, int Kh, int Kw, int P, int Cout)
+static size_t conv_workspace_plain(const Call &call, int n_layers, int B, int C, int Kh, int Kw, int P, int Cout)
 {
     const int p_slices = (P + kBK - 1) / kBK, n_im2col = C * Kh * Kw, k_slices = B * p_slices;
-    const int unit = t_exact ? p_slices : 1;
+    auto bytes = [&](int M, int N, int tile_n) {
+        return tc_workspace_bytes(make_plan(call, M, N, k_slices, n_layers, call.exact ? p_slices : 1, tile_n));
+    };
     // the wide and the narrow form of a layer that gathers several taps at a time: either can be chosen at call time
-    const size_t narrow = conv_swapped(Cout, n_im2col) ? tc_workspace_bytes(n_im2col, Cout, k_slices, n_layers, unit)
-                                                       : tc_workspace_bytes(Cout, n_im2col, k_slices, n_layers, unit);
-    size_t wide = Kw > 1 ? tc_workspace_bytes(Cout, n_im2col, k_slices, n_layers, unit, kWideN) : 0;
+    const size_t narrow = conv_swapped(Cout, n_im2col) ? bytes(n_im2col, Cout, kBN) : bytes(Cout, n_im2col, kBN);
+    size_t wide = Kw > 1 ? bytes(Cout, n_im2col, kWideN) : 0;
     if (Kw == 5 || Kw == 7) {           // whole tuples of five or seven columns
-        const size_t w = tc_workspace_bytes(Cout, n_im2col, k_slices, n_layers, unit, kWideN / Kw * Kw);
+        const size_t w = bytes(Cout, n_im2col, kWideN / Kw * Kw);
         wide = wide > w ? wide : w;
     }
     return narrow > wide ? narrow : wide;
 }
 
 // Workspace of one launch over n_layers layers of this geometry (n_layers <= kMaxBatch).
-static size_t conv_workspace_group(int n_layers, int B, int C, int Kh, int Kw, int sh, int sw, int ph, int pw, int P,
+static size_t conv_workspace_group(const Call &call, int n_layers, int B, int C, int Kh, int Kw, int sh, int sw, int ph, int pw, int P,
                                    int Cout, int H, int W, int Ho, int Wo)
 {
     // the larger of the in-place form and the repacked one, so that either can be chosen at call time
-    size_t need = conv_workspace_plain(n_layers, B, C, Kh, Kw, P, Cout);
-    const int mode = repack_mode(B, C, Cout, Kh, Kw, sh, sw, ph, pw, P, W, Ho, Wo);
+    size_t need = conv_workspace_plain(call, n_layers, B, C, Kh, Kw, P, Cout);
+    const int mode = repack_mode(call, B, C, Cout, Kh, Kw, sh, sw, ph, pw, P, W, Ho, Wo);
     const size_t x_bytes = round_up(sizeof(float) * (size_t)B * C * P, 256);
     const size_t d_bytes = round_up(sizeof(float) * (size_t)B * Cout * P, 256);
     if (mode == kRepackPadW) {
         const int Wo4 = (Wo + 3) / 4 * 4;
         const size_t xp = round_up(sizeof(float) * (size_t)B * C * H * (sw * Wo4), 256);
         const size_t dp = round_up(sizeof(float) * (size_t)B * Cout * Ho * Wo4, 256);
-        const size_t r = round_up(conv_workspace_plain(n_layers, B, C, Kh, Kw, Ho * Wo4, Cout), 256) + n_layers * (xp + dp);
+        const size_t r = round_up(conv_workspace_plain(call, n_layers, B, C, Kh, Kw, Ho * Wo4, Cout), 256) + n_layers * (xp + dp);
         need = need > r ? need : r;
     } else if (mode == kRepackPlanes) {
-        const size_t r = round_up(conv_workspace_plain(n_layers, B, C, 1, 1, P, Cout), 256) + n_layers * x_bytes;
+        const size_t r = round_up(conv_workspace_plain(call, n_layers, B, C, 1, 1, P, Cout), 256) + n_layers * x_bytes;
         need = need > r ? need : r;
     } else if (mode == kRepackFlat) {
-        const size_t r = round_up(conv_workspace_plain(n_layers, 1, C, 1, 1, B * P, Cout), 256) +
+        const size_t r = round_up(conv_workspace_plain(call, n_layers, 1, C, 1, 1, B * P, Cout), 256) +
                          n_layers * (x_bytes + d_bytes);
         need = need > r ? need : r;
     }
@@ -539,29 +543,29 @@ size_t tc_conv_workspace_bytes(int n_layers, int B, int C, int H, int W, int Kh,
                                int Ho, int Wo, int Cout, bool exact)
 {
     const int P = Ho * Wo;
-    ExactScope scope(exact);
+    const Call call(exact);
     // more layers than one launch takes are processed group after group in the same workspace
     const int first = n_layers < kMaxBatch ? n_layers : kMaxBatch;
-    size_t need = conv_workspace_group(first, B, C, Kh, Kw, sh, sw, ph, pw, P, Cout, H, W, Ho, Wo);
+    size_t need = conv_workspace_group(call, first, B, C, Kh, Kw, sh, sw, ph, pw, P, Cout, H, W, Ho, Wo);
     const int rest = n_layers > kMaxBatch ? n_layers % kMaxBatch : 0;
     if (rest) {
-        const size_t r = conv_workspace_group(rest, B, C, Kh, Kw, sh, sw, ph, pw, P, Cout, H, W, Ho, Wo);
+        const size_t r = conv_workspace_group(call, rest, B, C, Kh, Kw, sh, sw, ph, pw, P, Cout, H, W, Ho, Wo);
         need = need > r ? need : r;
     }
     return need;
 }
 
-static vgc_status conv_group(int n_layers, const float *const *x, const float *const *delta, float *const *S, int B,
+static vgc_status conv_group(const Call &call, int n_layers, const float *const *x, const float *const *delta, float *const *S, int B,
                              int C, int H, int W, int Cout, int Kh, int Kw, int sh, int sw, int ph, int pw, int Ho,
                              int Wo, float scale, int accumulate, void *ws, size_t ws_bytes, cudaStream_t st)
 {
     const int P = Ho * Wo, n_im2col = C * Kh * Kw;
-    const int mode = repack_mode(B, C, Cout, Kh, Kw, sh, sw, ph, pw, P, W, Ho, Wo);
+    const int mode = repack_mode(call, B, C, Cout, Kh, Kw, sh, sw, ph, pw, P, W, Ho, Wo);
     // one run of the output per warp; more when there are many
     auto blocks_for = [](size_t values) { const size_t b = (values + 8 * kRepackRun - 1) / (8 * kRepackRun); return (unsigned)(b < 1 ? 1 : (b > 148 * 32 ? 148 * 32 : b)); };
     if (mode == kRepackPadW) {
         const int Wo4 = (Wo + 3) / 4 * 4, Wx = sw * Wo4;              // padded widths of the errors and of x
-        const size_t inner = round_up(conv_workspace_plain(n_layers, B, C, Kh, Kw, Ho * Wo4, Cout), 256);
+        const size_t inner = round_up(conv_workspace_plain(call, n_layers, B, C, Kh, Kw, Ho * Wo4, Cout), 256);
         const size_t xp = round_up(sizeof(float) * (size_t)B * C * H * Wx, 256);
         const size_t dp = round_up(sizeof(float) * (size_t)B * Cout * Ho * Wo4, 256);
         if (ws_bytes < inner + n_layers * (xp + dp)) return VGC_ERR_WORKSPACE;
@@ -577,12 +581,12 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
         }
         VGC_CUDA_OK(launch_kernel(kAllL1, sqgrad_repack, dim3(blocks_for((size_t)B * ((size_t)C * H * Wx > (size_t)Cout * Ho * Wo4 ? (size_t)C * H * Wx : (size_t)Cout * Ho * Wo4)), 2 * n_layers), dim3(256), 0, st, true, jobs));
         count_launch();
-        return conv_group(n_layers, xr, dr, S, B, C, H, Wx, Cout, Kh, Kw, sh, sw, ph, 1, Ho, Wo4, scale, accumulate, ws, inner, st);
+        return conv_group(call, n_layers, xr, dr, S, B, C, H, Wx, Cout, Kh, Kw, sh, sw, ph, 1, Ho, Wo4, scale, accumulate, ws, inner, st);
     }
     if (mode != kRepackNone) {
         const bool flat = mode == kRepackFlat;
-        const size_t inner = round_up(flat ? conv_workspace_plain(n_layers, 1, C, 1, 1, B * P, Cout)
-                                           : conv_workspace_plain(n_layers, B, C, 1, 1, P, Cout), 256);
+        const size_t inner = round_up(flat ? conv_workspace_plain(call, n_layers, 1, C, 1, 1, B * P, Cout)
+                                           : conv_workspace_plain(call, n_layers, B, C, 1, 1, P, Cout), 256);
         const size_t x_bytes = round_up(sizeof(float) * (size_t)B * C * P, 256);
         const size_t d_bytes = flat ? round_up(sizeof(float) * (size_t)B * Cout * P, 256) : 0;
         if (ws_bytes < inner + n_layers * (x_bytes + d_bytes)) return VGC_ERR_WORKSPACE;
@@ -601,9 +605,9 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
         VGC_CUDA_OK(launch_kernel(kAllL1, sqgrad_repack, dim3(blocks_for((size_t)B * (flat && Cout > C ? Cout : C) * P), n_jobs), dim3(256), 0, st, true, jobs));
         count_launch();
         if (flat)
-            return conv_group(n_layers, xr, dr, S, 1, C, B * P, 1, Cout, 1, 1, 1, 1, 0, 0, B * P, 1, scale, accumulate, ws,
+            return conv_group(call, n_layers, xr, dr, S, 1, C, B * P, 1, Cout, 1, 1, 1, 1, 0, 0, B * P, 1, scale, accumulate, ws,
                               inner, st);
-        return conv_group(n_layers, xr, dr, S, B, C, Ho, Wo, Cout, 1, 1, 1, 1, 0, 0, Ho, Wo, scale, accumulate, ws, inner, st);
+        return conv_group(call, n_layers, xr, dr, S, B, C, Ho, Wo, Cout, 1, 1, 1, 1, 0, 0, Ho, Wo, scale, accumulate, ws, inner, st);
     }
     // which tiles TMA can deliver: rows of P positions with a 16-byte pitch, at least one slice long; the input
     // tile only when the im2col view is the tensor itself (1x1 kernel, stride 1, no padding)
@@ -619,18 +623,25 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
                             ? (Wo % 4 == 0 ? 4 : 2) : 0;
     // seven taps at a time: Kw = 7, stride 2, pad 3
     const bool taps7 = !in_tma && err_tma && Kw == 7 && sw == 2 && pw == 3 && W == 2 * Wo && Wo % 4 == 0;
-    // with few output channels the roles are swapped -- except in the three-tap form, where keeping the errors as
-    // the A operand (in tensor memory, half of its rows unused) measures faster than both operands in shared memory
-    // a square kernel that keeps the width: its input rows by TMA (the per-example form where it can take wide tiles)
-    // (wide tiles of the per-example form: an example fits one accumulator run, or parts of examples leave as plain sums)
-    auto short_runs = [&](int tile_n) {
-        return !t_exact || p_slices <= kChunk || make_plan(Cout, n_im2col, k_slices, n_layers, p_slices, tile_n).parts > 0;
-    };
-    const bool halo = !in_tma && err_tma && (Kw == 5 || Kw == 7) && Kh == Kw && sh == 1 && sw == 1 && 2 * pw == Kw - 1 &&
-                      Wo == W && W % 2 == 0 && H * W % 4 == 0 && short_runs(kWideN / Kw * Kw);
+    const bool ex = call.exact;
+    const int unit = ex ? p_slices : 1;
+    // the launch's plan: made once, it decides between forms below and is what is launched
+    auto plan_of = [&](int M, int N, int tile_n) { return make_plan(call, M, N, k_slices, n_layers, unit, tile_n); };
+    // wide tiles of the per-example form: an example fits one accumulator run, or parts of examples leave as plain sums
+    auto wide_fits = [&](const Plan &p) { return !ex || p_slices <= kChunk || p.parts > 0; };
+    Plan plan = {};
+    // a square kernel that keeps the width: its input rows by TMA
+    bool halo = !in_tma && err_tma && (Kw == 5 || Kw == 7) && Kh == Kw && sh == 1 && sw == 1 && 2 * pw == Kw - 1 && Wo == W &&
+                W % 2 == 0 && H * W % 4 == 0;
+    if (halo) {
+        plan = plan_of(Cout, n_im2col, kWideN / Kw * Kw);
+        halo = wide_fits(plan);
+    }
+    // with few output channels the roles are swapped -- except where several taps are gathered at a time: there keeping the errors
+    // as the A operand (in tensor memory, half of its rows unused) measures faster than both operands in shared memory
     const bool swapped = conv_swapped(Cout, n_im2col) && !taps && !taps_s2 && !taps7 && !halo;
     // both tiles by TMA: A in tensor memory, cross terms in bf16 (the per-example form keeps tf32 cross terms)
-    const bool tma_bf = err_tma && in_tma && !t_exact;
+    const bool tma_bf = err_tma && in_tma && !ex;
     const int rows_err = swapped ? kBN : kBM, rows_in = swapped ? kBM : kBN;
     Batch bt = {};
     uint32_t tx_err = 0, tx_in = 0;
@@ -671,8 +682,6 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
         prm.wo_magic = by_wo.magic;
         prm.wo_shift = by_wo.shift;
     }
-    const bool ex = t_exact;
-    const int unit = ex ? p_slices : 1;
     KernelFn fn = nullptr;
 #define VGC_TC_FN(A, B_, AT) (ex ? (KernelFn)sqgrad_tc<kMajorK, A, B_, AT, true> : (KernelFn)sqgrad_tc<kMajorK, A, B_, AT, false>)
     if (!swapped) {     // S[o][idx]: m = o, n = idx
@@ -680,22 +689,27 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
         if (halo) {
             const bool by4 = W % 4 == 0;
             fn = wide_halo_kernel(Kw == 5 ? (by4 ? kHalo5x4 : kHalo5x2) : (by4 ? kHalo7x4 : kHalo7x2), ex);
-            return tc_launch(fn, bt, n_layers, prm, Cout, n_im2col, k_slices, ws, ws_bytes, st, unit, kWideN / Kw * Kw);
+            return tc_launch(fn, bt, plan, prm, ws, ws_bytes, st);
         }
         if (taps || taps_s2 || taps7) {
             // Wide tiles where they are fewer than narrow ones (128 channels 28 x 28, batch 32: 47.9 -> 43.0 us, now 38.6; but 9 channels
             // 16 x 16 to 958, 81 columns: 25.0 us narrow, 28.7 wide).  The wide per-example form adds an example's sums up within
             // one accumulator run.
             const int mode = taps ? (taps == 4 ? kGatherTaps4 : kGatherTaps2) : taps_s2 ? (taps_s2 == 4 ? kGatherTaps4S2 : kGatherTaps2S2) : kGatherTaps7S2;
-            const bool wide = (n_im2col + kWideN - 1) / kWideN < (n_im2col + kBN - 1) / kBN && short_runs(kWideN);
+            bool wide = (n_im2col + kWideN - 1) / kWideN < (n_im2col + kBN - 1) / kBN;
+            if (wide) {
+                plan = plan_of(Cout, n_im2col, kWideN);
+                wide = wide_fits(plan);
+            }
+            if (!wide) plan = plan_of(Cout, n_im2col, kBN);
             fn = wide ? wide_taps_kernel(mode, ex) : narrow_taps_kernel(mode, ex);
-            return tc_launch(fn, bt, n_layers, prm, Cout, n_im2col, k_slices, ws, ws_bytes, st, unit, wide ? kWideN : kBN);
+            return tc_launch(fn, bt, plan, prm, ws, ws_bytes, st);
         }
         if (tma_bf) fn = sqgrad_tc<kMajorK, kTma, kTma, true, false, true>;
         else if (err_tma && in_tma) fn = sqgrad_tc<kMajorK, kTma, kTma, true, true>;
         else if (err_tma) fn = VGC_TC_FN(kTma, kGatherIm2col, true);
         else fn = VGC_TC_FN(kGatherErr, kGatherIm2col, false);
-        return tc_launch(fn, bt, n_layers, prm, Cout, n_im2col, k_slices, ws, ws_bytes, st, unit);
+        return tc_launch(fn, bt, plan_of(Cout, n_im2col, kBN), prm, ws, ws_bytes, st);
     }
     prm.ld_m = 1; prm.ld_n = n_im2col;   // m = idx, n = o
     if (tma_bf) fn = sqgrad_tc<kMajorK, kTma, kTma, true, false, true>;
@@ -703,7 +717,7 @@ static vgc_status conv_group(int n_layers, const float *const *x, const float *c
     else if (err_tma) fn = VGC_TC_FN(kGatherIm2col, kTma, false);
     else fn = VGC_TC_FN(kGatherIm2col, kGatherErr, false);
 #undef VGC_TC_FN
-    return tc_launch(fn, bt, n_layers, prm, n_im2col, Cout, k_slices, ws, ws_bytes, st, unit);
+    return tc_launch(fn, bt, plan_of(n_im2col, Cout, kBN), prm, ws, ws_bytes, st);
 }
 
 // n_layers layers of one geometry; x, delta, S are host arrays of device pointers
@@ -711,10 +725,10 @@ vgc_status tc_sqgrad_conv(int n_layers, const float *const *x, const float *cons
                           int H, int W, int Cout, int Kh, int Kw, int sh, int sw, int ph, int pw, int Ho, int Wo,
                           float scale, int accumulate, void *ws, size_t ws_bytes, cudaStream_t st, bool exact)
 {
-    ExactScope scope(exact);
+    const Call call(exact);
     for (int l0 = 0; l0 < n_layers; l0 += kMaxBatch) {
         const int nl = n_layers - l0 < kMaxBatch ? n_layers - l0 : kMaxBatch;
-        const vgc_status rc = conv_group(nl, x + l0, delta + l0, S + l0, B, C, H, W, Cout, Kh, Kw, sh, sw, ph, pw, Ho, Wo,
+        const vgc_status rc = conv_group(call, nl, x + l0, delta + l0, S + l0, B, C, H, W, Cout, Kh, Kw, sh, sw, ph, pw, Ho, Wo,
                                          scale, accumulate, ws, ws_bytes, st);
         if (rc != VGC_OK) return rc;
     }

@@ -2,6 +2,8 @@
 of unequal length, every way a tile gets its rows, several layers in a call.
 
 Checked against PyTorch in fp64.  Bound 1e-5 of the same statistic of absolute values: signed sums can cancel."""
+import threading
+
 import pytest
 import torch
 
@@ -39,3 +41,39 @@ def test_parts(B, C, H, Cout, k, stride, accumulate):
         want = torch.einsum("bop,bip->boi", dd, cols).square().sum(0).reshape(S.shape) * 0.5 + o
         most = torch.einsum("bop,bip->boi", dd.abs(), cols.abs()).square().sum(0).reshape(S.shape) * 0.5 + o
         assert float(((S.double() - want).abs() / most).max()) < 1e-5
+
+
+def test_hint_that_changes_during_calls():
+    """The planning hint decides whether examples are cut up, and so which kernels can run: a call goes by one reading of it, whatever
+    another thread sets meanwhile."""
+    B, C, H, Cout = 2, 64, 28, 64
+    gen = torch.Generator("cuda").manual_seed(3)
+    x, d = torch.rand(B, C, H, H, device="cuda", generator=gen), torch.rand(B, Cout, H, H, device="cuda", generator=gen)
+    cols, dd = torch.nn.functional.unfold(x.double(), 3, padding=1), d.double().reshape(B, Cout, -1)
+    want = torch.einsum("bop,bip->boi", dd, cols).square().sum(0).reshape(-1)
+    need = 0
+    for hint in (2, 1):
+        vgc.vgc_sqgrad_plan_hint(hint)
+        need = max(need, vgc.vgc_sqgrad_conv_exact_workspace_bytes(B, C, H, H, Cout, 3, 3, 1, 1, 1, 1))
+    ws, stop = torch.zeros(need, dtype=torch.uint8, device="cuda"), threading.Event()
+
+    def toggle():
+        hint = vgc.load_library().vgc_sqgrad_plan_hint
+        while not stop.is_set():
+            for _ in range(50):
+                hint(2)
+                hint(1)
+
+    thread = threading.Thread(target=toggle)
+    thread.start()
+    try:
+        worst = 0.0
+        for _ in range(2000):
+            S = torch.empty(Cout * C * 9, device="cuda")
+            vgc.vgc_sqgrad_conv_exact(x, d, (3, 3), (1, 1), (1, 1), 1.0, S, False, ws)
+            worst = max(worst, float(((S.double() - want).abs() / want).max()))
+    finally:
+        stop.set()
+        thread.join()
+        vgc.vgc_sqgrad_plan_hint(1)
+    assert worst < 1e-5
