@@ -335,7 +335,9 @@ static vgc_status tc_launch(KernelFn kernel, const Batch &bt, const Plan &plan, 
     prm.tile_n = tile_n; prm.tiles_x = plan.tiles_x; prm.tiles_y = plan.tiles_y;
     prm.chunk = kChunk;
     prm.status = static_cast<uint32_t *>(ws);
-    prm.partial = reinterpret_cast<float *>(static_cast<char *>(ws) + 256);
+    // partial tiles are read and written 16 bytes at a time, the caller's workspace may start anywhere: the status word's 256 bytes
+    // have room to round down
+    prm.partial = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(ws) + 256) & ~(uintptr_t)15);
     VGC_CUDA_OK(launch_kernel(kernel, dim3((unsigned)plan.blocks), dim3(kThreadsTc), kSmemBytes, st, true, bt, prm));
     count_launch();
     if (plan.partials) {
