@@ -282,7 +282,8 @@ vgc_status vgc_decode_sum(const vgc_message_view *msgs, int W, const uint32_t *g
  * and copy the message back: counters_host[4] = {nnz, n_criterion, n_dropped, dev_status} and the
  * first min(nnz, capacity) words into words_host.  Host buffers should be pinned.  Unlike the other
  * entry points this one WAITS for the stream (twice where the words have to be copied, which takes their
- * count on the host first: messages of more than 2^18 words, words_host or counters_host not page-locked).  `out` holds device pointers as for vgc_compress; r, v are device state.
+ * count on the host first: messages of more than 2^18 words, words_host (min(capacity, 2^18) words of it) or counters_host not
+ * page-locked).  `out` holds device pointers as for vgc_compress; r, v are device state.
  *
  * The results are those of this order.  The copies themselves run ahead, on a stream of the library's own behind
  * what `stream` holds at the call: a layer's kernels wait for that layer's copies only, and g arrives under the last

@@ -9,7 +9,9 @@
 // 351 -> 261 us, of which the copies are 205).  Where a staging buffer lies over another one or over memory that an earlier
 // layer's kernels write, copies and kernels take turns on the caller's stream.
 // The message goes home by a kernel that writes the counters and, up to kDirectWords, the words to host memory, where that memory is
-// page-locked: the call waits for the stream once.  Copies need the word count on the host first: two waits (MLP as above: 258 against 245 us).
+// page-locked as far as the message can reach: the call waits for the stream once.  Copies need the word count on the host first: two waits (MLP as above: 258 against 245 us).
+#include <cuda.h>
+
 #include <mutex>
 
 #include "vgc_common.cuh"
@@ -126,15 +128,28 @@ message_to_host(const vgc_message out, uint32_t *words_host, uint32_t *counters_
     for (uint32_t i = 4 * whole + first; i < kept; i += step) words_host[i] = out.words[i];
 }
 
-// The address under which kernels reach a page-locked host buffer; nullptr for other memory.
-uint32_t *device_view(const void *host)
+// The address under which kernels reach `bytes` bytes of host memory: all of them in one page-locked allocation or registration
+// (the runtime says of the first byte only whether it is), on a 4-byte boundary.  nullptr for other memory.
+uint32_t *device_view(const void *host, size_t bytes)
 {
-    cudaPointerAttributes attr;
-    if (cudaPointerGetAttributes(&attr, host) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return attr.type == cudaMemoryTypeHost ? static_cast<uint32_t *>(attr.devicePointer) : nullptr;
+    typedef CUresult (*AttributesFn)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const AttributesFn fn = [] {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const bool ok = cudaGetDriverEntryPoint("cuPointerGetAttributes", &p, cudaEnableDefault, &found) == cudaSuccess;
+        return ok && found == cudaDriverEntryPointSuccess ? reinterpret_cast<AttributesFn>(p) : nullptr;
+    }();
+    const uintptr_t first = reinterpret_cast<uintptr_t>(host);
+    if (!fn || (first & 3u)) return nullptr;
+    unsigned type = 0, managed = 0;
+    CUdeviceptr seen = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *into[5] = {&type, &managed, &seen, &start, &size};
+    // (memory that CUDA does not know: all of them zero)
+    if (fn(5, what, into, (CUdeviceptr)first) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed || seen != (CUdeviceptr)first) return nullptr;
+    return first >= start && first - start <= size && bytes <= size - (first - start) ? reinterpret_cast<uint32_t *>(seen) : nullptr;
 }
 
 struct LayerSizes {
@@ -230,7 +245,9 @@ extern "C" vgc_status vgc_step_host(const vgc_layer_host *layers, int n_layers, 
     vgc_status rc = vgc_compress(g_dev, s_dev, r, v, n, group_offsets, K, alpha, zeta, out, ws_compress, ws_compress_bytes,
                                  stream);
     if (rc != VGC_OK) return rc;
-    uint32_t *const words_view = out->capacity ? device_view(words_host) : nullptr, *const counters_view = device_view(counters_host);
+    const uint32_t most_words = out->capacity < kDirectWords ? out->capacity : kDirectWords;        // that the kernel may write
+    uint32_t *const words_view = most_words ? device_view(words_host, (size_t)most_words * 4) : nullptr;
+    uint32_t *const counters_view = device_view(counters_host, 16);
     if (words_view && counters_view) {
         VGC_CUDA_OK(vgc::launch_kernel(message_to_host, dim3(64), dim3(256), 0, st, true, *out, words_view, counters_view));
         vgc::count_launch();

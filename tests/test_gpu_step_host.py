@@ -151,3 +151,35 @@ def test_message_goes_home_by_a_kernel_or_by_copies(sizes, pinned, shift):
     assert got == (want["nnz"], want["n_criterion"], want["n_dropped"], 0)
     assert np.array_equal(words[:want["nnz"]].numpy().view(np.uint32), want["words"])
     assert bool((words[want["nnz"]:] == -1).all())
+
+
+@pytest.mark.parametrize("place", ["whole", "begins page-locked", "counters off by two bytes", "words off by two bytes"])
+def test_results_where_a_kernel_cannot_write(place):
+    """Results that are page-locked only in part, or lie on no word boundary, are copied: the number of launches tells which way they
+    went."""
+    step, launches = Step(7, "own"), vgc.vgc_kernel_launch_count
+
+    def launched(words, counters):
+        step.words, step.counters = words, counters
+        before = launches()
+        step.check(vgc.MessageBuffers(step.n, step.K, step.n))
+        return launches() - before
+
+    by_copies = launched(step.words, step.counters)                          # ordinary memory
+    room = torch.zeros(4 * step.n + 3 * 4096, dtype=torch.uint8)
+    first = -room.data_ptr() % 4096
+    base, more = memoryview(room.numpy())[first:], torch.zeros(64, dtype=torch.uint8).pin_memory()
+    locked = (4 * step.want["nnz"] // 4096 + 1) * 4096                       # the message fits, the buffer does not
+    assert locked + 4096 < 4 * step.n and step.want["nnz"] < 1 << 18
+    if not place.startswith("begins"):
+        locked = 4 * step.n + 4096
+    at = [2 if place.startswith(what) else 0 for what in ("words", "counters")]
+    rt = torch.cuda.cudart()
+    assert rt.cudaHostRegister(room.data_ptr() + first, locked, 0) == rt.cudaError.success
+    try:
+        count = launched(torch.frombuffer(base[at[0]:at[0] + 4 * step.n], dtype=torch.int32),
+                         torch.frombuffer(memoryview(more.numpy())[at[1]:at[1] + 16], dtype=torch.int32))
+    finally:
+        torch.cuda.synchronize()
+        assert rt.cudaHostUnregister(room.data_ptr() + first) == rt.cudaError.success
+    assert count - by_copies == (1 if place == "whole" else 0)
