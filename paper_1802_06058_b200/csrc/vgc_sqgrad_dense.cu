@@ -78,10 +78,11 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 
 // kFew: fewer than 32 examples (see the epilogue; the check costs an added layer 6 %, so it is compiled for these only)
 // kBf: the two cross terms take bf16 copies of hi and lo, 16 deep an instruction: a third fewer instructions and so less of the
-// accumulator's bias, but their rounding shows in sums of few terms (largest error of 1024 x 1024 sums, 64 examples: 1.7e-6 in
-// tf32, 2.9e-6 with bf16; 192: 3.4e-6, 3.3e-6; 512: 3.6e-6, 3.0e-6), hence from kBfLeast examples on (512 examples, 2048 x 2048:
-// 27.9 -> 26.0 us; 256 examples, 1024 x 1024: 9.4 -> 8.7).
-constexpr int kBfLeast = 192;
+// accumulator's bias, but their rounding shows in sums of few terms: largest error, of 1024 x 1024 to 2048 x 2048 sums and 4096 x 1024,
+// squares of normals (of positive parts of normals), in tf32 / with bf16: 64 examples 1.7e-6 / 2.9e-6; 192 4.1e-6 / 4.0e-6 (3.7e-6 / 3.9e-6);
+// 256, a whole run of the accumulator, 5.1e-6 / 4.6e-6 (4.6e-6 / 4.3e-6); 512 4.5e-6 / 4.0e-6 (3.8e-6 / 3.7e-6).  Hence from kBfLeast examples
+// on (512 examples, 2048 x 2048: 27.9 -> 26.0 us; 256 examples, 1024 x 1024: 9.4 -> 8.7).
+constexpr int kBfLeast = 256;
 template <bool kAccumulate, int kN, bool kFew, bool kBf>
 __global__ void __launch_bounds__(Shape<kAccumulate, kN>::kThreads, 1)
 sqgrad_dense(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,

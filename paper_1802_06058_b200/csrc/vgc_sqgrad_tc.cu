@@ -323,6 +323,19 @@ static size_t tc_workspace_bytes(const Plan &p)
     return 256 + (p.partials ? (size_t)(p.parts ? 1 : 2) * p.blocks * kBM * slot_columns(p.tile_n) * sizeof(float) : 0);
 }
 
+// Whether the cross terms of a layer of 192-column tiles take bf16 copies: where that loses nothing.  The copies' rounding adds up to
+// 2^-18 of a product, of either sign, so that it averages out over many terms; a third fewer instructions save up to 4 x 2^-23 of the
+// accumulator's truncation for every slice it runs.  From six slices a run on the second outweighs the first in the worst case.  Largest
+// error of squared sums of normals (positive parts of normals), 3 and 5 taps, 1 to 128 tiles, bf16 over tf32 (B200): runs of one slice,
+// 768 to 2048 terms 0.96 - 1.5 (1.12 - 2.3); of four slices, 128 terms 0.94 - 1.2 (1.09 - 1.66); of six to eight, 192 to 384 terms 0.86 - 1.02
+// (0.89 - 1.16), 512 to 768 terms 0.79 - 0.88 (0.80 - 0.97), 1024 and more 0.79 - 0.88 (0.77 - 0.95).  Root mean square: 0.77 - 0.84 there.
+static bool bf16_cross_better(const Plan &p, long long terms)
+{
+    const long long range = (long long)p.units_total / p.blocks * p.unit;         // slices of a block
+    const long long run = range < p.k_slices ? range : p.k_slices;               // in one tile, the drains every kChunk apart
+    return run >= 6 && terms >= 1024;
+}
+
 static vgc_status tc_launch(KernelFn kernel, const Batch &bt, const Plan &plan, Params prm, void *ws, size_t ws_bytes, cudaStream_t st)
 {
     const int M = plan.M, N = plan.N, n_layers = plan.n_layers, tile_n = plan.tile_n;
@@ -631,6 +644,7 @@ static vgc_status conv_group(const Call &call, int n_layers, const float *const 
     auto plan_of = [&](int M, int N, int tile_n) { return make_plan(call, M, N, k_slices, n_layers, unit, tile_n); };
     // wide tiles of the per-example form: an example fits one accumulator run, or parts of examples leave as plain sums
     auto wide_fits = [&](const Plan &p) { return !ex || p_slices <= kChunk || p.parts > 0; };
+    auto bf_cross = [&](const Plan &p) { return bf16_cross_better(p, (long long)B * P); };
     Plan plan = {};
     // a square kernel that keeps the width: its input rows by TMA
     bool halo = !in_tma && err_tma && (Kw == 5 || Kw == 7) && Kh == Kw && sh == 1 && sw == 1 && 2 * pw == Kw - 1 && Wo == W &&
@@ -690,7 +704,7 @@ static vgc_status conv_group(const Call &call, int n_layers, const float *const 
         prm.ld_m = n_im2col; prm.ld_n = 1;
         if (halo) {
             const bool by4 = W % 4 == 0;
-            fn = wide_halo_kernel(Kw == 5 ? (by4 ? kHalo5x4 : kHalo5x2) : (by4 ? kHalo7x4 : kHalo7x2), ex);
+            fn = wide_halo_kernel(Kw == 5 ? (by4 ? kHalo5x4 : kHalo5x2) : (by4 ? kHalo7x4 : kHalo7x2), ex, bf_cross(plan));
             return tc_launch(fn, bt, plan, prm, ws, ws_bytes, st);
         }
         if (taps || taps_s2 || taps7) {
@@ -704,7 +718,7 @@ static vgc_status conv_group(const Call &call, int n_layers, const float *const 
                 wide = wide_fits(plan);
             }
             if (!wide) plan = plan_of(Cout, n_im2col, kBN);
-            fn = wide ? wide_taps_kernel(mode, ex) : narrow_taps_kernel(mode, ex);
+            fn = wide ? wide_taps_kernel(mode, ex, bf_cross(plan)) : narrow_taps_kernel(mode, ex);
             return tc_launch(fn, bt, plan, prm, ws, ws_bytes, st);
         }
         if (tma_bf) fn = sqgrad_tc<kMajorK, kTma, kTma, true, false, true>;

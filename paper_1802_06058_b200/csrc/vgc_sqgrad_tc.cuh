@@ -11,11 +11,12 @@
 //      and in place (hi overwrites the raw tile, lo goes beside it), so both inherit the swizzled
 //      layout the tensor core wants,
 //   3. issues three tcgen05.mma per 8-deep step -- hi*hi, hi*lo, lo*hi -- into a TMEM
-//      accumulator (the dropped lo*lo term is 2^-22 relative).  In the TMA-fed K-major form and the
-//      wide form the two cross terms use bf16 copies of hi and lo instead (kind::f16, 16 deep per
-//      instruction): a cross term is 2^-11 of the product, so 8-bit operands leave an error below
-//      2^-18 of it, of either sign -- less than the third of the instructions saves of the
-//      accumulator's truncation bias (largest error of 3x3 layers 2.9e-6 -> 2.4e-6).
+//      accumulator (the dropped lo*lo term is 2^-22 relative).  In the TMA-fed K-major form, and in the
+//      wide form where accumulator runs are long and terms many (bf16_cross_better), the two cross terms
+//      use bf16 copies of hi and lo instead (kind::f16, 16 deep per instruction): a cross term is 2^-11 of
+//      the product, so 8-bit operands leave an error below 2^-18 of it, of either sign -- in such sums less
+//      than the third of the instructions saves of the accumulator's truncation bias (largest error of 128
+//      channels 28 x 28, batch 16: 2.9e-6 -> 2.4e-6).
 // The tensor core's fp32 accumulation is not trusted over long reductions: every kChunk k slices
 // the accumulator is drained by four epilogue warps (tcgen05.ld) and added, round-to-nearest, to
 // fp32 registers while the next chunk accumulates into the second TMEM buffer.
@@ -1432,8 +1433,8 @@ sqgrad_tc(const __grid_constant__ Batch bt, const Params prm)
 typedef void (*KernelFn)(const Batch, const Params);
 // The kernel's forms are compiled in several files: tiles of 192 columns whose B tile is gathered several taps at a time, the same with
 // the input rows by TMA, and 128-column tiles gathered several taps at a time.  mode: how the B tile gets its rows.
-KernelFn wide_taps_kernel(int mode, bool per_example);
-KernelFn wide_halo_kernel(int mode, bool per_example);
+KernelFn wide_taps_kernel(int mode, bool per_example, bool bf16_cross);
+KernelFn wide_halo_kernel(int mode, bool per_example, bool bf16_cross);
 KernelFn narrow_taps_kernel(int mode, bool per_example);
 
 }  // namespace tc

@@ -4,13 +4,20 @@
 namespace vgc {
 namespace tc {
 
-KernelFn wide_halo_kernel(int mode, bool per_example)
+template <int kMode>
+static KernelFn form(bool per_example, bool bf16_cross)
+{
+    if (per_example) return sqgrad_tc<kMajorK, kTma, kMode, true, true, false, kWideN>;
+    return bf16_cross ? sqgrad_tc<kMajorK, kTma, kMode, true, false, true, kWideN> : sqgrad_tc<kMajorK, kTma, kMode, true, false, false, kWideN>;
+}
+
+KernelFn wide_halo_kernel(int mode, bool per_example, bool bf16_cross)
 {
     switch (mode) {
-        case kHalo5x4: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kHalo5x4, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kHalo5x4, true, false, true, kWideN>;
-        case kHalo5x2: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kHalo5x2, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kHalo5x2, true, false, true, kWideN>;
-        case kHalo7x4: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kHalo7x4, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kHalo7x4, true, false, true, kWideN>;
-        case kHalo7x2: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kHalo7x2, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kHalo7x2, true, false, true, kWideN>;
+        case kHalo5x4: return form<kHalo5x4>(per_example, bf16_cross);
+        case kHalo5x2: return form<kHalo5x2>(per_example, bf16_cross);
+        case kHalo7x4: return form<kHalo7x4>(per_example, bf16_cross);
+        case kHalo7x2: return form<kHalo7x2>(per_example, bf16_cross);
         default: return nullptr;
     }
 }

@@ -4,14 +4,21 @@
 namespace vgc {
 namespace tc {
 
-KernelFn wide_taps_kernel(int mode, bool per_example)
+template <int kMode>
+static KernelFn form(bool per_example, bool bf16_cross)
+{
+    if (per_example) return sqgrad_tc<kMajorK, kTma, kMode, true, true, false, kWideN>;
+    return bf16_cross ? sqgrad_tc<kMajorK, kTma, kMode, true, false, true, kWideN> : sqgrad_tc<kMajorK, kTma, kMode, true, false, false, kWideN>;
+}
+
+KernelFn wide_taps_kernel(int mode, bool per_example, bool bf16_cross)
 {
     switch (mode) {
-        case kGatherTaps4: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps4, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps4, true, false, true, kWideN>;
-        case kGatherTaps2: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps2, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps2, true, false, true, kWideN>;
-        case kGatherTaps4S2: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps4S2, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps4S2, true, false, true, kWideN>;
-        case kGatherTaps2S2: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps2S2, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps2S2, true, false, true, kWideN>;
-        case kGatherTaps7S2: return per_example ? (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps7S2, true, true, false, kWideN> : (KernelFn)sqgrad_tc<kMajorK, kTma, kGatherTaps7S2, true, false, true, kWideN>;
+        case kGatherTaps4: return form<kGatherTaps4>(per_example, bf16_cross);
+        case kGatherTaps2: return form<kGatherTaps2>(per_example, bf16_cross);
+        case kGatherTaps4S2: return form<kGatherTaps4S2>(per_example, bf16_cross);
+        case kGatherTaps2S2: return form<kGatherTaps2S2>(per_example, bf16_cross);
+        case kGatherTaps7S2: return form<kGatherTaps7S2>(per_example, bf16_cross);
         default: return nullptr;
     }
 }

@@ -62,7 +62,7 @@ def test_added_is_one_fp32_addition(B, n_in, n_out):
     assert torch.equal(T, want)
 
 
-@pytest.mark.parametrize("B", [191, 192, 193, 224, 257, 512])
+@pytest.mark.parametrize("B", [191, 192, 193, 224, 255, 256, 257, 512])
 @pytest.mark.parametrize("n_in,n_out", [(1024, 1024), (1000, 132), (4096, 1300), (132, 2052)])
 def test_cross_terms_in_bf16(B, n_in, n_out):
     """Around the number of examples from which the two cross terms take bf16 copies (each a 2^-11 of the product, the copies good

@@ -78,3 +78,23 @@ def test_infinities_stay_where_they_are_read(H, W, k):
     finite = torch.isfinite(want)
     assert bool(finite[:, 0].all()) and not bool(finite.all()) and bool(torch.isfinite(S[finite]).all())
     assert float(((S.double() - want)[finite].abs() / want[finite]).max()) < 1e-5
+
+
+@pytest.mark.parametrize("C,H,W,Cout,k,stride", [(64, 4, 8, 512, 3, 1), (64, 8, 16, 512, 3, 2), (3, 8, 16, 512, 7, 2), (32, 4, 8, 512, 5, 1),
+                                                 (16, 4, 8, 512, 7, 1), (64, 2, 16, 512, 3, 1), (64, 16, 2, 512, 3, 1)])
+def test_few_terms(C, H, W, Cout, k, stride):
+    """Sums of 32 terms, most of them one term's: all parts are tf32 there.  One slice, twelve instructions that truncate (2^-23 of the sum
+    each at most), two cross terms of 2^-11 of the product with 11 bits read of a part (2^-21 each), 2^-22 dropped, two roundings
+    (2^-24 each); bf16 copies add up to 2^-18."""
+    gen = torch.Generator("cuda").manual_seed(C + k)
+    x = torch.randn(1, C, H, W, device="cuda", generator=gen)
+    d = torch.randn(1, Cout, H // stride, W // stride, device="cuda", generator=gen)
+    d *= torch.exp(2 * torch.randn(d.shape, device="cuda", generator=gen))
+    ws = torch.zeros(max(256, vgc.vgc_sqgrad_conv_workspace_bytes(1, C, H, W, Cout, k, k, stride, stride, k // 2, k // 2)), dtype=torch.uint8, device="cuda")
+    S = torch.zeros(Cout, C * k * k, device="cuda")
+    vgc.vgc_sqgrad_conv(x, d, (k, k), (stride, stride), (k // 2, k // 2), 1.0, S, False, ws)
+    cols = torch.nn.functional.unfold(x.double(), k, padding=k // 2, stride=stride)[0]
+    want = d.double().reshape(Cout, -1).square() @ cols.square().t()
+    some = want > 0                                                          # (taps that only ever read padding)
+    assert torch.equal(S > 0, some)
+    assert float(((S.double() - want).abs() / want)[some].max()) < 12 * 2.0 ** -23 + 2 * 2.0 ** -21 + 2.0 ** -22 + 2 * 2.0 ** -24
