@@ -263,9 +263,10 @@ static Plan make_plan(const Call &call, int M, int N, int k_slices, int n_layers
         // idle: parts of an example, a block each, at most two waves of them; costs as above, a wave's start about 5 slices.
         const long long waves_now = even ? (units + blocks - 1) / blocks : ((tiles + blocks - 1) / blocks) * upt;
         long long best = waves_now * unit_min + (even ? 14 : 0);
-        for (int q = 1; q < unit_min; ++q) {
+        const long long most = 2 * kSmCount / units;
+        for (long long want = most < unit_min ? most : unit_min; want > 1; --want) {          // parts of ever more slices
+            const int q = (int)((unit_min + want - 1) / want);
             const long long n_parts = (unit_min + q - 1) / q, n = units * n_parts;
-            if (n > 2 * kSmCount) continue;
             const long long cost = ((n + kSmCount - 1) / kSmCount) * (q + 5) + 14;
             if (cost < best) { best = cost; p.parts = (int)n_parts; p.part_slices = q; }
         }
