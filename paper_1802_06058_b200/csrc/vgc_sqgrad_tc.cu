@@ -226,6 +226,12 @@ struct Plan {
 // stores), up to 1.6 times (9 examples, 544 channels 14 x 14 to 48, 3x3 stride 2: 31.5 -> 19.3 us), none slower by more than the runs of
 // one side differ; 10 is 2 % faster than 14, 4 as fast as 6 but for small networks (ResNet-50, 128 x 128, 3 examples: 378 -> 367).
 constexpr int kCombineSlices = 4;
+// The price of a combine pass where examples may be cut into parts (either candidate there ends in one).  Its blocks have a warp per
+// example and few examples to share, so that many tiles take long: one example, 512 channels 32 x 32 to 300, 3 taps (72 tiles), 30.6 us in
+// whole tiles, 57.8 in two parts, which a price of 4 chooses; 256 channels 24 x 24 to 16, 5 taps (34 tiles), 26.5, 25.9; 3 channels 24 x 24
+// to 48, 7 taps (1 tile), 27.2, 10.4.  Of 61 such layers 4 makes 38 faster and 23 up to 1.9 times slower; no drawn size of four
+// examples and more depends on it.
+constexpr int kPartsCombineSlices = 14;
 static Plan make_plan(const Call &call, int M, int N, int k_slices, int n_layers, int unit_min, int tile_n)
 {
     Plan p;
@@ -260,14 +266,14 @@ static Plan make_plan(const Call &call, int M, int N, int k_slices, int n_layers
     p.parts = p.part_slices = 0;
     if (unit_min > 1 && call.concurrent == 1) {
         // Few long examples, which the form that adds up an example's products before it squares them keeps whole, leave SMs
-        // idle: parts of an example, a block each, at most two waves of them; costs as above, a wave's start about 5 slices.
+        // idle: parts of an example, a block each, at most two waves of them; a wave's start costs about 5 slices.
         const long long waves_now = even ? (units + blocks - 1) / blocks : ((tiles + blocks - 1) / blocks) * upt;
-        long long best = waves_now * unit_min + (even ? 14 : 0);
+        long long best = waves_now * unit_min + (even ? kPartsCombineSlices : 0);
         const long long most = 2 * kSmCount / units;
         for (long long want = most < unit_min ? most : unit_min; want > 1; --want) {          // parts of ever more slices
             const int q = (int)((unit_min + want - 1) / want);
             const long long n_parts = (unit_min + q - 1) / q, n = units * n_parts;
-            const long long cost = ((n + kSmCount - 1) / kSmCount) * (q + 5) + 14;
+            const long long cost = ((n + kSmCount - 1) / kSmCount) * (q + 5) + kPartsCombineSlices;
             if (cost < best) { best = cost; p.parts = (int)n_parts; p.part_slices = q; }
         }
         if (p.parts) {

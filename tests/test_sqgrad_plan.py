@@ -4,7 +4,7 @@ import time
 
 import paper_1802_06058_b200 as vgc
 
-SMS, SLICE, ROWS, COMBINE = 148, 32, 128, 4
+SMS, SLICE, ROWS, COMBINE, PARTS_COMBINE = 148, 32, 128, 4, 14
 
 
 def _up(a, b):
@@ -23,12 +23,12 @@ def _partial_tiles(M, N, examples, slices, tile_n, layers):
         blocks = even_blocks
     slot = ROWS * (192 if tile_n > 128 else 128) * 4
     if slices > 1:
-        best = (_up(units, blocks) if even else _up(tiles, blocks) * examples) * slices + (14 if even else 0)
+        best = (_up(units, blocks) if even else _up(tiles, blocks) * examples) * slices + (PARTS_COMBINE if even else 0)
         parts = 0
         for q in range(1, slices):
             n = units * _up(slices, q)
-            if n <= 2 * SMS and _up(n, SMS) * (q + 5) + 14 < best:
-                best, parts = _up(n, SMS) * (q + 5) + 14, n
+            if n <= 2 * SMS and _up(n, SMS) * (q + 5) + PARTS_COMBINE < best:
+                best, parts = _up(n, SMS) * (q + 5) + PARTS_COMBINE, n
         if parts:
             return parts * slot
     total, upt = (units, examples) if even else (tiles, 1)
