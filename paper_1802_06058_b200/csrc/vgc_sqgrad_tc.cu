@@ -653,7 +653,8 @@ static vgc_status conv_group(const Call &call, int n_layers, const float *const 
     auto wide_fits = [&](const Plan &p) { return !ex || p_slices <= kChunk || p.parts > 0; };
     auto bf_cross = [&](const Plan &p) { return bf16_cross_better(p, (long long)B * P); };
     Plan plan = {};
-    // a square kernel that keeps the width: its input rows by TMA
+    // a square kernel that keeps the width: its input rows by TMA, however few its columns (280 layers of 1 to 8 channels, 8 x 8 to 64 x 64,
+    // against the element-wise gather: 0.65 - 0.86 of its time on average for each number of channels and taps, at worst 1.02)
     bool halo = !in_tma && err_tma && (Kw == 5 || Kw == 7) && Kh == Kw && sh == 1 && sw == 1 && 2 * pw == Kw - 1 && Wo == W &&
                 W % 2 == 0 && H * W % 4 == 0;
     if (halo) {

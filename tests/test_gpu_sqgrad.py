@@ -241,7 +241,8 @@ def test_empty_batch_clears_or_keeps_the_result():
 
 @pytest.mark.parametrize("n_layers", [1, 3, 9])
 @pytest.mark.parametrize("B,C,H,Cout,k,s,p", [(3, 96, 12, 160, 1, 1, 0), (2, 40, 12, 48, 3, 1, 1), (4, 70, 7, 130, 1, 1, 0),
-                                              (2, 96, 16, 160, 1, 2, 0), (2, 24, 9, 20, 3, 2, 1), (8, 256, 14, 64, 1, 1, 0)])
+                                              (2, 96, 16, 160, 1, 2, 0), (2, 24, 9, 20, 3, 2, 1), (8, 256, 14, 64, 1, 1, 0),
+                                              (8, 10, 12, 130, 5, 1, 2), (3, 3, 10, 40, 5, 1, 2), (2, 5, 12, 140, 7, 1, 3), (3, 4, 6, 30, 7, 1, 3)])
 def test_batch_of_layers_matches_the_oracle_layer_by_layer(n_layers, B, C, H, Cout, k, s, p):
     gen = torch.Generator(device="cuda"); gen.manual_seed(n_layers * 100 + C)
     Ho = (H + 2 * p - k) // s + 1

@@ -77,7 +77,8 @@ def test_one_position_equals_the_position_statistic():
 
 
 @pytest.mark.parametrize("n_layers", [3, 9])
-@pytest.mark.parametrize("B,C,H,Cout,k,s,p", [(3, 96, 12, 160, 1, 1, 0), (2, 24, 16, 130, 3, 1, 1), (2, 40, 7, 130, 3, 1, 1)])
+@pytest.mark.parametrize("B,C,H,Cout,k,s,p", [(3, 96, 12, 160, 1, 1, 0), (2, 24, 16, 130, 3, 1, 1), (2, 40, 7, 130, 3, 1, 1),
+                                              (3, 9, 8, 130, 5, 1, 2), (3, 3, 10, 40, 5, 1, 2), (2, 5, 12, 140, 7, 1, 3), (3, 4, 6, 30, 7, 1, 3)])
 def test_exact_batch(n_layers, B, C, H, Cout, k, s, p):
     gen = torch.Generator(device="cuda"); gen.manual_seed(n_layers + C)
     Ho = (H + 2 * p - k) // s + 1

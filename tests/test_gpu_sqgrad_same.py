@@ -1,5 +1,6 @@
 """Convolutions of 3, 5 and 7 taps that keep the width (5 and 7: input rows by TMA): widths of every remainder, planes of less than a
-tile's rows, channels around the edges of tiles, both statistics.
+tile's rows, channels around the edges of tiles, both statistics; sums of few terms, and of as many as make the cross terms' operands
+bf16, there also at stride 2.
 
 Checked against PyTorch in fp64.  Bound 1e-5 relative to each entry of the squared sums (all terms positive, three products per
 term drop less than 2^-18 of it, an accumulator run loses less than 2e-6) and, for the per-example statistic, of the same sums
@@ -98,3 +99,19 @@ def test_few_terms(C, H, W, Cout, k, stride):
     some = want > 0                                                          # (taps that only ever read padding)
     assert torch.equal(S > 0, some)
     assert float(((S.double() - want).abs() / want)[some].max()) < 12 * 2.0 ** -23 + 2 * 2.0 ** -21 + 2.0 ** -22 + 2 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("C,H,Cout,k,stride,B", [(320, 8, 1024, 3, 1, 15), (320, 8, 1024, 3, 1, 16), (320, 6, 1000, 3, 1, 28), (320, 6, 1000, 3, 1, 29),
+                                                 (320, 16, 1024, 3, 2, 15), (320, 16, 1024, 3, 2, 16), (320, 12, 1024, 3, 2, 29), (64, 16, 1024, 7, 2, 15),
+                                                 (64, 16, 1024, 7, 2, 16), (64, 8, 1000, 5, 1, 15), (65, 8, 1000, 5, 1, 16), (64, 10, 1024, 5, 1, 10),
+                                                 (64, 10, 1024, 5, 1, 11), (48, 8, 1024, 7, 1, 15), (49, 8, 1024, 7, 1, 16), (48, 6, 900, 7, 1, 29)])
+def test_many_terms(C, H, Cout, k, stride, B):
+    """About 1024 terms in long accumulator runs, from where on the cross terms take bf16 copies, in every form of wide tiles."""
+    x = torch.randn(B, C, H, H, device="cuda", generator=torch.Generator("cuda").manual_seed(B + C))
+    d = torch.randn(B, Cout, H // stride, H // stride, device="cuda", generator=torch.Generator("cuda").manual_seed(k)) * 1e-3
+    ws = torch.zeros(vgc.vgc_sqgrad_conv_workspace_bytes(B, C, H, H, Cout, k, k, stride, stride, k // 2, k // 2), dtype=torch.uint8, device="cuda")
+    S = torch.full((Cout, C * k * k), -1.0, device="cuda")
+    vgc.vgc_sqgrad_conv(x, d, (k, k), (stride, stride), (k // 2, k // 2), 0.5, S, False, ws)
+    cols = torch.nn.functional.unfold(x.double(), k, padding=k // 2, stride=stride).square()
+    want = torch.einsum("bop,bip->oi", d.double().reshape(B, Cout, -1).square(), cols) * 0.5
+    assert int(ws[:4].view(torch.int32)) == 0 and float(((S.double() - want).abs() / want).max()) < 1e-5
