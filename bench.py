@@ -225,9 +225,9 @@ class HotPath:
             for li, spec in enumerate(self.layers):
                 M, N, K = spec.gemm_mnk(B)
                 self.flops_useful += 2 * M * N * K
-                # fp32 accuracy costs three TF32 products per algorithmic one; the TMA-fed form (1x1 convs) and tiles of 192
-                # columns (the 3x3 and 7x7 convs) take their two cross terms in bf16, at half the TF32 cost each
-                bf16_cross = spec.kind == "conv" and not exact_conv
+                # fp32 accuracy costs three TF32 products per algorithmic one; the TMA-fed form (1x1 convs) and, from 1024 terms
+                # on, tiles of 192 columns (the 3x3 and 7x7 convs) take their two cross terms in bf16, at half the TF32 cost each
+                bf16_cross = spec.kind == "conv" and not exact_conv and (spec.k == 1 or K >= 1024)
                 self.flops_issued += 2 * M * N * K * (2.0 if bf16_cross else 3.0)
             for g in self.groups:
                 spec = self.layers[g[0]]
@@ -760,7 +760,8 @@ def profile_kernels():
         ("1x1 on 7x7 planes: repacked channel-major (layer-4 expansion)", 2, 8, 512, 7, 2048, 1, 1, 0),
         ("1x1 stride 2: subsampled planes (layer-3 downsample)", 1, 8, 512, 28, 1024, 1, 2, 0),
         ("3x3 on 7x7 planes: padded planes + three taps (layer-4)", 1, 8, 512, 7, 512, 3, 1, 1),
-        ("5x5: element-wise gather (not a ResNet shape)", 1, 4, 64, 28, 128, 5, 1, 2),
+        ("5x5: input rows by TMA (not a ResNet shape)", 1, 8, 64, 28, 128, 5, 1, 2),
+        ("5x5 on odd planes: element-wise gather, errors too (not a ResNet shape)", 1, 8, 64, 27, 128, 5, 1, 2),
     ]
     for name, nl, B, C, H, Cout, k, st, pd in conv_cases:
         Ho = (H + 2 * pd - k) // st + 1
@@ -774,14 +775,16 @@ def profile_kernels():
         print(json.dumps({"case": "sqgrad_conv: " + name, "layers": nl, "B": B, "M": Cout, "N": C * k * k, "K": B * Ho * Ho,
                           "gflop": nl * 2 * Cout * C * k * k * B * Ho * Ho / 1e9}))
     # per-example statistic (kExact), dense layers (tensor cores and CUDA cores)
-    B, C, H, Cout = 8, 256, 14, 256
-    x = torch.randn(B, C, H, H, device=dev); d = torch.randn(B, Cout, H, H, device=dev) * 1e-4
-    S = torch.empty(Cout * C * 9, device=dev)
-    ws = torch.zeros(vgc.vgc_sqgrad_conv_exact_workspace_bytes(B, C, H, H, Cout, 3, 3, 1, 1, 1, 1), dtype=torch.uint8, device=dev)
-    for _ in range(2):
-        vgc.vgc_sqgrad_conv_exact(x, d, (3, 3), (1, 1), (1, 1), 1.0, S, ws=ws)
-    print(json.dumps({"case": "sqgrad_conv_exact: 3x3 layer-3 shape, per-example statistic", "B": B}))
-    for B, n_in, n_out, what in ((32, 2048, 1000, "tensor cores (fc of ResNet-50)"), (8, 1000, 333, "CUDA cores (batch < 32)")):
+    for B, C, H, Cout, k, what in ((8, 256, 14, 256, 3, "3x3 layer-3 shape"), (6, 288, 56, 96, 1, "1x1, few long examples: cut into parts")):
+        x = torch.randn(B, C, H, H, device=dev); d = torch.randn(B, Cout, H, H, device=dev) * 1e-4
+        S = torch.empty(Cout * C * k * k, device=dev)
+        ws = torch.zeros(vgc.vgc_sqgrad_conv_exact_workspace_bytes(B, C, H, H, Cout, k, k, 1, 1, k // 2, k // 2), dtype=torch.uint8, device=dev)
+        for _ in range(2):
+            vgc.vgc_sqgrad_conv_exact(x, d, (k, k), (1, 1), (k // 2, k // 2), 1.0, S, ws=ws)
+        torch.cuda.synchronize()
+        print(json.dumps({"case": "sqgrad_conv_exact: " + what + ", per-example statistic", "B": B}))
+    for B, n_in, n_out, what in ((64, 4096, 4096, "tensor cores, tf32 cross terms"), (512, 2048, 2048, "tensor cores, bf16 cross terms"),
+                                 (32, 512, 1000, "CUDA cores (up to 2^25 multiply-adds)"), (1024, 2048, 1000, "more than 512 examples")):
         x = torch.randn(B, n_in, device=dev); d = torch.randn(B, n_out, device=dev)
         S = torch.empty(n_out * n_in, device=dev)
         ws = torch.zeros(vgc.vgc_sqgrad_linear_workspace_bytes(B, n_in, n_out), dtype=torch.uint8, device=dev)

@@ -82,13 +82,14 @@ __device__ __forceinline__ float value_of(uint32_t word, const int32_t *gexp, co
 // lies in one stretch of u: DRAM pages are opened once for the words of all of them.  Shorter messages make groups of their
 // own, so that a piece is at least about half full whatever the lengths (one group for all took 4.5 ms for 64
 // messages into 138 M elements, one of 6.9 M words and the others empty; now 127 us).
-// Warps: one block's per SM where there is less than one word per 40 elements of a large buffer, but words enough that what they
-// touch does not stay in L2 (16 M elements, 0.35 M words: 11.7 us with one block per SM, 7.3 with two; 138 M, 0.22 M words: 6.4, 4.6; 68 M,
-// 1.5 M: 51.9, 50.0; 100 M, 1.9 M: 69.0, 72.2; 138 M, 0.9 M: 40.7, 43.1), two and a half blocks' otherwise -- DRAM is what
-// bounds it (a touched 64 bytes is read, and read again and written when its half-filled line leaves L2), more in flight only
-// widens the stretch.  138 M elements, us, with 1 / 2 / 2.5 / 3 / 4 blocks per SM: 64 messages, 2.7 M words 95 / 103 / 103 / 103 / 102,
-// 8.9 M words 230 / 173 / 172 / 223 / 271; 4 messages, 11 M words 272 / 189 / 175 / 170 / 200; 32 M elements, 7 messages, 2 M words
-// 55 / 41 / 39 / 40 / 40.
+// Warps: two and a half blocks' per SM; one block's where three things hold: a large buffer (kFlatLarge), less than one word per kFlatThin
+// elements, and words enough that what they touch does not stay in L2 (kFlatMany).  us, one block per SM / two: 16 M elements, 0.35 M
+// words 11.7 / 7.3; 68 M, 1.5 M 51.9 / 50.0; 100 M, 1.9 M 69.0 / 72.2; 138 M, 0.22 M 6.4 / 4.6; 138 M, 0.9 M 40.7 / 43.1.  (The line between 68 M
+// and 138 M elements is drawn at 100.7 M: just below it one block would be 4 % faster.)  DRAM is what bounds it, with accesses of 32 to
+// 64 bytes in random order -- 138 M elements, 2.7 M words: 76 bytes read and up to 34 written per 64 touched, 92 us for what a copy moves
+// in 40 --, and more in flight only widens the stretch.  138 M elements, us, with 1 / 2 / 2.5 / 3 / 4 blocks per SM: 64 messages, 2.7 M words
+// 95 / 103 / 103 / 103 / 102, 8.9 M words 230 / 173 / 172 / 223 / 271; 4 messages, 11 M words 272 / 189 / 175 / 170 / 200; 32 M elements, 7 messages,
+// 2 M words 55 / 41 / 39 / 40 / 40.
 constexpr int kFlatThreads = 256, kPiece = 32, kFlatFewest = kSmCount, kFlatMost = kSmCount * 5 / 2;
 constexpr uint32_t kFlatThin = 40;
 constexpr uint32_t kFlatMany = 1u << 19;             // words
