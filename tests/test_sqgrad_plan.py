@@ -62,6 +62,7 @@ def test_parts_of_examples():
 
 def test_long_examples_are_planned_as_fast_as_short_ones():
     """8.4 million slices an example: trying every part length took 0.1 s a query."""
+    vgc.load_library()
     start = time.perf_counter()
     for _ in range(50):
         assert vgc.vgc_sqgrad_conv_exact_workspace_bytes(1, 1, 16384, 16384, 16, 3, 3, 1, 1, 1, 1) > 256
